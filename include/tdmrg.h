@@ -328,7 +328,11 @@ const char* tdmrg_last_global_error(void);
  * Kernel-level entry points (device pointers, complex FP64 interleaved re/im, row-major).
  * They run one hot-path operation in isolation, for parity tests and measurement.
  * Arguments are sizes and device pointers owned by the caller; nothing is allocated
- * except where noted; each entry states whether it synchronises `stream`.
+ * except where noted; each entry states whether it synchronises `stream`.  Complex FP64
+ * contractions take a workspace (the digits of their operands) from a stream-ordered pool of
+ * the library for the length of the call; the pool keeps at most 512 MB between calls and gives
+ * it back when the last model is destroyed.  TDMRG_ERR_TIMEOUT if a bounded pipeline wait of a
+ * contraction gave up.
  * ---------------------------------------------------------------------------------- */
 
 /* Effective Hamiltonian of one site (the site step of Eq. S1):

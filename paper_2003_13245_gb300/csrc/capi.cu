@@ -1,5 +1,6 @@
 // extern "C" boundary of libtdmrg: argument checks, exception-to-status translation and
 // the kernel-level entry points.  Every computation runs in the CUDA kernels of the engine.
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -45,6 +46,7 @@ struct tdmrg_batch {
 };
 
 static thread_local std::string g_err;
+static std::atomic<int> g_models{0};     // live model handles
 
 namespace tdmrg {
 void set_global_error(const char* msg) { g_err = msg; }
@@ -108,6 +110,29 @@ tdmrg::MatRef mat(const void* p, long long rs, long long cs, long long sb = 0, l
                   int conj = 0) {
   return tdmrg::MatRef{(const cplx*)p, rs, cs, sb, sr, conj};
 }
+
+// digit workspace of one entry point's FP64 contractions, given back when it returns
+struct ZgHold {
+  tdmrg::ZgWork w;
+  cudaStream_t s;
+  explicit ZgHold(cudaStream_t st) : s(st) {
+    w.pooled = true;
+    CK(tdmrg::zg_pool_alloc(reinterpret_cast<void**>(&w.status), sizeof(int), s));
+    CK(cudaMemsetAsync(w.status, 0, sizeof(int), s));
+  }
+  ~ZgHold() {
+    tdmrg::zg_free(w, s);
+    cudaFreeAsync(w.status, s);
+  }
+  ZgHold(const ZgHold&) = delete;
+  // waits for the stream; throws when a bounded pipeline wait gave up
+  void finish() {
+    int hs = 0;
+    CK(cudaMemcpyAsync(&hs, w.status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (hs) throw Failure{TDMRG_ERR_TIMEOUT, "tensor-core pipeline wait timed out"};
+  }
+};
 
 // device temporaries of one entry point, freed when it returns
 struct DevBufs {
@@ -214,6 +239,7 @@ int tdmrg_model_create(int N, int modes, const double* omega, const double* g, d
     delete h;
     return rc;
   }
+  ++g_models;
   *out = h;
   return TDMRG_OK;
 }
@@ -454,6 +480,8 @@ int tdmrg_model_destroy(tdmrg_model* h) {
   if (!h) return TDMRG_OK;
   if (h->eng) cudaStreamSynchronize(h->eng->stream());
   delete h;
+  // the last model gives the pool's memory back to the device
+  if (--g_models == 0) tdmrg::zg_pool_trim();
   return TDMRG_OK;
 }
 
@@ -756,9 +784,11 @@ int tdmrg_kernel_heff(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
     TempMpo W(Dl, Dr, d, W_host);
     cudaStream_t s = (cudaStream_t)stream;
     if (precision == TDMRG_PREC_C128) {
-      tdmrg::Ctx c{s, (tdmrg::cplx*)X, (tdmrg::cplx*)Y};
+      ZgHold zg(s);
+      tdmrg::Ctx c{s, (tdmrg::cplx*)X, (tdmrg::cplx*)Y, &zg.w};
       tdmrg::heff_f64(c, W.m.s[0], Ml, Mr, d * d, d, (const tdmrg::cplx*)L,
                       (const tdmrg::cplx*)R, (const tdmrg::cplx*)A, (tdmrg::cplx*)out, nullptr);
+      zg.finish();
     } else {
       int* st = nullptr;
       CK(cudaMalloc(&st, sizeof(int)));
@@ -808,6 +838,7 @@ int tdmrg_kernel_heff_timed(int Ml, int Mr, int d, int Dl, int Dr, const double*
     CK(cudaMemsetAsync(st, 0, sizeof(int), s));
     const int Dm = Dl > Dr ? Dl : Dr;
     tdmrg::TcBufs b{};
+    ZgHold zg(s);
     cplx *X = nullptr, *Y = nullptr;
     if (precision == TDMRG_PREC_C64_3XTF32) {
       b.envA = (float*)get(sizeof(float) * 4 * (size_t)Dl * Ml * pad4(Ml));
@@ -827,7 +858,7 @@ int tdmrg_kernel_heff_timed(int Ml, int Mr, int d, int Dl, int Dr, const double*
       if (precision == TDMRG_PREC_C64_3XTF32)
         tdmrg::heff_tc_apply(s, b, W.m.s[0], Ml, Mr, D, d, (const cplx*)A, (cplx*)out);
       else
-        tdmrg::heff_f64(tdmrg::Ctx{s, X, Y}, W.m.s[0], Ml, Mr, D, d, (const cplx*)L,
+        tdmrg::heff_f64(tdmrg::Ctx{s, X, Y, &zg.w}, W.m.s[0], Ml, Mr, D, d, (const cplx*)L,
                         (const cplx*)R, (const cplx*)A, (cplx*)out, nullptr);
     };
     once();   // warm-up
@@ -846,6 +877,7 @@ int tdmrg_kernel_heff_timed(int Ml, int Mr, int d, int Dl, int Dr, const double*
     CK(cudaMemcpyAsync(&hs, st, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (hs) throw Failure{TDMRG_ERR_TIMEOUT, "tensor-core pipeline wait timed out"};
+    zg.finish();
     *ms_per_matvec = ms / reps;
   });
 }
@@ -984,7 +1016,8 @@ int tdmrg_kernel_heff_vjp(int Ml, int Mr, int d, int Dl, int Dr, const double* W
     for (int w = 0; w < Dr; ++w)
       CK(tdmrg::ztranspose(Mr, Mr, (const cplx*)R + (size_t)w * Mr * Mr, Rh + (size_t)w * Mr * Mr,
                            1, s));
-    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y};
+    ZgHold zg(s);
+    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y, &zg.w};
     // Abar = H_eff(L^dagger, W^T conj, R^dagger) ybar
     tdmrg::heff_f64(c, Wc.m.s[0], Ml, Mr, D, d, Lh, Rh, (const cplx*)ybar, (cplx*)Abar, nullptr);
     // Lbar = conj(env_right(R, bra = ybar, W, ket = A)); Rbar = conj(env_left(L, ybar, W, A))
@@ -994,7 +1027,7 @@ int tdmrg_kernel_heff_vjp(int Ml, int Mr, int d, int Dl, int Dr, const double* W
     tdmrg::env_left_f64(c, W.m.s[0], Ml, Mr, Ml, Mr, D, d, (const cplx*)L, (const cplx*)ybar,
                         (const cplx*)A, (cplx*)Rbar);
     CK(tdmrg::zconj((long long)Dr * Mr * Mr, (cplx*)Rbar, s));
-    CK(cudaStreamSynchronize(s));
+    zg.finish();
   });
 }
 
@@ -1041,10 +1074,11 @@ int tdmrg_kernel_env_left(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int
     return fail(nullptr, TDMRG_ERR_ARG, "env_left: bad arguments");
   return guarded(nullptr, [&] {
     TempMpo W(Dl, Dr, d, W_host);
-    tdmrg::Ctx c{(cudaStream_t)stream, (tdmrg::cplx*)X, (tdmrg::cplx*)Y};
+    ZgHold zg((cudaStream_t)stream);
+    tdmrg::Ctx c{(cudaStream_t)stream, (tdmrg::cplx*)X, (tdmrg::cplx*)Y, &zg.w};
     tdmrg::env_left_f64(c, W.m.s[0], Ml1, Mr1, Ml2, Mr2, d * d, d, (const tdmrg::cplx*)L,
                         (const tdmrg::cplx*)bra, (const tdmrg::cplx*)ket, (tdmrg::cplx*)Lout);
-    CK(cudaStreamSynchronize((cudaStream_t)stream));
+    zg.finish();
   });
 }
 
@@ -1250,7 +1284,7 @@ int site_exp_vjp_impl(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
     cplx* Er = buf.get(nr);
     cplx* t = nparam > 0 ? buf.get(n) : nullptr;
     cplx* part = nparam > 0 ? buf.get(257) : nullptr;
-    tdmrg::Ctx c{s, X, Y};
+    tdmrg::Ctx c{s, X, Y, eng.zg()};
     const cplx* Ld = (const cplx*)L;
     const cplx* Rd = (const cplx*)R;
     auto heff = [&](const cplx* in, cplx* out, const int* skip) {
@@ -1337,7 +1371,7 @@ int tdmrg_kernel_bond_exp_vjp(int M, int Dw, const void* L, const void* R, const
     CK(cudaMalloc(&a, sizeof(cplx) * (size_t)mm));
     CK(cudaMalloc(&b, sizeof(cplx) * (size_t)mm));
     CK(cudaMalloc(&T, sizeof(cplx) * (size_t)Dw * mm));
-    tdmrg::Ctx c{s, X, nullptr};
+    tdmrg::Ctx c{s, X, nullptr, eng.zg()};
     const cplx* Ld = (const cplx*)L;
     const cplx* Rd = (const cplx*)R;
     auto kmv = [&](const cplx* in, cplx* out, const int* skip) {
@@ -1358,14 +1392,14 @@ int tdmrg_kernel_bond_exp_vjp(int M, int Dw, const void* L, const void* R, const
       const cplx k = {wn[q] * tau_re, -wn[q] * tau_im};
       // T_w = conj(R_w) b^H;  Lbar_w += k a T_w
       CK(tdmrg::zgemm(M, M, M, Dw, 1, one, MatRef{Rd, M, 1, mm, 0, 1}, MatRef{b, 1, M, 0, 0, 1},
-                      zero, T, M, mm, nullptr, s));
+                      zero, T, M, mm, nullptr, s, eng.zg()));
       CK(tdmrg::zgemm(M, M, M, Dw, 1, k, MatRef{a, M, 1, 0, 0, 0}, MatRef{T, M, 1, mm, 0, 0}, one,
-                      (cplx*)Lbar, M, mm, nullptr, s));
+                      (cplx*)Lbar, M, mm, nullptr, s, eng.zg()));
       // T_w = conj(L_w) conj(b);  Rbar_w += k a^T T_w
       CK(tdmrg::zgemm(M, M, M, Dw, 1, one, MatRef{Ld, M, 1, mm, 0, 1}, MatRef{b, M, 1, 0, 0, 1},
-                      zero, T, M, mm, nullptr, s));
+                      zero, T, M, mm, nullptr, s, eng.zg()));
       CK(tdmrg::zgemm(M, M, M, Dw, 1, k, MatRef{a, 1, M, 0, 0, 0}, MatRef{T, M, 1, mm, 0, 0}, one,
-                      (cplx*)Rbar, M, mm, nullptr, s));
+                      (cplx*)Rbar, M, mm, nullptr, s, eng.zg()));
     }
     eng.sync_and_check();
   });
@@ -1379,6 +1413,7 @@ int tdmrg_kernel_qr_vjp(int m, int n, const void* Q, const void* R, const void* 
     using tdmrg::cplx;
     using tdmrg::MatRef;
     cudaStream_t s = (cudaStream_t)stream;
+    ZgHold zg(s);
     cplx *Ru = nullptr, *M = nullptr, *S = nullptr, *rhs = nullptr;
     struct Free {
       cplx** p[4];
@@ -1397,16 +1432,16 @@ int tdmrg_kernel_qr_vjp(int m, int n, const void* Q, const void* R, const void* 
     CK(tdmrg::triu_inplace(n, Ru, s));
     // M = R Rbar^H - Qbar^H Q
     CK(tdmrg::zgemm(n, n, n, 1, 1, one, MatRef{(const cplx*)R, n, 1, 0, 0, 0},
-                    MatRef{Ru, 1, n, 0, 0, 1}, zero, M, n, 0, nullptr, s));
+                    MatRef{Ru, 1, n, 0, 0, 1}, zero, M, n, 0, nullptr, s, &zg.w));
     CK(tdmrg::zgemm(n, n, m, 1, 1, mone, MatRef{(const cplx*)Qbar, 1, n, 0, 0, 1},
-                    MatRef{(const cplx*)Q, n, 1, 0, 0, 0}, one, M, n, 0, nullptr, s));
+                    MatRef{(const cplx*)Q, n, 1, 0, 0, 0}, one, M, n, 0, nullptr, s, &zg.w));
     CK(tdmrg::herm_lower(n, M, S, s));
     // rhs = Qbar + Q S;  Ybar R^H = rhs
     CK(cudaMemcpyAsync(rhs, Qbar, sizeof(cplx) * (size_t)m * n, cudaMemcpyDeviceToDevice, s));
     CK(tdmrg::zgemm(m, n, n, 1, 1, one, MatRef{(const cplx*)Q, n, 1, 0, 0, 0},
-                    MatRef{S, n, 1, 0, 0, 0}, one, rhs, n, 0, nullptr, s));
+                    MatRef{S, n, 1, 0, 0, 0}, one, rhs, n, 0, nullptr, s, &zg.w));
     CK(tdmrg::solve_rh(m, n, (const cplx*)R, rhs, (cplx*)Ybar, s));
-    CK(cudaStreamSynchronize(s));
+    zg.finish();
   });
 }
 
@@ -1442,7 +1477,8 @@ int tdmrg_kernel_env_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr, const 
                            0, s));
     CK(cudaMemcpyAsync(Gc, G, sizeof(cplx) * (size_t)ng, cudaMemcpyDeviceToDevice, s));
     CK(tdmrg::zconj(ng, Gc, s));
-    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y};
+    ZgHold zg(s);
+    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y, &zg.w};
     const cplx* Ed = (const cplx*)E;
     const cplx* Bd = (const cplx*)bra;
     const cplx* Kd = (const cplx*)ket;
@@ -1474,7 +1510,7 @@ int tdmrg_kernel_env_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr, const 
         tdmrg::env_right_f64(c, dWp.m.s[0], Ml, Mr, Ml, Mr, D, d, Ed, Bd, Kd, tmp);
       theta_bar[p] = dot_re((const cplx*)G, tmp, ng, part, s);
     }
-    CK(cudaStreamSynchronize(s));
+    zg.finish();
   });
 }
 
@@ -1499,7 +1535,8 @@ int tdmrg_kernel_expansion_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr,
     cplx* Z = buf.get((long long)Dmax * per);
     cplx* tmp = buf.get((long long)Dmax * per);
     cplx* part = buf.get(257);
-    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y};
+    ZgHold zg(s);
+    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y, &zg.w};
     const cplx one = {1.0, 0.0}, zero = {0.0, 0.0};
     const cplx* Ed = (const cplx*)E;
     const cplx* Ad = (const cplx*)A;
@@ -1515,11 +1552,11 @@ int tdmrg_kernel_expansion_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr,
       // Abar[y][(u,t,c)] = sum_{w,x} conj(L[w,x,y]) Z[w][x][(u,t,c)]
       CK(tdmrg::zgemm(Ml, D * Mr, Ml, 1, Dl, one, mat(Ed, 1, Ml, 0, (long long)Ml * Ml, 1),
                       mat(Z, (long long)D * Mr, 1, 0, per), zero, (cplx*)Abar, (long long)D * Mr,
-                      0, nullptr, s));
+                      0, nullptr, s, &zg.w));
       // Lbar[w][x][y] = sum_k Z[w][x][k] conj(A[y][k])
       CK(tdmrg::zgemm(Ml, Ml, D * Mr, Dl, 1, one, mat(Z, (long long)D * Mr, 1, per),
                       mat(Ad, 1, (long long)D * Mr, 0, 0, 1), zero, (cplx*)Ebar, Ml,
-                      (long long)Ml * Ml, nullptr, s));
+                      (long long)Ml * Ml, nullptr, s, &zg.w));
     } else {
       // Pb[(w,y)][(s,t,b)] = conj(Xbar[(s,t,b)][(w,y)])   (X = P^H)
       CK(tdmrg::ztranspose(D * Mr, Dl * Ml, (const cplx*)Xbar, Pb, 1, s));
@@ -1528,10 +1565,10 @@ int tdmrg_kernel_expansion_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr,
       // Abar[(y,u,t)][c] = sum_{v,b} Z[v][(y,u,t)][b] conj(R[v][b][c])
       CK(tdmrg::zgemm(Ml * D, Mr, Mr, 1, Dr, one, mat(Z, Mr, 1, 0, per),
                       mat(Ed, Mr, 1, 0, (long long)Mr * Mr, 1), zero, (cplx*)Abar, Mr, 0,
-                      nullptr, s));
+                      nullptr, s, &zg.w));
       // Rbar[v][b][c] = sum_k Z[v][k][b] conj(A[k][c])
       CK(tdmrg::zgemm(Mr, Mr, Ml * D, Dr, 1, one, mat(Z, 1, Mr, per), mat(Ad, Mr, 1, 0, 0, 1),
-                      zero, (cplx*)Ebar, Mr, (long long)Mr * Mr, nullptr, s));
+                      zero, (cplx*)Ebar, Mr, (long long)Mr * Mr, nullptr, s, &zg.w));
     }
     // theta_bar[p] = Re <Pb, partial(E, dW_p, A)>  (the candidates are linear in W)
     for (int p = 0; p < nparam; ++p) {
@@ -1547,7 +1584,7 @@ int tdmrg_kernel_expansion_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr,
         tdmrg::right_partial_f64(c, dWp.m.s[0], Ml, D, d, Mr, Mr, Ed, Ad, tmp, nullptr);
       theta_bar[p] = dot_re(Pb, tmp, (long long)np * per, part, s);
     }
-    CK(cudaStreamSynchronize(s));
+    zg.finish();
   });
 }
 
@@ -1563,6 +1600,7 @@ int tdmrg_kernel_qr_vjp_completed(int m, int n, const int* accepted, const void*
     return fail(nullptr, TDMRG_ERR_ARG, "qr_vjp_completed: completed columns need Xsel, Xselbar");
   return guarded(nullptr, [&] {
     cudaStream_t s = (cudaStream_t)stream;
+    ZgHold zg(s);
     const cplx one = {1.0, 0.0}, mone = {-1.0, 0.0}, zero = {0.0, 0.0};
     const size_t cb = sizeof(cplx);
     const cudaMemcpyKind dd = cudaMemcpyDeviceToDevice;
@@ -1598,35 +1636,35 @@ int tdmrg_kernel_qr_vjp_completed(int m, int n, const int* accepted, const void*
       CK(cudaMemcpyAsync(RbS + (size_t)i * n, Rb + (size_t)S[i] * n, cb * n, dd, s));
     }
     // the factorised matrix Y = Q_S R_S, and Z = [Y_S | Xsel]
-    CK(tdmrg::zgemm(m, n, ns, 1, 1, one, mat(Qp, n, 1), mat(RS, n, 1), zero, Yr, n, 0, nullptr, s));
+    CK(tdmrg::zgemm(m, n, ns, 1, 1, one, mat(Qp, n, 1), mat(RS, n, 1), zero, Yr, n, 0, nullptr, s, &zg.w));
     for (int i = 0; i < ns; ++i) col(Z, n, i, Yr, n, S[i]);
     for (int i = 0; i < nk; ++i) col(Z, n, ns + i, Xsel, nk, i);
     // R_Z = triu(Qp^H Z) with its accepted block taken from R
     CK(tdmrg::zgemm(n, n, m, 1, 1, one, mat(Qp, 1, n, 0, 0, 1), mat(Z, n, 1), zero, Rp, n, 0,
-                    nullptr, s));
+                    nullptr, s, &zg.w));
     CK(tdmrg::triu_inplace(n, Rp, s));
     for (int j = 0; j < ns; ++j)
       CK(cudaMemcpy2DAsync(Rp + j, cb * n, RS + S[j], cb * n, cb, (size_t)ns, dd, s));
     // Qbar_S += Y Rbar_S^H  (the R_S = Q_S^H Y term)
     if (ns > 0)
       CK(tdmrg::zgemm(m, ns, n, 1, 1, one, mat(Yr, n, 1), mat(RbS, 1, n, 0, 0, 1), one, Qbp, n, 0,
-                      nullptr, s));
+                      nullptr, s, &zg.w));
     // Zbar = full-rank QR VJP of Z = Qp R_Z with Rbar_Z = 0:
     //   M = -Qbp^H Qp, S = Hermitian fold of M, Zbar R_Z^H = Qbp + Qp S
     CK(tdmrg::zgemm(n, n, m, 1, 1, mone, mat(Qbp, 1, n, 0, 0, 1), mat(Qp, n, 1), zero, Mt, n, 0,
-                    nullptr, s));
+                    nullptr, s, &zg.w));
     CK(tdmrg::herm_lower(n, Mt, Sh, s));
     CK(cudaMemcpyAsync(rhs, Qbp, cb * (size_t)mn, dd, s));
-    CK(tdmrg::zgemm(m, n, n, 1, 1, one, mat(Qp, n, 1), mat(Sh, n, 1), one, rhs, n, 0, nullptr, s));
+    CK(tdmrg::zgemm(m, n, n, 1, 1, one, mat(Qp, n, 1), mat(Sh, n, 1), one, rhs, n, 0, nullptr, s, &zg.w));
     CK(tdmrg::solve_rh(m, n, Rp, rhs, Zb, s));
     // Ybar = Q_S Rbar_S + Zbar_S scattered to the positions S;  Xselbar = Zbar_K
     CK(tdmrg::zgemm(m, n, ns, 1, 1, one, mat(Qp, n, 1), mat(RbS, n, 1), zero, (cplx*)Ybar, n, 0,
-                    nullptr, s));
+                    nullptr, s, &zg.w));
     CK(cudaMemsetAsync(T, 0, cb * (size_t)mn, s));
     for (int i = 0; i < ns; ++i) col(T, n, S[i], Zb, n, i);
     CK(tdmrg::zaxpy(mn, one, T, (cplx*)Ybar, s));
     for (int i = 0; i < nk; ++i) col((cplx*)Xselbar, nk, i, Zb, n, ns + i);
-    CK(cudaStreamSynchronize(s));
+    zg.finish();
   });
 }
 
@@ -1648,7 +1686,7 @@ int tdmrg_kernel_krylov_dense(int n, const void* H, const void* v, void* out, do
                                 [&](const tdmrg::cplx* in, tdmrg::cplx* o, const int* skip) {
                                   tdmrg::MatRef a{Hd, n, 1, 0, 0, 0}, b{in, 1, 1, 0, 0, 0};
                                   CK(tdmrg::zgemm(n, 1, n, 1, 1, one, a, b, zero, o, 1, 0, skip,
-                                                  (cudaStream_t)stream));
+                                                  (cudaStream_t)stream, eng.zg()));
                                 });
     eng.sync_and_check();
     if (kused) *kused = used;

@@ -61,19 +61,19 @@ void heff_f64(const Ctx& c, const DevMpoSite& W, int Ml, int Mr, int D, int d, c
   const long long per = (long long)Ml * D * Mr;
   // X[(w,a)][(s,c)] = sum_y L[w,a,y] in[y,(s,c)]
   CK(zgemm(W.Dl * Ml, D * Mr, Ml, 1, 1, ONE, mref(Lenv, Ml, 1), mref(in, (long long)D * Mr, 1),
-           ZERO, c.X, (long long)D * Mr, 0, skip, c.st));
+           ZERO, c.X, (long long)D * Mr, 0, skip, c.st, c.ws));
   // Y[v][a][s][t][c] = sum_{w,u} W[w,v,s,u] X[w][a][u][t][c]
   CK(mpo_mix(W.lr, Ml, d, Mr, c.X, per, c.Y, per, skip, c.st));
   // out[(a,s)][b] = sum_{v,c} Y[v][(a,s)][c] R[v][b][c]
   CK(zgemm(Ml * D, Mr, Mr, 1, W.Dr, ONE, mref(c.Y, Mr, 1, 0, per),
-           mref(Renv, 1, Mr, 0, (long long)Mr * Mr), ZERO, out, Mr, 0, skip, c.st));
+           mref(Renv, 1, Mr, 0, (long long)Mr * Mr), ZERO, out, Mr, 0, skip, c.st, c.ws));
 }
 
 void left_partial_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Ml2, int D, int d, int Mr2,
                       const cplx* Lenv, const cplx* ket, cplx* Y, const int* skip) {
   const long long per = (long long)Ml1 * D * Mr2;
   CK(zgemm(W.Dl * Ml1, D * Mr2, Ml2, 1, 1, ONE, mref(Lenv, Ml2, 1),
-           mref(ket, (long long)D * Mr2, 1), ZERO, c.X, (long long)D * Mr2, 0, skip, c.st));
+           mref(ket, (long long)D * Mr2, 1), ZERO, c.X, (long long)D * Mr2, 0, skip, c.st, c.ws));
   CK(mpo_mix(W.lr, Ml1, d, Mr2, c.X, per, Y, per, skip, c.st));
 }
 
@@ -82,7 +82,7 @@ void right_partial_f64(const Ctx& c, const DevMpoSite& W, int Ml2, int D, int d,
   const long long per = (long long)Ml2 * D * Mr1;
   // X[v][(y,s)][b] = sum_c ket[(y,s)][c] R[v][b][c]
   CK(zgemm(Ml2 * D, Mr1, Mr2, W.Dr, 1, ONE, mref(ket, Mr2, 1),
-           mref(Renv, 1, Mr2, (long long)Mr1 * Mr2), ZERO, c.X, Mr1, per, skip, c.st));
+           mref(Renv, 1, Mr2, (long long)Mr1 * Mr2), ZERO, c.X, Mr1, per, skip, c.st, c.ws));
   CK(mpo_mix(W.rl, Ml2, d, Mr1, c.X, per, Y, per, skip, c.st));
 }
 
@@ -92,7 +92,7 @@ void env_left_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Mr1, int Ml2, 
   const long long per = (long long)Ml1 * D * Mr2;
   // Lout[v][b][c] = sum_{(a,s)} conj(bra[(a,s)][b]) Y[v][(a,s)][c]
   CK(zgemm(Mr1, Mr2, Ml1 * D, W.Dr, 1, ONE, mref(bra, 1, Mr1, 0, 0, 1), mref(c.Y, Mr2, 1, per),
-           ZERO, Lout, Mr2, (long long)Mr1 * Mr2, nullptr, c.st));
+           ZERO, Lout, Mr2, (long long)Mr1 * Mr2, nullptr, c.st, c.ws));
 }
 
 void env_right_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Mr1, int Ml2, int Mr2, int D,
@@ -102,16 +102,16 @@ void env_right_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Mr1, int Ml2,
   // Rout[w][a][y] = sum_{(s,b)} conj(bra[a][(s,b)]) Y[w][y][(s,b)]
   CK(zgemm(Ml1, Ml2, D * Mr1, W.Dl, 1, ONE, mref(bra, (long long)D * Mr1, 1, 0, 0, 1),
            mref(c.Y, 1, (long long)D * Mr1, per), ZERO, Rout, Ml2, (long long)Ml1 * Ml2,
-           nullptr, c.st));
+           nullptr, c.st, c.ws));
 }
 
 void bond_f64(const Ctx& c, int M, int Dw, const cplx* Lenv, const cplx* Renv, const cplx* in,
               cplx* out, const int* skip) {
   const long long mm = (long long)M * M;
   CK(zgemm(Dw * M, M, M, 1, 1, ONE, mref(Lenv, M, 1), mref(in, M, 1), ZERO, c.X, M, 0, skip,
-           c.st));
+           c.st, c.ws));
   CK(zgemm(M, M, M, 1, Dw, ONE, mref(c.X, M, 1, 0, mm), mref(Renv, 1, M, 0, mm), ZERO, out, M,
-           0, skip, c.st));
+           0, skip, c.st, c.ws));
 }
 
 // ------------------------------------------------------------------------------------
@@ -402,6 +402,7 @@ Engine::Engine(const ModelParams& p) : P(p) {
   rebuild_mpos();
   CK(cudaMalloc(&status_, sizeof(int) * 4));
   CK(cudaMemset(status_, 0, sizeof(int) * 4));
+  zws_.status = status_ + 2;
   bs_.noconv = status_ + 3;
   CK(cudaMalloc(&lz_, sizeof(LzState)));
   CK(cudaMalloc(&scal_, sizeof(double) * 8));
@@ -454,6 +455,7 @@ Engine::~Engine() {
                   (void*)bs_.bar, (void*)bs_.mv})
     if (p) cudaFree(p);
   if (h_mv_) cudaFreeHost(h_mv_);
+  zg_free(zws_, st_);
 }
 
 void Engine::rebuild_mpos() {
@@ -578,6 +580,7 @@ void Engine::alloc_mps(DevMps& s, int M) {
   maxxy = std::max(maxxy, (long long)Dmax * maxbond * maxbond);
   ensure_workspace(maxsite, maxxy, maxbond, maxbond);
   if (mixed()) alloc_tc(s);
+  else alloc_zg(s);
   if (maxenv > env_tmp_size_) {
     for (int i = 0; i < 2; ++i) {
       if (env_tmp_[i]) cudaFree(env_tmp_[i]);
@@ -585,6 +588,24 @@ void Engine::alloc_mps(DevMps& s, int M) {
     }
     env_tmp_size_ = maxenv;
   }
+}
+
+// The digit workspace of the largest contraction of a sweep, so that it does not grow between
+// captured steps (graph mode holds its address).
+void Engine::alloc_zg(const DevMps& s) {
+  size_t need = 0;
+  const int Dm = std::max(H_.maxD, J_.maxD);
+  for (int k = 0; k < s.L(); ++k) {
+    const int Ml = s.Mb[k], Mr = s.Mb[k + 1], D = s.D[k];
+    need = std::max(need, zgemm_digits_bytes(Dm * Ml, D * Mr, Ml, 1, 1, 1, 1));
+    need = std::max(need, zgemm_digits_bytes(Ml * D, Mr, Mr, Dm, 1, 1, Dm));
+    need = std::max(need, zgemm_digits_bytes(Ml * D, Mr, Mr, 1, Dm, 1, 1));
+    need = std::max(need, zgemm_digits_bytes(Mr, Mr, Ml * D, Dm, 1, 1, Dm));
+    need = std::max(need, zgemm_digits_bytes(Ml, Ml, D * Mr, Dm, 1, 1, Dm));
+  }
+  zws_.fixed = false;
+  CK(zg_reserve(zws_, need, st_));
+  zws_.fixed = graphs_;
 }
 
 void Engine::alloc_tc(const DevMps& s) {
@@ -838,7 +859,7 @@ void Engine::absorb_left(const cplx* C, int M, cplx* A, long long ncols) {
     CK(tc_gemm(Cp, At, g, st_));
   } else {
     CK(zgemm(M, (int)ncols, M, 1, 1, ONE, mref(C, M, 1), mref(A, ncols, 1), ZERO, T1_, ncols, 0,
-             nullptr, st_));
+             nullptr, st_, &zws_));
   }
   CK(cudaMemcpyAsync(A, T1_, sizeof(cplx) * (size_t)M * ncols, cudaMemcpyDeviceToDevice, st_));
 }
@@ -856,7 +877,7 @@ void Engine::absorb_right(cplx* A, long long nrows, const cplx* C, int M) {
     CK(tc_gemm(Ap, Ct, g, st_));
   } else {
     CK(zgemm((int)nrows, M, M, 1, 1, ONE, mref(A, M, 1), mref(C, M, 1), ZERO, T1_, M, 0, nullptr,
-             st_));
+             st_, &zws_));
   }
   CK(cudaMemcpyAsync(A, T1_, sizeof(cplx) * (size_t)M * nrows, cudaMemcpyDeviceToDevice, st_));
 }
@@ -1002,6 +1023,7 @@ void Engine::set_graphs(bool on, int qr_cap) {
     twin_on_ = false;
   }
   graphs_ = on;
+  zws_.fixed = on;
   qr_gcap_ = qr_cap;
   if (on && st_ == 0) {
     if (!own_stream_) CK(cudaStreamCreateWithFlags(&own_stream_, cudaStreamNonBlocking));

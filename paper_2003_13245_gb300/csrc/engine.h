@@ -45,6 +45,7 @@ struct Ctx {
   cudaStream_t st;
   cplx* X;
   cplx* Y;
+  ZgWork* ws = nullptr;    // workspace of the contractions' digit products
 };
 // out[a,s,t,b] = sum L[w,a,y] W[w,v,s,u] in[y,u,t,c] R[v,b,c]  (bra dims = ket dims)
 void heff_f64(const Ctx& c, const DevMpoSite& W, int Ml, int Mr, int D, int d, const cplx* Lenv,
@@ -196,6 +197,7 @@ class Engine {
   static void free_mpo(DevMpo& m);
   cudaStream_t stream() const { return st_; }
   cplx* X() { return X_; }
+  ZgWork* zg() { return &zws_; }
   cplx* Y() { return Y_; }
 
   // Lanczos exponential exp(tau M) v for a matvec callback (device pointers); returns the
@@ -262,7 +264,7 @@ class Engine {
   void site_update(DevMps& s, int k, double hr, double hi);
   void shift_right(DevMps& s, int k, const cplx* center, cplx* Cbond);
   void shift_left(DevMps& s, int k, const cplx* center, cplx* Cbond);
-  Ctx ctx() const { return Ctx{st_, X_, Y_}; }
+  Ctx ctx() { return Ctx{st_, X_, Y_, &zws_}; }
   bool mixed() const { return precision_ != 0; }
   double tic();
   void toc(double& acc, double t0);
@@ -271,6 +273,7 @@ class Engine {
   void env_right_any(const DevMpoSite& W, int Ml1, int Mr1, int Ml2, int Mr2, int D, int d,
                      const cplx* Renv, const cplx* bra, const cplx* ket, cplx* Rout);
   void alloc_tc(const DevMps& s);
+  void alloc_zg(const DevMps& s);
   void absorb_left(const cplx* C, int M, cplx* A, long long ncols);
   void absorb_right(cplx* A, long long nrows, const cplx* C, int M);
   void set_ones(cplx* p);
@@ -348,6 +351,7 @@ class Engine {
   unsigned char qr_ev_bulk_[QR_EV] = {};   // the QR of event pair i has m >= 4096
   cudaEvent_t lz_ev_[2 * QR_EV] = {};
   int lz_ev_n_ = 0;
+  ZgWork zws_{};                         // FP64 contractions (digit products)
   TcBufs tcb_{};
   BondScratch bs_{};
   unsigned long long* h_mv_ = nullptr;   // pinned copy of the device Krylov-vector counter

@@ -302,7 +302,7 @@ void Engine::exp_vjp_nodes(long long n, const cplx* v, const cplx* ybar, double 
     cplx* d = tp.get((long long)h.size());
     CK(cudaMemcpyAsync(d, h.data(), sizeof(cplx) * h.size(), cudaMemcpyHostToDevice, st_));
     CK(zgemm(nodes, (int)n, k1, 1, 1, kOne, mr(d, k1, 1), mr(basis, n, 1), kZero, Bq, n, 0,
-             nullptr, st_));
+             nullptr, st_, &zws_));
     CK(cudaStreamSynchronize(st_));
   } else {
     CK(cudaMemsetAsync(Bq, 0, sizeof(cplx) * (size_t)nodes * n, st_));
@@ -314,7 +314,7 @@ void Engine::exp_vjp_nodes(long long n, const cplx* v, const cplx* ybar, double 
     cplx* d = tp.get((long long)h.size());
     CK(cudaMemcpyAsync(d, h.data(), sizeof(cplx) * h.size(), cudaMemcpyHostToDevice, st_));
     CK(zgemm(nodes, (int)n, k2, 1, 1, kOne, mr(d, k2, 1), mr(V_, n, 1), kZero, Aq, n, 0,
-             nullptr, st_));
+             nullptr, st_, &zws_));
     CK(cudaStreamSynchronize(st_));
   } else {
     CK(cudaMemsetAsync(Aq, 0, sizeof(cplx) * (size_t)nodes * n, st_));
@@ -430,7 +430,7 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
     copy(nxt_lr[k], A[k + 1], n[k + 1]);
     const long long ncols = (long long)D[k + 1] * Mb[k + 2];
     CK(zgemm(Mr, (int)ncols, Mr, 1, 1, kOne, mr(c_lr[k], Mr, 1), mr(nxt_lr[k], ncols, 1), kZero,
-             A[k + 1], ncols, 0, nullptr, st_));
+             A[k + 1], ncols, 0, nullptr, st_, &zws_));
     copy(A[k], Q_lr[k], n[k]);
   }
   // right to left
@@ -473,7 +473,7 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
     copy(nxt_rl[k], A[k - 1], n[k - 1]);
     const long long nrows = (long long)Mb[k - 1] * D[k - 1];
     CK(zgemm((int)nrows, Ml, Ml, 1, 1, kOne, mr(nxt_rl[k], Ml, 1), mr(c_rl[k], Ml, 1), kZero,
-             A[k - 1], Ml, 0, nullptr, st_));
+             A[k - 1], Ml, 0, nullptr, st_, &zws_));
     copy(A[k], Qs_rl[k], n[k]);
   }
   // optional normalisation of the output center: A0 <- A0 / ||A0||, log ||A0||^2 reported
@@ -601,10 +601,10 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
         // theta_p = Re sum_q k_q <a_q, H_eff(dW_p) b_q> = Re sum dW_p . G, G accumulated over
         // the nodes: U = L b_q, V = conj(a_q) R, then one contraction over (x, t, c)
         CK(zgemm(W.Dl * Ml, D[k] * Mr, Ml, 1, 1, kOne, mr(Le, Ml, 1), mr(b, (long long)D[k] * Mr, 1),
-                 kZero, X_, (long long)D[k] * Mr, 0, nullptr, st_));
+                 kZero, X_, (long long)D[k] * Mr, 0, nullptr, st_, &zws_));
         CK(zgemm(Ml * D[k], Mr, Mr, W.Dr, 1, kOne, mr(a, Mr, 1, 1),
                  mrb(Re, Mr, 1, (long long)Mr * Mr), kZero, Y_, Mr, (long long)Ml * D[k] * Mr,
-                 nullptr, st_));
+                 nullptr, st_, &zws_));
         CK(param_gram(W.Dl, W.Dr, Ml, dd[k], Mr, X_, Y_, kcc, Gacc, st_));
       } else {
         for (int p = 0; p < np; ++p) {
@@ -650,13 +650,13 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
       const cplx kk = {kq[q].real(), kq[q].imag()};  // w_q conj(tau)
       // Lbar_w += k a conj(R_w) b^H;  Rbar_w += k a^T conj(L_w) conj(b)
       CK(zgemm(M, M, M, Dw, 1, kOne, mrb(Re, M, 1, mm, 1), mr(b, 1, M, 1), kZero, El, M, mm,
-               nullptr, st_));
+               nullptr, st_, &zws_));
       CK(zgemm(M, M, M, Dw, 1, kk, mr(a, M, 1), mrb(El, M, 1, mm), kOne, Lbar, M, mm, nullptr,
-               st_));
+               st_, &zws_));
       CK(zgemm(M, M, M, Dw, 1, kOne, mrb(Le, M, 1, mm, 1), mr(b, M, 1, 1), kZero, El, M, mm,
-               nullptr, st_));
+               nullptr, st_, &zws_));
       CK(zgemm(M, M, M, Dw, 1, kk, mr(a, 1, M), mrb(El, M, 1, mm), kOne, Rbar, M, mm, nullptr,
-               st_));
+               st_, &zws_));
     }
     CK(cudaStreamSynchronize(st_));
   };
@@ -714,9 +714,9 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
       const long long nrows = (long long)Mb[k - 1] * D[k - 1];
       // A[k-1] = nxt c:  cbar = nxt^H abar,  abar <- abar c^H
       CK(zgemm(Ml, Ml, (int)nrows, 1, 1, kOne, mr(nxt_rl[k], 1, Ml, 1), mr(ab[k - 1], Ml, 1),
-               kZero, b1, Ml, 0, nullptr, st_));
+               kZero, b1, Ml, 0, nullptr, st_, &zws_));
       CK(zgemm((int)nrows, Ml, Ml, 1, 1, kOne, mr(ab[k - 1], Ml, 1), mr(c_rl[k], 1, Ml, 1), kZero,
-               s1, Ml, 0, nullptr, st_));
+               s1, Ml, 0, nullptr, st_, &zws_));
       copy(ab[k - 1], s1, n[k - 1]);
       // c = exp(-h K(Lenv[k], Rnew[k-1])) Cm
       bond_vjp(Ml, Dl, Lenv[k], Rnew[k - 1], Cm_rl[k], b1, b2, e1, e2);
@@ -778,9 +778,9 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
       const long long ncols = (long long)D[k + 1] * Mb[k + 2];
       // A[k+1] = c nxt:  cbar = abar nxt^H,  abar <- c^H abar
       CK(zgemm(Mr, Mr, (int)ncols, 1, 1, kOne, mr(ab[k + 1], ncols, 1), mr(nxt_lr[k], 1, ncols, 1),
-               kZero, b1, Mr, 0, nullptr, st_));
+               kZero, b1, Mr, 0, nullptr, st_, &zws_));
       CK(zgemm(Mr, (int)ncols, Mr, 1, 1, kOne, mr(c_lr[k], 1, Mr, 1), mr(ab[k + 1], ncols, 1),
-               kZero, s1, ncols, 0, nullptr, st_));
+               kZero, s1, ncols, 0, nullptr, st_, &zws_));
       copy(ab[k + 1], s1, n[k + 1]);
       // c = exp(-h K(Lenv[k+1], Rin[k])) R
       bond_vjp(Mr, Dr, Lenv[k + 1], Rin[k], R_lr[k], b1, b2, e1, e2);
@@ -1120,7 +1120,7 @@ void Engine::canonicalize_vjp(int M, cplx* const* psi0, const cplx* const* gbar,
     copy(nxt[k], A[k - 1], z.n[k - 1]);
     const long long nrows = (long long)z.Mb[k - 1] * z.D[k - 1];
     CK(zgemm((int)nrows, Ml, Ml, 1, 1, kOne, mr(nxt[k], Ml, 1), mr(Cm[k], Ml, 1), kZero, A[k - 1],
-             Ml, 0, nullptr, st_));
+             Ml, 0, nullptr, st_, &zws_));
     copy(A[k], Qs[k], z.n[k]);
   }
   cplx* part = tp.get(257);
@@ -1172,9 +1172,9 @@ void Engine::canonicalize_vjp(int M, cplx* const* psi0, const cplx* const* gbar,
     const long long nrows = (long long)z.Mb[k - 1] * z.D[k - 1];
     // A[k-1] = nxt Cm:  Cmbar = nxt^H abar,  abar <- abar Cm^H
     CK(zgemm(Ml, Ml, (int)nrows, 1, 1, kOne, mr(nxt[k], 1, Ml, 1), mr(ab[k - 1], Ml, 1), kZero,
-             cmb, Ml, 0, nullptr, st_));
+             cmb, Ml, 0, nullptr, st_, &zws_));
     CK(zgemm((int)nrows, Ml, Ml, 1, 1, kOne, mr(ab[k - 1], Ml, 1), mr(Cm[k], 1, Ml, 1), kZero, t1,
-             Ml, 0, nullptr, st_));
+             Ml, 0, nullptr, st_, &zws_));
     copy(ab[k - 1], t1, z.n[k - 1]);
     // Renv[k-1] = env_right(Renv[k], Qs, W, Qs)
     call(tdmrg_kernel_env_vjp(1, Ml, Mr, z.d[k], W.Dl, W.Dr, Wd[k].data(), np,

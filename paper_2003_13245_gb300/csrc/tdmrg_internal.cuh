@@ -25,11 +25,38 @@ struct MatRef {
   int conj;
 };
 
+// Workspace of the digit products of zgemm (zgemm_digits.cu) for calls on one stream at a time:
+// the digits of both operands and split-K partials.  It grows on demand up to kZgMaxBytes unless
+// `fixed` (captured graphs hold its address).  `pooled` workspaces live for one call of a
+// kernel-level entry point and come from the library's stream-ordered pool; the others belong to
+// an engine.  *status (device) is set to 3 when a bounded pipeline wait gives up.
+struct ZgWork {
+  void* p = nullptr;
+  size_t bytes = 0;
+  int* status = nullptr;
+  bool fixed = false, pooled = false;
+};
+constexpr size_t kZgMaxBytes = (size_t)2 << 30;
+// grows w to at least min(bytes, kZgMaxBytes) (contents lost); leaves it as it is when fixed
+cudaError_t zg_reserve(ZgWork& w, size_t bytes, cudaStream_t s);
+void zg_free(ZgWork& w, cudaStream_t s);
+// a block of the library's stream-ordered pool (cudaFreeAsync gives it back)
+cudaError_t zg_pool_alloc(void** p, size_t bytes, cudaStream_t s);
+// returns the memory the pool holds for later calls to the device
+void zg_pool_trim();
+
 // C_b = alpha * sum_{r < nred} op(A_{b,r}) op(B_{b,r}) + beta * C_b, b < nbatch.
-// C row-major with leading dimension ldc and batch stride sc.
+// C row-major with leading dimension ldc and batch stride sc.  With a workspace the product is
+// taken on the tensor cores in exact digit products (zgemm_digits.cu), otherwise (and for the
+// shapes where that is not faster) by FP64 FMAs.
 cudaError_t zgemm(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef A, MatRef B,
                   cplx beta, cplx* C, long long ldc, long long sc, const int* skip,
-                  cudaStream_t s);
+                  cudaStream_t s, ZgWork* ws = nullptr);
+// the digit-product form alone; *taken = false when the workspace cannot hold one tile
+cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef A,
+                         MatRef B, cplx beta, cplx* C, long long ldc, long long sc,
+                         const int* skip, const ZgWork& ws, cudaStream_t s, bool* taken);
+size_t zgemm_digits_bytes(int m, int n, int k, int nbatch, int nred, int nbA, int nbB);
 
 // Sparse MPO mixing over the channel and the physical (P) level of a site:
 // Y[wo][a][s][t][b] = sum_{blocks of wo} sum_u op[s][u] X[wi][a][u][t][b].

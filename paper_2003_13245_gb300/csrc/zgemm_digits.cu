@@ -1,0 +1,780 @@
+// Complex FP64 GEMM on the tensor cores: both operands are written as sums of 8-bit digits and
+// the digit products are summed exactly (the splitting of Ozaki, Ogita, Oishi and Rump,
+// "Error-free transformations of matrix multiplication", with a truncated product sum).
+//
+// Why: GB300 issues about 2 FP64 FMAs per clock per SM, so a 64 x 64 x 64 complex tile of
+// zgemm_kernel holds an SM for ~0.27 ms; its tensor cores take 4096 fp16 multiply-adds per clock.
+//
+// Split (digit_split_kernel): a row of 128 consecutive k of an operand is scaled by the power of
+// two 2^E above its largest component and rounded to a 56-bit integer in units of 2^(E-55), which
+// is written as seven signed base-256 digits (-128..128), each an exact fp16.  All of it is integer
+// arithmetic.  Re and im parts share E.  The digits are stored as the shared-memory image of the
+// tile they will be staged in (8 x 16 byte core matrices), so a stage is one contiguous block.
+//
+// Product (digit_gemm_kernel): one CTA computes a 128 x 32 tile of C.  For every digit i of the
+// 128-row operand one tcgen05.mma (kind::f16, FP32 accumulation) multiplies it with the digits
+// j = 0 .. min(6, 7 - i) of the 32-column operand at once (N = 32 per digit), because digit pair
+// (i, j) goes to the accumulator of level i + j and both the digits in shared memory and the
+// levels in TMEM are contiguous: 4 x 7 instructions per 16-deep k step.  A digit product is at
+// most 2^14; over one chunk of 128 k a level of p pairs sums to at most p 2^22, an integer that
+// FP32 holds exactly.  After each chunk eight warps read the levels back and combine them in
+// 64-bit integers; the chunk's result is rounded once to FP64 and the chunks are added in FP64.
+//
+// Error: the operands carry 56 bits below the chunk's largest entry and the dropped pairs
+// (i + j > 7) are below 2^-62 of it, so an entry is off by about 2^-56 sqrt(K) max|a| max|b| and
+// one rounding; the FMA kernel rounds every partial sum.
+//
+// Bound: the tensor pipe in the main loop (28 instructions, ~2300 clocks per k step of 128 x 32),
+// plus the integer epilogue, which cannot overlap it (eight re and im levels fill all 512 TMEM
+// columns).  72 KB per stage from L2, three stages, one CTA per SM.  Measured on GB300 against the
+// FMA kernel: 896 x 8192 x 128 0.28 against 6.2 ms (27 TFLOP/s, tensor pipe 39 %); 8192 x 128 x 128
+// summed over seven channels 0.35 against 7.3 ms; 128 x 128 x 8192, seven batches, 0.55 against
+// 34 ms; 64 x 64 x 256, seven batches, 35 against 1048 us; 16 x 16 x 4 21 against 68 us.
+#include "tdmrg_internal.cuh"
+
+#include <mutex>
+
+namespace tdmrg {
+
+namespace {
+
+constexpr int ND = 7;                         // digits
+constexpr int NL = 8;                         // levels i + j kept
+constexpr int PT = 128, QT = 32;              // tile rows (operand P) and columns (operand Q)
+constexpr int KS = 16;                        // k per stage
+constexpr int KC = 128;                       // k per chunk (one scale per row and chunk)
+constexpr int STEPS = KC / KS;
+constexpr int P_BLOCK = 2 * ND * PT * KS * 2; // 57344 bytes per stage
+constexpr int Q_BLOCK = 2 * ND * QT * KS * 2; // 14336
+constexpr int STAGE = P_BLOCK + Q_BLOCK;
+constexpr int NST = 3;
+constexpr int GEMM_THREADS = 320;             // TMA warp, MMA warp, eight epilogue warps
+constexpr size_t GEMM_SMEM = (size_t)NST * STAGE + 256 + 128;
+constexpr int TMEM_COLS = 512;
+constexpr int E_NONFINITE = 1 << 20;          // scale of a row that holds an Inf or a NaN
+constexpr long long WAIT_CYCLES = 4000000000LL;
+
+struct Operand {
+  const cplx* p;
+  long long rs, ks, sb, sr;   // strides of row, k, batch, reduction term
+  int conj;
+  int rows, nb;               // rows; batches stored (1 when the batches share the operand)
+  int tile;                   // PT or QT
+  int tiles;                  // row tiles
+  unsigned char* dig;         // [nb][tiles][steps] blocks
+  int* ex;                    // [nb][chunks][tiles * tile]
+};
+
+struct SplitArgs {
+  Operand o[2];
+  int K, nred, ksteps, chunks;   // k steps and chunks of one reduction term
+  int blocks0;                   // blocks of operand 0
+  const int* skip;
+};
+
+constexpr int SR = 16;                        // rows of a split block
+constexpr int S_LD = KC + 1;
+
+// One block: 16 rows x one chunk of 128 k of one operand.
+__global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
+  if (A.skip && *A.skip) return;
+  __shared__ cplx s_v[SR * S_LD];
+  __shared__ int s_e[SR];
+  const bool second = (int)blockIdx.x >= A.blocks0;
+  const Operand& o = A.o[second ? 1 : 0];
+  int id = blockIdx.x - (second ? A.blocks0 : 0);
+  const int tc = A.nred * A.chunks;
+  const int chunk = id % tc;
+  id /= tc;
+  const int groups = o.tiles * (o.tile / SR);
+  const int r0 = (id % groups) * SR;
+  const int b = id / groups;
+  const int red = chunk / A.chunks, c = chunk % A.chunks;
+  const int k0 = c * KC, kn = min(KC, A.K - k0);
+  const int steps = (kn + KS - 1) / KS;
+  const cplx* src = o.p + (long long)b * o.sb + (long long)red * o.sr;
+  if (threadIdx.x < SR) s_e[threadIdx.x] = 0;
+  // load in the order that is contiguous in memory
+  const bool kfast = o.ks == 1;
+  for (int e = threadIdx.x; e < SR * KC; e += 256) {
+    const int r = kfast ? e / KC : e % SR, k = kfast ? e % KC : e / SR;
+    cplx v = make_double2(0.0, 0.0);
+    if (r0 + r < o.rows && k < kn) v = src[(long long)(r0 + r) * o.rs + (long long)(k0 + k) * o.ks];
+    s_v[r * S_LD + k] = v;
+  }
+  __syncthreads();
+  const int r = threadIdx.x & (SR - 1), g = threadIdx.x / SR;      // row, group of 8 k
+  const cplx* mine = s_v + r * S_LD + g * 8;
+  int e = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const cplx v = mine[i];
+    e = max(e, (__double2hiint(v.x) >> 20) & 0x7ff);
+    e = max(e, (__double2hiint(v.y) >> 20) & 0x7ff);
+  }
+  atomicMax(&s_e[r], e);
+  __syncthreads();
+  const int em = s_e[r];
+  if (g == 0)
+    o.ex[((long long)b * tc + chunk) * ((long long)o.tiles * o.tile) + r0 + r] =
+        em == 0x7ff ? E_NONFINITE : max(em, 1) - 1022;
+  if (g >= 2 * steps) return;
+  const int emax = max(em, 1);
+  const bool bad = em == 0x7ff;
+  const int row = r0 + r, tile = row / o.tile, rt = row % o.tile;
+  const int ks = g >> 1, kh = g & 1;
+  const long long step = (long long)red * A.ksteps + (long long)c * STEPS + ks;
+  const int block = 2 * ND * o.tile * KS * 2;
+  unsigned char* dst = o.dig +
+      (((long long)b * o.tiles + tile) * ((long long)A.nred * A.ksteps) + step) * block;
+  const bool wide = o.tile == PT;
+#pragma unroll
+  for (int part = 0; part < 2; ++part) {
+    unsigned long long w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const double x = part == 0 ? mine[i].x : mine[i].y;
+      const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+      const int ex = (int)(bits >> 52) & 0x7ff;
+      unsigned long long mant = bits & 0xfffffffffffffULL;
+      if (ex) mant |= 1ULL << 52;
+      const int sh = max(ex, 1) - emax + 2;
+      unsigned long long v;
+      if (sh >= 0) v = mant << sh;
+      else if (sh >= -54) v = (mant + (1ULL << (-sh - 1))) >> (-sh);
+      else v = 0;
+      if (bad) v = 0;
+      const bool neg = ((bits >> 63) != 0) != (part == 1 && o.conj != 0);
+      w[i] = (neg ? 0ULL - v : v) + 0x0080808080808080ULL;
+    }
+#pragma unroll
+    for (int l = 0; l < ND; ++l) {
+      uint32_t h[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t mask = l == 0 ? 0xffffu : 0xffu;
+        const uint32_t a = (uint32_t)(w[2 * q] >> (48 - 8 * l)) & mask;
+        const uint32_t c2 = (uint32_t)(w[2 * q + 1] >> (48 - 8 * l)) & mask;
+        // 0x6400 + u is the fp16 number 1024 + u; subtracting 1152 leaves the signed digit
+        const uint32_t pk = (0x64006400u + a) + (c2 << 16);
+        uint32_t d;
+        asm("sub.f16x2 %0, %1, %2;" : "=r"(d) : "r"(pk), "r"(0x64806480u));
+        h[q] = d;
+      }
+      long long off;
+      if (wide)                      // [part][digit][k half][row group][8 rows][16 B]
+        off = (((part * ND + l) * 2 + kh) * (PT / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
+      else                           // [part][k half][digit][row group][8 rows][16 B]
+        off = (((part * 2 + kh) * ND + l) * (QT / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
+      *reinterpret_cast<uint4*>(dst + off) = make_uint4(h[0], h[1], h[2], h[3]);
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// bounded wait (about 2 s); gives up at once when another role of the CTA has
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* fail,
+                                          int* status) {
+  if (mbar_try(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try(bar, parity)) {
+    if (*fail) return false;
+    if (clock64() - t0 > WAIT_CYCLES) {
+      *fail = 1;
+      atomicExch(status, 3);
+      return false;
+    }
+  }
+  return true;
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
+                                          uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_u32(dst)),
+      "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+// K-major operand without swizzle: 8-row x 16-byte core matrices, `lbo` bytes between the two of
+// a k step, 128 bytes between row groups
+__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
+  d |= (uint64_t)(lbo >> 4) << 16;
+  d |= (uint64_t)(128 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+// D f32, A and B fp16, both K-major, M = 128
+__host__ __device__ constexpr uint32_t idesc(int negA, int n) {
+  return (1u << 4) | ((uint32_t)negA << 13) | ((uint32_t)(n >> 3) << 17) |
+         ((uint32_t)(PT >> 4) << 24);
+}
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id,
+                                        uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(id), "r"(acc));
+}
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+          smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr));
+}
+
+// T * 2^e, |T| < 2^63, rounded to nearest: integer arithmetic while the result is a normal number
+__device__ __forceinline__ double pack(long long T, int e) {
+  if (T == 0) return 0.0;
+  const unsigned long long u = T < 0 ? 0ULL - (unsigned long long)T : (unsigned long long)T;
+  const int lz = __clzll((long long)u);
+  const int be = e + 63 - lz + 1023;               // biased exponent
+  if (be < 1 || be > 2045) {                       // rare: let the library round and saturate
+    return scalbn((double)T, e);
+  }
+  const unsigned long long m = u << lz;
+  const unsigned long long rnd = (m >> 11) + ((m & 0x400) && ((m & 0xbff) != 0) ? 1 : 0);
+  unsigned long long bits = ((unsigned long long)(be - 1) << 52) + rnd;   // the hidden bit adds 1
+  if (T < 0) bits |= 1ULL << 63;
+  return __longlong_as_double((long long)bits);
+}
+
+struct GemmArgs {
+  const unsigned char* pd;
+  const unsigned char* qd;
+  const int* pe;
+  const int* qe;
+  long long p_b, q_b;          // bytes between batches (0: shared)
+  long long pe_b, qe_b;        // exponents between batches
+  int p_rows, q_rows;          // output extent along P and Q
+  int p_tiles, q_tiles;
+  int ksteps, chunks, nred;    // per reduction term
+  int ksplit, per_split;       // chunks (over all terms) of one split
+  cplx* C;
+  long long cp, cq, sc;        // output strides along P, along Q, between batches
+  cplx* part;                  // split-K partials [ksplit][nbatch][p_rows][q_rows] (cp = 1)
+  int nbatch;
+  cplx alpha, beta;
+  int plain;                   // alpha = 1, beta = 0
+  int* status;
+  const int* skip;
+};
+
+__global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __grid_constant__ GemmArgs A) {
+  if (A.skip && *A.skip) return;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + NST * STAGE);
+  uint64_t* empty = full + NST;
+  uint64_t* acc_full = empty + NST;
+  uint64_t* acc_empty = acc_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
+  volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* issued = fail + 1;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int pt = blockIdx.y, qt = blockIdx.x;
+  const int bz = blockIdx.z / A.ksplit, sp = blockIdx.z % A.ksplit;
+  const int all = A.nred * A.chunks;
+  const int cbeg = sp * A.per_split, cend = min(all, cbeg + A.per_split);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, 8);
+    *fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  if (threadIdx.x == 0) {
+    // producer: one contiguous block of each operand per k step
+    const long long tsteps = (long long)A.nred * A.ksteps;
+    const unsigned char* P = A.pd + bz * A.p_b + (long long)pt * tsteps * P_BLOCK;
+    const unsigned char* Q = A.qd + bz * A.q_b + (long long)qt * tsteps * Q_BLOCK;
+    int t = 0;
+    bool live = true;
+    for (int ch = cbeg; ch < cend && live; ++ch) {
+      const int red = ch / A.chunks, c = ch % A.chunks;
+      const int ns = min(STEPS, A.ksteps - c * STEPS);
+      for (int k = 0; k < ns; ++k, ++t) {
+        const int s = t % NST;
+        if (t >= NST && !mbar_wait(&empty[s], (t / NST - 1) & 1, fail, A.status)) {
+          live = false;
+          break;
+        }
+        const long long step = (long long)red * A.ksteps + c * STEPS + k;
+        unsigned char* st = smem + s * STAGE;
+        mbar_expect_tx(&full[s], STAGE);
+        bulk_load(st, P + step * P_BLOCK, P_BLOCK, &full[s]);
+        bulk_load(st + P_BLOCK, Q + step * Q_BLOCK, Q_BLOCK, &full[s]);
+      }
+    }
+    *issued = t;
+  } else if (threadIdx.x == 32) {
+    // MMA issuer
+    int t = 0;
+    bool live = true;
+    for (int ch = cbeg; ch < cend && live; ++ch) {
+      const int ns = min(STEPS, A.ksteps - (ch % A.chunks) * STEPS);
+      const int local = ch - cbeg;
+      if (local > 0 && !mbar_wait(acc_empty, (local - 1) & 1, fail, A.status)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      for (int k = 0; k < ns; ++k, ++t) {
+        const int s = t % NST;
+        if (!mbar_wait(&full[s], (t / NST) & 1, fail, A.status)) {
+          live = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t p0 = smem_u32(smem + s * STAGE), q0 = p0 + P_BLOCK;
+        const uint64_t qr = sdesc(q0, ND * QT * 16), qi = sdesc(q0 + Q_BLOCK / 2, ND * QT * 16);
+#pragma unroll
+        for (int i = 0; i < ND; ++i) {
+          // digits j = 0 .. min(6, 7 - i) of Q: levels i .. i + j
+          const uint32_t n = QT * (NL - i < ND ? NL - i : ND);
+          // a chunk's first write of a level does not accumulate: digit 0 starts levels 0-6;
+          // level 7 starts with digit pair (1, 6), which is cut off the others of digit 1
+          const uint32_t acc = (k > 0 || i > 0) ? 1u : 0u;
+          const bool cut = i == 1 && k == 0;
+          const uint32_t m = cut ? n - QT : n;
+          const uint64_t pr = sdesc(p0 + i * (PT * KS * 2), PT * 16);
+          const uint64_t pi = sdesc(p0 + (ND + i) * (PT * KS * 2), PT * 16);
+          const uint32_t d_re = tmem + i * QT, d_im = tmem + NL * QT + i * QT;
+          mma_f16(d_re, pr, qr, idesc(0, m), acc);
+          mma_f16(d_im, pr, qi, idesc(0, m), acc);
+          if (cut) {
+            constexpr uint32_t last = (ND - 1) * QT * 16;       // digit 6 of Q
+            mma_f16(d_re + m, pr, sdesc(q0 + last, ND * QT * 16), idesc(0, QT), 0u);
+            mma_f16(d_im + m, pr, sdesc(q0 + Q_BLOCK / 2 + last, ND * QT * 16), idesc(0, QT), 0u);
+          }
+          mma_f16(d_re, pi, qi, idesc(1, n), 1u);
+          mma_f16(d_im, pi, qr, idesc(0, n), 1u);
+        }
+        mma_commit(&empty[s]);
+      }
+      if (live) mma_commit(acc_full);
+    }
+  } else if (warp >= 2) {
+    // epilogue: warp w reads TMEM lanes 32 (w mod 4)..; warps 2-5 the first 16 columns of every
+    // level, warps 6-9 the others
+    const int quad = warp & 3, half = (warp - 2) >> 2;
+    const int prow = pt * PT + quad * 32 + lane;
+    const int qcol0 = qt * QT + half * 16;
+    const long long pext = (long long)A.p_tiles * PT, qext = (long long)A.q_tiles * QT;
+    const int* pe = A.pe + bz * A.pe_b + prow;
+    const int* qe = A.qe + bz * A.qe_b + qcol0;
+    const uint32_t base = tmem + ((uint32_t)(quad * 32) << 16) + half * 16;
+    double re[16], im[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) re[c] = im[c] = 0.0;
+    bool ok = true;
+    for (int ch = cbeg; ch < cend; ++ch) {
+      const int local = ch - cbeg;
+      const int ep = __ldg(pe + ch * pext);
+      ok = mbar_wait(acc_full, local & 1, fail, A.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int blk = 0; blk < 4; ++blk) {          // (columns 0-7, 8-15) x (re, im)
+        const int c0 = (blk >> 1) * 8;
+        const bool imag = blk & 1;
+        uint32_t v[NL][8];
+#pragma unroll
+        for (int l = 0; l < NL; ++l)
+          tmem_ld8(base + (imag ? NL * QT : 0) + l * QT + c0, v[l]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          // the asm volatile loads are complete: tie the values to the wait
+          int S[NL];
+#pragma unroll
+          for (int l = 0; l < NL; ++l) {
+            asm volatile("" : "+r"(v[l][c]));
+            S[l] = __float2int_rn(__uint_as_float(v[l][c]));
+          }
+          // the sum is hi 2^32 + lo in units of level 7 (|hi| < 2^49, |lo| < 2^50): 62 bits of it,
+          // from the top of hi down
+          const long long hi = S[0] * 16777216LL + S[1] * 65536LL + S[2] * 256LL + S[3];
+          const long long lo = S[4] * 16777216LL + S[5] * 65536LL + S[6] * 256LL + S[7];
+          const int sh = min(32, __clzll(hi < 0 ? -hi : hi) - 2);
+          const long long T = (long long)((unsigned long long)hi << sh) + (lo >> (32 - sh));
+          const int eq = __ldg(qe + ch * qext + c0 + c);
+          double x = pack(T, ep + eq - 38 - sh);
+          if (ep == E_NONFINITE || eq == E_NONFINITE) x = __longlong_as_double(0x7ff8000000000000LL);
+          if (imag) im[c0 + c] = local == 0 ? x : im[c0 + c] + x;
+          else re[c0 + c] = local == 0 ? x : re[c0 + c] + x;
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty);
+    }
+    if (ok && prow < A.p_rows) {
+      if (A.ksplit > 1) {
+        cplx* D = A.part + (((long long)sp * A.nbatch + bz) * A.q_rows) * A.p_rows + prow;
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          if (qcol0 + c < A.q_rows) D[(long long)(qcol0 + c) * A.p_rows] = make_double2(re[c], im[c]);
+      } else {
+        cplx* D = A.C + bz * A.sc + prow * A.cp;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          if (qcol0 + c < A.q_rows) {
+            cplx v = make_double2(re[c], im[c]);
+            cplx* d = D + (qcol0 + c) * A.cq;
+            if (!A.plain) {
+              v = make_double2(A.alpha.x * re[c] - A.alpha.y * im[c],
+                               A.alpha.x * im[c] + A.alpha.y * re[c]);
+              if (A.beta.x != 0.0 || A.beta.y != 0.0) {
+                const cplx o = *d;
+                v.x += A.beta.x * o.x - A.beta.y * o.y;
+                v.y += A.beta.x * o.y + A.beta.y * o.x;
+              }
+            }
+            *d = v;
+          }
+        }
+      }
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && *fail) {
+    // a failed pipeline may still have copies in flight: the last one of each stage lands
+    // (bounded) before the shared memory is released
+    const int n = *issued;
+    for (int s = 0; s < NST; ++s) {
+      int last = -1;
+      for (int u = s; u < n; u += NST) last = u;
+      int none = 0;
+      if (last >= 0) mbar_wait(&full[s], (last / NST) & 1, &none, A.status);
+    }
+  }
+  __syncwarp();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(TMEM_COLS));
+  }
+}
+
+// C = alpha sum_s part_s + beta C, splits in order
+__global__ void __launch_bounds__(256) digit_reduce_kernel(GemmArgs A) {
+  if (A.skip && *A.skip) return;
+  const long long mn = (long long)A.p_rows * A.q_rows, total = mn * A.nbatch;
+  for (long long e = blockIdx.x * 256LL + threadIdx.x; e < total; e += (long long)gridDim.x * 256) {
+    const cplx* p = A.part + e;
+    cplx v = p[0];
+    for (int s = 1; s < A.ksplit; ++s) {
+      const cplx u = p[(long long)s * total];
+      v.x += u.x;
+      v.y += u.y;
+    }
+    const long long b = e / mn, r = e % mn;
+    cplx* d = A.C + b * A.sc + (r % A.p_rows) * A.cp + (r / A.p_rows) * A.cq;
+    if (!A.plain) {
+      v = make_double2(A.alpha.x * v.x - A.alpha.y * v.y, A.alpha.x * v.y + A.alpha.y * v.x);
+      if (A.beta.x != 0.0 || A.beta.y != 0.0) {
+        const cplx o = *d;
+        v.x += A.beta.x * o.x - A.beta.y * o.y;
+        v.y += A.beta.x * o.y + A.beta.y * o.x;
+      }
+    }
+    *d = v;
+  }
+}
+
+constexpr size_t ALIGN = 256;
+size_t up(size_t x) { return (x + ALIGN - 1) & ~(ALIGN - 1); }
+
+struct Plan {
+  int ksteps, chunks, tc;
+  size_t row_p, row_q;       // bytes of one 128-row tile of P, one 32-row tile of Q (with scales)
+};
+Plan plan_of(int k, int nred) {
+  Plan p;
+  p.ksteps = (k + KS - 1) / KS;
+  p.chunks = (k + KC - 1) / KC;
+  p.tc = p.chunks * nred;
+  p.row_p = (size_t)p.ksteps * nred * P_BLOCK + (size_t)p.tc * PT * sizeof(int);
+  p.row_q = (size_t)p.ksteps * nred * Q_BLOCK + (size_t)p.tc * QT * sizeof(int);
+  return p;
+}
+
+}  // namespace
+
+namespace {
+// splits of the chunk loop that fill the GPU when there are few tiles
+int splits_of(long long ntile, int chunks) {
+  const long long ks = (148 + ntile - 1) / ntile;
+  return (int)(ks < chunks ? ks : chunks);
+}
+}  // namespace
+
+size_t zgemm_digits_bytes(int m, int n, int k, int nbatch, int nred, int nbA, int nbB) {
+  const Plan p = plan_of(k, nred);
+  auto need = [&](int pr, int qr, int nbp, int nbq) {
+    const size_t tp = (pr + PT - 1) / PT, tq = (qr + QT - 1) / QT;
+    const int ks = splits_of((long long)(tp * tq) * nbatch, p.tc);
+    return tp * nbp * p.row_p + tq * nbq * p.row_q +
+           (ks > 1 ? sizeof(cplx) * (size_t)pr * qr * nbatch * ks : 0);
+  };
+  const size_t a = need(m, n, nbA, nbB), b = need(n, m, nbB, nbA);
+  return (a > b ? a : b) + 8 * ALIGN;
+}
+
+// C_b = alpha sum_r A_{b,r} B_{b,r} + beta C_b by digit products; *taken = false (and nothing is
+// launched) when the workspace cannot hold one tile row of each operand.
+cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef A, MatRef B,
+                         cplx beta, cplx* C, long long ldc, long long sc, const int* skip,
+                         const ZgWork& ws, cudaStream_t s, bool* taken) {
+  *taken = false;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(digit_gemm_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)GEMM_SMEM);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const Plan pl = plan_of(k, nred);
+  // the 128-row operand P is the side that pads least; on a tie the columns of C, whose stores
+  // are then contiguous across the lanes
+  auto tiles = [](int a, int t) { return (long long)(a + t - 1) / t; };
+  const bool swap = tiles(n, PT) * tiles(m, QT) <= tiles(m, PT) * tiles(n, QT);
+  Operand a{A.p, A.rs, A.cs, A.sb, A.sr, A.conj, m, A.sb == 0 ? 1 : nbatch, 0, 0, nullptr, nullptr};
+  Operand b{B.p, B.cs, B.rs, B.sb, B.sr, B.conj, n, B.sb == 0 ? 1 : nbatch, 0, 0, nullptr, nullptr};
+  Operand P = swap ? b : a, Q = swap ? a : b;
+  const long long cp = swap ? 1 : ldc, cq = swap ? ldc : 1;
+  P.tile = PT;
+  Q.tile = QT;
+  const int pt_all = (int)tiles(P.rows, PT), qt_all = (int)tiles(Q.rows, QT);
+  // slabs of the batch, then of the rows of P, then of Q, that fit the workspace
+  const size_t room = ws.bytes > 8 * ALIGN ? ws.bytes - 8 * ALIGN : 0;
+  int nb = nbatch, np = pt_all, nq = qt_all;
+  auto fits = [&](int bb, int pp, int qq) {
+    return (size_t)pp * (P.nb == 1 ? 1 : bb) * pl.row_p +
+               (size_t)qq * (Q.nb == 1 ? 1 : bb) * pl.row_q <= room;
+  };
+  if (!fits(1, 1, 1)) return cudaSuccess;
+  if (!fits(nb, np, nq)) {
+    nb = 1;
+    while (np > 1 && !fits(1, np, nq)) np = (np + 1) / 2;
+    while (nq > 1 && !fits(1, np, nq)) nq = (nq + 1) / 2;
+  }
+  for (int b0 = 0; b0 < nbatch; b0 += nb)
+    for (int p0 = 0; p0 < pt_all; p0 += np)
+      for (int q0 = 0; q0 < qt_all; q0 += nq) {
+        const int bb = b0 + nb < nbatch ? nb : nbatch - b0;
+        Operand p = P, q = Q;
+        p.tiles = p0 + np < pt_all ? np : pt_all - p0;
+        q.tiles = q0 + nq < qt_all ? nq : qt_all - q0;
+        p.rows = P.rows - p0 * PT < p.tiles * PT ? P.rows - p0 * PT : p.tiles * PT;
+        q.rows = Q.rows - q0 * QT < q.tiles * QT ? Q.rows - q0 * QT : q.tiles * QT;
+        p.p += (long long)p0 * PT * P.rs + (long long)b0 * P.sb;
+        q.p += (long long)q0 * QT * Q.rs + (long long)b0 * Q.sb;
+        p.nb = P.nb == 1 ? 1 : bb;
+        q.nb = Q.nb == 1 ? 1 : bb;
+        // carve the workspace
+        unsigned char* w = reinterpret_cast<unsigned char*>(
+            (reinterpret_cast<uintptr_t>(ws.p) + ALIGN - 1) & ~(uintptr_t)(ALIGN - 1));
+        unsigned char* end = static_cast<unsigned char*>(ws.p) + ws.bytes;
+        const long long tsteps = (long long)nred * pl.ksteps;
+        const size_t pbytes = (size_t)p.tiles * tsteps * P_BLOCK;
+        const size_t qbytes = (size_t)q.tiles * tsteps * Q_BLOCK;
+        p.dig = w;
+        w += up(pbytes * p.nb);
+        q.dig = w;
+        w += up(qbytes * q.nb);
+        p.ex = reinterpret_cast<int*>(w);
+        w += up(sizeof(int) * (size_t)p.nb * pl.tc * p.tiles * PT);
+        q.ex = reinterpret_cast<int*>(w);
+        w += up(sizeof(int) * (size_t)q.nb * pl.tc * q.tiles * QT);
+        SplitArgs sa{};
+        sa.o[0] = p;
+        sa.o[1] = q;
+        sa.K = k;
+        sa.nred = nred;
+        sa.ksteps = pl.ksteps;
+        sa.chunks = pl.chunks;
+        sa.skip = skip;
+        const long long blk0 = (long long)p.nb * p.tiles * (PT / SR) * pl.tc;
+        const long long blk1 = (long long)q.nb * q.tiles * (QT / SR) * pl.tc;
+        sa.blocks0 = (int)blk0;
+        if (blk0 + blk1 > 0x7fffffffLL) return cudaErrorInvalidValue;
+        count_launch();
+        digit_split_kernel<<<(unsigned)(blk0 + blk1), 256, 0, s>>>(sa);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        GemmArgs g{};
+        g.pd = p.dig;
+        g.qd = q.dig;
+        g.pe = p.ex;
+        g.qe = q.ex;
+        g.p_b = p.nb == 1 ? 0 : (long long)pbytes;
+        g.q_b = q.nb == 1 ? 0 : (long long)qbytes;
+        g.pe_b = p.nb == 1 ? 0 : (long long)pl.tc * p.tiles * PT;
+        g.qe_b = q.nb == 1 ? 0 : (long long)pl.tc * q.tiles * QT;
+        g.p_rows = p.rows;
+        g.q_rows = q.rows;
+        g.p_tiles = p.tiles;
+        g.q_tiles = q.tiles;
+        g.ksteps = pl.ksteps;
+        g.chunks = pl.chunks;
+        g.nred = nred;
+        g.C = C + (long long)b0 * sc + (long long)p0 * PT * cp + (long long)q0 * QT * cq;
+        g.cp = cp;
+        g.cq = cq;
+        g.sc = sc;
+        g.nbatch = bb;
+        g.alpha = alpha;
+        g.beta = beta;
+        g.plain = alpha.x == 1.0 && alpha.y == 0.0 && beta.x == 0.0 && beta.y == 0.0;
+        g.status = ws.status;
+        g.skip = skip;
+        // split the chunks when the tiles leave SMs idle
+        const long long ntile = (long long)p.tiles * q.tiles * bb;
+        int ks = splits_of(ntile, pl.tc);
+        const size_t one = sizeof(cplx) * (size_t)p.rows * q.rows * bb;
+        while (ks > 1 && w + one * ks > end) --ks;
+        g.per_split = (pl.tc + ks - 1) / ks;
+        g.ksplit = (pl.tc + g.per_split - 1) / g.per_split;
+        g.part = reinterpret_cast<cplx*>(w);
+        if ((long long)bb * g.ksplit > 65535 || p.tiles > 65535) return cudaErrorInvalidValue;
+        count_launch();
+        digit_gemm_kernel<<<dim3(q.tiles, p.tiles, bb * g.ksplit), GEMM_THREADS, GEMM_SMEM, s>>>(g);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (g.ksplit > 1) {
+          long long blocks = ((long long)p.rows * q.rows * bb + 255) / 256;
+          if (blocks > 152 * 8) blocks = 152 * 8;
+          count_launch();
+          digit_reduce_kernel<<<(int)blocks, 256, 0, s>>>(g);
+          if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+      }
+  *taken = true;
+  return cudaSuccess;
+}
+
+// ------------------------------------------------------------------------------------------
+// workspaces
+// ------------------------------------------------------------------------------------------
+namespace {
+// The library's stream-ordered pool, one per device, made at the first use.  It keeps at most
+// kPoolKeep bytes between calls (zg_pool_trim gives them back); CUDA's pools are safe with
+// several threads, and an allocation freed on one stream is handed to another only after it.
+constexpr unsigned long long kPoolKeep = 512ULL << 20;
+constexpr int kPoolDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kPoolDevices];
+
+cudaError_t pool_of(cudaMemPool_t* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kPoolDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+    unsigned long long keep = kPoolKeep;
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    g_pool[dev] = p;
+  }
+  *out = g_pool[dev];
+  return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t zg_pool_alloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaMemPool_t pool = nullptr;
+  const cudaError_t e = pool_of(&pool);
+  return e != cudaSuccess ? e : cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+cudaError_t zg_reserve(ZgWork& w, size_t bytes, cudaStream_t s) {
+  if (bytes > kZgMaxBytes) bytes = kZgMaxBytes;
+  if (w.fixed || bytes <= w.bytes) return cudaSuccess;
+  bytes = up(bytes + bytes / 8);      // room to grow without a new allocation
+  zg_free(w, s);
+  const cudaError_t e = w.pooled ? zg_pool_alloc(&w.p, bytes, s) : cudaMalloc(&w.p, bytes);
+  if (e != cudaSuccess) {
+    w.p = nullptr;
+    return e;
+  }
+  w.bytes = bytes;
+  return cudaSuccess;
+}
+
+void zg_free(ZgWork& w, cudaStream_t s) {
+  if (w.p) {
+    if (w.pooled) cudaFreeAsync(w.p, s);
+    else cudaFree(w.p);
+  }
+  w.p = nullptr;
+  w.bytes = 0;
+}
+
+void zg_pool_trim() {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  for (cudaMemPool_t p : g_pool)
+    if (p) cudaMemPoolTrimTo(p, 0);
+}
+
+}  // namespace tdmrg
