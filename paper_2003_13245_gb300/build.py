@@ -13,7 +13,7 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libtdmrg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU_SOURCES = ["kernels_f64.cu", "zgemm_digits.cu", "qr_blocked.cu", "kernels_tc.cu", "bond_krylov.cu",
+CU_SOURCES = ["kernels_f64.cu", "zgemm_digits.cu", "qr_blocked.cu", "qr_tensor.cu", "kernels_tc.cu", "bond_krylov.cu",
               "lanczos_step.cu", "engine.cu", "step_adjoint.cu", "capi.cu", "noalloc.cu",
               "fgr.cu"]
 CXX_SOURCES = ["model.cpp", "small_exp.cpp"]

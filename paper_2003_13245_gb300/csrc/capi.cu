@@ -1150,13 +1150,18 @@ int tdmrg_kernel_gauge_qr_blocked(int m, int n, const void* Y, int p, const void
     unsigned char* acc = nullptr;
     int* st = status;
     const long long qlen = tdmrg::gauge_qr_blocked_scratch(n, sms);
+    tdmrg::ZgWork qw;
+    qw.pooled = true;
     struct Free {
       tdmrg::QrScratch& w;
       tdmrg::cplx*& qb;
       unsigned char*& acc;
       int*& st;
       bool own;
+      tdmrg::ZgWork& qw;
+      cudaStream_t s;
       ~Free() {
+        tdmrg::zg_free(qw, s);
         if (w.part) cudaFree(w.part);
         if (w.partn) cudaFree(w.partn);
         if (w.bar) cudaFree(w.bar);
@@ -1164,7 +1169,10 @@ int tdmrg_kernel_gauge_qr_blocked(int m, int n, const void* Y, int p, const void
         if (acc) cudaFree(acc);
         if (own && st) cudaFree(st);
       }
-    } fr{W, qb, acc, st, status == nullptr};
+    } fr{W, qb, acc, st, status == nullptr, qw, s};
+    CK(tdmrg::zg_reserve(qw, tdmrg::gauge_qr_tensor_bytes(m, n, sms), s));
+    W.dig = static_cast<unsigned char*>(qw.p);
+    W.dig_bytes = qw.bytes;
     CK(cudaMalloc(&W.part, sizeof(tdmrg::cplx) * 2 * (size_t)sms * (n + 1)));
     CK(cudaMalloc(&W.partn, sizeof(double) * 2 * (size_t)sms));
     CK(cudaMalloc(&W.bar, sizeof(unsigned) * 2));

@@ -456,6 +456,7 @@ Engine::~Engine() {
     if (p) cudaFree(p);
   if (h_mv_) cudaFreeHost(h_mv_);
   zg_free(zws_, st_);
+  zg_free(qws_, st_);
 }
 
 void Engine::rebuild_mpos() {
@@ -580,7 +581,7 @@ void Engine::alloc_mps(DevMps& s, int M) {
   maxxy = std::max(maxxy, (long long)Dmax * maxbond * maxbond);
   ensure_workspace(maxsite, maxxy, maxbond, maxbond);
   if (mixed()) alloc_tc(s);
-  else alloc_zg(s);
+  alloc_zg(s);
   if (maxenv > env_tmp_size_) {
     for (int i = 0; i < 2; ++i) {
       if (env_tmp_[i]) cudaFree(env_tmp_[i]);
@@ -590,8 +591,8 @@ void Engine::alloc_mps(DevMps& s, int M) {
   }
 }
 
-// The digit workspace of the largest contraction of a sweep, so that it does not grow between
-// captured steps (graph mode holds its address).
+// The digit workspaces of the largest contraction and gauge QR of a sweep, so that they do not
+// grow between captured steps (graph mode holds their addresses).
 void Engine::alloc_zg(const DevMps& s) {
   size_t need = 0;
   const int Dm = std::max(H_.maxD, J_.maxD);
@@ -603,9 +604,16 @@ void Engine::alloc_zg(const DevMps& s) {
     need = std::max(need, zgemm_digits_bytes(Mr, Mr, Ml * D, Dm, 1, 1, Dm));
     need = std::max(need, zgemm_digits_bytes(Ml, Ml, D * Mr, Dm, 1, 1, Dm));
   }
-  zws_.fixed = false;
-  CK(zg_reserve(zws_, need, st_));
-  zws_.fixed = graphs_;
+  size_t qneed = 0;
+  for (int k = 0; k < s.L(); ++k) {
+    const int Ml = s.Mb[k], Mr = s.Mb[k + 1], D = s.D[k];
+    qneed = std::max(qneed, gauge_qr_tensor_bytes(Ml * D, Mr, qr_.gmax));
+    qneed = std::max(qneed, gauge_qr_tensor_bytes(D * Mr, Ml, qr_.gmax));
+  }
+  zws_.fixed = qws_.fixed = false;
+  if (!mixed()) CK(zg_reserve(zws_, need, st_));
+  CK(zg_reserve(qws_, qneed, st_));
+  zws_.fixed = qws_.fixed = graphs_;
 }
 
 void Engine::alloc_tc(const DevMps& s) {
@@ -803,6 +811,9 @@ void Engine::check_status() {
 void Engine::gauge_qr_dev(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* R, int* src) {
   const double t0 = tic();
   const bool timed = !capturing_;
+  CK(zg_reserve(qws_, gauge_qr_tensor_bytes(m, n, qr_.gmax), st_));
+  qr_.dig = static_cast<unsigned char*>(qws_.p);
+  qr_.dig_bytes = qws_.bytes;
   if (timed) {
     if (qr_ev_n_ == QR_EV) harvest_qr_events();
     CK(cudaEventRecord(qr_ev_[2 * qr_ev_n_], st_));
@@ -1023,7 +1034,7 @@ void Engine::set_graphs(bool on, int qr_cap) {
     twin_on_ = false;
   }
   graphs_ = on;
-  zws_.fixed = on;
+  zws_.fixed = qws_.fixed = on;
   qr_gcap_ = qr_cap;
   if (on && st_ == 0) {
     if (!own_stream_) CK(cudaStreamCreateWithFlags(&own_stream_, cudaStreamNonBlocking));

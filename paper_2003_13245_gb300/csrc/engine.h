@@ -352,6 +352,7 @@ class Engine {
   cudaEvent_t lz_ev_[2 * QR_EV] = {};
   int lz_ev_n_ = 0;
   ZgWork zws_{};                         // FP64 contractions (digit products)
+  ZgWork qws_{};                         // digits of the gauge QR
   TcBufs tcb_{};
   BondScratch bs_{};
   unsigned long long* h_mv_ = nullptr;   // pinned copy of the device Krylov-vector counter

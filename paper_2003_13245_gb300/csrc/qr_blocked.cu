@@ -390,6 +390,10 @@ cudaError_t gauge_qr_blocked(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cpl
                              cplx* scratch, long long scratch_len, unsigned char* acc,
                              const QrScratch& W, int* status, cudaStream_t s, int gcap,
                              double rank_tol, int* src) {
+  bool taken = false;
+  cudaError_t et = gauge_qr_tensor(m, n, Y, p, E, Q, R, scratch, scratch_len, acc, W, status, s,
+                                   gcap, rank_tol, src, &taken);
+  if (taken || et != cudaSuccess) return et;
   int G = gauge_qr_blocked_grid(m);
   if (gcap > 0 && G > gcap) G = gcap;
   const long long PS = (long long)n * QB + QB + QB * QB;

@@ -1,0 +1,920 @@
+// Gauge QR with its projections on the tensor cores: the factorisation, skipping and completion of
+// qr_blocked.cu (blocked Gram-Schmidt of 16 columns at a time, deterministic completion) in one
+// cooperative launch, with Q^H V, V^H V and Q P taken as exact digit products (the scheme of
+// zgemm_digits.cu) instead of FP64 FMAs.
+//
+// CTA g owns a slice of at most 128 rows of Y, Q and the working block V (shared memory, FP64).
+// The digits of the accepted columns of its slice are kept in global memory in the two operand
+// forms the products need (K = rows for Q^H V, K = columns for Q P); both are private to the CTA
+// and stream through a two-stage ring of bulk copies.  The first form has one scale per column,
+// the second one per row, with a bit to spare: a row that a later column outgrows is written
+// again from Q.
+//
+// Per block of 16 columns, repeated until the projection is negligible (two or three times):
+//  1. digits of V; P = Q^H V (accumulators in TMEM columns 0-255) and V^H V (columns 256-511);
+//     cross-CTA sums of both;
+//  2. V -= Q P.
+// A pass whose coefficients satisfy |P|^2 <= 2^-57 ||v||^2 leaves V^H V valid to rounding; it is the
+// last.  Then, as in qr_blocked.cu, Gram-Schmidt with skips inside the block in Gram form with a
+// guard against cancellation; the triangular inverse is built beside it, so that the new columns
+// are one product V M.  Columns whose projected norm is already below the rank threshold are
+// skipped together.
+//
+// Completion of skipped positions runs the same blocks over the candidates (columns of E, then
+// unit vectors); the first pass rejects every candidate in the span of the accepted columns at
+// once (residual^2 = ||e||^2 - |P|^2 <= 1e-4 ||e||^2), so 16 rejections cost one pass.
+//
+// Bound: latency.  A pass of a block takes ~20 us (four grid barriers of ~1.3 us, two tensor-core
+// products of 4-10 us, reading their levels back, the digits), the serial 16-column factorisation
+// ~16 us and the FP64 product V M 5-10 us; the FP64 work per column no longer grows with the
+// number of accepted columns.
+//
+// Measured on GB300 against qr_blocked.cu (FP64 FMAs), us, columns nearly parallel so that every
+// block takes two passes; "rank 2": all but two columns are completed from 7 n candidates of
+// which n lie in the span:
+//                     152 CTAs                          76 CTAs (two lanes)
+//   m x n        full rank    rank 2              full rank    rank 2
+//   64 x 16       97 / 109     754 / 235
+//   144 x 64     374 / 378    3312 / 661
+//   512 x 128    845 / 859    7934 / 1334
+//   2048 x 128  1156 / 845   12461 / 1351        1658 / 847   12275 / 1351
+//   8192 x 128  2682 / 1022  19468 / 1765        4516 / 1255  25260 / 2302
+// Below nine columns the other kernel is the faster one at full rank (256 x 4: 55 against 95 us),
+// where such bonds, at the ends of a chain, mostly are.  About 32 rows per CTA: fewer rows raise the
+// number of partial sums, more the FP64 product V M.
+#include "umma.cuh"
+
+namespace tdmrg {
+
+using namespace dig;
+
+namespace {
+
+constexpr int QB = 16;                          // columns per block
+constexpr int QT_THREADS = 256;
+constexpr int MAXR = 128;                       // rows of a CTA
+constexpr int MAXN = 128;                       // columns
+constexpr int MINN = 9;                         // fewer: qr_blocked.cu (one block, no projection)
+constexpr int GROUP = 2 * ND * 2 * 128;         // digits of 8 rows x 16 k: 3584 bytes
+constexpr int RING = 16 * GROUP;                // one k step of 128 rows: 57344 bytes
+constexpr int BSTEP = 2 * ND * 2 * 2 * 128;     // 16 columns x 16 k: 7168 bytes
+constexpr int BDIG = 8 * BSTEP;                 // 57344 bytes
+constexpr int E_EMPTY = -100000;
+constexpr int TMEM_COLS = 512;
+constexpr int IM = NL * QB;                     // im levels after the re levels
+
+struct QtArgs {
+  int m, n, p;
+  QrRef Y, E;
+  cplx* Q;
+  cplx* R;
+  cplx* part;               // [G][PS]
+  cplx* fin;                // [PS]
+  int PS;
+  unsigned char* dig;       // per CTA: form 1 then form 2
+  long long dig_cta;        // bytes of one CTA
+  int rows;                 // rows of a CTA
+  unsigned* bar;
+  int* status;
+  long long wait;
+  unsigned char* acc_out;
+  int* src_out;
+  double rank_tol, complete_tol;
+};
+
+__device__ __forceinline__ double wsum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__device__ bool qt_barrier(const QtArgs& A, unsigned& epoch, int* s_ok) {
+  const unsigned G = gridDim.x;
+  __syncthreads();
+  ++epoch;
+  if (threadIdx.x == 0) {
+    volatile unsigned* vbar = A.bar;
+    volatile int* vstat = A.status;
+    const unsigned target = epoch * G;
+    __threadfence();
+    atomicAdd(A.bar, 1u);
+    int ok = 1;
+    const long long t0 = clock64();
+    while (*vbar < target) {
+      if (*vstat) { ok = 0; break; }
+      if (clock64() - t0 > A.wait) {
+        atomicExch(A.status, 1);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+    *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// fin[0..cnt) = sum over the CTAs of part[.][0..cnt) in a fixed order; every CTA sums a slice of the
+// entries
+__device__ bool qt_reduce(const QtArgs& A, int cnt, unsigned& ep, int* s_ok) {
+  const int G = gridDim.x;
+  if (!qt_barrier(A, ep, s_ok)) return false;
+  const int per = (cnt + G - 1) / G;
+  const int lo = blockIdx.x * per, hi = min(cnt, lo + per);
+  // L lanes per entry, so that one round of loads covers the slice where possible
+  int L = 32;
+  while (L > 1 && per * L > QT_THREADS) L >>= 1;
+  const int sub = threadIdx.x & (L - 1);
+  for (int e0 = lo; e0 < hi; e0 += QT_THREADS / L) {
+    const int e = e0 + threadIdx.x / L;
+    double ax = 0.0, ay = 0.0;
+    if (e < hi) {
+      const cplx* src = A.part + e;
+#pragma unroll 4
+      for (int g = sub; g < G; g += L) {
+        const cplx u = __ldcg(src + (long long)g * A.PS);
+        ax += u.x;
+        ay += u.y;
+      }
+    }
+    for (int o = L >> 1; o > 0; o >>= 1) {
+      ax += __shfl_xor_sync(0xffffffffu, ax, o);
+      ay += __shfl_xor_sync(0xffffffffu, ay, o);
+    }
+    if (sub == 0 && e < hi) A.fin[e] = make_double2(ax, ay);
+  }
+  return qt_barrier(A, ep, s_ok);
+}
+
+__device__ __forceinline__ cplx qt_load(const QrRef& Y, long long r, long long c) {
+  const long long off = r * Y.rs + (c < Y.cb ? c * Y.cs : (c % Y.cb) * Y.cs + (c / Y.cb) * Y.cbs);
+  const cplx v = Y.p[off];
+  return Y.conj ? make_double2(v.x, -v.y) : v;
+}
+
+struct Pipe {
+  uint64_t* full;           // [2] ring stages
+  uint64_t* empty;          // [2]
+  uint64_t* done;           // one GEMM's accumulators
+  uint32_t it;              // ring steps used so far
+  uint32_t gemms;           // GEMMs completed so far
+  volatile int* fail;
+  int* status;
+};
+
+// Issued by thread 0.  D += sum over S k steps of A_s B_s: A from `src` (step s at s * stride,
+// `bytes` of it) through the ring, B in shared memory at bdig + s * BSTEP.  conj: Q^H V (re = ArBr
+// + AiBi, im = ArBi - AiBr), else Q P (re = ArBr - AiBi, im = ArBi + AiBr).  gram: also V^H V of
+// the same B tiles into columns 256.. (A = the B tile itself, its rows beyond 16 unused).
+__device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, const unsigned char* bdig,
+                        const unsigned char* src, long long stride, uint32_t bytes, int S,
+                        bool conj, int gram_steps) {
+  bool ok = true;
+  const uint32_t it0 = P.it;
+  int issued = 0;
+  auto load = [&](int s) {
+    const int st = (it0 + s) & 1;
+    mbar_expect_tx(&P.full[st], bytes);
+    bulk_load(ring + st * RING, src + s * stride, bytes, &P.full[st]);
+    ++issued;
+  };
+  auto tile = [&](uint32_t a, uint32_t lbo, uint32_t sbo, uint32_t apart, uint32_t adig, uint32_t b,
+                  uint32_t d, bool first) {
+    const uint64_t br = sdesc(b, ND * 256), bi = sdesc(b + BSTEP / 2, ND * 256);
+#pragma unroll
+    for (int i = 0; i < ND; ++i) {
+      const uint32_t n = QB * (NL - i < ND ? NL - i : ND);
+      const uint32_t acc = (!first || i > 0) ? 1u : 0u;
+      const bool cut = i == 1 && first;          // level 7 starts with digit pair (1, 6)
+      const uint32_t mm = cut ? n - QB : n;
+      const uint64_t ar = sdesc(a + i * adig, lbo, sbo), ai = sdesc(a + apart + i * adig, lbo, sbo);
+      const uint32_t dr = d + i * QB, di = d + IM + i * QB;
+      mma_f16(dr, ar, br, idesc(0, mm), acc);
+      mma_f16(di, ar, bi, idesc(0, mm), acc);
+      if (cut) {
+        mma_f16(dr + mm, ar, sdesc(b + (ND - 1) * 256, ND * 256), idesc(0, QB), 0u);
+        mma_f16(di + mm, ar, sdesc(b + BSTEP / 2 + (ND - 1) * 256, ND * 256), idesc(0, QB), 0u);
+      }
+      mma_f16(dr, ai, bi, idesc(conj ? 0 : 1, n), 1u);
+      mma_f16(di, ai, br, idesc(conj ? 1 : 0, n), 1u);
+    }
+  };
+  for (int s = 0; s < S && s < 2; ++s) load(s);
+  const uint32_t b0 = smem_u32(bdig);
+  for (int s = 0; s < gram_steps; ++s)
+    tile(b0 + s * BSTEP, ND * 256, 128, BSTEP / 2, 256, b0 + s * BSTEP, tmem + 2 * IM, s == 0);
+  for (int s = 0; s < S; ++s) {
+    const int st = (it0 + s) & 1;
+    const uint32_t par = ((it0 + s) >> 1) & 1;
+    if (!mbar_wait(&P.full[st], par, P.fail, P.status, 1)) {
+      ok = false;
+      break;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tile(smem_u32(ring + st * RING), 128, GROUP, GROUP / 2, 256, b0 + s * BSTEP, tmem, s == 0);
+    mma_commit(&P.empty[st]);
+    if (s + 2 < S) {
+      if (!mbar_wait(&P.empty[st], par, P.fail, P.status, 1)) {
+        ok = false;
+        break;
+      }
+      load(s + 2);
+    }
+  }
+  mma_commit(P.done);
+  P.it += S;
+  if (!ok) {
+    // copies in flight land (bounded) before the shared memory can be released
+    int none = 0;
+    for (int s = issued > 2 ? issued - 2 : 0; s < issued; ++s)
+      mbar_wait(&P.full[(it0 + s) & 1], ((it0 + s) >> 1) & 1, &none, P.status, 1);
+  }
+}
+
+// the thread's 8 complex results of one accumulator set: lane = row, columns t0 .. t0 + 7
+__device__ __forceinline__ void qt_read(uint32_t addr, int eA, const int* eB, cplx (&out)[8]) {
+#pragma unroll
+  for (int c0 = 0; c0 < 8; c0 += 4) {
+    const int e[4] = {eB[c0], eB[c0 + 1], eB[c0 + 2], eB[c0 + 3]};
+    double x[2][4];
+    read_levels4<2>(addr + c0, QB, IM, eA, e, x);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) out[c0 + c] = make_double2(x[0][c], x[1][c]);
+  }
+}
+
+// 4 consecutive k of one part (re or im) of a row as digits: 8-byte stores, 256 bytes per digit
+__device__ __forceinline__ void qt_store(const cplx* x, int stride, int live, int part, int emax,
+                                         bool bad, unsigned char* dst) {
+  unsigned long long w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    w[i] = i < live ? digits_of(part == 0 ? x[i * stride].x : x[i * stride].y, emax, false, bad)
+                    : 0x0080808080808080ULL;
+#pragma unroll
+  for (int l = 0; l < ND; ++l)
+    *reinterpret_cast<uint2*>(dst + l * 256) =
+        make_uint2(digit_pair(w[0], w[1], l), digit_pair(w[2], w[3], l));
+}
+
+struct Shared {
+  cplx G[QB][QB];            // Gram matrix of the block
+  cplx R[QB][QB];            // its triangular factor
+  cplx M[QB][QB];            // and the inverse
+  cplx u[2][QB], y[QB];      // factors of one step (u of alternate steps)
+  double inv;
+  double quarter[QB];        // a quarter of the projected norm^2
+  double hh[8][QB];          // partial sums of |P|^2
+  double lim[QB];            // completion: smallest residual norm of a candidate that is taken
+  int em[QB];                // largest biased exponent of a column (digit scale)
+  int ev[QB];                // its digit scale E
+  int idx[MAXN];             // column of Q of every accepted vector, in order of acceptance
+  int ec[MAXN];              // form 1: scale of every accepted vector (this CTA's rows)
+  int er[MAXR];              // form 2: scale of every row (E_EMPTY: nothing but zeros so far)
+  int rnew[MAXR];            // largest biased exponent of a row's new entries
+  int acc[MAXN];             // accepted (main factorisation) or filled (completion)
+  int take[QB];
+  int src[QB];               // block column of the block's i-th accepted vector
+  int drop[QB];              // skipped before the in-block factorisation
+  double red[32];
+  int ok, fail, done, stop, last, any;
+  uint32_t tmem;
+  uint64_t bar[5];
+};
+
+}  // namespace
+
+__global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A) {
+  extern __shared__ unsigned char raw[];
+  unsigned char* base =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~(uintptr_t)127);
+  unsigned char* ring = base;                                   // 2 * RING
+  unsigned char* bdig = base + 2 * RING;                        // BDIG
+  cplx* V = reinterpret_cast<cplx*>(bdig + BDIG);               // [QB][MAXR + 1]
+  constexpr int LDV = MAXR + 1;
+  cplx* H = reinterpret_cast<cplx*>(ring + RING);               // [MAXN][QB], in stage 1
+  __shared__ Shared S;
+
+  const int m = A.m, n = A.n;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r0 = blockIdx.x * A.rows;
+  const int nr = max(0, min(m, r0 + A.rows) - r0);
+  const int rsteps = (A.rows + 15) / 16, rgroups = (A.rows + 7) / 8;
+  const int ngroups = (n + 7) / 8;
+  unsigned char* d1 = A.dig + blockIdx.x * A.dig_cta;           // [rstep][column group][GROUP]
+  unsigned char* d2 = d1 + (long long)rsteps * ngroups * GROUP; // [column step][row group][GROUP]
+  const long long s1 = (long long)ngroups * GROUP, s2 = (long long)rgroups * GROUP;
+  cplx* mypart = A.part + (long long)blockIdx.x * A.PS;
+  unsigned ep = 0;
+  bool alive = true;
+
+  Pipe P{&S.bar[0], &S.bar[2], &S.bar[4], 0, 0, &S.fail, A.status};
+  if (tid == 0) {
+    for (int i = 0; i < 5; ++i) mbar_init(&S.bar[i], 1);
+    S.fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&S.tmem)),
+                 "r"(TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (blockIdx.x == 0)
+    for (int e = tid; e < n * n; e += QT_THREADS) A.R[e] = make_double2(0.0, 0.0);
+  for (int i = tid; i < n; i += QT_THREADS) S.acc[i] = 0;
+  for (int i = tid; i < MAXR; i += QT_THREADS) S.er[i] = E_EMPTY;
+  // ||Y||_F (summed over the CTAs with the first block's Gram matrix)
+  {
+    double s = 0.0;
+    for (long long e = tid; e < (long long)nr * n; e += QT_THREADS) {
+      const bool cfast = A.Y.cs == 1;
+      const int r = (int)(cfast ? e / n : e % nr), c = (int)(cfast ? e % n : e / nr);
+      const cplx y = qt_load(A.Y, r0 + r, c);
+      s = fma(y.x, y.x, fma(y.y, y.y, s));
+    }
+    s = wsum(s);
+    if (lane == 0) S.red[warp] = s;
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int w = 0; w < QT_THREADS / 32; ++w) t += S.red[w];
+      mypart[QB * QB] = make_double2(t, 0.0);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = S.tmem;
+  double thr = 0.0, thr2 = 0.0;       // known after the first reduction
+  int na = 0;               // accepted vectors
+  int j0 = 0;               // next column of Y (main) -- n when the factorisation is done
+  int open = 0;             // completion: next position to look at
+  long long cand = 0;       // completion: next candidate
+  bool main_phase = true, started = false;
+
+  while (alive) {
+    int bsz;
+    if (main_phase) {
+      bsz = min(QB, n - j0);
+    } else {
+      if (na >= n) break;
+      const long long left = (long long)A.p + m - cand;
+      if (left <= 0) {
+        if (tid == 0 && blockIdx.x == 0) atomicExch(A.status, 2);
+        break;
+      }
+      bsz = (int)(left < QB ? left : QB);
+    }
+    // ---- load the block (missing columns are zero)
+    {
+      const QrRef& src = main_phase ? A.Y : A.E;
+      const long long c0 = main_phase ? j0 : cand;
+      const bool rfast = src.rs == 1;
+      for (int e = tid; e < QB * nr; e += QT_THREADS) {
+        const int t = rfast ? e / nr : e % QB, r = rfast ? e % nr : e / QB;
+        cplx v = make_double2(0.0, 0.0);
+        if (t < bsz) {
+          if (main_phase || c0 + t < A.p) v = qt_load(src, r0 + r, c0 + t);
+          else if (c0 + t - A.p == r0 + r) v.x = 1.0;
+        }
+        V[t * LDV + r] = v;
+      }
+    }
+    if (tid < QB) S.drop[tid] = tid < bsz ? 0 : 1;
+    __syncthreads();
+    // ---- projection passes
+    cplx racc[MAXN / QB];
+    bool all_dropped = false;
+    for (int pass = 0; pass < 4; ++pass) {
+      // digits of V, one scale per column (two columns per warp)
+      const bool gram = pass > 0 || na == 0;
+      {
+        int e2[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int t = 2 * warp + u;
+          int e = 0;
+          double s = 0.0;
+          for (int r = lane; r < nr; r += 32) {
+            const cplx v = V[t * LDV + r];
+            e = max(e, max(bexp(v.x), bexp(v.y)));
+            if (!gram) s = fma(v.x, v.x, fma(v.y, v.y, s));
+          }
+          e2[u] = __reduce_max_sync(0xffffffffu, e);
+          if (!gram) {                     // the norms alone (the first pass needs no more)
+            s = wsum(s);
+            if (lane == 0) mypart[na * QB + t] = make_double2(s, 0.0);
+          }
+          if (lane == 0) S.ev[t] = e2[u] == 0x7ff ? E_NONFINITE : max(e2[u], 1) - 1022;
+        }
+        for (int k = lane; k < 16 * rsteps; k += 32) {     // column, part, group of 4 rows
+          const int u = k & 1, part = (k >> 1) & 1, q = k >> 2;
+          const int t = 2 * warp + u, em = u ? e2[1] : e2[0];
+          qt_store(V + t * LDV + q * 4, 1, min(4, nr - q * 4), part, max(em, 1), em == 0x7ff,
+                   bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
+                       t * 16 + (q & 1) * 8);
+        }
+      }
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncthreads();
+      if (tid == 0)
+        qt_gemm(P, tmem, ring, bdig, d1, s1, (uint32_t)((na + 7) / 8 * GROUP), na > 0 ? rsteps : 0,
+                true, gram ? rsteps : 0);
+      __syncwarp();
+      alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
+      ++P.gemms;
+      alive = __syncthreads_and(alive ? 1 : 0) != 0;
+      if (!alive) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      {
+        const int quad = warp & 3, t0 = (warp >> 2) * 8;
+        const int row = quad * 32 + lane;
+        const uint32_t addr = tmem + ((uint32_t)(quad * 32) << 16) + t0;
+        cplx out[8];
+        if (quad * 32 < na) {
+          qt_read(addr, S.ec[min(row, na - 1)], S.ev + t0, out);
+          if (row < na)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) mypart[row * QB + t0 + c] = out[c];
+        }
+        if (gram && quad == 0) {
+          qt_read(addr + 2 * IM, S.ev[lane & 15], S.ev + t0, out);
+          if (lane < QB)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) mypart[na * QB + lane * QB + t0 + c] = out[c];
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (!qt_reduce(A, na * QB + (gram ? QB * QB : QB) + (started ? 0 : 1), ep, &S.ok)) {
+        alive = false;
+        break;
+      }
+      if (!started) {
+        started = true;
+        const double y2 = __ldcg(&A.fin[QB * QB]).x;
+        if (!(y2 < 1.7976931348623157e308)) {
+          // Inf or NaN in Y: every column is skipped
+          bsz = n;
+          all_dropped = true;
+          break;
+        }
+        thr = A.rank_tol * sqrt(y2);
+        thr2 = thr * thr;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // P into shared memory, |P|^2 and its scale per column
+      cplx hreg[MAXN / QB];
+      {
+        const int t = tid & 15, q = tid >> 4;
+        if (tid < QB) S.em[tid] = 0;
+#pragma unroll
+        for (int k = 0; k < MAXN / QB; ++k)
+          hreg[k] = k * QB + q < na ? __ldcg(&A.fin[(k * QB + q) * QB + t]) : make_double2(0.0, 0.0);
+        if (gram) S.G[q][t] = __ldcg(&A.fin[na * QB + tid]);
+        else if (q == 0) S.G[t][t] = __ldcg(&A.fin[na * QB + t]);
+        __syncthreads();
+        int e = 0;
+#pragma unroll
+        for (int k = 0; k < MAXN / QB; ++k)
+          if (k * QB < na) {
+            const cplx h = hreg[k];
+            if (k * QB + q < na) H[(k * QB + q) * QB + t] = h;
+            e = max(e, max(bexp(h.x), bexp(h.y)));
+          }
+        atomicMax(&S.em[t], e);
+      }
+      // |P|^2, R's coefficients and what to do with each column; rejections of candidates are
+      // wanted before Q P, all else runs while the tensor cores form it
+      auto decide = [&] {
+        const int t = tid & 15;
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < MAXN / QB; ++k)
+          if (k * QB < na) s = fma(hreg[k].x, hreg[k].x, fma(hreg[k].y, hreg[k].y, s));
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (lane < 16) S.hh[warp][t] = s;
+        // R accumulates over the passes in registers (CTA 0 writes it)
+        if (main_phase && blockIdx.x == 0)
+#pragma unroll
+          for (int k = 0; k < MAXN / QB; ++k)
+            if (k * QB < na) {
+              if (pass == 0) racc[k] = hreg[k];
+              else racc[k] = make_double2(racc[k].x + hreg[k].x, racc[k].y + hreg[k].y);
+            }
+        __syncthreads();
+        if (tid < QB) {
+          const double vv = S.G[tid][tid].x;
+          double h = 0.0;
+          for (int w = 0; w < QT_THREADS / 32; ++w) h += S.hh[w][tid];
+          int drop = S.drop[tid];
+          if (main_phase) {
+            if (!(vv > thr2)) drop = 1;
+          } else if (pass == 0) {
+            S.lim[tid] = A.complete_tol * sqrt(vv);
+            // in the span of the accepted vectors (or zero, or not finite)
+            if (!(vv - h > A.complete_tol * A.complete_tol * vv)) drop = 1;
+          }
+          S.drop[tid] = drop;
+          S.quarter[tid] = 0.25 * vv;
+          // the Gram matrix stands when the projection leaves it unchanged to rounding
+          const bool more = !drop && (!gram || h > 6.9e-18 * vv);
+          const unsigned mm = __ballot_sync(0xffffu, more), dd = __ballot_sync(0xffffu, !drop);
+          if (tid == 0) {
+            S.last = mm == 0;
+            S.any = dd != 0;
+          }
+        }
+        __syncthreads();
+      };
+      const bool first = na == 0 || (!main_phase && pass == 0);
+      if (first) {
+        decide();
+        if (!S.any) {
+          all_dropped = true;
+          break;
+        }
+      } else {
+        __syncthreads();
+      }
+      if (na > 0) {
+        // V -= Q P
+        const int isteps = (na + 15) / 16;
+        {
+          const int t = tid & 15;
+          const int em = max(S.em[t], 1);
+          const bool bad = em == 0x7ff;
+          if (tid < QB) S.ev[t] = bad ? E_NONFINITE : em - 1022;
+          for (int k = tid >> 4; k < 8 * isteps; k += 16) {     // part, group of 4 columns of Q
+            const int part = k & 1, q = k >> 1;
+            qt_store(H + q * 4 * QB + t, QB, min(4, na - q * 4), part, em, bad,
+                     bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
+                         t * 16 + (q & 1) * 8);
+          }
+        }
+        asm volatile("fence.proxy.async;" ::: "memory");
+        __syncthreads();
+        if (tid == 0)
+          qt_gemm(P, tmem, ring, bdig, d2, s2, (uint32_t)s2, isteps, false, 0);
+        __syncwarp();
+        if (!first) decide();
+        alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
+        ++P.gemms;
+        alive = __syncthreads_and(alive ? 1 : 0) != 0;
+        if (!alive) break;
+        if (!S.any) {
+          all_dropped = true;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int quad = warp & 3, t0 = (warp >> 2) * 8;
+        if (quad * 32 < nr) {
+          cplx out[8];
+          const int r = quad * 32 + lane;
+          qt_read(tmem + ((uint32_t)(quad * 32) << 16) + t0, S.er[min(r, nr - 1)], S.ev + t0, out);
+          if (r < nr)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              cplx& v = V[(t0 + c) * LDV + r];
+              v = make_double2(v.x - out[c].x, v.y - out[c].y);
+            }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      }
+      if (S.last) break;
+    }
+    if (!alive) break;
+    if (all_dropped) {
+      if (main_phase) {
+        if (blockIdx.x == 0) {
+          const int t = tid & 15, q = tid >> 4;
+#pragma unroll
+          for (int k = 0; k < MAXN / QB; ++k)
+            if (k * QB + q < na && t < bsz)
+              A.R[(long long)S.idx[k * QB + q] * n + j0 + t] = racc[k];
+        }
+        j0 += bsz;
+      } else {
+        cand += bsz;
+      }
+    } else {
+      // ---- Gram-Schmidt with skips inside the block (Gram form, right-looking), the inverse of
+      // the triangular factor beside it.  Thread e holds the pair (a, b), a <= b, numbered by
+      // falling b: at step s the pairs with b > s are the first ones.  It carries G_ab until row a
+      // is taken (then R_ab), and the inverse's M_ab from then on; both are updated by the same
+      // product of a column factor u_a (conj(R_sa) for a > s, M_as for a <= s) and R_sb.
+      const int room = n - na;             // completion: positions left
+      if (warp < 5) {
+        int b = QB - 1, rem = tid;
+        while (b >= 0 && rem > b) rem -= b-- + 1;
+        const int a = rem;                 // b < 0: no pair
+        cplx g = b >= 0 ? S.G[a][b] : make_double2(0.0, 0.0);
+        int taken = 0, s = 0;
+        for (; s < bsz; ++s) {
+          if (a == s && b == s) {
+            // positive doubles compare like their bits (a negative rho is below everything):
+            // integer comparisons keep the FP64 pipe out of the serial chain
+            const double rho = g.x;
+            const long long rb = __double_as_longlong(rho);
+            int take = 0;
+            double inv = 0.0, nrm = 0.0;
+            if (!main_phase && taken >= room) take = -1;
+            else if (!S.drop[s]) {
+              // cancellation inside the block: this column starts the next block
+              if (taken > 0 && rb < __double_as_longlong(S.quarter[s])) take = -1;
+              else if (rb > 0) {
+                inv = bexp(rho) > 0 ? rsqrt_series(rho) : rsqrt(rho);
+                nrm = rho * inv;
+                const double lim = main_phase ? thr : S.lim[s];
+                take = __double_as_longlong(nrm) > __double_as_longlong(lim) ? 1 : 0;
+                if (!take) inv = 0.0;
+              }
+            }
+            S.take[s] = take;
+            S.inv = inv;
+            if (take >= 0) S.R[s][s] = make_double2(take ? nrm : 0.0, 0.0);
+            S.M[s][s] = make_double2(take > 0 ? inv : 0.0, 0.0);
+            S.u[s & 1][s] = make_double2(inv, 0.0);
+          }
+          asm volatile("bar.sync 1, 160;" ::: "memory");
+          const int take = S.take[s];
+          if (take < 0) break;
+          if (take > 0) {
+            const double inv = S.inv;
+            ++taken;
+            if (a == s && b > s) {         // row s of R
+              g = make_double2(g.x * inv, g.y * inv);
+              S.R[s][b] = g;
+              S.y[b] = g;
+              S.u[s & 1][b] = make_double2(g.x, -g.y);
+              g = make_double2(0.0, 0.0);
+            } else if (b == s && a < s) {  // column s of the inverse
+              g = make_double2(g.x * inv, g.y * inv);
+              S.M[a][s] = g;
+              S.u[s & 1][a] = g;
+            }
+            asm volatile("bar.sync 1, 160;" ::: "memory");
+            if (b > s) {
+              const cplx u = S.u[s & 1][a], y = S.y[b];
+              g.x = fma(-u.x, y.x, g.x);
+              g.x = fma(u.y, y.y, g.x);
+              g.y = fma(-u.x, y.y, g.y);
+              g.y = fma(-u.y, y.x, g.y);
+            }
+          } else {
+            if (a == s && b > s) {
+              S.R[s][b] = make_double2(0.0, 0.0);
+              g = make_double2(0.0, 0.0);
+            } else if (b == s && a < s) {
+              S.M[a][s] = make_double2(0.0, 0.0);
+            }
+            asm volatile("bar.sync 1, 160;" ::: "memory");
+          }
+        }
+        if (tid == 0) S.done = s;
+      }
+      __syncthreads();
+      const int done = S.done;
+      // ---- the new columns q_t = sum_{s <= t} v_s M_st: warp w takes columns w and 15 - w, the
+      // lanes the rows (MAXR / 32 rows each)
+      {
+        cplx q[2][MAXR / 32];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int t = u == 0 ? warp : QB - 1 - warp;
+          const bool on = t < done && S.take[t] > 0;
+#pragma unroll
+          for (int k = 0; k < MAXR / 32; ++k) {
+            q[u][k] = make_double2(0.0, 0.0);
+            const int r = k * 32 + lane;
+            if (on && k * 32 < nr) {
+              double x = 0.0, y = 0.0, x2 = 0.0, y2b = 0.0;
+              for (int s = 0; s <= t; ++s) {
+                if (S.take[s] <= 0) continue;      // (a skipped vector may hold Inf or NaN)
+                const cplx v = V[s * LDV + min(r, nr - 1)], c = S.M[s][t];
+                x = fma(v.x, c.x, x);
+                x2 = fma(-v.y, c.y, x2);
+                y = fma(v.x, c.y, y);
+                y2b = fma(v.y, c.x, y2b);
+              }
+              q[u][k] = make_double2(x + x2, y + y2b);
+            }
+          }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int t = u == 0 ? warp : QB - 1 - warp;
+          if (t < done && S.take[t] > 0)
+#pragma unroll
+            for (int k = 0; k < MAXR / 32; ++k) {
+              const int r = k * 32 + lane;
+              if (r < nr) V[t * LDV + r] = q[u][k];
+            }
+        }
+        __syncthreads();
+      }
+      // ---- bookkeeping: S.em[t] = position of column t among the accepted vectors, -1 if none
+      if (tid == 0) {
+        int a = na, pos = open;
+        for (int t = 0; t < QB; ++t) S.em[t] = -1;
+        for (int t = 0; t < done; ++t) {
+          if (S.take[t] <= 0) continue;
+          int col;
+          if (main_phase) {
+            col = j0 + t;
+          } else {
+            while (S.acc[pos]) ++pos;
+            col = pos;
+            if (A.src_out && blockIdx.x == 0) A.src_out[col] = (int)(cand + t);
+          }
+          S.acc[col] = 1;
+          S.idx[a] = col;
+          S.src[a - na] = t;
+          S.em[t] = a++;
+        }
+        S.any = a;
+        S.last = pos;
+      }
+      __syncthreads();
+      const int na1 = S.any;
+      open = S.last;
+      // digits of the new columns are wanted while a column or a position is left
+      const bool more = na1 < n;
+      // form 2 is written two bytes at a time: a k step is cleared when its first column comes
+      // (its unused columns must be zero)
+      if (more)
+        for (int k = (na + 15) / 16; k * 16 < na1; ++k)
+          for (int e = tid; e < s2 / 16; e += QT_THREADS)
+            reinterpret_cast<uint4*>(d2 + k * s2)[e] = make_uint4(0u, 0u, 0u, 0u);
+      // ---- Q in FP64, and its digits in both operand forms
+      for (int r = tid; r < nr; r += QT_THREADS) S.rnew[r] = 0;
+      if (tid < QB) S.ev[tid] = 0;
+      __syncthreads();
+      for (int e = tid; e < QB * nr; e += QT_THREADS) {
+        const int t = e % QB, r = e / QB;
+        const int a = S.em[t];
+        if (a >= 0) {
+          const cplx v = V[t * LDV + r];
+          A.Q[(long long)(r0 + r) * n + S.idx[a]] = v;
+          const int ex = max(bexp(v.x), bexp(v.y));
+          atomicMax(&S.rnew[r], ex);
+          atomicMax(&S.ev[t], ex);
+        }
+      }
+      __syncthreads();
+      {
+        const int t = tid & 15, g = tid >> 4;
+        const int a = S.em[t];
+        if (more && a >= 0) {
+          const int em = max(S.ev[t], 1);
+          if (g == 0) S.ec[a] = em - 1022;
+          for (int k = g; k < 8 * rsteps; k += 16) {
+            const int part = k & 1, q = k >> 1;
+            qt_store(V + t * LDV + q * 4, 1, min(4, nr - q * 4), part, em, em == 0x7ff,
+                     d1 + (q >> 2) * s1 + (a >> 3) * GROUP + part * (GROUP / 2) +
+                         ((q >> 1) & 1) * 128 + (a & 7) * 16 + (q & 1) * 8);
+          }
+        }
+        for (int r = g; more && r < nr; r += 16) {
+          // this row's scale; outgrown: all its columns again (the 16 threads of a row agree)
+          int er = S.er[r];
+          const int en = S.rnew[r] - 1022;
+          const bool grown = S.rnew[r] > 0 && en > er;
+          if (grown) er = en + 1;
+          const int first = grown ? 0 : na;
+          for (int c = first + t; c < na1; c += 16) {
+            const cplx v = c < na ? A.Q[(long long)(r0 + r) * n + S.idx[c]]
+                                  : V[S.src[c - na] * LDV + r];
+            unsigned char* dst = d2 + (c >> 4) * s2 + (r >> 3) * GROUP + ((c >> 3) & 1) * 128 +
+                                 (r & 7) * 16 + (c & 7) * 2;
+            const unsigned long long wr = digits_of(v.x, er + 1022, false, false);
+            const unsigned long long wi = digits_of(v.y, er + 1022, false, false);
+#pragma unroll
+            for (int l = 0; l < ND; ++l) {
+              const uint32_t d = digit_pair(wr, wi, l);
+              *reinterpret_cast<unsigned short*>(dst + l * 256) = (unsigned short)d;
+              *reinterpret_cast<unsigned short*>(dst + GROUP / 2 + l * 256) =
+                  (unsigned short)(d >> 16);
+            }
+          }
+          __syncwarp(0xffffu << (lane & 16));      // the row's 16 threads (the other half may be done)
+          if (t == 0) S.er[r] = er;
+        }
+      }
+      if (main_phase && blockIdx.x == 0)
+        for (int e = tid; e < done * done; e += QT_THREADS) {
+          const int s = e / done, t = e % done;
+          if (s <= t) A.R[(long long)(j0 + s) * n + j0 + t] = S.R[s][t];
+        }
+      if (main_phase && blockIdx.x == 0) {
+        const int t = tid & 15, q = tid >> 4;
+#pragma unroll
+        for (int k = 0; k < MAXN / QB; ++k)
+          if (k * QB + q < na && t < done)
+            A.R[(long long)S.idx[k * QB + q] * n + j0 + t] = racc[k];
+      }
+      na = na1;
+      if (main_phase) j0 += done;
+      else cand += done;
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncthreads();
+    }
+    if (main_phase && j0 >= n) {
+      main_phase = false;
+      if (blockIdx.x == 0)
+        for (int i = tid; i < n; i += QT_THREADS) A.acc_out[i] = (unsigned char)S.acc[i];
+    }
+    __syncthreads();
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(TMEM_COLS));
+  }
+}
+
+namespace {
+struct QtPlan {
+  int G, rows;
+  long long dig_cta;
+};
+// about 32 rows per CTA, at most MAXR
+bool qt_plan(int m, int n, int cap, QtPlan& p) {
+  if (n > MAXN || n < MINN || cap < 1) return false;
+  long long g = ((long long)m + 31) / 32;
+  if (g > cap) g = cap;
+  p.rows = (int)((m + g - 1) / g);
+  if (p.rows > MAXR) return false;
+  p.G = (m + p.rows - 1) / p.rows;
+  p.dig_cta = ((long long)((p.rows + 15) / 16) * ((n + 7) / 8) +
+               (long long)((n + 15) / 16) * ((p.rows + 7) / 8)) * GROUP;
+  return true;
+}
+constexpr size_t QT_SMEM = 2 * (size_t)RING + BDIG + sizeof(cplx) * QB * (MAXR + 1) + 128;
+}  // namespace
+
+size_t gauge_qr_tensor_bytes(int m, int n, int sms) {
+  if (n > MAXN || n < MINN || m > (long long)MAXR * sms) return 0;
+  const long long G = (m + 31) / 32 < sms ? (m + 31) / 32 : sms;
+  return (size_t)((m + 16 * G) * ((n + 7) / 8) / 16 + (m + 8 * G) * (long long)((n + 15) / 16) / 8 +
+                  32) * GROUP;
+}
+
+cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* R, cplx* scratch,
+                            long long scratch_len, unsigned char* acc, const QrScratch& W,
+                            int* status, cudaStream_t s, int gcap, double rank_tol, int* src,
+                            bool* taken) {
+  *taken = false;
+  int cap = W.gmax;
+  if (gcap > 0 && gcap < cap) cap = gcap;
+  QtPlan pl;
+  if (!W.dig || !qt_plan(m, n, cap, pl)) return cudaSuccess;
+  const long long PS = (long long)n * QB + QB + QB * QB;
+  if ((size_t)pl.G * pl.dig_cta > W.dig_bytes || pl.G * PS + PS > scratch_len) return cudaSuccess;
+  static bool attr = false;
+  cudaError_t e;
+  if (!attr) {
+    e = cudaFuncSetAttribute(gauge_qr_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)QT_SMEM);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  if ((e = cudaMemsetAsync(W.bar, 0, 2 * sizeof(unsigned), s)) != cudaSuccess) return e;
+  QtArgs a{};
+  a.m = m; a.n = n; a.p = p;
+  a.Y = Y; a.E = p > 0 ? E : Y;
+  a.Q = Q; a.R = R;
+  a.part = scratch;
+  a.fin = scratch + (long long)pl.G * PS;
+  a.PS = (int)PS;
+  a.dig = W.dig;
+  a.dig_cta = pl.dig_cta;
+  a.rows = pl.rows;
+  a.bar = W.bar;
+  a.status = status;
+  a.wait = W.wait > 0 ? W.wait : kBarrierWaitCycles;
+  a.acc_out = acc;
+  a.src_out = src;
+  a.rank_tol = rank_tol;
+  a.complete_tol = 1e-2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pl.G);
+  cfg.blockDim = dim3(QT_THREADS);
+  cfg.dynamicSmemBytes = QT_SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  count_launch();
+  *taken = true;
+  return cudaLaunchKernelEx(&cfg, gauge_qr_tensor_kernel, a);
+}
+
+}  // namespace tdmrg

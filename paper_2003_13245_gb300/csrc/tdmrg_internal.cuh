@@ -143,6 +143,9 @@ struct QrScratch {
   int gmax = 0;
   int nmax = 0;
   long long wait = 0;         // grid-barrier wait limit in clock cycles (0: ~2 s)
+  // digits of Q for the tensor-core factorisation (gauge_qr_tensor_bytes; none: it is not used)
+  unsigned char* dig = nullptr;
+  size_t dig_bytes = 0;
 };
 // the default limit of every bounded grid-barrier wait: about 2 s at 2 GHz
 constexpr long long kBarrierWaitCycles = 4000000000LL;
@@ -170,6 +173,15 @@ cudaError_t gauge_qr_blocked(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cpl
                              cplx* scratch, long long scratch_len, unsigned char* acc,
                              const QrScratch& W, int* status, cudaStream_t s, int gcap = 0,
                              double rank_tol = 1e-12, int* src = nullptr);
+
+// the factorisation and completion of gauge_qr_blocked with the projections on the tensor cores
+// (qr_tensor.cu), one launch; *taken = false and nothing launched when the factor does not fit it
+// (n > 128, more than 128 rows per CTA, no digit workspace)
+cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* R, cplx* scratch,
+                            long long scratch_len, unsigned char* acc, const QrScratch& W,
+                            int* status, cudaStream_t s, int gcap, double rank_tol, int* src,
+                            bool* taken);
+size_t gauge_qr_tensor_bytes(int m, int n, int sms);
 
 // dst[j][i] = conj?(src[i][j]) for an m x n source.
 cudaError_t ztranspose(int m, int n, const cplx* src, cplx* dst, int conj, cudaStream_t s);

@@ -30,16 +30,16 @@
 // FMA kernel: 896 x 8192 x 128 0.28 against 6.2 ms (27 TFLOP/s, tensor pipe 39 %); 8192 x 128 x 128
 // summed over seven channels 0.35 against 7.3 ms; 128 x 128 x 8192, seven batches, 0.55 against
 // 34 ms; 64 x 64 x 256, seven batches, 35 against 1048 us; 16 x 16 x 4 21 against 68 us.
-#include "tdmrg_internal.cuh"
+#include "umma.cuh"
 
 #include <mutex>
 
 namespace tdmrg {
 
+using namespace dig;
+
 namespace {
 
-constexpr int ND = 7;                         // digits
-constexpr int NL = 8;                         // levels i + j kept
 constexpr int PT = 128, QT = 32;              // tile rows (operand P) and columns (operand Q)
 constexpr int KS = 16;                        // k per stage
 constexpr int KC = 128;                       // k per chunk (one scale per row and chunk)
@@ -51,8 +51,6 @@ constexpr int NST = 3;
 constexpr int GEMM_THREADS = 320;             // TMA warp, MMA warp, eight epilogue warps
 constexpr size_t GEMM_SMEM = (size_t)NST * STAGE + 256 + 128;
 constexpr int TMEM_COLS = 512;
-constexpr int E_NONFINITE = 1 << 20;          // scale of a row that holds an Inf or a NaN
-constexpr long long WAIT_CYCLES = 4000000000LL;
 
 struct Operand {
   const cplx* p;
@@ -109,8 +107,7 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const cplx v = mine[i];
-    e = max(e, (__double2hiint(v.x) >> 20) & 0x7ff);
-    e = max(e, (__double2hiint(v.y) >> 20) & 0x7ff);
+    e = max(e, max(bexp(v.x), bexp(v.y)));
   }
   atomicMax(&s_e[r], e);
   __syncthreads();
@@ -132,35 +129,13 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
   for (int part = 0; part < 2; ++part) {
     unsigned long long w[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const double x = part == 0 ? mine[i].x : mine[i].y;
-      const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-      const int ex = (int)(bits >> 52) & 0x7ff;
-      unsigned long long mant = bits & 0xfffffffffffffULL;
-      if (ex) mant |= 1ULL << 52;
-      const int sh = max(ex, 1) - emax + 2;
-      unsigned long long v;
-      if (sh >= 0) v = mant << sh;
-      else if (sh >= -54) v = (mant + (1ULL << (-sh - 1))) >> (-sh);
-      else v = 0;
-      if (bad) v = 0;
-      const bool neg = ((bits >> 63) != 0) != (part == 1 && o.conj != 0);
-      w[i] = (neg ? 0ULL - v : v) + 0x0080808080808080ULL;
-    }
+    for (int i = 0; i < 8; ++i)
+      w[i] = digits_of(part == 0 ? mine[i].x : mine[i].y, emax, part == 1 && o.conj != 0, bad);
 #pragma unroll
     for (int l = 0; l < ND; ++l) {
       uint32_t h[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t mask = l == 0 ? 0xffffu : 0xffu;
-        const uint32_t a = (uint32_t)(w[2 * q] >> (48 - 8 * l)) & mask;
-        const uint32_t c2 = (uint32_t)(w[2 * q + 1] >> (48 - 8 * l)) & mask;
-        // 0x6400 + u is the fp16 number 1024 + u; subtracting 1152 leaves the signed digit
-        const uint32_t pk = (0x64006400u + a) + (c2 << 16);
-        uint32_t d;
-        asm("sub.f16x2 %0, %1, %2;" : "=r"(d) : "r"(pk), "r"(0x64806480u));
-        h[q] = d;
-      }
+      for (int q = 0; q < 4; ++q) h[q] = digit_pair(w[2 * q], w[2 * q + 1], l);
       long long off;
       if (wide)                      // [part][digit][k half][row group][8 rows][16 B]
         off = (((part * ND + l) * 2 + kh) * (PT / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
@@ -169,108 +144,6 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
       *reinterpret_cast<uint4*>(dst + off) = make_uint4(h[0], h[1], h[2], h[3]);
     }
   }
-}
-
-// ------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait (about 2 s); gives up at once when another role of the CTA has
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* fail,
-                                          int* status) {
-  if (mbar_try(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try(bar, parity)) {
-    if (*fail) return false;
-    if (clock64() - t0 > WAIT_CYCLES) {
-      *fail = 1;
-      atomicExch(status, 3);
-      return false;
-    }
-  }
-  return true;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
-                                          uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-// K-major operand without swizzle: 8-row x 16-byte core matrices, `lbo` bytes between the two of
-// a k step, 128 bytes between row groups
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)(lbo >> 4) << 16;
-  d |= (uint64_t)(128 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-// D f32, A and B fp16, both K-major, M = 128
-__host__ __device__ constexpr uint32_t idesc(int negA, int n) {
-  return (1u << 4) | ((uint32_t)negA << 13) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(PT >> 4) << 24);
-}
-__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id,
-                                        uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(id), "r"(acc));
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7])
-      : "r"(taddr));
-}
-
-// T * 2^e, |T| < 2^63, rounded to nearest: integer arithmetic while the result is a normal number
-__device__ __forceinline__ double pack(long long T, int e) {
-  if (T == 0) return 0.0;
-  const unsigned long long u = T < 0 ? 0ULL - (unsigned long long)T : (unsigned long long)T;
-  const int lz = __clzll((long long)u);
-  const int be = e + 63 - lz + 1023;               // biased exponent
-  if (be < 1 || be > 2045) {                       // rare: let the library round and saturate
-    return scalbn((double)T, e);
-  }
-  const unsigned long long m = u << lz;
-  const unsigned long long rnd = (m >> 11) + ((m & 0x400) && ((m & 0xbff) != 0) ? 1 : 0);
-  unsigned long long bits = ((unsigned long long)(be - 1) << 52) + rnd;   // the hidden bit adds 1
-  if (T < 0) bits |= 1ULL << 63;
-  return __longlong_as_double((long long)bits);
 }
 
 struct GemmArgs {
@@ -346,7 +219,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
       const int ns = min(STEPS, A.ksteps - c * STEPS);
       for (int k = 0; k < ns; ++k, ++t) {
         const int s = t % NST;
-        if (t >= NST && !mbar_wait(&empty[s], (t / NST - 1) & 1, fail, A.status)) {
+        if (t >= NST && !mbar_wait(&empty[s], (t / NST - 1) & 1, fail, A.status, 3)) {
           live = false;
           break;
         }
@@ -365,11 +238,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
     for (int ch = cbeg; ch < cend && live; ++ch) {
       const int ns = min(STEPS, A.ksteps - (ch % A.chunks) * STEPS);
       const int local = ch - cbeg;
-      if (local > 0 && !mbar_wait(acc_empty, (local - 1) & 1, fail, A.status)) break;
+      if (local > 0 && !mbar_wait(acc_empty, (local - 1) & 1, fail, A.status, 3)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       for (int k = 0; k < ns; ++k, ++t) {
         const int s = t % NST;
-        if (!mbar_wait(&full[s], (t / NST) & 1, fail, A.status)) {
+        if (!mbar_wait(&full[s], (t / NST) & 1, fail, A.status, 3)) {
           live = false;
           break;
         }
@@ -419,39 +292,24 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
     for (int ch = cbeg; ch < cend; ++ch) {
       const int local = ch - cbeg;
       const int ep = __ldg(pe + ch * pext);
-      ok = mbar_wait(acc_full, local & 1, fail, A.status);
+      const int eqv = __ldg(qe + ch * qext + (lane & 15));      // column lane & 15
+      ok = mbar_wait(acc_full, local & 1, fail, A.status, 3);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-      for (int blk = 0; blk < 4; ++blk) {          // (columns 0-7, 8-15) x (re, im)
-        const int c0 = (blk >> 1) * 8;
+      for (int blk = 0; blk < 8; ++blk) {          // four columns of re, then of im
+        const int c0 = (blk >> 1) * 4;
         const bool imag = blk & 1;
-        uint32_t v[NL][8];
+        int eq[4];
 #pragma unroll
-        for (int l = 0; l < NL; ++l)
-          tmem_ld8(base + (imag ? NL * QT : 0) + l * QT + c0, v[l]);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int c = 0; c < 4; ++c) eq[c] = __shfl_sync(0xffffffffu, eqv, c0 + c);
+        double x[1][4];
+        read_levels4<1>(base + (imag ? NL * QT : 0) + c0, QT, 0, ep, eq, x);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          // the asm volatile loads are complete: tie the values to the wait
-          int S[NL];
-#pragma unroll
-          for (int l = 0; l < NL; ++l) {
-            asm volatile("" : "+r"(v[l][c]));
-            S[l] = __float2int_rn(__uint_as_float(v[l][c]));
-          }
-          // the sum is hi 2^32 + lo in units of level 7 (|hi| < 2^49, |lo| < 2^50): 62 bits of it,
-          // from the top of hi down
-          const long long hi = S[0] * 16777216LL + S[1] * 65536LL + S[2] * 256LL + S[3];
-          const long long lo = S[4] * 16777216LL + S[5] * 65536LL + S[6] * 256LL + S[7];
-          const int sh = min(32, __clzll(hi < 0 ? -hi : hi) - 2);
-          const long long T = (long long)((unsigned long long)hi << sh) + (lo >> (32 - sh));
-          const int eq = __ldg(qe + ch * qext + c0 + c);
-          double x = pack(T, ep + eq - 38 - sh);
-          if (ep == E_NONFINITE || eq == E_NONFINITE) x = __longlong_as_double(0x7ff8000000000000LL);
-          if (imag) im[c0 + c] = local == 0 ? x : im[c0 + c] + x;
-          else re[c0 + c] = local == 0 ? x : re[c0 + c] + x;
+        for (int c = 0; c < 4; ++c) {
+          if (imag) im[c0 + c] = local == 0 ? x[0][c] : im[c0 + c] + x[0][c];
+          else re[c0 + c] = local == 0 ? x[0][c] : re[c0 + c] + x[0][c];
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -497,7 +355,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
       int last = -1;
       for (int u = s; u < n; u += NST) last = u;
       int none = 0;
-      if (last >= 0) mbar_wait(&full[s], (last / NST) & 1, &none, A.status);
+      if (last >= 0) mbar_wait(&full[s], (last / NST) & 1, &none, A.status, 3);
     }
   }
   __syncwarp();
