@@ -83,7 +83,7 @@ int fail(tdmrg_model* h, int code, const char* msg) {
 // a dense host W[Dl][Dr][d][d] (complex interleaved) as a one-site device MPO
 struct TempMpo {
   tdmrg::DevMpo m;
-  TempMpo(int Dl, int Dr, int d, const double* W) {
+  TempMpo(int Dl, int Dr, int d, const double* W, cudaStream_t st) {
     tdmrg::MpoSite s;
     s.Dl = Dl;
     s.Dr = Dr;
@@ -99,7 +99,7 @@ struct TempMpo {
         }
         if (nz) s.blocks.push_back({wl, wr, op});
       }
-    Engine::upload_mpo({s}, m);
+    Engine::upload_mpo({s}, m, true, st);
   }
   ~TempMpo() { Engine::free_mpo(m); }
 };
@@ -134,17 +134,22 @@ struct ZgHold {
   }
 };
 
-// device temporaries of one entry point, freed when it returns
+// device temporaries of one entry point, from the library's stream-ordered pool, given back when it
+// returns (cudaMalloc and cudaFree cost 10-100 us a call and stop the device)
 struct DevBufs {
+  cudaStream_t s;
   std::vector<void*> p;
-  cplx* get(long long n) {
+  explicit DevBufs(cudaStream_t st) : s(st) {}
+  DevBufs(const DevBufs&) = delete;
+  void* bytes(size_t n) {
     void* q = nullptr;
-    CK(cudaMalloc(&q, sizeof(cplx) * (size_t)(n > 0 ? n : 1)));
+    CK(tdmrg::zg_pool_alloc(&q, n > 0 ? n : 16, s));
     p.push_back(q);
-    return (cplx*)q;
+    return q;
   }
+  cplx* get(long long n) { return (cplx*)bytes(sizeof(cplx) * (size_t)(n > 0 ? n : 1)); }
   ~DevBufs() {
-    for (void* q : p) cudaFree(q);
+    for (void* q : p) cudaFreeAsync(q, s);
   }
 };
 
@@ -781,7 +786,7 @@ int tdmrg_kernel_heff(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
   if (precision != TDMRG_PREC_C128 && precision != TDMRG_PREC_C64_3XTF32)
     return fail(nullptr, TDMRG_ERR_ARG, "heff: unknown precision");
   return guarded(nullptr, [&] {
-    TempMpo W(Dl, Dr, d, W_host);
+    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
     cudaStream_t s = (cudaStream_t)stream;
     if (precision == TDMRG_PREC_C128) {
       ZgHold zg(s);
@@ -790,8 +795,8 @@ int tdmrg_kernel_heff(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
                       (const tdmrg::cplx*)R, (const tdmrg::cplx*)A, (tdmrg::cplx*)out, nullptr);
       zg.finish();
     } else {
-      int* st = nullptr;
-      CK(cudaMalloc(&st, sizeof(int)));
+      DevBufs mem(s);
+      int* st = (int*)mem.bytes(sizeof(int));
       CK(cudaMemsetAsync(st, 0, sizeof(int), s));
       tdmrg::TcWork w = tdmrg::heff_tc_carve((float*)ws32, Ml, Mr, d * d, Dl, Dr, st);
       tdmrg::heff_tc_envs(s, w, Ml, Mr, Dl, Dr, (const tdmrg::cplx*)L, (const tdmrg::cplx*)R);
@@ -799,7 +804,6 @@ int tdmrg_kernel_heff(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
       int hs = 0;
       CK(cudaMemcpyAsync(&hs, st, sizeof(int), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
-      cudaFree(st);
       if (hs) throw Failure{TDMRG_ERR_TIMEOUT, "tensor-core pipeline wait timed out"};
     }
     CK(cudaStreamSynchronize(s));
@@ -817,7 +821,7 @@ int tdmrg_kernel_heff_timed(int Ml, int Mr, int d, int Dl, int Dr, const double*
   return guarded(nullptr, [&] {
     using tdmrg::cplx;
     using tdmrg::pad4;
-    TempMpo W(Dl, Dr, d, W_host);
+    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
     cudaStream_t s = (cudaStream_t)stream;
     const int D = d * d;
     const long long site = (long long)Ml * D * Mr;
@@ -995,20 +999,11 @@ int tdmrg_kernel_heff_vjp(int Ml, int Mr, int d, int Dl, int Dr, const double* W
           Wt[dst] = W_host[src];
           Wt[dst + 1] = -W_host[src + 1];
         }
-    TempMpo W(Dl, Dr, d, W_host);
-    TempMpo Wc(Dl, Dr, d, Wt.data());
-    cplx* Lh = nullptr;
-    cplx* Rh = nullptr;
-    struct Free {
-      cplx*& a;
-      cplx*& b;
-      ~Free() {
-        if (a) cudaFree(a);
-        if (b) cudaFree(b);
-      }
-    } fr{Lh, Rh};
-    CK(cudaMalloc(&Lh, sizeof(cplx) * (size_t)Dl * Ml * Ml));
-    CK(cudaMalloc(&Rh, sizeof(cplx) * (size_t)Dr * Mr * Mr));
+    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
+    TempMpo Wc(Dl, Dr, d, Wt.data(), (cudaStream_t)stream);
+    DevBufs mem(s);
+    cplx* Lh = mem.get((long long)Dl * Ml * Ml);
+    cplx* Rh = mem.get((long long)Dr * Mr * Mr);
     // per-channel Hermitian conjugates of the environments
     for (int w = 0; w < Dl; ++w)
       CK(tdmrg::ztranspose(Ml, Ml, (const cplx*)L + (size_t)w * Ml * Ml, Lh + (size_t)w * Ml * Ml,
@@ -1037,20 +1032,12 @@ int tdmrg_kernel_zgemm_tc(int M, int N, int K, const void* A, const void* B, int
   return guarded(nullptr, [&] {
     cudaStream_t s = (cudaStream_t)stream;
     tdmrg::TcOperand a{nullptr, M, K, tdmrg::pad4(K), 1}, b{nullptr, N, K, tdmrg::pad4(K), 1};
-    int* st = nullptr;
-    float* part = nullptr;
+    DevBufs mem(s);
     const long long part_len = 2LL * M * N * 64;      // room for a split-K of up to 64
-    CK(cudaMalloc(&a.p, sizeof(float) * a.floats()));
-    CK(cudaMalloc(&b.p, sizeof(float) * b.floats()));
-    CK(cudaMalloc(&st, sizeof(int)));
-    CK(cudaMalloc(&part, sizeof(float) * part_len));
-    struct F {
-      void* x[4];
-      ~F() {
-        for (void* p : x)
-          if (p) cudaFree(p);
-      }
-    } f{{a.p, b.p, st, part}};
+    a.p = (float*)mem.bytes(sizeof(float) * a.floats());
+    b.p = (float*)mem.bytes(sizeof(float) * b.floats());
+    int* st = (int*)mem.bytes(sizeof(int));
+    float* part = (float*)mem.bytes(sizeof(float) * part_len);
     CK(cudaMemsetAsync(st, 0, sizeof(int), s));
     CK(tdmrg::split_f64((const tdmrg::cplx*)A, 0, K, 1, 0, a, s));
     CK(tdmrg::split_f64((const tdmrg::cplx*)B, 0, K, 1, 0, b, s));
@@ -1073,7 +1060,7 @@ int tdmrg_kernel_env_left(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int
       !bra || !ket || !Lout || !X || !Y)
     return fail(nullptr, TDMRG_ERR_ARG, "env_left: bad arguments");
   return guarded(nullptr, [&] {
-    TempMpo W(Dl, Dr, d, W_host);
+    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
     ZgHold zg((cudaStream_t)stream);
     tdmrg::Ctx c{(cudaStream_t)stream, (tdmrg::cplx*)X, (tdmrg::cplx*)Y, &zg.w};
     tdmrg::env_left_f64(c, W.m.s[0], Ml1, Mr1, Ml2, Mr2, d * d, d, (const tdmrg::cplx*)L,
@@ -1094,23 +1081,13 @@ int tdmrg_kernel_gauge_qr(int m, int n, const void* Y, int p, const void* E, voi
     tdmrg::QrScratch W{};
     W.gmax = sms;
     W.nmax = n;
+    DevBufs mem(s);
+    W.part = mem.get(2 * (long long)sms * (n + 1));
+    W.partn = (double*)mem.bytes(sizeof(double) * 2 * (size_t)sms);
+    W.bar = (unsigned*)mem.bytes(sizeof(unsigned) * 2);
     int* st = status;
-    struct Free {
-      tdmrg::QrScratch& w;
-      int*& st;
-      bool own;
-      ~Free() {
-        if (w.part) cudaFree(w.part);
-        if (w.partn) cudaFree(w.partn);
-        if (w.bar) cudaFree(w.bar);
-        if (own && st) cudaFree(st);
-      }
-    } fr{W, st, status == nullptr};
-    CK(cudaMalloc(&W.part, sizeof(tdmrg::cplx) * 2 * (size_t)sms * (n + 1)));
-    CK(cudaMalloc(&W.partn, sizeof(double) * 2 * (size_t)sms));
-    CK(cudaMalloc(&W.bar, sizeof(unsigned) * 2));
     if (!st) {
-      CK(cudaMalloc(&st, sizeof(int)));
+      st = (int*)mem.bytes(sizeof(int));
       CK(cudaMemsetAsync(st, 0, sizeof(int), s));
     }
     tdmrg::QrRef y{(const tdmrg::cplx*)Y, n, 1, 1LL << 60, 0, 0};
@@ -1146,40 +1123,18 @@ int tdmrg_kernel_gauge_qr_blocked(int m, int n, const void* Y, int p, const void
     tdmrg::QrScratch W{};
     W.gmax = sms;
     W.nmax = n;
-    tdmrg::cplx* qb = nullptr;
-    unsigned char* acc = nullptr;
-    int* st = status;
+    DevBufs mem(s);
+    W.part = mem.get(2 * (long long)sms * (n + 1));
+    W.partn = (double*)mem.bytes(sizeof(double) * 2 * (size_t)sms);
+    W.bar = (unsigned*)mem.bytes(sizeof(unsigned) * 2);
     const long long qlen = tdmrg::gauge_qr_blocked_scratch(n, sms);
-    tdmrg::ZgWork qw;
-    qw.pooled = true;
-    struct Free {
-      tdmrg::QrScratch& w;
-      tdmrg::cplx*& qb;
-      unsigned char*& acc;
-      int*& st;
-      bool own;
-      tdmrg::ZgWork& qw;
-      cudaStream_t s;
-      ~Free() {
-        tdmrg::zg_free(qw, s);
-        if (w.part) cudaFree(w.part);
-        if (w.partn) cudaFree(w.partn);
-        if (w.bar) cudaFree(w.bar);
-        if (qb) cudaFree(qb);
-        if (acc) cudaFree(acc);
-        if (own && st) cudaFree(st);
-      }
-    } fr{W, qb, acc, st, status == nullptr, qw, s};
-    CK(tdmrg::zg_reserve(qw, tdmrg::gauge_qr_tensor_bytes(m, n, sms), s));
-    W.dig = static_cast<unsigned char*>(qw.p);
-    W.dig_bytes = qw.bytes;
-    CK(cudaMalloc(&W.part, sizeof(tdmrg::cplx) * 2 * (size_t)sms * (n + 1)));
-    CK(cudaMalloc(&W.partn, sizeof(double) * 2 * (size_t)sms));
-    CK(cudaMalloc(&W.bar, sizeof(unsigned) * 2));
-    CK(cudaMalloc(&qb, sizeof(tdmrg::cplx) * (size_t)qlen));
-    CK(cudaMalloc(&acc, (size_t)n + 16));
+    tdmrg::cplx* qb = mem.get(qlen);
+    unsigned char* acc = (unsigned char*)mem.bytes((size_t)n + 16);
+    W.dig_bytes = tdmrg::gauge_qr_tensor_bytes(m, n, sms);
+    if (W.dig_bytes) W.dig = (unsigned char*)mem.bytes(W.dig_bytes);
+    int* st = status;
     if (!st) {
-      CK(cudaMalloc(&st, sizeof(int)));
+      st = (int*)mem.bytes(sizeof(int));
       CK(cudaMemsetAsync(st, 0, sizeof(int), s));
     }
     tdmrg::QrRef y{(const tdmrg::cplx*)Y, n, 1, 1LL << 60, 0, 0};
@@ -1214,27 +1169,16 @@ int tdmrg_kernel_bond_exp(int M, int Dw, const void* L, const void* R, const voi
     W.maxn = n;
     W.maxDw = Dw;
     W.gmax = sms;
-    tdmrg::cplx* V = nullptr;
-    int* st = nullptr;
-    struct Free {
-      tdmrg::BondScratch& w;
-      tdmrg::cplx*& V;
-      int*& st;
-      ~Free() {
-        for (void* p : {(void*)w.W, (void*)w.T, (void*)w.P, (void*)w.part, (void*)w.partn,
-                        (void*)w.bar, (void*)w.mv, (void*)V, (void*)st})
-          if (p) cudaFree(p);
-      }
-    } fr{W, V, st};
-    CK(cudaMalloc(&W.W, sizeof(tdmrg::cplx) * (size_t)n));
-    CK(cudaMalloc(&W.T, sizeof(float2) * (size_t)Dw * n));
-    CK(cudaMalloc(&W.P, sizeof(float2) * (size_t)Dw * n));
-    CK(cudaMalloc(&W.part, sizeof(tdmrg::cplx) * 2 * (size_t)sms * (tdmrg::KMAX + 1)));
-    CK(cudaMalloc(&W.partn, sizeof(double) * 2 * (size_t)sms));   // 2 * gmax
-    CK(cudaMalloc(&W.bar, sizeof(unsigned) * 2));
-    CK(cudaMalloc(&W.mv, sizeof(unsigned long long)));
-    CK(cudaMalloc(&V, sizeof(tdmrg::cplx) * (size_t)kcap * n));
-    CK(cudaMalloc(&st, sizeof(int)));
+    DevBufs mem(s);
+    W.W = mem.get(n);
+    W.T = (float2*)mem.bytes(sizeof(float2) * (size_t)Dw * n);
+    W.P = (float2*)mem.bytes(sizeof(float2) * (size_t)Dw * n);
+    W.part = mem.get(2 * (long long)sms * (tdmrg::KMAX + 1));
+    W.partn = (double*)mem.bytes(sizeof(double) * 2 * (size_t)sms);   // 2 * gmax
+    W.bar = (unsigned*)mem.bytes(sizeof(unsigned) * 2);
+    W.mv = (unsigned long long*)mem.bytes(sizeof(unsigned long long));
+    tdmrg::cplx* V = mem.get((long long)kcap * n);
+    int* st = (int*)mem.bytes(sizeof(int));
     CK(cudaMemsetAsync(W.mv, 0, sizeof(unsigned long long), s));
     CK(cudaMemsetAsync(st, 0, sizeof(int), s));
     CK(tdmrg::bond_exp_fused(M, Dw, (const tdmrg::cplx*)L, (const tdmrg::cplx*)R,
@@ -1269,12 +1213,12 @@ int site_exp_vjp_impl(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
     const size_t site = (size_t)Dl * Dr * D;
     const long long n = (long long)Ml * D * Mr;
     const long long nl = (long long)Dl * Ml * Ml, nr = (long long)Dr * Mr * Mr;
-    TempMpo W(Dl, Dr, d, W_host);
+    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
     std::vector<std::unique_ptr<TempMpo>> dWs(nparam);
     for (int p = 0; p < nparam; ++p) {
       theta_bar[p] = 0.0;
       if (any_nonzero(dW_host + 2 * site * p, 2 * site))
-        dWs[p].reset(new TempMpo(Dl, Dr, d, dW_host + 2 * site * p));
+        dWs[p].reset(new TempMpo(Dl, Dr, d, dW_host + 2 * site * p, (cudaStream_t)stream));
     }
     tdmrg::ModelParams P;
     P.N = 3;
@@ -1283,7 +1227,7 @@ int site_exp_vjp_impl(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
     eng.set_krylov(tol, tdmrg::KMAX, 0);
     eng.ensure_workspace(n, n, 1, 1);
     const long long xy = (long long)std::max(Dl, Dr) * n;
-    DevBufs buf;
+    DevBufs buf(s);
     cplx* X = buf.get(xy);
     cplx* Y = buf.get(xy);
     cplx* a = buf.get(n);
@@ -1367,18 +1311,11 @@ int tdmrg_kernel_bond_exp_vjp(int M, int Dw, const void* L, const void* R, const
     eng.set_stream(s);
     eng.set_krylov(tol, tdmrg::KMAX, 0);
     eng.ensure_workspace(mm, mm, 1, 1);
-    cplx *X = nullptr, *a = nullptr, *b = nullptr, *T = nullptr;
-    struct Free {
-      cplx** p[4];
-      ~Free() {
-        for (auto q : p)
-          if (*q) cudaFree(*q);
-      }
-    } fr{{&X, &a, &b, &T}};
-    CK(cudaMalloc(&X, sizeof(cplx) * (size_t)Dw * mm));
-    CK(cudaMalloc(&a, sizeof(cplx) * (size_t)mm));
-    CK(cudaMalloc(&b, sizeof(cplx) * (size_t)mm));
-    CK(cudaMalloc(&T, sizeof(cplx) * (size_t)Dw * mm));
+    DevBufs mem(s);
+    cplx* X = mem.get(Dw * mm);
+    cplx* a = mem.get(mm);
+    cplx* b = mem.get(mm);
+    cplx* T = mem.get(Dw * mm);
     tdmrg::Ctx c{s, X, nullptr, eng.zg()};
     const cplx* Ld = (const cplx*)L;
     const cplx* Rd = (const cplx*)R;
@@ -1422,18 +1359,11 @@ int tdmrg_kernel_qr_vjp(int m, int n, const void* Q, const void* R, const void* 
     using tdmrg::MatRef;
     cudaStream_t s = (cudaStream_t)stream;
     ZgHold zg(s);
-    cplx *Ru = nullptr, *M = nullptr, *S = nullptr, *rhs = nullptr;
-    struct Free {
-      cplx** p[4];
-      ~Free() {
-        for (auto q : p)
-          if (*q) cudaFree(*q);
-      }
-    } fr{{&Ru, &M, &S, &rhs}};
-    CK(cudaMalloc(&Ru, sizeof(cplx) * (size_t)n * n));
-    CK(cudaMalloc(&M, sizeof(cplx) * (size_t)n * n));
-    CK(cudaMalloc(&S, sizeof(cplx) * (size_t)n * n));
-    CK(cudaMalloc(&rhs, sizeof(cplx) * (size_t)m * n));
+    DevBufs mem(s);
+    cplx* Ru = mem.get((long long)n * n);
+    cplx* M = mem.get((long long)n * n);
+    cplx* S = mem.get((long long)n * n);
+    cplx* rhs = mem.get((long long)m * n);
     const cplx one = {1.0, 0.0}, mone = {-1.0, 0.0}, zero = {0.0, 0.0};
     // entries of Rbar below the diagonal are structural zeros of R
     CK(cudaMemcpyAsync(Ru, Rbar, sizeof(cplx) * (size_t)n * n, cudaMemcpyDeviceToDevice, s));
@@ -1465,13 +1395,13 @@ int tdmrg_kernel_env_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr, const 
     cudaStream_t s = (cudaStream_t)stream;
     const int D = d * d;
     const size_t site = (size_t)Dl * Dr * D;
-    TempMpo W(Dl, Dr, d, W_host);
+    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
     const std::vector<double> Wt = transpose_conj_ops(W_host, Dl, Dr, d);
-    TempMpo Wc(Dl, Dr, d, Wt.data());
+    TempMpo Wc(Dl, Dr, d, Wt.data(), (cudaStream_t)stream);
     const int Me = side == 0 ? Ml : Mr, De = side == 0 ? Dl : Dr;   // E (environment in)
     const int Mg = side == 0 ? Mr : Ml, Dg = side == 0 ? Dr : Dl;   // G (environment out)
     const long long ne = (long long)De * Me * Me, ng = (long long)Dg * Mg * Mg;
-    DevBufs buf;
+    DevBufs buf(s);
     cplx* Eh = buf.get(ne);     // E^dagger per channel
     cplx* Gt = buf.get(ng);     // G^T per channel
     cplx* Gc = buf.get(ng);     // conj G
@@ -1511,7 +1441,7 @@ int tdmrg_kernel_env_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr, const 
         theta_bar[p] = 0.0;
         continue;
       }
-      TempMpo dWp(Dl, Dr, d, dW);
+      TempMpo dWp(Dl, Dr, d, dW, (cudaStream_t)stream);
       if (side == 0)
         tdmrg::env_left_f64(c, dWp.m.s[0], Ml, Mr, Ml, Mr, D, d, Ed, Bd, Kd, tmp);
       else
@@ -1537,8 +1467,8 @@ int tdmrg_kernel_expansion_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr,
     const long long per = (long long)Ml * D * Mr;
     const int Dmax = Dl > Dr ? Dl : Dr;
     const std::vector<double> Wt = transpose_conj_ops(W_host, Dl, Dr, d);
-    TempMpo Wc(Dl, Dr, d, Wt.data());
-    DevBufs buf;
+    TempMpo Wc(Dl, Dr, d, Wt.data(), (cudaStream_t)stream);
+    DevBufs buf(s);
     cplx* Pb = buf.get((long long)Dmax * per);    // Xbar in the channel-major partial layout
     cplx* Z = buf.get((long long)Dmax * per);
     cplx* tmp = buf.get((long long)Dmax * per);
@@ -1585,7 +1515,7 @@ int tdmrg_kernel_expansion_vjp(int side, int Ml, int Mr, int d, int Dl, int Dr,
         theta_bar[p] = 0.0;
         continue;
       }
-      TempMpo dWp(Dl, Dr, d, dW);
+      TempMpo dWp(Dl, Dr, d, dW, (cudaStream_t)stream);
       if (side == 0)
         tdmrg::left_partial_f64(c, dWp.m.s[0], Ml, Ml, D, d, Mr, Ed, Ad, tmp, nullptr);
       else
@@ -1615,7 +1545,7 @@ int tdmrg_kernel_qr_vjp_completed(int m, int n, const int* accepted, const void*
     std::vector<int> order(S);
     order.insert(order.end(), K.begin(), K.end());
     const long long mn = (long long)m * n, nn = (long long)n * n;
-    DevBufs buf;
+    DevBufs buf(s);
     cplx* Qp = buf.get(mn);
     cplx* Z = buf.get(mn);
     cplx* Yr = buf.get(mn);

@@ -312,7 +312,8 @@ void bond_tc_apply(cudaStream_t st, const TcBufs& b, int M, int Dw, const cplx* 
 // ------------------------------------------------------------------------------------
 // MPO upload
 // ------------------------------------------------------------------------------------
-void Engine::upload_mpo(const std::vector<MpoSite>& W, DevMpo& out) {
+void Engine::upload_mpo(const std::vector<MpoSite>& W, DevMpo& out, bool pooled,
+                        cudaStream_t stream) {
   free_mpo(out);
   out.s.resize(W.size());
   out.maxD = 1;
@@ -358,8 +359,13 @@ void Engine::upload_mpo(const std::vector<MpoSite>& W, DevMpo& out) {
     const size_t int_bytes = sizeof(int) * (size_t)(h.Dr + 1 + nb + h.Dl + 1 + nb);
     const size_t total = 2 * ops_bytes + 2 * ops32_bytes + int_bytes + 64;
     char* mem = nullptr;
-    CK(cudaMalloc(&mem, total));
+    if (pooled)
+      CK(zg_pool_alloc(reinterpret_cast<void**>(&mem), total, stream));
+    else
+      CK(cudaMalloc(&mem, total));
     s.mem = mem;
+    s.pooled = pooled;
+    s.stream = stream;
     cplx* d_olr = reinterpret_cast<cplx*>(mem);
     cplx* d_orl = d_olr + (size_t)nb * d * d;
     float2* d_flr = reinterpret_cast<float2*>(d_orl + (size_t)nb * d * d);
@@ -372,16 +378,24 @@ void Engine::upload_mpo(const std::vector<MpoSite>& W, DevMpo& out) {
     std::vector<float2> flr(olr.size()), frl(orl.size());
     for (size_t e = 0; e < olr.size(); ++e) flr[e] = make_float2((float)olr[e].x, (float)olr[e].y);
     for (size_t e = 0; e < orl.size(); ++e) frl[e] = make_float2((float)orl[e].x, (float)orl[e].y);
-    if (nb > 0) {
-      CK(cudaMemcpy(d_flr, flr.data(), ops32_bytes, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d_frl, frl.data(), ops32_bytes, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d_olr, olr.data(), ops_bytes, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d_orl, orl.data(), ops_bytes, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d_lrc, ilr_chan.data(), sizeof(int) * nb, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d_rlc, irl_chan.data(), sizeof(int) * nb, cudaMemcpyHostToDevice));
-    }
-    CK(cudaMemcpy(d_lrs, ilr_start.data(), sizeof(int) * (h.Dr + 1), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(d_rls, irl_start.data(), sizeof(int) * (h.Dl + 1), cudaMemcpyHostToDevice));
+    // one host image, one copy
+    std::vector<char> host(total, 0);
+    auto put = [&](const void* dev, const void* src, size_t bytes) {
+      if (bytes) std::memcpy(host.data() + (static_cast<const char*>(dev) - mem), src, bytes);
+    };
+    put(d_olr, olr.data(), ops_bytes);
+    put(d_orl, orl.data(), ops_bytes);
+    put(d_flr, flr.data(), ops32_bytes);
+    put(d_frl, frl.data(), ops32_bytes);
+    put(d_lrs, ilr_start.data(), sizeof(int) * (h.Dr + 1));
+    put(d_lrc, ilr_chan.data(), sizeof(int) * nb);
+    put(d_rls, irl_start.data(), sizeof(int) * (h.Dl + 1));
+    put(d_rlc, irl_chan.data(), sizeof(int) * nb);
+    // (a copy from pageable memory has taken its source when the call returns)
+    if (pooled)
+      CK(cudaMemcpyAsync(mem, host.data(), total, cudaMemcpyHostToDevice, stream));
+    else
+      CK(cudaMemcpy(mem, host.data(), total, cudaMemcpyHostToDevice));
     s.lr = MixTable{h.Dr, d_lrs, d_lrc, d_olr, d_flr, nb};
     s.rl = MixTable{h.Dl, d_rls, d_rlc, d_orl, d_frl, nb};
   }
@@ -389,7 +403,10 @@ void Engine::upload_mpo(const std::vector<MpoSite>& W, DevMpo& out) {
 
 void Engine::free_mpo(DevMpo& m) {
   for (auto& s : m.s)
-    if (s.mem) cudaFree(s.mem);
+    if (s.mem) {
+      if (s.pooled) cudaFreeAsync(s.mem, s.stream);
+      else cudaFree(s.mem);
+    }
   m.s.clear();
 }
 

@@ -21,6 +21,8 @@ struct DevMpoSite {
   int Dl = 0, Dr = 0, d = 0, nblk = 0;
   MixTable lr{}, rl{};               // lr: in = wl, out = wr;  rl: in = wr, out = wl
   void* mem = nullptr;               // one allocation holding all tables
+  bool pooled = false;               // from the stream-ordered pool, given back on `stream`
+  cudaStream_t stream = 0;
   std::vector<MpoBlock> host;
 };
 
@@ -193,7 +195,9 @@ class Engine {
   ModelParams P;
 
   void ensure_workspace(long long maxsite, long long maxxy, int maxbond, int maxm);
-  static void upload_mpo(const std::vector<MpoSite>& W, DevMpo& out);
+  // with a stream (pooled true) the tables come from the stream-ordered pool and are copied on it
+  static void upload_mpo(const std::vector<MpoSite>& W, DevMpo& out, bool pooled = false,
+                         cudaStream_t stream = 0);
   static void free_mpo(DevMpo& m);
   cudaStream_t stream() const { return st_; }
   cplx* X() { return X_; }
