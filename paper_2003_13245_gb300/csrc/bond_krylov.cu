@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
   unsigned epoch = 0;
   __shared__ cplx h1[NV], h2[NV], cc[KMAX];
   __shared__ double alpha[KMAX], beta[KMAX + 1], red[BT / 32];
-  __shared__ double s_nrm, s_b0, s_scale;
+  __shared__ double s_nrm, s_b0, s_inv;
   __shared__ int s_done, s_k, s_second;
 
   const int M = A.M, Dw = A.Dw;
@@ -274,19 +274,20 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
       const int lane = threadIdx.x;
       double yr, yi, err;
       bool done, bd;
+      double nb, inv1;
       lzc::tridiag_step(j, h1[j].x + h2[j].x, s_nrm, A.tr, A.ti, A.tol, A.kcap, A.fixed, alpha,
-                        beta, true, yr, yi, done, err, bd);
+                        beta, true, yr, yi, done, err, bd, nb, inv1);
       if (done && lane <= j) cc[lane] = make_double2(s_b0 * yr, s_b0 * yi);
       if (lane == 0) {
         s_done = done ? 1 : 0;
         s_k = j + 1;
-        s_scale = sqrt(s_nrm);
+        s_inv = inv1;
       }
     }
     __syncthreads();
     k = s_k;
     if (s_done) break;
-    inv = 1.0 / s_scale;
+    inv = s_inv;
     for (int e = threadIdx.x; e < len; e += BT)
       A.V[(size_t)(j + 1) * n + e0 + e] = make_double2(ws[e].x * inv, ws[e].y * inv);
     src = A.W;

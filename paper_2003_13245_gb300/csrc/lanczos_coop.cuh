@@ -6,8 +6,9 @@
 // (lanczos_step.cu).  All sums have a fixed order, so results do not depend on timing.
 #pragma once
 
-#include "tdmrg_internal.cuh"
+#include "fp64_util.cuh"
 #include "lanczos_exp.cuh"
+#include "tdmrg_internal.cuh"
 
 namespace tdmrg {
 namespace lzc {
@@ -74,18 +75,23 @@ __device__ __forceinline__ void slice_dots(const cplx* V, long long n, const cpl
   }
 }
 
-// The same partial dots with every thread of the CTA on every vector (for large slices): the
-// vectors are taken four at a time, each thread sums its elements (stride blockDim), then a
-// warp tree and the warps in order.  red: 8 * (blockDim / 32) doubles of shared memory.
+// The same partial dots with every thread of the CTA on every vector (for large slices), and
+// with `norm` the slice's ||w||^2: the vectors are taken four at a time, each thread sums its
+// elements (stride blockDim), then warp v adds the threads' sums of value v in a fixed order (one
+// warp per value: a tree in every warp would cost each of them five FP64 additions per value).
+// red: 9 * blockDim doubles of shared memory.
 __device__ __forceinline__ void slice_dots_block(const cplx* V, long long n, const cplx* w,
                                                  long long e0, int len, int i0, int i1,
-                                                 cplx* part, double* red) {
+                                                 cplx* part, double* norm, double* red) {
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int T = blockDim.x;
   for (int c0 = i0; c0 < i1; c0 += 4) {
     const int nv = min(4, i1 - c0);
-    double sr[4] = {0.0, 0.0, 0.0, 0.0}, si[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int e = threadIdx.x; e < len; e += blockDim.x) {
+    const bool nrm = norm && c0 == i0;
+    double sr[4] = {0.0, 0.0, 0.0, 0.0}, si[4] = {0.0, 0.0, 0.0, 0.0}, sn = 0.0;
+    for (int e = threadIdx.x; e < len; e += T) {
       const cplx b = w[e];
+      if (nrm) sn = fma(b.x, b.x, fma(b.y, b.y, sn));
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         if (v < nv) {
@@ -98,24 +104,23 @@ __device__ __forceinline__ void slice_dots_block(const cplx* V, long long n, con
       }
     }
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      if (v < nv) {                 // uniform across the CTA
-        sr[v] = wsum(sr[v]);
-        si[v] = wsum(si[v]);
-        if (lane == 0) {
-          red[(wv * 4 + v) * 2] = sr[v];
-          red[(wv * 4 + v) * 2 + 1] = si[v];
-        }
+    for (int v = 0; v < 4; ++v)
+      if (v < nv) {
+        red[(2 * v) * T + threadIdx.x] = sr[v];
+        red[(2 * v + 1) * T + threadIdx.x] = si[v];
       }
-    }
+    if (nrm) red[8 * T + threadIdx.x] = sn;
     __syncthreads();
-    if ((int)threadIdx.x < nv) {
-      double x = 0.0, y = 0.0;
-      for (int u = 0; u < nw; ++u) {
-        x += red[(u * 4 + threadIdx.x) * 2];
-        y += red[(u * 4 + threadIdx.x) * 2 + 1];
+    const int live = min(T, (len + 31) & ~31);      // threads that summed anything
+    for (int v = wv; v < 9; v += nw) {
+      if (v < 8 ? v >= 2 * nv : !nrm) continue;
+      double x = 0.0;
+      for (int u = lane; u < live; u += 32) x += red[v * T + u];
+      x = wsum(x);
+      if (lane == 0) {
+        if (v == 8) norm[blockIdx.x] = x;
+        else reinterpret_cast<double*>(part + (size_t)blockIdx.x * NV + c0 + (v >> 1))[v & 1] = x;
       }
-      part[(size_t)blockIdx.x * NV + c0 + threadIdx.x] = make_double2(x, y);
     }
     __syncthreads();
   }
@@ -183,17 +188,26 @@ __device__ __forceinline__ void reduce_norm(const double* partn, int G, double* 
 
 // Lanczos vector j done: alpha_j = Re(h1[j] + h2[j]), beta_{j+1} = sqrt(nrm2).  Warp 0 extends
 // the tridiagonal T (alpha[0..j), beta[1..j] read from `alpha`, `beta`; alpha[j], beta[j+1]
-// stored there when `store`), evaluates y = exp(tau T) e_1 (lane i returns y_i in yr, yi) and
-// decides whether to stop: breakdown, kcap vectors, or beta_{j+1} |y_j| < tol unless the
-// dimension is fixed.  Every lane returns the same done / err / breakdown.  Call from the 32
-// lanes of one warp.
+// stored there when `store`) and decides whether to stop: breakdown, kcap vectors, or
+// beta_{j+1} |y_j| < tol, y = exp(tau T) e_1, unless the dimension is fixed.  Where the run goes on
+// for sure -- a fixed dimension not reached, or a single-precision estimate above 8 tol -- the FP64
+// exponential (10-15 us of serial FP64) is left out; otherwise it decides, and lane i returns y_i
+// in yr, yi when done.  Every lane returns the same done / err / breakdown, beta_{j+1} in nb and
+// its reciprocal in inv.  Call from the 32 lanes of one warp.
 __device__ __forceinline__ void tridiag_step(int j, double aj, double nrm2, double tr, double ti,
                                              double tol, int kcap, int fixed, double* alpha,
                                              double* beta, bool store, double& yr, double& yi,
-                                             bool& done, double& err, bool& breakdown) {
+                                             bool& done, double& err, bool& breakdown, double& nb,
+                                             double& inv) {
   const int lane = threadIdx.x & 31;
   const int kk = j + 1;
-  const double nb = sqrt(nrm2);
+  if (bexp(nrm2) > 0 && bexp(nrm2) < 0x7ff && nrm2 > 0.0) {
+    inv = rsqrt_series(nrm2);
+    nb = nrm2 * inv;
+  } else {
+    nb = sqrt(nrm2);
+    inv = 1.0 / nb;
+  }
   const double a = lane < j ? alpha[lane] : (lane == j ? aj : 0.0);
   const double bl = (lane >= 1 && lane < kk) ? beta[lane] : 0.0;
   const double br = (lane + 1 < kk) ? beta[lane + 1] : 0.0;
@@ -201,6 +215,24 @@ __device__ __forceinline__ void tridiag_step(int j, double aj, double nrm2, doub
   if (store && lane == 0) {
     alpha[j] = aj;
     beta[j + 1] = nb;
+  }
+  yr = yi = err = 0.0;
+  breakdown = false;
+  // nb against 1e-12 of the largest entry, from the upper words first (2^-20 below their numbers)
+  const int top = __reduce_max_sync(0xffffffffu, max(__double2hiint(fabs(a)), __double2hiint(fabs(bl))));
+  const double low = __hiloint2double(top, 0);
+  const bool clear = nb > 2e-12 * low && low > 1e-290;
+  if (clear && kk < kcap) {
+    if (fixed) {
+      done = false;
+      return;
+    }
+    const float e32 = lz_last_entry32((float)a, (float)bl, (float)br, kk, (float)tr, (float)ti);
+    const float est = (float)nb * e32;
+    if (est > 8.f * (float)tol && est < 3e38f) {
+      done = false;
+      return;
+    }
   }
   const double scale = lz_warp_max(fmax(fabs(a), fabs(bl)));
   const double sigma = lz_exp_shifted(a, bl, br, kk, tr, ti, yr, yi);

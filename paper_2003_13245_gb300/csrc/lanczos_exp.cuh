@@ -158,4 +158,56 @@ __device__ __forceinline__ void lz_shift_factor(double sigma, double tr, double 
   }
 }
 
+// |(exp(tau T_k) e_1)_{k-1}| in single precision, for the stopping test only: the same shift and
+// sub-steps.  Entry k-1 of the series starts at the k-1-th power with a product of off-diagonals
+// and no cancellation, so its relative error is a few 1e-6 where the test is decided (beyond the
+// spread of the spectrum); the caller keeps a factor of 8.  Not finite or zero where single
+// precision over- or underflows.  All 32 lanes call it.
+__device__ __forceinline__ float lz_last_entry32(float a, float bl, float br, int k, float tr,
+                                                 float ti) {
+  const int lane = threadIdx.x & 31;
+  const bool in = lane < k;
+  const float rad = fabsf(bl) + fabsf(br);
+  float lo = in ? a - rad : 3e38f, hi = in ? a + rad : -3e38f;
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  const float sigma = 0.5f * (lo + hi);
+  const float as = in ? a - sigma : 0.f;
+  float tnorm = fabsf(as) + rad;
+  for (int o = 16; o > 0; o >>= 1) tnorm = fmaxf(tnorm, __shfl_xor_sync(0xffffffffu, tnorm, o));
+  const float tabs = sqrtf(tr * tr + ti * ti);
+  const float want = ceilf(tabs * tnorm);
+  if (!(want <= 256.f)) return __int_as_float(0x7fc00000);       // long series: the caller's FP64
+  const int nsub = want >= 1.f ? (int)want : 1;
+  const float sr = tr / nsub, si = ti / nsub;
+  // terms from order k-1 on reach entry k-1: the sum runs to k-1 + 8 (x <= 1: the rest is 1e-9 of
+  // it at most, and less than the factor kept for any k)
+  const int nq = min(k + 7, 40);
+  float yr = lane == 0 ? 1.f : 0.f, yi = 0.f;
+  for (int st = 0; st < nsub; ++st) {
+    float ur = yr, ui = yi, ar = yr, ai = yi;
+    for (int q = 1; q <= nq; ++q) {
+      const float ur_u = __shfl_up_sync(0xffffffffu, ur, 1), ur_d = __shfl_down_sync(0xffffffffu, ur, 1);
+      const float ui_u = __shfl_up_sync(0xffffffffu, ui, 1), ui_d = __shfl_down_sync(0xffffffffu, ui, 1);
+      const float inv = __fdividef(1.f, (float)q);
+      const float xr = as * ur + (lane >= 1 ? bl * ur_u : 0.f) + (lane < 31 ? br * ur_d : 0.f);
+      const float xi = as * ui + (lane >= 1 ? bl * ui_u : 0.f) + (lane < 31 ? br * ui_d : 0.f);
+      const float cr = sr * inv, ci = si * inv;
+      ur = cr * xr - ci * xi;
+      ui = cr * xi + ci * xr;
+      ar += ur;
+      ai += ui;
+    }
+    yr = ar;
+    yi = ai;
+  }
+  const float lr = __shfl_sync(0xffffffffu, yr, k - 1), li = __shfl_sync(0xffffffffu, yi, k - 1);
+  // (the squares of 1e-20 would underflow)
+  const float big = fmaxf(fabsf(lr), fabsf(li)), small = fminf(fabsf(lr), fabsf(li));
+  const float r = big > 0.f ? small / big : 0.f;
+  return big * sqrtf(1.f + r * r) * (tr != 0.f ? expf(tr * sigma) : 1.f);
+}
+
 }  // namespace tdmrg

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(LT) lz_step_kernel(LzStepArgs A) {
   // converged in an earlier launch (the host queues one step ahead of its poll)
   if (*reinterpret_cast<volatile int*>(&S->done)) return;
   __shared__ cplx h1[NV], h2[NV];
-  __shared__ double red[8 * (LT / 32)];
+  __shared__ double red[9 * LT];
   __shared__ double alpha[KMAX], beta[KMAX + 1];
   __shared__ double s_nrm, s_inv;
   __shared__ int s_done, s_second;
@@ -52,8 +52,8 @@ __global__ void __launch_bounds__(LT) lz_step_kernel(LzStepArgs A) {
   for (int i = threadIdx.x; i <= j; i += blockDim.x) beta[i] = i > 0 ? __ldcg(&S->beta[i]) : 0.0;
 
   const int lo = j > 0 ? j - 1 : 0;
-  lzc::slice_dots_block(A.V, n, w, e0, len, lo, j + 1, part1, red);
-  lzc::slice_norm(w, len, red, A.partn + A.G);      // ||w||^2 before the projection
+  lzc::slice_dots_block(A.V, n, w, e0, len, lo, j + 1, part1,
+                        A.partn + A.G /* ||w||^2 before the projection */, red);
   if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
   lzc::reduce_dots(part1, A.G, lo, j + 1, h1);
   lzc::reduce_norm(A.partn + A.G, A.G, &s_nrm);
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(LT) lz_step_kernel(LzStepArgs A) {
   }
   __syncthreads();
   if (s_second) {
-    lzc::slice_dots_block(A.V, n, w, e0, len, 0, j + 1, part2, red);
+    lzc::slice_dots_block(A.V, n, w, e0, len, 0, j + 1, part2, nullptr, red);
     if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
     lzc::reduce_dots(part2, A.G, 0, j + 1, h2);
     lzc::slice_project(A.V, n, w, e0, len, 0, j + 1, h2);
@@ -85,9 +85,9 @@ __global__ void __launch_bounds__(LT) lz_step_kernel(LzStepArgs A) {
     const double aj = h1[j].x + h2[j].x;          // alpha_j = Re <q_j, H q_j>
     double yr, yi, err;
     bool done, bd;
+    double nb, inv;
     lzc::tridiag_step(j, aj, s_nrm, A.tr, A.ti, A.tol, A.kcap, A.fixed, alpha, beta, false, yr,
-                      yi, done, err, bd);
-    const double nb = sqrt(s_nrm);
+                      yi, done, err, bd, nb, inv);
     if (blockIdx.x == 0) {
       if (lane == 0) {
         S->h1[j] = h1[j];
@@ -108,12 +108,12 @@ __global__ void __launch_bounds__(LT) lz_step_kernel(LzStepArgs A) {
           S->done = 1;
         }
       } else if (lane == 0) {
-        S->inv = 1.0 / nb;
+        S->inv = inv;
       }
     }
     if (lane == 0) {
       s_done = done ? 1 : 0;
-      s_inv = done ? 0.0 : 1.0 / nb;
+      s_inv = done ? 0.0 : inv;
     }
   }
   __syncthreads();

@@ -2,6 +2,7 @@
 // bounded waits, bulk copies, tcgen05 kind::f16 on K-major tiles without swizzle, the split of an
 // FP64 number into seven signed base-256 digits and the reassembly of the level sums.
 #pragma once
+#include "fp64_util.cuh"
 #include "tdmrg_internal.cuh"
 
 namespace tdmrg {
@@ -94,9 +95,6 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 }
-
-// biased exponent of a double (2047: Inf or NaN)
-__device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
 // x (negated if neg) in units of 2^(E - 55), E = emax - 1022 and |x| < 2^E, rounded, plus 128 in
 // each of its seven base-256 digits: digit l (l = 0 the highest) is bits 48 - 8 l .. of it, less
@@ -206,20 +204,6 @@ __device__ __forceinline__ void read_levels4(uint32_t taddr, uint32_t ldl, uint3
         x[p][c] = from_levels_any(u, eA, eB[c]);
       }
   }
-}
-
-// 1 / sqrt(x) for a positive normal x: single-precision seed y, then the series of
-// (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ... for e = 1 - x y^2 (|e| < 2^-20, so the next term is below
-// 2^-61).  Five FP64 instructions: a warp-wide one holds its pipe for 64 clocks here.
-__device__ __forceinline__ double rsqrt_series(double x) {
-  const long long b = __double_as_longlong(x);
-  const int k = ((int)(b >> 52) - 1023) >> 1;                  // x = xs 4^k, xs in [1, 4)
-  const double xs = __longlong_as_double(b - (long long)(2 * k) * (1LL << 52));
-  const double y0 = (double)rsqrtf(__double2float_rn(xs));
-  const double t = xs * y0;
-  const double e = fma(-t, y0, 1.0);
-  const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
-  return __longlong_as_double(__double_as_longlong(y) - (long long)k * (1LL << 52));
 }
 
 }  // namespace dig
