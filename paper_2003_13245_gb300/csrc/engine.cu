@@ -62,47 +62,60 @@ void heff_f64(const Ctx& c, const DevMpoSite& W, int Ml, int Mr, int D, int d, c
   // X[(w,a)][(s,c)] = sum_y L[w,a,y] in[y,(s,c)]
   CK(zgemm(W.Dl * Ml, D * Mr, Ml, 1, 1, ONE, mref(Lenv, Ml, 1), mref(in, (long long)D * Mr, 1),
            ZERO, c.X, (long long)D * Mr, 0, skip, c.st, c.ws));
+  // out[(a,s)][b] = sum_{v,c} Y[v][(a,s)][c] R[v][b][c],
   // Y[v][a][s][t][c] = sum_{w,u} W[w,v,s,u] X[w][a][u][t][c]
-  CK(mpo_mix(W.lr, Ml, d, Mr, c.X, per, c.Y, per, skip, c.st));
-  // out[(a,s)][b] = sum_{v,c} Y[v][(a,s)][c] R[v][b][c]
-  CK(zgemm(Ml * D, Mr, Mr, 1, W.Dr, ONE, mref(c.Y, Mr, 1, 0, per),
-           mref(Renv, 1, Mr, 0, (long long)Mr * Mr), ZERO, out, Mr, 0, skip, c.st, c.ws));
+  CK(zgemm_mixed(Ml * D, Mr, Mr, 1, W.Dr, mref(c.Y, Mr, 1, 0, per),
+                 mref(Renv, 1, Mr, 0, (long long)Mr * Mr), out, Mr, 0, W.lr, Ml, Mr, c.X, c.Y, true,
+                 skip, c.st, c.ws));
 }
+
+namespace {
+void left_x_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Ml2, int D, int Mr2,
+                const cplx* Lenv, const cplx* ket, const int* skip) {
+  CK(zgemm(W.Dl * Ml1, D * Mr2, Ml2, 1, 1, ONE, mref(Lenv, Ml2, 1),
+           mref(ket, (long long)D * Mr2, 1), ZERO, c.X, (long long)D * Mr2, 0, skip, c.st, c.ws));
+}
+void right_x_f64(const Ctx& c, const DevMpoSite& W, int Ml2, int D, int Mr1, int Mr2,
+                 const cplx* Renv, const cplx* ket, const int* skip) {
+  // X[v][(y,s)][b] = sum_c ket[(y,s)][c] R[v][b][c]
+  CK(zgemm(Ml2 * D, Mr1, Mr2, W.Dr, 1, ONE, mref(ket, Mr2, 1),
+           mref(Renv, 1, Mr2, (long long)Mr1 * Mr2), ZERO, c.X, Mr1, (long long)Ml2 * D * Mr1, skip,
+           c.st, c.ws));
+}
+}  // namespace
 
 void left_partial_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Ml2, int D, int d, int Mr2,
                       const cplx* Lenv, const cplx* ket, cplx* Y, const int* skip) {
   const long long per = (long long)Ml1 * D * Mr2;
-  CK(zgemm(W.Dl * Ml1, D * Mr2, Ml2, 1, 1, ONE, mref(Lenv, Ml2, 1),
-           mref(ket, (long long)D * Mr2, 1), ZERO, c.X, (long long)D * Mr2, 0, skip, c.st, c.ws));
+  left_x_f64(c, W, Ml1, Ml2, D, Mr2, Lenv, ket, skip);
   CK(mpo_mix(W.lr, Ml1, d, Mr2, c.X, per, Y, per, skip, c.st));
 }
 
 void right_partial_f64(const Ctx& c, const DevMpoSite& W, int Ml2, int D, int d, int Mr1, int Mr2,
                        const cplx* Renv, const cplx* ket, cplx* Y, const int* skip) {
   const long long per = (long long)Ml2 * D * Mr1;
-  // X[v][(y,s)][b] = sum_c ket[(y,s)][c] R[v][b][c]
-  CK(zgemm(Ml2 * D, Mr1, Mr2, W.Dr, 1, ONE, mref(ket, Mr2, 1),
-           mref(Renv, 1, Mr2, (long long)Mr1 * Mr2), ZERO, c.X, Mr1, per, skip, c.st, c.ws));
+  right_x_f64(c, W, Ml2, D, Mr1, Mr2, Renv, ket, skip);
   CK(mpo_mix(W.rl, Ml2, d, Mr1, c.X, per, Y, per, skip, c.st));
 }
 
 void env_left_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Mr1, int Ml2, int Mr2, int D,
                   int d, const cplx* Lenv, const cplx* bra, const cplx* ket, cplx* Lout) {
-  left_partial_f64(c, W, Ml1, Ml2, D, d, Mr2, Lenv, ket, c.Y, nullptr);
+  left_x_f64(c, W, Ml1, Ml2, D, Mr2, Lenv, ket, nullptr);
   const long long per = (long long)Ml1 * D * Mr2;
   // Lout[v][b][c] = sum_{(a,s)} conj(bra[(a,s)][b]) Y[v][(a,s)][c]
-  CK(zgemm(Mr1, Mr2, Ml1 * D, W.Dr, 1, ONE, mref(bra, 1, Mr1, 0, 0, 1), mref(c.Y, Mr2, 1, per),
-           ZERO, Lout, Mr2, (long long)Mr1 * Mr2, nullptr, c.st, c.ws));
+  CK(zgemm_mixed(Mr1, Mr2, Ml1 * D, W.Dr, 1, mref(bra, 1, Mr1, 0, 0, 1), mref(c.Y, Mr2, 1, per),
+                 Lout, Mr2, (long long)Mr1 * Mr2, W.lr, Ml1, Mr2, c.X, c.Y, false, nullptr, c.st,
+                 c.ws));
 }
 
 void env_right_f64(const Ctx& c, const DevMpoSite& W, int Ml1, int Mr1, int Ml2, int Mr2, int D,
                    int d, const cplx* Renv, const cplx* bra, const cplx* ket, cplx* Rout) {
-  right_partial_f64(c, W, Ml2, D, d, Mr1, Mr2, Renv, ket, c.Y, nullptr);
+  right_x_f64(c, W, Ml2, D, Mr1, Mr2, Renv, ket, nullptr);
   const long long per = (long long)Ml2 * D * Mr1;
   // Rout[w][a][y] = sum_{(s,b)} conj(bra[a][(s,b)]) Y[w][y][(s,b)]
-  CK(zgemm(Ml1, Ml2, D * Mr1, W.Dl, 1, ONE, mref(bra, (long long)D * Mr1, 1, 0, 0, 1),
-           mref(c.Y, 1, (long long)D * Mr1, per), ZERO, Rout, Ml2, (long long)Ml1 * Ml2,
-           nullptr, c.st, c.ws));
+  CK(zgemm_mixed(Ml1, Ml2, D * Mr1, W.Dl, 1, mref(bra, (long long)D * Mr1, 1, 0, 0, 1),
+                 mref(c.Y, 1, (long long)D * Mr1, per), Rout, Ml2, (long long)Ml1 * Ml2, W.rl, Ml2,
+                 Mr1, c.X, c.Y, false, nullptr, c.st, c.ws));
 }
 
 void bond_f64(const Ctx& c, int M, int Dw, const cplx* Lenv, const cplx* Renv, const cplx* in,
@@ -354,50 +367,84 @@ void Engine::upload_mpo(const std::vector<MpoSite>& W, DevMpo& out, bool pooled,
       }
       irl_start[h.Dl] = pos;
     }
-    const size_t ops_bytes = sizeof(cplx) * (size_t)nb * d * d;
-    const size_t ops32_bytes = sizeof(float2) * (size_t)nb * d * d;
-    const size_t int_bytes = sizeof(int) * (size_t)(h.Dr + 1 + nb + h.Dl + 1 + nb);
-    const size_t total = 2 * ops_bytes + 2 * ops32_bytes + int_bytes + 64;
-    char* mem = nullptr;
-    if (pooled)
-      CK(zg_pool_alloc(reinterpret_cast<void**>(&mem), total, stream));
-    else
-      CK(cudaMalloc(&mem, total));
-    s.mem = mem;
-    s.pooled = pooled;
-    s.stream = stream;
-    cplx* d_olr = reinterpret_cast<cplx*>(mem);
-    cplx* d_orl = d_olr + (size_t)nb * d * d;
-    float2* d_flr = reinterpret_cast<float2*>(d_orl + (size_t)nb * d * d);
-    float2* d_frl = d_flr + (size_t)nb * d * d;
-    int* ip = reinterpret_cast<int*>(d_frl + (size_t)nb * d * d);
-    int* d_lrs = ip;
-    int* d_lrc = d_lrs + h.Dr + 1;
-    int* d_rls = d_lrc + nb;
-    int* d_rlc = d_rls + h.Dl + 1;
+    // nonzero entries by output channel and level, in the order of the dense tables
+    auto sparse = [&](const std::vector<int>& st, const std::vector<int>& chan,
+                      const std::vector<cplx>& op, int Dout, std::vector<int>& start,
+                      std::vector<int2>& cu, std::vector<cplx>& val) {
+      start.assign((size_t)Dout * d + 1, 0);
+      for (int wo = 0; wo < Dout; ++wo)
+        for (int sg = 0; sg < d; ++sg) {
+          for (int q = st[wo]; q < st[wo + 1]; ++q)
+            for (int u = 0; u < d; ++u) {
+              const cplx v = op[((size_t)q * d + sg) * d + u];
+              if (v.x != 0.0 || v.y != 0.0) {
+                cu.push_back(make_int2(chan[q], u));
+                val.push_back(make_double2(v.x, v.y == 0.0 ? 0.0 : v.y));
+              }
+            }
+          start[(size_t)wo * d + sg + 1] = (int)cu.size();
+        }
+    };
+    std::vector<int> slr, srl;
+    std::vector<int2> clr, crl;
+    std::vector<cplx> vlr, vrl;
+    sparse(ilr_start, ilr_chan, olr, h.Dr, slr, clr, vlr);
+    sparse(irl_start, irl_chan, orl, h.Dl, srl, crl, vrl);
     std::vector<float2> flr(olr.size()), frl(orl.size());
     for (size_t e = 0; e < olr.size(); ++e) flr[e] = make_float2((float)olr[e].x, (float)olr[e].y);
     for (size_t e = 0; e < orl.size(); ++e) frl[e] = make_float2((float)orl[e].x, (float)orl[e].y);
-    // one host image, one copy
-    std::vector<char> host(total, 0);
-    auto put = [&](const void* dev, const void* src, size_t bytes) {
-      if (bytes) std::memcpy(host.data() + (static_cast<const char*>(dev) - mem), src, bytes);
+    // one host image of all tables, one copy
+    std::vector<char> host;
+    auto put = [&](const void* src, size_t bytes) {
+      const size_t at = host.size();
+      host.resize(at + ((bytes + 15) & ~(size_t)15));
+      if (bytes) std::memcpy(host.data() + at, src, bytes);
+      return at;
     };
-    put(d_olr, olr.data(), ops_bytes);
-    put(d_orl, orl.data(), ops_bytes);
-    put(d_flr, flr.data(), ops32_bytes);
-    put(d_frl, frl.data(), ops32_bytes);
-    put(d_lrs, ilr_start.data(), sizeof(int) * (h.Dr + 1));
-    put(d_lrc, ilr_chan.data(), sizeof(int) * nb);
-    put(d_rls, irl_start.data(), sizeof(int) * (h.Dl + 1));
-    put(d_rlc, irl_chan.data(), sizeof(int) * nb);
+    const size_t o_olr = put(olr.data(), sizeof(cplx) * olr.size());
+    const size_t o_orl = put(orl.data(), sizeof(cplx) * orl.size());
+    const size_t o_vlr = put(vlr.data(), sizeof(cplx) * vlr.size());
+    const size_t o_vrl = put(vrl.data(), sizeof(cplx) * vrl.size());
+    const size_t o_flr = put(flr.data(), sizeof(float2) * flr.size());
+    const size_t o_frl = put(frl.data(), sizeof(float2) * frl.size());
+    const size_t o_clr = put(clr.data(), sizeof(int2) * clr.size());
+    const size_t o_crl = put(crl.data(), sizeof(int2) * crl.size());
+    const size_t o_lrs = put(ilr_start.data(), sizeof(int) * ilr_start.size());
+    const size_t o_lrc = put(ilr_chan.data(), sizeof(int) * ilr_chan.size());
+    const size_t o_rls = put(irl_start.data(), sizeof(int) * irl_start.size());
+    const size_t o_rlc = put(irl_chan.data(), sizeof(int) * irl_chan.size());
+    const size_t o_slr = put(slr.data(), sizeof(int) * slr.size());
+    const size_t o_srl = put(srl.data(), sizeof(int) * srl.size());
+    char* mem = nullptr;
+    if (pooled)
+      CK(zg_pool_alloc(reinterpret_cast<void**>(&mem), host.size(), stream));
+    else
+      CK(cudaMalloc(&mem, host.size()));
+    s.mem = mem;
+    s.pooled = pooled;
+    s.stream = stream;
     // (a copy from pageable memory has taken its source when the call returns)
     if (pooled)
-      CK(cudaMemcpyAsync(mem, host.data(), total, cudaMemcpyHostToDevice, stream));
+      CK(cudaMemcpyAsync(mem, host.data(), host.size(), cudaMemcpyHostToDevice, stream));
     else
-      CK(cudaMemcpy(mem, host.data(), total, cudaMemcpyHostToDevice));
-    s.lr = MixTable{h.Dr, d_lrs, d_lrc, d_olr, d_flr, nb};
-    s.rl = MixTable{h.Dl, d_rls, d_rlc, d_orl, d_frl, nb};
+      CK(cudaMemcpy(mem, host.data(), host.size(), cudaMemcpyHostToDevice));
+    auto table = [&](int Dout, size_t st, size_t ch, size_t op, size_t f32, size_t sps, size_t spc,
+                     size_t spv) {
+      MixTable t{};
+      t.Dout = Dout;
+      t.start = reinterpret_cast<int*>(mem + st);
+      t.chan = reinterpret_cast<int*>(mem + ch);
+      t.ops = reinterpret_cast<cplx*>(mem + op);
+      t.ops32 = reinterpret_cast<float2*>(mem + f32);
+      t.nblk = nb;
+      t.d = d;
+      t.sp_start = reinterpret_cast<int*>(mem + sps);
+      t.sp_cu = reinterpret_cast<int2*>(mem + spc);
+      t.sp_val = reinterpret_cast<cplx*>(mem + spv);
+      return t;
+    };
+    s.lr = table(h.Dr, o_lrs, o_lrc, o_olr, o_flr, o_slr, o_clr, o_vlr);
+    s.rl = table(h.Dl, o_rls, o_rlc, o_orl, o_frl, o_srl, o_crl, o_vrl);
   }
 }
 

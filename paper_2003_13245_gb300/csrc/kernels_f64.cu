@@ -2,6 +2,7 @@
 // the environment updates and the bond step), sparse MPO channel mixing, the one-launch
 // norm, the start and final combination of a Lanczos run, and the column-wise cooperative
 // gauge QR (completion pass and kernel-level entry points).
+#include "mix.cuh"
 #include "tdmrg_internal.cuh"
 
 #include <atomic>
@@ -124,6 +125,33 @@ __global__ void __launch_bounds__(256) zgemm_kernel(int m, int n, int k, int nre
   }
 }
 
+cudaError_t zgemm_mixed(int m, int n, int k, int nbatch, int nred, MatRef A, MatRef B, cplx* C,
+                        long long ldc, long long sc, const MixTable& T, int Ma, int Mb,
+                        const cplx* X, cplx* Y, bool mixA, const int* skip, cudaStream_t s,
+                        ZgWork* ws) {
+  const cplx one = {1.0, 0.0}, zero = {0.0, 0.0};
+  const long long per = (long long)Ma * T.d * T.d * Mb;
+  if (ws && ws->status && (long long)k * nred > 1 && per < 0x7fffffffLL) {
+    MatRef a = A, b = B;
+    MatRef& x = mixA ? a : b;
+    x.p = X;
+    x.mix = &T;
+    x.xs = per;
+    x.dmb = T.d * Mb;
+    cudaError_t e = zg_reserve(*ws, zgemm_digits_bytes(m, n, k, nbatch, nred, A.sb == 0 ? 1 : nbatch,
+                                                       B.sb == 0 ? 1 : nbatch), s);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    else if (e != cudaSuccess) return e;
+    bool taken = false;
+    if (ws->p) e = zgemm_digits(m, n, k, nbatch, nred, one, a, b, zero, C, ldc, sc, skip, *ws, s,
+                                &taken);
+    if (taken || (ws->p && e != cudaSuccess)) return e;
+  }
+  const cudaError_t e = mpo_mix(T, Ma, T.d, Mb, X, per, Y, per, skip, s);
+  return e != cudaSuccess ? e
+                          : zgemm(m, n, k, nbatch, nred, one, A, B, zero, C, ldc, sc, skip, s, ws);
+}
+
 // With a workspace every product of two or more terms goes to the digit products: measured on
 // GB300 they are faster from the smallest shapes (4 x 4 x 4: 18.6 against 68 us, a 64 x 64 tile
 // of FMAs being the least this kernel does; 64 x 64 x 256, 7 batches: 35 against 1048 us) to the
@@ -156,42 +184,37 @@ cudaError_t zgemm(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef 
 // ------------------------------------------------------------------------------------
 // MPO channel mixing
 // ------------------------------------------------------------------------------------
-__global__ void mpo_mix_kernel(int Dout, int Ma, int d, int Mb, const int* start,
-                               const int* chan, const cplx* ops, const cplx* X, long long xs,
-                               cplx* Y, long long ys, const int* skip) {
+// blockIdx.y is one output channel and level (wo, s), whose few nonzero entries are the same for
+// the whole block; the threads run over (a, t, b), contiguous in t and b.  Bound by the reads of X
+// (mostly from L2) and the write of Y; entries of 1 cost no FP64 instruction, real ones two.
+__global__ void __launch_bounds__(256) mpo_mix_kernel(int Ma, int d, int Mb, const int* start,
+                                                      const int2* cu, const cplx* val,
+                                                      const cplx* X, long long xs, cplx* Y,
+                                                      long long ys, const int* skip) {
   if (skip && *skip) return;
-  const long long per = (long long)Ma * d * d * Mb;
-  const long long total = per * Dout;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    long long r = e;
-    const int b = (int)(r % Mb); r /= Mb;
-    const int tau = (int)(r % d); r /= d;
-    const int sig = (int)(r % d); r /= d;
-    const int a = (int)(r % Ma);
-    const int wo = (int)(r / Ma);
-    cplx acc = make_double2(0.0, 0.0);
-    for (int blk = start[wo]; blk < start[wo + 1]; ++blk) {
-      const cplx* op = ops + (long long)blk * d * d + sig * d;
-      const cplx* x = X + chan[blk] * xs + ((long long)a * d * d + tau) * Mb + b;
-      for (int u = 0; u < d; ++u) {
-        const cplx o = op[u];
-        if (o.x != 0.0 || o.y != 0.0) cfma(acc, o, x[(long long)u * d * Mb]);
-      }
-    }
-    Y[wo * ys + (e - (long long)wo * per)] = acc;
+  const int dmb = d * Mb, ddmb = d * dmb;
+  const int wo = blockIdx.y / d, sig = blockIdx.y % d;
+  const int lo = start[blockIdx.y], hi = start[blockIdx.y + 1];
+  const int total = Ma * dmb;
+  cplx* y = Y + wo * ys + (long long)sig * dmb;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
+    const int a = i / dmb, tb = i - a * dmb;
+    const long long off = (long long)a * ddmb + tb;
+    y[off] = mix_entries(lo, hi, cu, val, X + off, xs, dmb);
   }
 }
 
 cudaError_t mpo_mix(const MixTable& T, int Ma, int d, int Mb, const cplx* X, long long xs,
                     cplx* Y, long long ys, const int* skip, cudaStream_t s) {
-  const long long total = (long long)T.Dout * Ma * d * d * Mb;
-  if (total <= 0) return cudaSuccess;
+  const long long total = (long long)Ma * d * Mb;
+  if (total <= 0 || T.Dout <= 0) return cudaSuccess;
+  if (total > 0x7fffffffLL - 256 * 152 * 32 || (long long)T.Dout * d > 65535)
+    return cudaErrorInvalidValue;
   long long blocks = (total + 255) / 256;
-  if (blocks > 152 * 32) blocks = 152 * 32;
+  if (blocks > 152 * 16) blocks = 152 * 16;
   count_launch();
-  mpo_mix_kernel<<<(int)blocks, 256, 0, s>>>(T.Dout, Ma, d, Mb, T.start, T.chan, T.ops, X, xs,
-                                              Y, ys, skip);
+  mpo_mix_kernel<<<dim3((unsigned)blocks, T.Dout * d), 256, 0, s>>>(Ma, d, Mb, T.sp_start, T.sp_cu,
+                                                                    T.sp_val, X, xs, Y, ys, skip);
   return cudaGetLastError();
 }
 

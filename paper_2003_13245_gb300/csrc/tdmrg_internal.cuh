@@ -19,10 +19,16 @@ void count_launch(int n = 1);
 
 // Strided view of a matrix operand: element (i, j) = p[i * rs + j * cs] (conjugated if conj),
 // batch b / reduction term r shift the pointer by b * sb + r * sr.
+struct MixTable;
 struct MatRef {
   const cplx* p;
   long long rs, cs, sb, sr;
   int conj;
+  // zgemm_mixed: the operand is not stored but mixed on the fly, p = X[wi][a][u][t][b] (xs entries
+  // per channel, dmb = d * (extent of b)); the strides address Y[wo][a][s][t][b]
+  const MixTable* mix = nullptr;
+  long long xs = 0;
+  int dmb = 0;
 };
 
 // Workspace of the digit products of zgemm (zgemm_digits.cu) for calls on one stream at a time:
@@ -67,7 +73,18 @@ struct MixTable {
   const cplx* ops;       // d x d per block
   const float2* ops32;   // the same operators rounded to FP32 (mixed-precision path)
   int nblk;
+  // the nonzero entries by output channel and level (wo * d + s): input channel and level, value
+  int d;
+  const int* sp_start;   // Dout * d + 1
+  const int2* sp_cu;
+  const cplx* sp_val;
 };
+// zgemm of an operand A (or B) mixed from X: with a workspace the mixing happens where the operand
+// is split into digits, otherwise mpo_mix writes it to Y (Ma x d x d x Mb per channel) first
+cudaError_t zgemm_mixed(int m, int n, int k, int nbatch, int nred, MatRef A, MatRef B, cplx* C,
+                        long long ldc, long long sc, const MixTable& T, int Ma, int Mb,
+                        const cplx* X, cplx* Y, bool mixA, const int* skip, cudaStream_t s,
+                        ZgWork* ws);
 cudaError_t mpo_mix(const MixTable& T, int Ma, int d, int Mb, const cplx* X, long long xs,
                     cplx* Y, long long ys, const int* skip, cudaStream_t s);
 

@@ -30,6 +30,7 @@
 // FMA kernel: 896 x 8192 x 128 0.28 against 6.2 ms (27 TFLOP/s, tensor pipe 39 %); 8192 x 128 x 128
 // summed over seven channels 0.35 against 7.3 ms; 128 x 128 x 8192, seven batches, 0.55 against
 // 34 ms; 64 x 64 x 256, seven batches, 35 against 1048 us; 16 x 16 x 4 21 against 68 us.
+#include "mix.cuh"
 #include "umma.cuh"
 
 #include <mutex>
@@ -61,6 +62,14 @@ struct Operand {
   int tiles;                  // row tiles
   unsigned char* dig;         // [nb][tiles][steps] blocks
   int* ex;                    // [nb][chunks][tiles * tile]
+  // mixed on the fly (mix_start != NULL): p = X, the strides address Y
+  const int* mix_start;
+  const int2* mix_cu;
+  const cplx* mix_val;
+  long long xs;
+  int dmb, d, b0;             // b0: first batch of a slab
+  long long off0;             // offset of the first row of a slab
+  int by_red;                 // the channel is the reduction term (else the batch)
 };
 
 struct SplitArgs {
@@ -97,7 +106,17 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
   for (int e = threadIdx.x; e < SR * KC; e += 256) {
     const int r = kfast ? e / KC : e % SR, k = kfast ? e % KC : e / SR;
     cplx v = make_double2(0.0, 0.0);
-    if (r0 + r < o.rows && k < kn) v = src[(long long)(r0 + r) * o.rs + (long long)(k0 + k) * o.ks];
+    if (r0 + r < o.rows && k < kn) {
+      const long long off = (long long)(r0 + r) * o.rs + (long long)(k0 + k) * o.ks;
+      if (!o.mix_start) {
+        v = src[off];
+      } else {
+        const int idx = (int)(off + o.off0), sig = (idx / o.dmb) % o.d;
+        const int* st = o.mix_start + (o.by_red ? red : b + o.b0) * o.d + sig;
+        v = mix_entries(__ldg(st), __ldg(st + 1), o.mix_cu, o.mix_val, o.p + (idx - sig * o.dmb),
+                        o.xs, o.dmb);
+      }
+    }
     s_v[r * S_LD + k] = v;
   }
   __syncthreads();
@@ -449,8 +468,28 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
   // are then contiguous across the lanes
   auto tiles = [](int a, int t) { return (long long)(a + t - 1) / t; };
   const bool swap = tiles(n, PT) * tiles(m, QT) <= tiles(m, PT) * tiles(n, QT);
-  Operand a{A.p, A.rs, A.cs, A.sb, A.sr, A.conj, m, A.sb == 0 ? 1 : nbatch, 0, 0, nullptr, nullptr};
-  Operand b{B.p, B.cs, B.rs, B.sb, B.sr, B.conj, n, B.sb == 0 ? 1 : nbatch, 0, 0, nullptr, nullptr};
+  auto operand = [&](const MatRef& M, int rows, long long rs, long long ks) {
+    Operand o{};
+    o.p = M.p;
+    o.rs = rs;
+    o.ks = ks;
+    o.sb = M.sb;
+    o.sr = M.sr;
+    o.conj = M.conj;
+    o.rows = rows;
+    o.nb = M.sb == 0 ? 1 : nbatch;
+    if (M.mix) {
+      o.mix_start = M.mix->sp_start;
+      o.mix_cu = M.mix->sp_cu;
+      o.mix_val = M.mix->sp_val;
+      o.xs = M.xs;
+      o.dmb = M.dmb;
+      o.d = M.mix->d;
+      o.by_red = M.sr != 0;
+    }
+    return o;
+  };
+  const Operand a = operand(A, m, A.rs, A.cs), b = operand(B, n, B.cs, B.rs);
   Operand P = swap ? b : a, Q = swap ? a : b;
   const long long cp = swap ? 1 : ldc, cq = swap ? ldc : 1;
   P.tile = PT;
@@ -478,8 +517,15 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
         q.tiles = q0 + nq < qt_all ? nq : qt_all - q0;
         p.rows = P.rows - p0 * PT < p.tiles * PT ? P.rows - p0 * PT : p.tiles * PT;
         q.rows = Q.rows - q0 * QT < q.tiles * QT ? Q.rows - q0 * QT : q.tiles * QT;
-        p.p += (long long)p0 * PT * P.rs + (long long)b0 * P.sb;
-        q.p += (long long)q0 * QT * Q.rs + (long long)b0 * Q.sb;
+        for (Operand* o : {&p, &q}) {
+          const long long row0 = o == &p ? (long long)p0 * PT : (long long)q0 * QT;
+          if (o->mix_start) {
+            o->off0 = row0 * o->rs;
+            o->b0 = b0;
+          } else {
+            o->p += row0 * o->rs + (long long)b0 * o->sb;
+          }
+        }
         p.nb = P.nb == 1 ? 1 : bb;
         q.nb = Q.nb == 1 ? 1 : bb;
         // carve the workspace
