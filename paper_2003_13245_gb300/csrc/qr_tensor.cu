@@ -4,6 +4,7 @@
 // zgemm_digits.cu) instead of FP64 FMAs.
 //
 // CTA g owns a slice of at most 128 rows of Y, Q and the working block V (shared memory, FP64).
+// Up to 256 columns: the accepted vectors enter the products in tiles of 128.
 // The digits of the accepted columns of its slice are kept in global memory in the two operand
 // forms the products need (K = rows for Q^H V, K = columns for Q P); both are private to the CTA
 // and stream through a two-stage ring of bulk copies.  The first form has one scale per column,
@@ -34,10 +35,12 @@
 // which n lie in the span:
 //                     152 CTAs                          76 CTAs (two lanes)
 //   m x n        full rank    rank 2              full rank    rank 2
-//   64 x 16       97 / 109     754 / 235
-//   144 x 64     374 / 378    3312 / 661
-//   512 x 128    845 / 859    7934 / 1334
-//   2048 x 128  1156 / 845   12461 / 1351        1658 / 847   12275 / 1351
+//   64 x 16       98 / 109     748 / 231
+//   144 x 64     371 / 374    3152 / 641
+//   512 x 128    815 / 846    8258 / 1355
+//   512 x 256   2098 / 2018  23093 / 3204
+//   2048 x 128  1155 / 836   12395 / 1391        1658 / 847   12275 / 1351
+//   2048 x 144  1380 / 956   20269 / 1607
 //   8192 x 128  2682 / 1022  19468 / 1765        4516 / 1255  25260 / 2302
 // Below nine columns the other kernel is the faster one at full rank (256 x 4: 55 against 95 us),
 // where such bonds, at the ends of a chain, mostly are.  About 32 rows per CTA: fewer rows raise the
@@ -53,12 +56,14 @@ namespace {
 constexpr int QB = 16;                          // columns per block
 constexpr int QT_THREADS = 256;
 constexpr int MAXR = 128;                       // rows of a CTA
-constexpr int MAXN = 128;                       // columns
+constexpr int MAXN = 256;                       // columns
+constexpr int TILE = 128;                       // accepted vectors of one product
 constexpr int MINN = 9;                         // fewer: qr_blocked.cu (one block, no projection)
 constexpr int GROUP = 2 * ND * 2 * 128;         // digits of 8 rows x 16 k: 3584 bytes
 constexpr int RING = 16 * GROUP;                // one k step of 128 rows: 57344 bytes
 constexpr int BSTEP = 2 * ND * 2 * 2 * 128;     // 16 columns x 16 k: 7168 bytes
 constexpr int BDIG = 8 * BSTEP;                 // 57344 bytes
+constexpr int PASSES = 4;
 constexpr int E_EMPTY = -100000;
 constexpr int TMEM_COLS = 512;
 constexpr int IM = NL * QB;                     // im levels after the re levels
@@ -68,8 +73,8 @@ struct QtArgs {
   QrRef Y, E;
   cplx* Q;
   cplx* R;
-  cplx* part;               // [G][PS]
-  cplx* fin;                // [PS]
+  cplx* part;               // [2][G][PS], used in turn
+  cplx* fin;                // [PASSES][PS]
   int PS;
   unsigned char* dig;       // per CTA: form 1 then form 2
   long long dig_cta;        // bytes of one CTA
@@ -114,22 +119,33 @@ __device__ bool qt_barrier(const QtArgs& A, unsigned& epoch, int* s_ok) {
   return *s_ok != 0;
 }
 
-// fin[0..cnt) = sum over the CTAs of part[.][0..cnt) in a fixed order; every CTA sums a slice of the
-// entries
-__device__ bool qt_reduce(const QtArgs& A, int cnt, unsigned& ep, int* s_ok) {
+// fin[0..cnt) = sum over the CTAs of part[.][0..cnt) in a fixed order.  Every CTA sums a slice of
+// the entries and a second barrier makes all of them readable; where all partial sums are few,
+// every CTA sums them itself into its shared copy `own` (the same order, so the same result) and
+// the second barrier is left out (a CTA may then still read partial sums when another goes on:
+// two sets of them are used in turn).  Returns where to read the sums.
+constexpr int OWN = 512;                        // entries a CTA may sum for itself
+__device__ const cplx* qt_reduce(const QtArgs& A, int cnt, const cplx* part, cplx* fin, cplx* own,
+                                 unsigned& ep, int* s_ok) {
   const int G = gridDim.x;
-  if (!qt_barrier(A, ep, s_ok)) return false;
-  const int per = (cnt + G - 1) / G;
-  const int lo = blockIdx.x * per, hi = min(cnt, lo + per);
+  if (G > 1) {
+    if (!qt_barrier(A, ep, s_ok)) return nullptr;
+  } else {
+    __syncthreads();
+  }
+  const bool alone = cnt <= OWN && cnt * G <= 4096;
+  const int per = alone ? cnt : (cnt + G - 1) / G;
+  const int lo = alone ? 0 : blockIdx.x * per, hi = min(cnt, lo + per);
+  cplx* out = alone ? own : fin;
   // L lanes per entry, so that one round of loads covers the slice where possible
   int L = 32;
-  while (L > 1 && per * L > QT_THREADS) L >>= 1;
+  while (L > 1 && (per * L > QT_THREADS || L > G)) L >>= 1;
   const int sub = threadIdx.x & (L - 1);
   for (int e0 = lo; e0 < hi; e0 += QT_THREADS / L) {
     const int e = e0 + threadIdx.x / L;
     double ax = 0.0, ay = 0.0;
     if (e < hi) {
-      const cplx* src = A.part + e;
+      const cplx* src = part + e;
 #pragma unroll 4
       for (int g = sub; g < G; g += L) {
         const cplx u = __ldcg(src + (long long)g * A.PS);
@@ -141,9 +157,16 @@ __device__ bool qt_reduce(const QtArgs& A, int cnt, unsigned& ep, int* s_ok) {
       ax += __shfl_xor_sync(0xffffffffu, ax, o);
       ay += __shfl_xor_sync(0xffffffffu, ay, o);
     }
-    if (sub == 0 && e < hi) A.fin[e] = make_double2(ax, ay);
+    if (sub == 0 && e < hi) {
+      out[e] = make_double2(ax, ay);
+      if (alone && blockIdx.x == 0) fin[e] = make_double2(ax, ay);   // R is formed from it
+    }
   }
-  return qt_barrier(A, ep, s_ok);
+  if (alone) {
+    __syncthreads();
+    return own;
+  }
+  return qt_barrier(A, ep, s_ok) ? fin : nullptr;
 }
 
 __device__ __forceinline__ cplx qt_load(const QrRef& Y, long long r, long long c) {
@@ -163,10 +186,11 @@ struct Pipe {
 };
 
 // Issued by thread 0.  D += sum over S k steps of A_s B_s: A from `src` (step s at s * stride,
-// `bytes` of it) through the ring, B in shared memory at bdig + s * BSTEP.  conj: Q^H V (re = ArBr
+// `bytes` of it, at `off` of a stage) through the ring, B in shared memory at bdig + s * BSTEP.  conj: Q^H V (re = ArBr
 // + AiBi, im = ArBi - AiBr), else Q P (re = ArBr - AiBi, im = ArBi + AiBr).  gram: also V^H V of
 // the same B tiles into columns 256.. (A = the B tile itself, its rows beyond 16 unused).
-__device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, const unsigned char* bdig,
+__device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
+                        const unsigned char* bdig,
                         const unsigned char* src, long long stride, uint32_t bytes, int S,
                         bool conj, int gram_steps) {
   bool ok = true;
@@ -175,7 +199,7 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, const unsig
   auto load = [&](int s) {
     const int st = (it0 + s) & 1;
     mbar_expect_tx(&P.full[st], bytes);
-    bulk_load(ring + st * RING, src + s * stride, bytes, &P.full[st]);
+    bulk_load(ring + st * RING + off, src + s * stride, bytes, &P.full[st]);
     ++issued;
   };
   auto tile = [&](uint32_t a, uint32_t lbo, uint32_t sbo, uint32_t apart, uint32_t adig, uint32_t b,
@@ -268,11 +292,12 @@ struct Shared {
   double lim[QB];            // completion: smallest residual norm of a candidate that is taken
   int em[QB];                // largest biased exponent of a column (digit scale)
   int ev[QB];                // its digit scale E
-  int idx[MAXN];             // column of Q of every accepted vector, in order of acceptance
+  short idx[MAXN];           // column of Q of every accepted vector, in order of acceptance
+  cplx own[OWN];             // sums of a small reduction
   int ec[MAXN];              // form 1: scale of every accepted vector (this CTA's rows)
   int er[MAXR];              // form 2: scale of every row (E_EMPTY: nothing but zeros so far)
   int rnew[MAXR];            // largest biased exponent of a row's new entries
-  int acc[MAXN];             // accepted (main factorisation) or filled (completion)
+  unsigned char acc[MAXN];   // accepted (main factorisation) or filled (completion)
   int take[QB];
   int src[QB];               // block column of the block's i-th accepted vector
   int drop[QB];              // skipped before the in-block factorisation
@@ -304,6 +329,8 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
   unsigned char* d1 = A.dig + blockIdx.x * A.dig_cta;           // [rstep][column group][GROUP]
   unsigned char* d2 = d1 + (long long)rsteps * ngroups * GROUP; // [column step][row group][GROUP]
   const long long s1 = (long long)ngroups * GROUP, s2 = (long long)rgroups * GROUP;
+  const long long pset = (long long)gridDim.x * A.PS;
+  const cplx* part = A.part;
   cplx* mypart = A.part + (long long)blockIdx.x * A.PS;
   unsigned ep = 0;
   bool alive = true;
@@ -384,9 +411,10 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
     if (tid < QB) S.drop[tid] = tid < bsz ? 0 : 1;
     __syncthreads();
     // ---- projection passes
-    cplx racc[MAXN / QB];
+    bool private_r = false;   // some of the sums were not published
+    int npass = 0;            // passes whose coefficients belong to R
     bool all_dropped = false;
-    for (int pass = 0; pass < 4; ++pass) {
+    for (int pass = 0; pass < PASSES; ++pass) {
       // digits of V, one scale per column (two columns per warp)
       const bool gram = pass > 0 || na == 0;
       {
@@ -418,41 +446,58 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
       }
       asm volatile("fence.proxy.async;" ::: "memory");
       __syncthreads();
-      if (tid == 0)
-        qt_gemm(P, tmem, ring, bdig, d1, s1, (uint32_t)((na + 7) / 8 * GROUP), na > 0 ? rsteps : 0,
-                true, gram ? rsteps : 0);
-      __syncwarp();
-      alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
-      ++P.gemms;
-      alive = __syncthreads_and(alive ? 1 : 0) != 0;
-      if (!alive) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      {
+      // P and V^H V, a tile of accepted vectors at a time.  With at most 96 vectors in a tile they
+      // sit in its rows 32.., so that the warps of rows 0-31 have the Gram matrix alone.
+      for (int i0 = 0; i0 == 0 || i0 < na; i0 += TILE) {
+        const int ni = min(TILE, na - i0);
+        const bool g0 = gram && i0 == 0;
+        const int shift = g0 && ni <= TILE - 32 ? 32 : 0;
+        if (tid == 0)
+          qt_gemm(P, tmem, ring, shift / 8 * GROUP, bdig, d1 + (long long)(i0 / 8) * GROUP, s1,
+                  (uint32_t)((ni + 7) / 8 * GROUP), ni > 0 ? rsteps : 0, true, g0 ? rsteps : 0);
+        __syncwarp();
+        alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
+        ++P.gemms;
+        alive = __syncthreads_and(alive ? 1 : 0) != 0;
+        if (!alive) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int quad = warp & 3, t0 = (warp >> 2) * 8;
-        const int row = quad * 32 + lane;
+        const int row = quad * 32 + lane - shift;
         const uint32_t addr = tmem + ((uint32_t)(quad * 32) << 16) + t0;
         cplx out[8];
-        if (quad * 32 < na) {
-          qt_read(addr, S.ec[min(row, na - 1)], S.ev + t0, out);
-          if (row < na)
+        if (quad * 32 >= shift && quad * 32 - shift < ni) {
+          qt_read(addr, S.ec[i0 + min(row, ni - 1)], S.ev + t0, out);
+          if (row < ni)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) mypart[row * QB + t0 + c] = out[c];
+            for (int c = 0; c < 8; ++c) mypart[(i0 + row) * QB + t0 + c] = out[c];
         }
-        if (gram && quad == 0) {
+        if (g0 && quad == 0) {
           qt_read(addr + 2 * IM, S.ev[lane & 15], S.ev + t0, out);
           if (lane < QB)
 #pragma unroll
             for (int c = 0; c < 8; ++c) mypart[na * QB + lane * QB + t0 + c] = out[c];
         }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        if (i0 + TILE < na) {
+          __syncthreads();
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      if (!qt_reduce(A, na * QB + (gram ? QB * QB : QB) + (started ? 0 : 1), ep, &S.ok)) {
+      if (!alive) break;
+      cplx* fin = A.fin + (long long)pass * A.PS;
+      const int cnt = na * QB + (gram ? QB * QB : QB) + (started ? 0 : 1);
+      const cplx* sum = qt_reduce(A, cnt, part, fin, S.own, ep, &S.ok);
+      if (!sum) {
         alive = false;
         break;
       }
+      mypart += part == A.part ? pset : -pset;
+      part = part == A.part ? A.part + pset : A.part;
+      if (sum == S.own) private_r = true;
+      auto take_sum = [&](int e) { return sum == S.own ? S.own[e] : __ldcg(sum + e); };
       if (!started) {
         started = true;
-        const double y2 = __ldcg(&A.fin[QB * QB]).x;
+        const double y2 = take_sum(QB * QB).x;
         if (!(y2 < 1.7976931348623157e308)) {
           // Inf or NaN in Y: every column is skipped
           bsz = n;
@@ -463,45 +508,42 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         thr2 = thr * thr;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // P into shared memory, |P|^2 and its scale per column
-      cplx hreg[MAXN / QB];
-      {
+      if (gram) S.G[tid >> 4][tid & 15] = take_sum(na * QB + tid);
+      else if (tid < QB) S.G[tid][tid] = take_sum(na * QB + tid);
+      // one tile of P: into shared memory, its |P|^2 and its scale per column
+      cplx hreg[TILE / QB];
+      double hsum = 0.0;
+      auto load_p = [&](int i0) {
         const int t = tid & 15, q = tid >> 4;
         if (tid < QB) S.em[tid] = 0;
 #pragma unroll
-        for (int k = 0; k < MAXN / QB; ++k)
-          hreg[k] = k * QB + q < na ? __ldcg(&A.fin[(k * QB + q) * QB + t]) : make_double2(0.0, 0.0);
-        if (gram) S.G[q][t] = __ldcg(&A.fin[na * QB + tid]);
-        else if (q == 0) S.G[t][t] = __ldcg(&A.fin[na * QB + t]);
+        for (int k = 0; k < TILE / QB; ++k) {
+          const int i = i0 + k * QB + q;
+          hreg[k] = i < na ? take_sum(i * QB + t) : make_double2(0.0, 0.0);
+        }
         __syncthreads();
         int e = 0;
 #pragma unroll
-        for (int k = 0; k < MAXN / QB; ++k)
-          if (k * QB < na) {
+        for (int k = 0; k < TILE / QB; ++k)
+          if (i0 + k * QB < na) {
             const cplx h = hreg[k];
-            if (k * QB + q < na) H[(k * QB + q) * QB + t] = h;
+            if (i0 + k * QB + q < na) H[(k * QB + q) * QB + t] = h;
             e = max(e, max(bexp(h.x), bexp(h.y)));
           }
         atomicMax(&S.em[t], e);
-      }
-      // |P|^2, R's coefficients and what to do with each column; rejections of candidates are
-      // wanted before Q P, all else runs while the tensor cores form it
+      };
+      auto square_p = [&](int i0) {
+#pragma unroll
+        for (int k = 0; k < TILE / QB; ++k)
+          if (i0 + k * QB < na)
+            hsum = fma(hreg[k].x, hreg[k].x, fma(hreg[k].y, hreg[k].y, hsum));
+      };
+      // what to do with each column; rejections of candidates are wanted before Q P, all else runs
+      // while the tensor cores form it
       auto decide = [&] {
         const int t = tid & 15;
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < MAXN / QB; ++k)
-          if (k * QB < na) s = fma(hreg[k].x, hreg[k].x, fma(hreg[k].y, hreg[k].y, s));
-        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        const double s = hsum + __shfl_xor_sync(0xffffffffu, hsum, 16);
         if (lane < 16) S.hh[warp][t] = s;
-        // R accumulates over the passes in registers (CTA 0 writes it)
-        if (main_phase && blockIdx.x == 0)
-#pragma unroll
-          for (int k = 0; k < MAXN / QB; ++k)
-            if (k * QB < na) {
-              if (pass == 0) racc[k] = hreg[k];
-              else racc[k] = make_double2(racc[k].x + hreg[k].x, racc[k].y + hreg[k].y);
-            }
         __syncthreads();
         if (tid < QB) {
           const double vv = S.G[tid][tid].x;
@@ -529,17 +571,24 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
       };
       const bool first = na == 0 || (!main_phase && pass == 0);
       if (first) {
+        for (int i0 = 0; i0 < na; i0 += TILE) {
+          load_p(i0);
+          square_p(i0);
+          if (i0 + TILE < na) __syncthreads();
+        }
         decide();
         if (!S.any) {
           all_dropped = true;
           break;
         }
-      } else {
-        __syncthreads();
       }
-      if (na > 0) {
-        // V -= Q P
-        const int isteps = (na + 15) / 16;
+      // V -= Q P, a tile of accepted vectors at a time
+      for (int i0 = 0; i0 < na; i0 += TILE) {
+        if (!first || na > TILE) {
+          load_p(i0);
+          __syncthreads();
+        }
+        const int ni = min(TILE, na - i0), isteps = (ni + 15) / 16;
         {
           const int t = tid & 15;
           const int em = max(S.em[t], 1);
@@ -547,7 +596,7 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
           if (tid < QB) S.ev[t] = bad ? E_NONFINITE : em - 1022;
           for (int k = tid >> 4; k < 8 * isteps; k += 16) {     // part, group of 4 columns of Q
             const int part = k & 1, q = k >> 1;
-            qt_store(H + q * 4 * QB + t, QB, min(4, na - q * 4), part, em, bad,
+            qt_store(H + q * 4 * QB + t, QB, min(4, ni - q * 4), part, em, bad,
                      bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
                          t * 16 + (q & 1) * 8);
           }
@@ -555,17 +604,17 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         asm volatile("fence.proxy.async;" ::: "memory");
         __syncthreads();
         if (tid == 0)
-          qt_gemm(P, tmem, ring, bdig, d2, s2, (uint32_t)s2, isteps, false, 0);
+          qt_gemm(P, tmem, ring, 0, bdig, d2 + (long long)(i0 / 16) * s2, s2, (uint32_t)s2, isteps,
+                  false, 0);
         __syncwarp();
-        if (!first) decide();
+        if (!first) {
+          square_p(i0);
+          if (i0 + TILE >= na) decide();
+        }
         alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
         ++P.gemms;
         alive = __syncthreads_and(alive ? 1 : 0) != 0;
         if (!alive) break;
-        if (!S.any) {
-          all_dropped = true;
-          break;
-        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int quad = warp & 3, t0 = (warp >> 2) * 8;
         if (quad * 32 < nr) {
@@ -583,18 +632,33 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
+      npass = pass + 1;
+      if (!alive) break;
+      if (!S.any) {
+        all_dropped = true;
+        break;
+      }
       if (S.last) break;
     }
     if (!alive) break;
+    // rows of the accepted vectors in R's new columns: the sum of the passes' coefficients (the CTAs
+    // share the rows where they can all read the sums, else CTA 0 kept them)
+    auto write_r = [&](int cols) {
+      if (private_r && blockIdx.x != 0) return;
+      const int first = private_r ? 0 : blockIdx.x, G = private_r ? 1 : gridDim.x;
+      for (int e = first * QT_THREADS + tid; e < na * QB; e += G * QT_THREADS) {
+        const int i = e >> 4, t = e & 15;
+        cplx r = make_double2(0.0, 0.0);
+        for (int q = 0; q < npass; ++q) {
+          const cplx h = __ldcg(A.fin + (long long)q * A.PS + e);
+          r = make_double2(r.x + h.x, r.y + h.y);
+        }
+        if (t < cols) A.R[(long long)S.idx[i] * n + j0 + t] = r;
+      }
+    };
     if (all_dropped) {
       if (main_phase) {
-        if (blockIdx.x == 0) {
-          const int t = tid & 15, q = tid >> 4;
-#pragma unroll
-          for (int k = 0; k < MAXN / QB; ++k)
-            if (k * QB + q < na && t < bsz)
-              A.R[(long long)S.idx[k * QB + q] * n + j0 + t] = racc[k];
-        }
+        write_r(bsz);
         j0 += bsz;
       } else {
         cand += bsz;
@@ -731,7 +795,7 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
             if (A.src_out && blockIdx.x == 0) A.src_out[col] = (int)(cand + t);
           }
           S.acc[col] = 1;
-          S.idx[a] = col;
+          S.idx[a] = (short)col;
           S.src[a - na] = t;
           S.em[t] = a++;
         }
@@ -809,13 +873,7 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
           const int s = e / done, t = e % done;
           if (s <= t) A.R[(long long)(j0 + s) * n + j0 + t] = S.R[s][t];
         }
-      if (main_phase && blockIdx.x == 0) {
-        const int t = tid & 15, q = tid >> 4;
-#pragma unroll
-        for (int k = 0; k < MAXN / QB; ++k)
-          if (k * QB + q < na && t < done)
-            A.R[(long long)S.idx[k * QB + q] * n + j0 + t] = racc[k];
-      }
+      if (main_phase) write_r(done);
       na = na1;
       if (main_phase) j0 += done;
       else cand += done;
@@ -875,7 +933,7 @@ cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx
   QtPlan pl;
   if (!W.dig || !qt_plan(m, n, cap, pl)) return cudaSuccess;
   const long long PS = (long long)n * QB + QB + QB * QB;
-  if ((size_t)pl.G * pl.dig_cta > W.dig_bytes || pl.G * PS + PS > scratch_len) return cudaSuccess;
+  if ((size_t)pl.G * pl.dig_cta > W.dig_bytes || (2 * (long long)pl.G + PASSES) * PS > scratch_len) return cudaSuccess;
   static bool attr = false;
   cudaError_t e;
   if (!attr) {
@@ -890,7 +948,7 @@ cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx
   a.Y = Y; a.E = p > 0 ? E : Y;
   a.Q = Q; a.R = R;
   a.part = scratch;
-  a.fin = scratch + (long long)pl.G * PS;
+  a.fin = scratch + 2 * (long long)pl.G * PS;      // PASSES * PS
   a.PS = (int)PS;
   a.dig = W.dig;
   a.dig_cta = pl.dig_cta;

@@ -193,7 +193,7 @@ cudaError_t gauge_qr_blocked(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cpl
 
 // the factorisation and completion of gauge_qr_blocked with the projections on the tensor cores
 // (qr_tensor.cu), one launch; *taken = false and nothing launched when the factor does not fit it
-// (n > 128, more than 128 rows per CTA, no digit workspace)
+// (n < 9 or n > 256, more than 128 rows per CTA, no digit workspace)
 cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* R, cplx* scratch,
                             long long scratch_len, unsigned char* acc, const QrScratch& W,
                             int* status, cudaStream_t s, int gcap, double rank_tol, int* src,

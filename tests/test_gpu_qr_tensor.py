@@ -1,5 +1,5 @@
 """The tensor-core gauge QR at the edges of its tiling (blocks of 16 columns, row slices of 32 to
-128 rows per CTA, at most 128 columns), with the column layouts the sweep uses, rank deficiency
+128 rows per CTA, tiles of 128 accepted vectors, at most 256 columns), with the column layouts the sweep uses, rank deficiency
 with candidates in and out of the span, and columns near the rank threshold."""
 import numpy as np
 import pytest
@@ -33,7 +33,8 @@ def run(Y, E=None):
 
 
 @pytest.mark.parametrize("m,n", [(1, 1), (2, 2), (16, 16), (17, 17), (33, 15), (31, 31), (65, 32),
-                                 (128, 128), (129, 127), (1000, 33), (4097, 113), (19000, 100)])
+                                 (128, 128), (129, 127), (1000, 33), (4097, 113), (19000, 100), (129, 129), (300, 144),
+                                 (2000, 256), (256, 255)])
 def test_full_rank(m, n):
     """Columns of very different size, mixed: Q has orthonormal columns, QR = Y to rounding and R
     is upper triangular with a positive diagonal, which fixes both uniquely.  Both products round
@@ -47,7 +48,7 @@ def test_full_rank(m, n):
     assert np.all(np.diag(R).real > 0) and np.abs(np.diag(R).imag).max() == 0.0
 
 
-@pytest.mark.parametrize("m,n,rank", [(20, 16, 1), (40, 17, 16), (300, 48, 20), (2000, 128, 65),
+@pytest.mark.parametrize("m,n,rank", [(20, 16, 1), (40, 17, 16), (300, 48, 20), (2000, 128, 65), (700, 200, 30), (600, 256, 140),
                                       (513, 96, 0)])
 def test_completion_follows_the_candidates(m, n, rank):
     """Columns beyond the rank are skipped (their residual is rounding); the skipped positions are
