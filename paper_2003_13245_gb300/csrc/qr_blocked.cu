@@ -383,9 +383,9 @@ int gauge_qr_blocked_grid(int m) {
 
 long long gauge_qr_blocked_scratch(int n, int gmax) {
   const long long PS = (long long)n * QB + QB + QB * QB;
-  // complex entries: two sets of partials of every CTA and their sums (of up to four passes,
+  // complex entries: two sets of partials of every CTA and their sums (of up to five passes,
   // qr_tensor.cu; this kernel uses one set and one sum)
-  return (2LL * gmax + 4) * PS;
+  return (2LL * gmax + 5) * PS;
 }
 
 cudaError_t gauge_qr_blocked(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* R,

@@ -11,37 +11,41 @@
 // the second one per row, with a bit to spare: a row that a later column outgrows is written
 // again from Q.
 //
-// Per block of 16 columns, repeated until the projection is negligible (two or three times):
+// Per block of 16 columns a pass is
 //  1. digits of V; P = Q^H V (accumulators in TMEM columns 0-255) and V^H V (columns 256-511);
 //     cross-CTA sums of both;
-//  2. V -= Q P.
-// A pass whose coefficients satisfy |P|^2 <= 2^-57 ||v||^2 leaves V^H V valid to rounding; it is the
-// last.  Then, as in qr_blocked.cu, Gram-Schmidt with skips inside the block in Gram form with a
-// guard against cancellation; the triangular inverse is built beside it, so that the new columns
-// are one product V M.  Columns whose projected norm is already below the rank threshold are
-// skipped together.
+//  2. V -= Q P, and P^H P (columns 256-511; every CTA for itself).
+// V^H V - P^H P is the Gram matrix of what is left, unless less than 1e-8 of some norm^2 is left:
+// then a second pass follows (before it, where next to nothing is left of any column, as with
+// dependent columns, their norms alone tell whether all of them are skipped).  Then, as in
+// qr_blocked.cu, Gram-Schmidt with skips inside the block in Gram form; the triangular inverse is
+// built beside it, so that the new columns are one product V M.  A column that keeps less than 1e-8
+// of its norm^2 starts the next block.  Where one kept less than a quarter, the rounding of the first
+// round shows: a second round projects the new columns (orthonormal to 1e-8) once more and corrects
+// them by the series of the Cholesky factor of 1 + E, without the serial chain.  Graded columns, as
+// a center matrix has them, thus take two passes for 16 columns instead of a block for every few.
 //
 // Completion of skipped positions runs the same blocks over the candidates (columns of E, then
 // unit vectors); the first pass rejects every candidate in the span of the accepted columns at
 // once (residual^2 = ||e||^2 - |P|^2 <= 1e-4 ||e||^2), so 16 rejections cost one pass.
 //
-// Bound: latency.  A pass of a block takes ~20 us (four grid barriers of ~1.3 us, two tensor-core
-// products of 4-10 us, reading their levels back, the digits), the serial 16-column factorisation
-// ~16 us and the FP64 product V M 5-10 us; the FP64 work per column no longer grows with the
-// number of accepted columns.
+// Bound: latency.  A pass of a block takes ~25 us (two to four grid barriers of ~1.3 us, two
+// tensor-core products of 4-10 us, reading their levels back, the digits), the serial 16-column
+// factorisation ~16 us and the FP64 product V M 3-10 us; the FP64 work per column does not grow
+// with the number of accepted columns.
 //
-// Measured on GB300 against qr_blocked.cu (FP64 FMAs), us, columns nearly parallel so that every
-// block takes two passes; "rank 2": all but two columns are completed from 7 n candidates of
-// which n lie in the span:
-//                     152 CTAs                          76 CTAs (two lanes)
-//   m x n        full rank    rank 2              full rank    rank 2
-//   64 x 16       98 / 109     748 / 231
-//   144 x 64     371 / 374    3152 / 641
-//   512 x 128    815 / 846    8258 / 1355
-//   512 x 256   2098 / 2018  23093 / 3204
-//   2048 x 128  1155 / 836   12395 / 1391        1658 / 847   12275 / 1351
-//   2048 x 144  1380 / 956   20269 / 1607
-//   8192 x 128  2682 / 1022  19468 / 1765        4516 / 1255  25260 / 2302
+// Measured on GB300 against qr_blocked.cu (FP64 FMAs), us.  "parallel": random columns, nearly
+// parallel; "graded": singular values from 1 to e^-9, mixed, for which the same kernel with one round
+// (a restart below a quarter) stands in the middle; "rank 2": all but two columns are completed from
+// 7 n candidates of which n lie in the span:
+//   m x n        parallel         graded                 rank 2
+//   64 x 16       99 /   81       257 / 449 /   79        743 /  157
+//   256 x 32     171 /  198       356 / 641 /  198       1549 /  290
+//   1024 x 64    388 /  450       706 / 914 /  450       3716 /  545
+//   256 x 128    825 /  994      1028 / 1150 / 1000      7537 / 1184
+//   1024 x 128   943 / 1001      1173 / 1183 / 1105      9622 / 1208
+//   8192 x 128  2681 / 1218      3913 / 1454 / 1231     19468 / 1552
+//   8192 x 128 on 76 CTAs (two lanes)  4514 / 1541 and (rank 2) 25140 / 1783
 // Below nine columns the other kernel is the faster one at full rank (256 x 4: 55 against 95 us),
 // where such bonds, at the ends of a chain, mostly are.  About 32 rows per CTA: fewer rows raise the
 // number of partial sums, more the FP64 product V M.
@@ -63,7 +67,10 @@ constexpr int GROUP = 2 * ND * 2 * 128;         // digits of 8 rows x 16 k: 3584
 constexpr int RING = 16 * GROUP;                // one k step of 128 rows: 57344 bytes
 constexpr int BSTEP = 2 * ND * 2 * 2 * 128;     // 16 columns x 16 k: 7168 bytes
 constexpr int BDIG = 8 * BSTEP;                 // 57344 bytes
-constexpr int PASSES = 4;
+constexpr int PASSES = 4;                       // projections of a block, at most (and a second round)
+// smallest part of a norm^2 that may be left where the rest is taken off in the Gram matrix
+// (rounding of 2^-53 is then up to 1e-8 of what is left; the second round takes that out)
+constexpr double KEEP = 1e-8;
 constexpr int E_EMPTY = -100000;
 constexpr int TMEM_COLS = 512;
 constexpr int IM = NL * QB;                     // im levels after the re levels
@@ -74,7 +81,7 @@ struct QtArgs {
   cplx* Q;
   cplx* R;
   cplx* part;               // [2][G][PS], used in turn
-  cplx* fin;                // [PASSES][PS]
+  cplx* fin;                // [PASSES + 1][PS]
   int PS;
   unsigned char* dig;       // per CTA: form 1 then form 2
   long long dig_cta;        // bytes of one CTA
@@ -123,7 +130,8 @@ __device__ bool qt_barrier(const QtArgs& A, unsigned& epoch, int* s_ok) {
 // the entries and a second barrier makes all of them readable; where all partial sums are few,
 // every CTA sums them itself into its shared copy `own` (the same order, so the same result) and
 // the second barrier is left out (a CTA may then still read partial sums when another goes on:
-// two sets of them are used in turn).  Returns where to read the sums.
+// two sets of them are used in turn).  Without `fin` (few entries) always so.  Returns where to
+// read the sums.
 constexpr int OWN = 512;                        // entries a CTA may sum for itself
 __device__ const cplx* qt_reduce(const QtArgs& A, int cnt, const cplx* part, cplx* fin, cplx* own,
                                  unsigned& ep, int* s_ok) {
@@ -133,7 +141,7 @@ __device__ const cplx* qt_reduce(const QtArgs& A, int cnt, const cplx* part, cpl
   } else {
     __syncthreads();
   }
-  const bool alone = cnt <= OWN && cnt * G <= 4096;
+  const bool alone = !fin || (cnt <= OWN && cnt * G <= 4096);
   const int per = alone ? cnt : (cnt + G - 1) / G;
   const int lo = alone ? 0 : blockIdx.x * per, hi = min(cnt, lo + per);
   cplx* out = alone ? own : fin;
@@ -159,7 +167,7 @@ __device__ const cplx* qt_reduce(const QtArgs& A, int cnt, const cplx* part, cpl
     }
     if (sub == 0 && e < hi) {
       out[e] = make_double2(ax, ay);
-      if (alone && blockIdx.x == 0) fin[e] = make_double2(ax, ay);   // R is formed from it
+      if (alone && fin && blockIdx.x == 0) fin[e] = make_double2(ax, ay);   // R is formed from it
     }
   }
   if (alone) {
@@ -186,9 +194,10 @@ struct Pipe {
 };
 
 // Issued by thread 0.  D += sum over S k steps of A_s B_s: A from `src` (step s at s * stride,
-// `bytes` of it, at `off` of a stage) through the ring, B in shared memory at bdig + s * BSTEP.  conj: Q^H V (re = ArBr
-// + AiBi, im = ArBi - AiBr), else Q P (re = ArBr - AiBi, im = ArBi + AiBr).  gram: also V^H V of
-// the same B tiles into columns 256.. (A = the B tile itself, its rows beyond 16 unused).
+// `bytes` of it, at `off` of a stage) through the ring, B in shared memory at bdig + s * BSTEP.
+// conj: Q^H V (re = ArBr + AiBi, im = ArBi - AiBr), else Q P (re = ArBr - AiBi, im = ArBi + AiBr).
+// gram_steps: also B^H B of the same B tiles into columns 256.. (A = the B tile itself, its rows
+// beyond 16 unused).
 __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
                         const unsigned char* bdig,
                         const unsigned char* src, long long stride, uint32_t bytes, int S,
@@ -203,7 +212,7 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
     ++issued;
   };
   auto tile = [&](uint32_t a, uint32_t lbo, uint32_t sbo, uint32_t apart, uint32_t adig, uint32_t b,
-                  uint32_t d, bool first) {
+                  uint32_t d, bool first, bool cj) {
     const uint64_t br = sdesc(b, ND * 256), bi = sdesc(b + BSTEP / 2, ND * 256);
 #pragma unroll
     for (int i = 0; i < ND; ++i) {
@@ -219,14 +228,15 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
         mma_f16(dr + mm, ar, sdesc(b + (ND - 1) * 256, ND * 256), idesc(0, QB), 0u);
         mma_f16(di + mm, ar, sdesc(b + BSTEP / 2 + (ND - 1) * 256, ND * 256), idesc(0, QB), 0u);
       }
-      mma_f16(dr, ai, bi, idesc(conj ? 0 : 1, n), 1u);
-      mma_f16(di, ai, br, idesc(conj ? 1 : 0, n), 1u);
+      mma_f16(dr, ai, bi, idesc(cj ? 0 : 1, n), 1u);
+      mma_f16(di, ai, br, idesc(cj ? 1 : 0, n), 1u);
     }
   };
   for (int s = 0; s < S && s < 2; ++s) load(s);
   const uint32_t b0 = smem_u32(bdig);
   for (int s = 0; s < gram_steps; ++s)
-    tile(b0 + s * BSTEP, ND * 256, 128, BSTEP / 2, 256, b0 + s * BSTEP, tmem + 2 * IM, s == 0);
+    tile(b0 + s * BSTEP, ND * 256, 128, BSTEP / 2, 256, b0 + s * BSTEP, tmem + 2 * IM, s == 0,
+         true);
   for (int s = 0; s < S; ++s) {
     const int st = (it0 + s) & 1;
     const uint32_t par = ((it0 + s) >> 1) & 1;
@@ -235,7 +245,8 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
       break;
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tile(smem_u32(ring + st * RING), 128, GROUP, GROUP / 2, 256, b0 + s * BSTEP, tmem, s == 0);
+    tile(smem_u32(ring + st * RING), 128, GROUP, GROUP / 2, 256, b0 + s * BSTEP, tmem, s == 0,
+         conj);
     mma_commit(&P.empty[st]);
     if (s + 2 < S) {
       if (!mbar_wait(&P.empty[st], par, P.fail, P.status, 1)) {
@@ -287,7 +298,7 @@ struct Shared {
   cplx M[QB][QB];            // and the inverse
   cplx u[2][QB], y[QB];      // factors of one step (u of alternate steps)
   double inv;
-  double quarter[QB];        // a quarter of the projected norm^2
+  double ref[QB];            // norm^2 of the column before the last projection
   double hh[8][QB];          // partial sums of |P|^2
   double lim[QB];            // completion: smallest residual norm of a candidate that is taken
   int em[QB];                // largest biased exponent of a column (digit scale)
@@ -302,7 +313,7 @@ struct Shared {
   int src[QB];               // block column of the block's i-th accepted vector
   int drop[QB];              // skipped before the in-block factorisation
   double red[32];
-  int ok, fail, done, stop, last, any;
+  int ok, fail, done, last, any, near, refine;
   uint32_t tmem;
   uint64_t bar[5];
 };
@@ -412,334 +423,401 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
     __syncthreads();
     // ---- projection passes
     bool private_r = false;   // some of the sums were not published
-    int npass = 0;            // passes whose coefficients belong to R
+    int npass = 0;            // passes of the first round
     bool all_dropped = false;
-    for (int pass = 0; pass < PASSES; ++pass) {
-      // digits of V, one scale per column (two columns per warp)
-      const bool gram = pass > 0 || na == 0;
-      {
-        int e2[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int t = 2 * warp + u;
-          int e = 0;
-          double s = 0.0;
-          for (int r = lane; r < nr; r += 32) {
-            const cplx v = V[t * LDV + r];
-            e = max(e, max(bexp(v.x), bexp(v.y)));
-            if (!gram) s = fma(v.x, v.x, fma(v.y, v.y, s));
-          }
-          e2[u] = __reduce_max_sync(0xffffffffu, e);
-          if (!gram) {                     // the norms alone (the first pass needs no more)
-            s = wsum(s);
-            if (lane == 0) mypart[na * QB + t] = make_double2(s, 0.0);
-          }
-          if (lane == 0) S.ev[t] = e2[u] == 0x7ff ? E_NONFINITE : max(e2[u], 1) - 1022;
-        }
-        for (int k = lane; k < 16 * rsteps; k += 32) {     // column, part, group of 4 rows
-          const int u = k & 1, part = (k >> 1) & 1, q = k >> 2;
-          const int t = 2 * warp + u, em = u ? e2[1] : e2[0];
-          qt_store(V + t * LDV + q * 4, 1, min(4, nr - q * 4), part, max(em, 1), em == 0x7ff,
-                   bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
-                       t * 16 + (q & 1) * 8);
-        }
-      }
-      asm volatile("fence.proxy.async;" ::: "memory");
-      __syncthreads();
-      // P and V^H V, a tile of accepted vectors at a time.  With at most 96 vectors in a tile they
-      // sit in its rows 32.., so that the warps of rows 0-31 have the Gram matrix alone.
-      for (int i0 = 0; i0 == 0 || i0 < na; i0 += TILE) {
-        const int ni = min(TILE, na - i0);
-        const bool g0 = gram && i0 == 0;
-        const int shift = g0 && ni <= TILE - 32 ? 32 : 0;
-        if (tid == 0)
-          qt_gemm(P, tmem, ring, shift / 8 * GROUP, bdig, d1 + (long long)(i0 / 8) * GROUP, s1,
-                  (uint32_t)((ni + 7) / 8 * GROUP), ni > 0 ? rsteps : 0, true, g0 ? rsteps : 0);
-        __syncwarp();
-        alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
-        ++P.gemms;
-        alive = __syncthreads_and(alive ? 1 : 0) != 0;
-        if (!alive) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int quad = warp & 3, t0 = (warp >> 2) * 8;
-        const int row = quad * 32 + lane - shift;
-        const uint32_t addr = tmem + ((uint32_t)(quad * 32) << 16) + t0;
-        cplx out[8];
-        if (quad * 32 >= shift && quad * 32 - shift < ni) {
-          qt_read(addr, S.ec[i0 + min(row, ni - 1)], S.ev + t0, out);
-          if (row < ni)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) mypart[(i0 + row) * QB + t0 + c] = out[c];
-        }
-        if (g0 && quad == 0) {
-          qt_read(addr + 2 * IM, S.ev[lane & 15], S.ev + t0, out);
-          if (lane < QB)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) mypart[na * QB + lane * QB + t0 + c] = out[c];
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        if (i0 + TILE < na) {
-          __syncthreads();
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        }
-      }
-      if (!alive) break;
-      cplx* fin = A.fin + (long long)pass * A.PS;
-      const int cnt = na * QB + (gram ? QB * QB : QB) + (started ? 0 : 1);
-      const cplx* sum = qt_reduce(A, cnt, part, fin, S.own, ep, &S.ok);
-      if (!sum) {
-        alive = false;
-        break;
-      }
-      mypart += part == A.part ? pset : -pset;
-      part = part == A.part ? A.part + pset : A.part;
-      if (sum == S.own) private_r = true;
-      auto take_sum = [&](int e) { return sum == S.own ? S.own[e] : __ldcg(sum + e); };
-      if (!started) {
-        started = true;
-        const double y2 = take_sum(QB * QB).x;
-        if (!(y2 < 1.7976931348623157e308)) {
-          // Inf or NaN in Y: every column is skipped
-          bsz = n;
-          all_dropped = true;
-          break;
-        }
-        thr = A.rank_tol * sqrt(y2);
-        thr2 = thr * thr;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (gram) S.G[tid >> 4][tid & 15] = take_sum(na * QB + tid);
-      else if (tid < QB) S.G[tid][tid] = take_sum(na * QB + tid);
-      // one tile of P: into shared memory, its |P|^2 and its scale per column
-      cplx hreg[TILE / QB];
-      double hsum = 0.0;
-      auto load_p = [&](int i0) {
-        const int t = tid & 15, q = tid >> 4;
-        if (tid < QB) S.em[tid] = 0;
-#pragma unroll
-        for (int k = 0; k < TILE / QB; ++k) {
-          const int i = i0 + k * QB + q;
-          hreg[k] = i < na ? take_sum(i * QB + t) : make_double2(0.0, 0.0);
-        }
-        __syncthreads();
-        int e = 0;
-#pragma unroll
-        for (int k = 0; k < TILE / QB; ++k)
-          if (i0 + k * QB < na) {
-            const cplx h = hreg[k];
-            if (i0 + k * QB + q < na) H[(k * QB + q) * QB + t] = h;
-            e = max(e, max(bexp(h.x), bexp(h.y)));
-          }
-        atomicMax(&S.em[t], e);
-      };
-      auto square_p = [&](int i0) {
-#pragma unroll
-        for (int k = 0; k < TILE / QB; ++k)
-          if (i0 + k * QB < na)
-            hsum = fma(hreg[k].x, hreg[k].x, fma(hreg[k].y, hreg[k].y, hsum));
-      };
-      // what to do with each column; rejections of candidates are wanted before Q P, all else runs
-      // while the tensor cores form it
-      auto decide = [&] {
-        const int t = tid & 15;
-        const double s = hsum + __shfl_xor_sync(0xffffffffu, hsum, 16);
-        if (lane < 16) S.hh[warp][t] = s;
-        __syncthreads();
-        if (tid < QB) {
-          const double vv = S.G[tid][tid].x;
-          double h = 0.0;
-          for (int w = 0; w < QT_THREADS / 32; ++w) h += S.hh[w][tid];
-          int drop = S.drop[tid];
-          if (main_phase) {
-            if (!(vv > thr2)) drop = 1;
-          } else if (pass == 0) {
-            S.lim[tid] = A.complete_tol * sqrt(vv);
-            // in the span of the accepted vectors (or zero, or not finite)
-            if (!(vv - h > A.complete_tol * A.complete_tol * vv)) drop = 1;
-          }
-          S.drop[tid] = drop;
-          S.quarter[tid] = 0.25 * vv;
-          // the Gram matrix stands when the projection leaves it unchanged to rounding
-          const bool more = !drop && (!gram || h > 6.9e-18 * vv);
-          const unsigned mm = __ballot_sync(0xffffu, more), dd = __ballot_sync(0xffffu, !drop);
-          if (tid == 0) {
-            S.last = mm == 0;
-            S.any = dd != 0;
-          }
-        }
-        __syncthreads();
-      };
-      const bool first = na == 0 || (!main_phase && pass == 0);
-      if (first) {
-        for (int i0 = 0; i0 < na; i0 += TILE) {
-          load_p(i0);
-          square_p(i0);
-          if (i0 + TILE < na) __syncthreads();
-        }
-        decide();
-        if (!S.any) {
-          all_dropped = true;
-          break;
-        }
-      }
-      // V -= Q P, a tile of accepted vectors at a time
-      for (int i0 = 0; i0 < na; i0 += TILE) {
-        if (!first || na > TILE) {
-          load_p(i0);
-          __syncthreads();
-        }
-        const int ni = min(TILE, na - i0), isteps = (ni + 15) / 16;
+    bool refine = false;      // second round: one pass over the block's new columns
+    for (;;) {
+      for (int pass = npass; pass <= PASSES; ++pass) {
+        // digits of V, one scale per column (two columns per warp)
         {
-          const int t = tid & 15;
-          const int em = max(S.em[t], 1);
-          const bool bad = em == 0x7ff;
-          if (tid < QB) S.ev[t] = bad ? E_NONFINITE : em - 1022;
-          for (int k = tid >> 4; k < 8 * isteps; k += 16) {     // part, group of 4 columns of Q
-            const int part = k & 1, q = k >> 1;
-            qt_store(H + q * 4 * QB + t, QB, min(4, ni - q * 4), part, em, bad,
+          int e2[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int t = 2 * warp + u;
+            int e = 0;
+            for (int r = lane; r < nr; r += 32) {
+              const cplx v = V[t * LDV + r];
+              e = max(e, max(bexp(v.x), bexp(v.y)));
+            }
+            e2[u] = __reduce_max_sync(0xffffffffu, e);
+            if (lane == 0) S.ev[t] = e2[u] == 0x7ff ? E_NONFINITE : max(e2[u], 1) - 1022;
+          }
+          for (int k = lane; k < 16 * rsteps; k += 32) {     // column, part, group of 4 rows
+            const int u = k & 1, part = (k >> 1) & 1, q = k >> 2;
+            const int t = 2 * warp + u, em = u ? e2[1] : e2[0];
+            qt_store(V + t * LDV + q * 4, 1, min(4, nr - q * 4), part, max(em, 1), em == 0x7ff,
                      bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
                          t * 16 + (q & 1) * 8);
           }
         }
         asm volatile("fence.proxy.async;" ::: "memory");
         __syncthreads();
-        if (tid == 0)
-          qt_gemm(P, tmem, ring, 0, bdig, d2 + (long long)(i0 / 16) * s2, s2, (uint32_t)s2, isteps,
-                  false, 0);
-        __syncwarp();
-        if (!first) {
-          square_p(i0);
-          if (i0 + TILE >= na) decide();
-        }
-        alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
-        ++P.gemms;
-        alive = __syncthreads_and(alive ? 1 : 0) != 0;
-        if (!alive) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int quad = warp & 3, t0 = (warp >> 2) * 8;
-        if (quad * 32 < nr) {
+        // P and V^H V, a tile of accepted vectors at a time.  With at most 96 vectors in a tile they
+        // sit in its rows 32.., so that the warps of rows 0-31 have the Gram matrix alone.
+        for (int i0 = 0; i0 == 0 || i0 < na; i0 += TILE) {
+          const int ni = min(TILE, na - i0);
+          const bool g0 = i0 == 0;
+          const int shift = g0 && ni <= TILE - 32 ? 32 : 0;
+          if (tid == 0)
+            qt_gemm(P, tmem, ring, shift / 8 * GROUP, bdig, d1 + (long long)(i0 / 8) * GROUP, s1,
+                    (uint32_t)((ni + 7) / 8 * GROUP), ni > 0 ? rsteps : 0, true, g0 ? rsteps : 0);
+          __syncwarp();
+          alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
+          ++P.gemms;
+          alive = __syncthreads_and(alive ? 1 : 0) != 0;
+          if (!alive) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const int quad = warp & 3, t0 = (warp >> 2) * 8;
+          const int row = quad * 32 + lane - shift;
+          const uint32_t addr = tmem + ((uint32_t)(quad * 32) << 16) + t0;
           cplx out[8];
-          const int r = quad * 32 + lane;
-          qt_read(tmem + ((uint32_t)(quad * 32) << 16) + t0, S.er[min(r, nr - 1)], S.ev + t0, out);
-          if (r < nr)
+          if (quad * 32 >= shift && quad * 32 - shift < ni) {
+            qt_read(addr, S.ec[i0 + min(row, ni - 1)], S.ev + t0, out);
+            if (row < ni)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              cplx& v = V[(t0 + c) * LDV + r];
-              v = make_double2(v.x - out[c].x, v.y - out[c].y);
-            }
+              for (int c = 0; c < 8; ++c) mypart[(i0 + row) * QB + t0 + c] = out[c];
+          }
+          if (g0 && quad == 0) {
+            qt_read(addr + 2 * IM, S.ev[lane & 15], S.ev + t0, out);
+            if (lane < QB)
+#pragma unroll
+              for (int c = 0; c < 8; ++c) mypart[na * QB + lane * QB + t0 + c] = out[c];
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          if (i0 + TILE < na) {
+            __syncthreads();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
+        if (!alive) break;
+        cplx* fin = A.fin + (long long)pass * A.PS;
+        const int cnt = na * QB + QB * QB + (started ? 0 : 1);
+        const cplx* sum = qt_reduce(A, cnt, part, fin, S.own, ep, &S.ok);
+        if (!sum) {
+          alive = false;
+          break;
+        }
+        mypart += part == A.part ? pset : -pset;
+        part = part == A.part ? A.part + pset : A.part;
+        if (sum == S.own) private_r = true;
+        if (!refine) npass = pass + 1;
+        auto take_sum = [&](int e) { return sum == S.own ? S.own[e] : __ldcg(sum + e); };
+        if (!started) {
+          started = true;
+          const double y2 = take_sum(QB * QB).x;
+          if (!(y2 < 1.7976931348623157e308)) {
+            // Inf or NaN in Y: every column is skipped
+            bsz = n;
+            all_dropped = true;
+            break;
+          }
+          thr = A.rank_tol * sqrt(y2);
+          thr2 = thr * thr;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      }
-      npass = pass + 1;
-      if (!alive) break;
-      if (!S.any) {
-        all_dropped = true;
-        break;
-      }
-      if (S.last) break;
-    }
-    if (!alive) break;
-    // rows of the accepted vectors in R's new columns: the sum of the passes' coefficients (the CTAs
-    // share the rows where they can all read the sums, else CTA 0 kept them)
-    auto write_r = [&](int cols) {
-      if (private_r && blockIdx.x != 0) return;
-      const int first = private_r ? 0 : blockIdx.x, G = private_r ? 1 : gridDim.x;
-      for (int e = first * QT_THREADS + tid; e < na * QB; e += G * QT_THREADS) {
-        const int i = e >> 4, t = e & 15;
-        cplx r = make_double2(0.0, 0.0);
-        for (int q = 0; q < npass; ++q) {
-          const cplx h = __ldcg(A.fin + (long long)q * A.PS + e);
-          r = make_double2(r.x + h.x, r.y + h.y);
+        S.G[tid >> 4][tid & 15] = take_sum(na * QB + tid);
+        // one tile of P: into shared memory, its |P|^2 and its scale per column
+        cplx hreg[TILE / QB];
+        double hsum = 0.0;
+        auto load_p = [&](int i0) {
+          const int t = tid & 15, q = tid >> 4;
+          if (tid < QB) S.em[tid] = 0;
+#pragma unroll
+          for (int k = 0; k < TILE / QB; ++k) {
+            const int i = i0 + k * QB + q;
+            hreg[k] = i < na ? take_sum(i * QB + t) : make_double2(0.0, 0.0);
+          }
+          __syncthreads();
+          int e = 0;
+#pragma unroll
+          for (int k = 0; k < TILE / QB; ++k)
+            if (i0 + k * QB < na) {
+              const cplx h = hreg[k];
+              if (i0 + k * QB + q < na) H[(k * QB + q) * QB + t] = h;
+              e = max(e, max(bexp(h.x), bexp(h.y)));
+            }
+          atomicMax(&S.em[t], e);
+        };
+        auto square_p = [&](int i0) {
+#pragma unroll
+          for (int k = 0; k < TILE / QB; ++k)
+            if (i0 + k * QB < na)
+              hsum = fma(hreg[k].x, hreg[k].x, fma(hreg[k].y, hreg[k].y, hsum));
+        };
+        // what to do with each column; rejections of candidates are wanted before Q P, all else runs
+        // while the tensor cores form it
+        auto decide = [&] {
+          const int t = tid & 15;
+          const double s = hsum + __shfl_xor_sync(0xffffffffu, hsum, 16);
+          if (lane < 16) S.hh[warp][t] = s;
+          __syncthreads();
+          if (tid < QB) {
+            const double vv = S.G[tid][tid].x;
+            double h = 0.0;
+            for (int w = 0; w < QT_THREADS / 32; ++w) h += S.hh[w][tid];
+            int drop = S.drop[tid];
+            if (main_phase) {
+              if (!(vv > thr2)) drop = 1;
+            } else if (pass == 0) {
+              S.lim[tid] = A.complete_tol * sqrt(vv);
+              // in the span of the accepted vectors (or zero, or not finite)
+              if (!(vv - h > A.complete_tol * A.complete_tol * vv)) drop = 1;
+            }
+            S.drop[tid] = drop;
+            S.ref[tid] = vv;
+            // first pass: V^H V - P^H P stands in for the Gram matrix of what is left, where that is
+            // not too small a part; later ones: V^H V as it is, where P does not change it
+            const bool more = !drop && (pass == 0 ? !(vv - h > KEEP * vv) : h > 6.9e-18 * vv);
+            const bool away = !drop && vv - h > 2e-15 * vv;
+            const unsigned mm = __ballot_sync(0xffffu, more), dd = __ballot_sync(0xffffu, !drop);
+            const unsigned aa = __ballot_sync(0xffffu, away);
+            if (tid == 0) {
+              S.last = mm == 0;
+              S.any = dd != 0;
+              S.near = main_phase && pass == 0 && aa == 0;
+            }
+          }
+          __syncthreads();
+        };
+        const bool first = !refine && pass == 0;
+        if (first) {
+          for (int i0 = 0; i0 < na; i0 += TILE) {
+            load_p(i0);
+            square_p(i0);
+            if (i0 + TILE < na) __syncthreads();
+          }
+          decide();
+          if (!S.any) {
+            all_dropped = true;
+            break;
+          }
         }
-        if (t < cols) A.R[(long long)S.idx[i] * n + j0 + t] = r;
-      }
-    };
-    if (all_dropped) {
-      if (main_phase) {
-        write_r(bsz);
-        j0 += bsz;
-      } else {
-        cand += bsz;
-      }
-    } else {
-      // ---- Gram-Schmidt with skips inside the block (Gram form, right-looking), the inverse of
-      // the triangular factor beside it.  Thread e holds the pair (a, b), a <= b, numbered by
-      // falling b: at step s the pairs with b > s are the first ones.  It carries G_ab until row a
-      // is taken (then R_ab), and the inverse's M_ab from then on; both are updated by the same
-      // product of a column factor u_a (conj(R_sa) for a > s, M_as for a <= s) and R_sb.
-      const int room = n - na;             // completion: positions left
-      if (warp < 5) {
-        int b = QB - 1, rem = tid;
-        while (b >= 0 && rem > b) rem -= b-- + 1;
-        const int a = rem;                 // b < 0: no pair
-        cplx g = b >= 0 ? S.G[a][b] : make_double2(0.0, 0.0);
-        int taken = 0, s = 0;
-        for (; s < bsz; ++s) {
-          if (a == s && b == s) {
-            // positive doubles compare like their bits (a negative rho is below everything):
-            // integer comparisons keep the FP64 pipe out of the serial chain
-            const double rho = g.x;
-            const long long rb = __double_as_longlong(rho);
-            int take = 0;
-            double inv = 0.0, nrm = 0.0;
-            if (!main_phase && taken >= room) take = -1;
-            else if (!S.drop[s]) {
-              // cancellation inside the block: this column starts the next block
-              if (taken > 0 && rb < __double_as_longlong(S.quarter[s])) take = -1;
-              else if (rb > 0) {
-                inv = bexp(rho) > 0 ? rsqrt_series(rho) : rsqrt(rho);
-                nrm = rho * inv;
-                const double lim = main_phase ? thr : S.lim[s];
-                take = __double_as_longlong(nrm) > __double_as_longlong(lim) ? 1 : 0;
-                if (!take) inv = 0.0;
+        // V -= Q P, a tile of accepted vectors at a time
+        for (int i0 = 0; i0 < na; i0 += TILE) {
+          if (!first || na > TILE) {
+            load_p(i0);
+            __syncthreads();
+          }
+          const int ni = min(TILE, na - i0), isteps = (ni + 15) / 16;
+          {
+            const int t = tid & 15;
+            const int em = max(S.em[t], 1);
+            const bool bad = em == 0x7ff;
+            if (tid < QB) S.ev[t] = bad ? E_NONFINITE : em - 1022;
+            for (int k = tid >> 4; k < 8 * isteps; k += 16) {     // part, group of 4 columns of Q
+              const int part = k & 1, q = k >> 1;
+              qt_store(H + q * 4 * QB + t, QB, min(4, ni - q * 4), part, em, bad,
+                       bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
+                           t * 16 + (q & 1) * 8);
+            }
+          }
+          asm volatile("fence.proxy.async;" ::: "memory");
+          __syncthreads();
+          // with a single pass also P^H P, which every CTA forms for itself
+          const bool corr = first && S.last;
+          if (tid == 0)
+            qt_gemm(P, tmem, ring, 0, bdig, d2 + (long long)(i0 / 16) * s2, s2, (uint32_t)s2, isteps,
+                    false, corr ? isteps : 0);
+          __syncwarp();
+          if (!first && !refine) {
+            square_p(i0);
+            if (i0 + TILE >= na) decide();
+          }
+          alive = mbar_wait(P.done, P.gemms & 1, P.fail, A.status, 1);
+          ++P.gemms;
+          alive = __syncthreads_and(alive ? 1 : 0) != 0;
+          if (!alive) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const int quad = warp & 3, t0 = (warp >> 2) * 8;
+          if (quad * 32 < nr) {
+            cplx out[8];
+            const int r = quad * 32 + lane;
+            qt_read(tmem + ((uint32_t)(quad * 32) << 16) + t0, S.er[min(r, nr - 1)], S.ev + t0, out);
+            if (r < nr)
+#pragma unroll
+              for (int c = 0; c < 8; ++c) {
+                cplx& v = V[(t0 + c) * LDV + r];
+                v = make_double2(v.x - out[c].x, v.y - out[c].y);
               }
-            }
-            S.take[s] = take;
-            S.inv = inv;
-            if (take >= 0) S.R[s][s] = make_double2(take ? nrm : 0.0, 0.0);
-            S.M[s][s] = make_double2(take > 0 ? inv : 0.0, 0.0);
-            S.u[s & 1][s] = make_double2(inv, 0.0);
           }
-          asm volatile("bar.sync 1, 160;" ::: "memory");
-          const int take = S.take[s];
-          if (take < 0) break;
-          if (take > 0) {
-            const double inv = S.inv;
-            ++taken;
-            if (a == s && b > s) {         // row s of R
-              g = make_double2(g.x * inv, g.y * inv);
-              S.R[s][b] = g;
-              S.y[b] = g;
-              S.u[s & 1][b] = make_double2(g.x, -g.y);
-              g = make_double2(0.0, 0.0);
-            } else if (b == s && a < s) {  // column s of the inverse
-              g = make_double2(g.x * inv, g.y * inv);
-              S.M[a][s] = g;
-              S.u[s & 1][a] = g;
+          if (corr && quad == 0) {
+            cplx out[8];
+            qt_read(tmem + 2 * IM + t0, S.ev[lane & 15], S.ev + t0, out);
+            if (lane < QB)
+#pragma unroll
+              for (int c = 0; c < 8; ++c) {
+                cplx& g = S.G[lane][t0 + c];
+                g = make_double2(g.x - out[c].x, g.y - out[c].y);
+              }
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncthreads();
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        if (!alive || refine) break;
+        if (!S.any) {
+          all_dropped = true;
+          break;
+        }
+        if (S.last || npass == PASSES) break;
+        if (S.near) {
+          // next to nothing is left of any column: their norms tell whether they are skipped, without
+          // another projection
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int t = 2 * warp + u;
+            double q = 0.0;
+            for (int r = lane; r < nr; r += 32) {
+              const cplx v = V[t * LDV + r];
+              q = fma(v.x, v.x, fma(v.y, v.y, q));
             }
-            asm volatile("bar.sync 1, 160;" ::: "memory");
-            if (b > s) {
-              const cplx u = S.u[s & 1][a], y = S.y[b];
-              g.x = fma(-u.x, y.x, g.x);
-              g.x = fma(u.y, y.y, g.x);
-              g.y = fma(-u.x, y.y, g.y);
-              g.y = fma(-u.y, y.x, g.y);
-            }
-          } else {
-            if (a == s && b > s) {
-              S.R[s][b] = make_double2(0.0, 0.0);
-              g = make_double2(0.0, 0.0);
-            } else if (b == s && a < s) {
-              S.M[a][s] = make_double2(0.0, 0.0);
-            }
-            asm volatile("bar.sync 1, 160;" ::: "memory");
+            q = wsum(q);
+            if (lane == 0) mypart[t] = make_double2(q, 0.0);
+          }
+          if (!qt_reduce(A, QB, part, nullptr, S.own, ep, &S.ok)) {
+            alive = false;
+            break;
+          }
+          mypart += part == A.part ? pset : -pset;
+          part = part == A.part ? A.part + pset : A.part;
+          if (tid < QB) {
+            const int drop = S.drop[tid] || !(S.own[tid].x > thr2);
+            S.drop[tid] = drop;
+            const unsigned dd = __ballot_sync(0xffffu, !drop);
+            if (tid == 0) S.any = dd != 0;
+          }
+          __syncthreads();
+          if (!S.any) {
+            all_dropped = true;
+            break;
           }
         }
-        if (tid == 0) S.done = s;
       }
-      __syncthreads();
+      if (!alive || all_dropped) break;
+      if (!refine) {
+        // ---- Gram-Schmidt with skips inside the block (Gram form, right-looking), the inverse of
+        // the triangular factor beside it.  Thread e holds the pair (a, b), a <= b, numbered by
+        // falling b: at step s the pairs with b > s are the first ones.  It carries G_ab until row a
+        // is taken (then R_ab), and the inverse's M_ab from then on; both are updated by the same
+        // product of a column factor u_a (conj(R_sa) for a > s, M_as for a <= s) and R_sb.
+        const int room = n - na;             // completion: positions left
+        if (tid == 0) S.refine = 0;
+        __syncthreads();
+        if (warp < 5) {
+          int b = QB - 1, rem = tid;
+          while (b >= 0 && rem > b) rem -= b-- + 1;
+          const int a = rem;                 // b < 0: no pair
+          cplx g = b >= 0 ? S.G[a][b] : make_double2(0.0, 0.0);
+          int taken = 0, s = 0;
+          for (; s < bsz; ++s) {
+            if (a == s && b == s) {
+              // positive doubles compare like their bits (a negative rho is below everything):
+              // integer comparisons keep the FP64 pipe out of the serial chain
+              const double rho = g.x;
+              const long long rb = __double_as_longlong(rho);
+              int take = 0;
+              double inv = 0.0, nrm = 0.0;
+              if (!main_phase && taken >= room) take = -1;
+              else if (!S.drop[s]) {
+                // cancellation inside the block: this column starts the next block
+                if (taken > 0 && rb < __double_as_longlong(KEEP * S.ref[s])) take = -1;
+                else if (rb > 0) {
+                  inv = bexp(rho) > 0 ? rsqrt_series(rho) : rsqrt(rho);
+                  nrm = rho * inv;
+                  const double lim = main_phase ? thr : S.lim[s];
+                  take = __double_as_longlong(nrm) > __double_as_longlong(lim) ? 1 : 0;
+                  if (!take) inv = 0.0;
+                  // much of it went with the projection or with the block's other columns: what is
+                  // left carries their rounding, the second round takes it out
+                  else if (rho < 0.25 * S.ref[s]) S.refine = 1;
+                }
+              }
+              S.take[s] = take;
+              S.inv = inv;
+              if (take >= 0) S.R[s][s] = make_double2(take ? nrm : 0.0, 0.0);
+              S.M[s][s] = make_double2(take > 0 ? inv : 0.0, 0.0);
+              S.u[s & 1][s] = make_double2(inv, 0.0);
+            }
+            asm volatile("bar.sync 1, 160;" ::: "memory");
+            const int take = S.take[s];
+            if (take < 0) break;
+            if (take > 0) {
+              const double inv = S.inv;
+              ++taken;
+              if (a == s && b > s) {         // row s of R
+                g = make_double2(g.x * inv, g.y * inv);
+                S.R[s][b] = g;
+                S.y[b] = g;
+                S.u[s & 1][b] = make_double2(g.x, -g.y);
+                g = make_double2(0.0, 0.0);
+              } else if (b == s && a < s) {  // column s of the inverse
+                g = make_double2(g.x * inv, g.y * inv);
+                S.M[a][s] = g;
+                S.u[s & 1][a] = g;
+              }
+              asm volatile("bar.sync 1, 160;" ::: "memory");
+              if (b > s) {
+                const cplx u = S.u[s & 1][a], y = S.y[b];
+                g.x = fma(-u.x, y.x, g.x);
+                g.x = fma(u.y, y.y, g.x);
+                g.y = fma(-u.x, y.y, g.y);
+                g.y = fma(-u.y, y.x, g.y);
+              }
+            } else {
+              if (a == s && b > s) {
+                S.R[s][b] = make_double2(0.0, 0.0);
+                g = make_double2(0.0, 0.0);
+              } else if (b == s && a < s) {
+                S.M[a][s] = make_double2(0.0, 0.0);
+              }
+              asm volatile("bar.sync 1, 160;" ::: "memory");
+            }
+          }
+          if (tid == 0) S.done = s;
+        }
+        __syncthreads();
+      } else {
+        // ---- second round: the columns are orthonormal up to E = V^H V - 1, |E| < 1e-6 (KEEP); the
+        // factor 1 + U and its inverse 1 - U + U^2, to third order
+        const int a = tid >> 4, b = tid & 15;
+        const bool on = a <= b && b < S.done && S.take[a] > 0 && S.take[b] > 0;
+        cplx g = make_double2(0.0, 0.0);
+        auto half = [&] {
+          if (a == b) g = make_double2(0.5 * g.x, 0.0);
+        };
+        if (on) {
+          g = S.G[a][b];
+          if (a == b) g.x -= 1.0;
+          half();
+        }
+        const cplx e1 = g;
+        S.M[a][b] = g;
+        __syncthreads();
+        if (on) {
+          cplx q = make_double2(0.0, 0.0);     // (U^H U)_ab
+          for (int k = 0; k <= a; ++k) {
+            const cplx x = S.M[k][a], y = S.M[k][b];
+            q.x = fma(x.x, y.x, fma(x.y, y.y, q.x));
+            q.y = fma(x.x, y.y, fma(-x.y, y.x, q.y));
+          }
+          g = q;
+          half();
+          g = make_double2(e1.x - g.x, e1.y - g.y);
+        }
+        S.G[a][b] = g;                         // U
+        __syncthreads();
+        cplx w = make_double2(0.0, 0.0);
+        if (on) {
+          w = make_double2((a == b ? 1.0 : 0.0) - g.x, -g.y);
+          for (int k = a; k <= b; ++k) {
+            const cplx x = S.G[a][k], y = S.G[k][b];
+            w.x = fma(x.x, y.x, fma(-x.y, y.y, w.x));
+            w.y = fma(x.x, y.y, fma(x.y, y.x, w.y));
+          }
+        }
+        S.M[a][b] = w;
+        __syncthreads();
+      }
       const int done = S.done;
       // ---- the new columns q_t = sum_{s <= t} v_s M_st: warp w takes columns w and 15 - w, the
       // lanes the rows (MAXR / 32 rows each)
@@ -780,6 +858,47 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         }
         __syncthreads();
       }
+      if (refine || !S.refine) break;
+      refine = true;
+      // skipped and put-off columns take no part in the second round
+      for (int e = tid; e < QB * nr; e += QT_THREADS) {
+        const int t = e / nr, r = e % nr;
+        if (t >= S.done || S.take[t] <= 0) V[t * LDV + r] = make_double2(0.0, 0.0);
+      }
+      __syncthreads();
+    }
+    if (!alive) break;
+    // rows of the accepted vectors in R's new columns: the sum of the passes' coefficients (the CTAs
+    // share the rows where they can all read the sums, else CTA 0 kept them)
+    auto write_r = [&](int cols) {
+      if (private_r && blockIdx.x != 0) return;
+      const int first = private_r ? 0 : blockIdx.x, G = private_r ? 1 : gridDim.x;
+      for (int e = first * QT_THREADS + tid; e < na * QB; e += G * QT_THREADS) {
+        const int i = e >> 4, t = e & 15;
+        cplx r = make_double2(0.0, 0.0);
+        for (int q = 0; q < npass; ++q) {
+          const cplx h = __ldcg(A.fin + (long long)q * A.PS + e);
+          r = make_double2(r.x + h.x, r.y + h.y);
+        }
+        if (refine)
+          for (int s = 0; s <= t; ++s)
+            if (S.take[s] > 0) {
+              const cplx h = __ldcg(A.fin + (long long)npass * A.PS + i * QB + s), f = S.R[s][t];
+              r.x = fma(h.x, f.x, fma(-h.y, f.y, r.x));
+              r.y = fma(h.x, f.y, fma(h.y, f.x, r.y));
+            }
+        if (t < cols) A.R[(long long)S.idx[i] * n + j0 + t] = r;
+      }
+    };
+    if (all_dropped) {
+      if (main_phase) {
+        write_r(bsz);
+        j0 += bsz;
+      } else {
+        cand += bsz;
+      }
+    } else {
+      const int done = S.done;
       // ---- bookkeeping: S.em[t] = position of column t among the accepted vectors, -1 if none
       if (tid == 0) {
         int a = na, pos = open;
@@ -871,7 +990,16 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
       if (main_phase && blockIdx.x == 0)
         for (int e = tid; e < done * done; e += QT_THREADS) {
           const int s = e / done, t = e % done;
-          if (s <= t) A.R[(long long)(j0 + s) * n + j0 + t] = S.R[s][t];
+          if (s > t) continue;
+          cplx r = S.R[s][t];
+          if (refine && S.take[s] > 0)       // (1 + U) R
+            for (int k = s; k <= t; ++k)
+              if (S.take[k] > 0) {
+                const cplx x = S.G[s][k], y = S.R[k][t];
+                r.x = fma(x.x, y.x, fma(-x.y, y.y, r.x));
+                r.y = fma(x.x, y.y, fma(x.y, y.x, r.y));
+              }
+          A.R[(long long)(j0 + s) * n + j0 + t] = r;
         }
       if (main_phase) write_r(done);
       na = na1;
@@ -933,7 +1061,7 @@ cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx
   QtPlan pl;
   if (!W.dig || !qt_plan(m, n, cap, pl)) return cudaSuccess;
   const long long PS = (long long)n * QB + QB + QB * QB;
-  if ((size_t)pl.G * pl.dig_cta > W.dig_bytes || (2 * (long long)pl.G + PASSES) * PS > scratch_len) return cudaSuccess;
+  if ((size_t)pl.G * pl.dig_cta > W.dig_bytes || (2 * (long long)pl.G + PASSES + 1) * PS > scratch_len) return cudaSuccess;
   static bool attr = false;
   cudaError_t e;
   if (!attr) {
@@ -948,7 +1076,7 @@ cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx
   a.Y = Y; a.E = p > 0 ? E : Y;
   a.Q = Q; a.R = R;
   a.part = scratch;
-  a.fin = scratch + 2 * (long long)pl.G * PS;      // PASSES * PS
+  a.fin = scratch + 2 * (long long)pl.G * PS;      // (PASSES + 1) * PS
   a.PS = (int)PS;
   a.dig = W.dig;
   a.dig_cta = pl.dig_cta;

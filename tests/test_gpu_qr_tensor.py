@@ -129,3 +129,19 @@ def test_nonfinite_input_takes_nothing(bad):
     ref, tri = np.linalg.qr(np.delete(E, 2, axis=1)[:, :20])
     ref = ref * (np.diag(tri) / np.abs(np.diag(tri)))
     assert np.abs(Q - ref).max() < 1e-10
+
+
+@pytest.mark.parametrize("span", [0.5, 3.0, 9.0, 20.0])
+@pytest.mark.parametrize("m,n", [(16, 16), (40, 17), (257, 40), (1200, 130)])
+def test_graded(m, n, span):
+    """Singular values from 1 to e^-span, mixed over the columns: what is left of a column inside its
+    block lies above a quarter, above 1e-8 (a second round) and below it (the next block).  Entries
+    of both products round sums of rows and columns of norm <= 1: 1e-13 as in test_full_rank."""
+    rng = np.random.default_rng(m + n)
+    U, _ = np.linalg.qr(random_complex(rng, (n, n)))
+    Y = np.linalg.qr(random_complex(rng, (m, n)))[0] @ (np.exp(-span * np.arange(n) / n)[:, None] * U)
+    Q, R = run(Y)
+    assert np.abs(Q.conj().T @ Q - np.eye(n)).max() < 1e-13
+    assert np.abs(Q @ R - Y).max() < 1e-13 * np.linalg.norm(Y, axis=0).max()
+    assert np.abs(np.tril(R, -1)).max() == 0.0
+    assert np.all(np.diag(R).real > 0) and np.abs(np.diag(R).imag).max() == 0.0
