@@ -71,6 +71,8 @@ constexpr int PASSES = 4;                       // projections of a block, at mo
 // smallest part of a norm^2 that may be left where the rest is taken off in the Gram matrix
 // (rounding of 2^-53 is then up to 1e-8 of what is left; the second round takes that out)
 constexpr double KEEP = 1e-8;
+// a correction whose coefficients are below it is formed in FP32: 16 terms of 2^-32 rounded at 2^-24
+constexpr double SMALL = 2.3283064365386963e-10;
 constexpr int E_EMPTY = -100000;
 constexpr int TMEM_COLS = 512;
 constexpr int IM = NL * QB;                     // im levels after the re levels
@@ -187,8 +189,10 @@ struct Pipe {
   uint64_t* full;           // [2] ring stages
   uint64_t* empty;          // [2]
   uint64_t* done;           // one GEMM's accumulators
+  uint64_t* side;           // Q P: its B^H B, which comes after
   uint32_t it;              // ring steps used so far
   uint32_t gemms;           // GEMMs completed so far
+  uint32_t sides;
   volatile int* fail;
   int* status;
 };
@@ -197,7 +201,8 @@ struct Pipe {
 // `bytes` of it, at `off` of a stage) through the ring, B in shared memory at bdig + s * BSTEP.
 // conj: Q^H V (re = ArBr + AiBi, im = ArBi - AiBr), else Q P (re = ArBr - AiBi, im = ArBi + AiBr).
 // gram_steps: also B^H B of the same B tiles into columns 256.. (A = the B tile itself, its rows
-// beyond 16 unused).
+// beyond 16 unused): with Q^H V while the first copies are on their way, with Q P behind it, so that
+// it runs while V is updated.
 __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
                         const unsigned char* bdig,
                         const unsigned char* src, long long stride, uint32_t bytes, int S,
@@ -234,9 +239,12 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
   };
   for (int s = 0; s < S && s < 2; ++s) load(s);
   const uint32_t b0 = smem_u32(bdig);
-  for (int s = 0; s < gram_steps; ++s)
-    tile(b0 + s * BSTEP, ND * 256, 128, BSTEP / 2, 256, b0 + s * BSTEP, tmem + 2 * IM, s == 0,
-         true);
+  auto gram = [&] {
+    for (int s = 0; s < gram_steps; ++s)
+      tile(b0 + s * BSTEP, ND * 256, 128, BSTEP / 2, 256, b0 + s * BSTEP, tmem + 2 * IM, s == 0,
+           true);
+  };
+  if (conj) gram();
   for (int s = 0; s < S; ++s) {
     const int st = (it0 + s) & 1;
     const uint32_t par = ((it0 + s) >> 1) & 1;
@@ -257,6 +265,10 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
     }
   }
   mma_commit(P.done);
+  if (!conj && gram_steps > 0) {
+    gram();
+    mma_commit(P.side);
+  }
   P.it += S;
   if (!ok) {
     // copies in flight land (bounded) before the shared memory can be released
@@ -315,7 +327,7 @@ struct Shared {
   double red[32];
   int ok, fail, done, last, any, near, refine;
   uint32_t tmem;
-  uint64_t bar[5];
+  uint64_t bar[6];
 };
 
 }  // namespace
@@ -346,9 +358,9 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
   unsigned ep = 0;
   bool alive = true;
 
-  Pipe P{&S.bar[0], &S.bar[2], &S.bar[4], 0, 0, &S.fail, A.status};
+  Pipe P{&S.bar[0], &S.bar[2], &S.bar[4], &S.bar[5], 0, 0, 0, &S.fail, A.status};
   if (tid == 0) {
-    for (int i = 0; i < 5; ++i) mbar_init(&S.bar[i], 1);
+    for (int i = 0; i < 6; ++i) mbar_init(&S.bar[i], 1);
     S.fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -426,6 +438,7 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
     int npass = 0;            // passes of the first round
     bool all_dropped = false;
     bool refine = false;      // second round: one pass over the block's new columns
+    bool small = false;       // it changes them by less than SMALL
     for (;;) {
       for (int pass = npass; pass <= PASSES; ++pass) {
         // digits of V, one scale per column (two columns per warp)
@@ -640,6 +653,13 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
                 v = make_double2(v.x - out[c].x, v.y - out[c].y);
               }
           }
+          if (corr) {
+            alive = mbar_wait(P.side, P.sides & 1, P.fail, A.status, 1);
+            ++P.sides;
+            alive = __syncthreads_and(alive ? 1 : 0) != 0;
+            if (!alive) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
           if (corr && quad == 0) {
             cplx out[8];
             qt_read(tmem + 2 * IM + t0, S.ev[lane & 15], S.ev + t0, out);
@@ -778,50 +798,74 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         __syncthreads();
       } else {
         // ---- second round: the columns are orthonormal up to E = V^H V - 1, |E| < 1e-6 (KEEP); the
-        // factor 1 + U and its inverse 1 - U + U^2, to third order
+        // factor 1 + U and its inverse 1 - W, W = U - U^2, to third order (the second-order terms,
+        // below 1e-12, in FP32)
         const int a = tid >> 4, b = tid & 15;
         const bool on = a <= b && b < S.done && S.take[a] > 0 && S.take[b] > 0;
+        float2* F = reinterpret_cast<float2*>(S.own);      // U to first order, U, then W
         cplx g = make_double2(0.0, 0.0);
-        auto half = [&] {
-          if (a == b) g = make_double2(0.5 * g.x, 0.0);
-        };
         if (on) {
           g = S.G[a][b];
-          if (a == b) g.x -= 1.0;
-          half();
+          if (a == b) g = make_double2(0.5 * (g.x - 1.0), 0.0);
         }
-        const cplx e1 = g;
-        S.M[a][b] = g;
+        F[tid] = make_float2((float)g.x, (float)g.y);
         __syncthreads();
         if (on) {
-          cplx q = make_double2(0.0, 0.0);     // (U^H U)_ab
+          float2 q = make_float2(0.0f, 0.0f);  // (U^H U)_ab
           for (int k = 0; k <= a; ++k) {
-            const cplx x = S.M[k][a], y = S.M[k][b];
-            q.x = fma(x.x, y.x, fma(x.y, y.y, q.x));
-            q.y = fma(x.x, y.y, fma(-x.y, y.x, q.y));
+            const float2 x = F[k * QB + a], y = F[k * QB + b];
+            q.x = fmaf(x.x, y.x, fmaf(x.y, y.y, q.x));
+            q.y = fmaf(x.x, y.y, fmaf(-x.y, y.x, q.y));
           }
-          g = q;
-          half();
-          g = make_double2(e1.x - g.x, e1.y - g.y);
+          if (a == b) q = make_float2(0.5f * q.x, 0.0f);
+          g = make_double2(g.x - q.x, g.y - q.y);
         }
         S.G[a][b] = g;                         // U
+        F[256 + tid] = make_float2((float)g.x, (float)g.y);
         __syncthreads();
-        cplx w = make_double2(0.0, 0.0);
+        cplx w = g;
         if (on) {
-          w = make_double2((a == b ? 1.0 : 0.0) - g.x, -g.y);
+          float2 q = make_float2(0.0f, 0.0f);  // (U^2)_ab
           for (int k = a; k <= b; ++k) {
-            const cplx x = S.G[a][k], y = S.G[k][b];
-            w.x = fma(x.x, y.x, fma(-x.y, y.y, w.x));
-            w.y = fma(x.x, y.y, fma(x.y, y.x, w.y));
+            const float2 x = F[256 + a * QB + k], y = F[256 + k * QB + b];
+            q.x = fmaf(x.x, y.x, fmaf(-x.y, y.y, q.x));
+            q.y = fmaf(x.x, y.y, fmaf(x.y, y.x, q.y));
           }
+          w = make_double2(w.x - q.x, w.y - q.y);
         }
-        S.M[a][b] = w;
-        __syncthreads();
+        S.M[a][b] = make_double2((on && a == b ? 1.0 : 0.0) - w.x, -w.y);
+        F[512 + tid] = make_float2((float)w.x, (float)w.y);
+        small = __syncthreads_and(fabs(w.x) < SMALL && fabs(w.y) < SMALL) != 0;
       }
       const int done = S.done;
       // ---- the new columns q_t = sum_{s <= t} v_s M_st: warp w takes columns w and 15 - w, the
-      // lanes the rows (MAXR / 32 rows each)
-      {
+      // lanes the rows (MAXR / 32 rows each).  A second round that changes little: v_t - sum v_s W_st,
+      // the sum in FP32
+      if (small) {
+        const float2* W = reinterpret_cast<const float2*>(S.own) + 512;
+        float2* F = reinterpret_cast<float2*>(ring);       // V, [QB][MAXR + 1]
+        for (int e = tid; e < QB * nr; e += QT_THREADS) {
+          const int t = e / nr, r = e - t * nr;
+          const cplx v = V[t * LDV + r];
+          F[t * LDV + r] = make_float2((float)v.x, (float)v.y);
+        }
+        __syncthreads();
+        for (int u = 0; u < 2; ++u) {
+          const int t = u == 0 ? warp : QB - 1 - warp;
+          if (t >= done || S.take[t] <= 0) continue;
+          for (int r = lane; r < nr; r += 32) {
+            float2 q = make_float2(0.0f, 0.0f);
+            for (int s = 0; s <= t; ++s) {
+              const float2 v = F[s * LDV + r], c = W[s * QB + t];
+              q.x = fmaf(v.x, c.x, fmaf(-v.y, c.y, q.x));
+              q.y = fmaf(v.x, c.y, fmaf(v.y, c.x, q.y));
+            }
+            cplx& v = V[t * LDV + r];
+            v = make_double2(v.x - q.x, v.y - q.y);
+          }
+        }
+        __syncthreads();
+      } else {
         cplx q[2][MAXR / 32];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -987,10 +1031,12 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
           if (t == 0) S.er[r] = er;
         }
       }
-      if (main_phase && blockIdx.x == 0)
-        for (int e = tid; e < done * done; e += QT_THREADS) {
-          const int s = e / done, t = e % done;
-          if (s > t) continue;
+      // the block's own part of R, a share of it to every CTA
+      if (main_phase)
+        for (int e = blockIdx.x * 32 + (tid & 31) + (tid >> 5) * 32 * gridDim.x; e < QB * QB;
+             e += QT_THREADS * gridDim.x) {
+          const int s = e >> 4, t = e & 15;
+          if (s > t || t >= done) continue;
           cplx r = S.R[s][t];
           if (refine && S.take[s] > 0)       // (1 + U) R
             for (int k = s; k <= t; ++k)
