@@ -198,6 +198,8 @@ __global__ void __launch_bounds__(128, NST == 2 ? 2 : 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  behind_next();
+  behind_wait();
 
   if (threadIdx.x == 0) {
     // producer
@@ -331,6 +333,8 @@ __global__ void __launch_bounds__(128, NST == 2 ? 2 : 1)
 
 // sum of the split-K partials into the requested output form
 __global__ void split_reduce_kernel(TcGemm g) {
+  behind_next();
+  behind_wait();
   const int ks = g.ksplit;
   const long long MN = (long long)g.M * g.N;
   const long long total = (long long)g.nbatch * MN;
@@ -400,6 +404,8 @@ cudaError_t make_map(CUtensorMap* m, const TcOperand& op, int box_rows) {
 // src[b*sb + row*rs + k*ks] (conjugated if conj)
 __global__ void split_f64_kernel(const double2* src, long long sb, long long rs, long long ks,
                                  int conj, float* dst, int nb, int rows, int K, int ld) {
+  behind_next();
+  behind_wait();
   const long long plane = (long long)nb * rows * ld;
   const long long total = (long long)nb * rows * K;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -423,6 +429,8 @@ __global__ void split_f64_kernel(const double2* src, long long sb, long long rs,
 // (the source is row-contiguous: consecutive rows are adjacent)
 __global__ void split_f64_t_kernel(const double2* src, long long sb, long long kstride, int conj,
                                    float* dst, int nb, int rows, int K, int ld) {
+  behind_next();
+  behind_wait();
   __shared__ double2 tile[32][33];
   const long long plane = (long long)nb * rows * ld;
   const int b = blockIdx.z;
@@ -456,6 +464,8 @@ constexpr int MIX_MAX_OPS = 5000;     // float2 entries: nblk * d * d (40 KB)
 __global__ void mix_split_kernel(int Dout, int Ma, int d, int Mb, const int* start,
                                  const int* chan, const float2* ops, int nblk, const float* X,
                                  long long xs, long long xplane, float* dst, int ld, int trans) {
+  behind_next();
+  behind_wait();
   __shared__ float2 s_ops[MIX_MAX_OPS];
   __shared__ int s_start[MIX_MAX_BLK + 1];
   __shared__ int s_chan[MIX_MAX_BLK];
@@ -513,6 +523,8 @@ __global__ void __launch_bounds__(256, D >= 10 ? 2 : (D >= 8 ? 3 : 4)) mix_split
                                                                 const float* X, long long xs,
                                                                 long long xplane, float* dst,
                                                                 int ld, int trans) {
+  behind_next();
+  behind_wait();
   __shared__ float2 s_ops[MIX_MAX_OPS];
   __shared__ int s_start[MIX_MAX_BLK + 1];
   __shared__ int s_chan[MIX_MAX_BLK];
@@ -570,6 +582,8 @@ __global__ void __launch_bounds__(256, D >= 10 ? 2 : (D >= 8 ? 3 : 4)) mix_split
 // split planes (natural operand layout [4][nb][rows][ld]) -> complex FP64 [nb][rows][K]
 __global__ void planes_to_f64_kernel(const float* P, int nb, int rows, int K, int ld,
                                      double2* out) {
+  behind_next();
+  behind_wait();
   const long long plane = (long long)nb * rows * ld;
   const long long total = (long long)nb * rows * K;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -713,16 +727,16 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, const TcGemm& g, cud
   dim3 grid((g.N + bn - 1) / bn, (g.M + BM - 1) / BM, g.nbatch * gg.ksplit);
   count_launch();
   if (bn == 128)
-    tc_zgemm_kernel<3, 128><<<grid, 128, smem_bytes(3, 128), s>>>(ma, mb, gg);
+    e = launch_behind(tc_zgemm_kernel<3, 128>, grid, 128, smem_bytes(3, 128), s, ma, mb, gg);
   else if ((long long)grid.x * grid.y * grid.z <= n_sms)
-    tc_zgemm_kernel<4, 64><<<grid, 128, smem_bytes(4, 64), s>>>(ma, mb, gg);
+    e = launch_behind(tc_zgemm_kernel<4, 64>, grid, 128, smem_bytes(4, 64), s, ma, mb, gg);
   else
-    tc_zgemm_kernel<2, 64><<<grid, 128, smem_bytes(2, 64), s>>>(ma, mb, gg);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_behind(tc_zgemm_kernel<2, 64>, grid, 128, smem_bytes(2, 64), s, ma, mb, gg);
+  if (e != cudaSuccess) return e;
   if (gg.ksplit > 1) {
     count_launch();
-    split_reduce_kernel<<<grid_for((long long)g.nbatch * g.M * g.N), 256, 0, s>>>(gg);
-    e = cudaGetLastError();
+    e = launch_behind(split_reduce_kernel, dim3(grid_for((long long)g.nbatch * g.M * g.N)), 256, 0, s,
+                      gg);
   }
   return e;
 }
@@ -762,18 +776,16 @@ cudaError_t split_f64(const cplx* src, long long sb, long long rs, long long ks,
                       const TcOperand& dst, cudaStream_t s) {
   const long long total = (long long)dst.nb * dst.rows * dst.K;
   count_launch();
-  split_f64_kernel<<<grid_for(total), 256, 0, s>>>(src, sb, rs, ks, conj, dst.p, dst.nb, dst.rows,
-                                                   dst.K, dst.ld);
-  return cudaGetLastError();
+  return launch_behind(split_f64_kernel, dim3(grid_for(total)), 256, 0, s, src, sb, rs, ks, conj, dst.p,
+                       dst.nb, dst.rows, dst.K, dst.ld);
 }
 
 cudaError_t split_f64_t(const cplx* src, long long sb, long long kstride, int conj,
                         const TcOperand& dst, cudaStream_t s) {
   dim3 grid((dst.rows + 31) / 32, (dst.K + 31) / 32, dst.nb);
   count_launch();
-  split_f64_t_kernel<<<grid, dim3(32, 8), 0, s>>>(src, sb, kstride, conj, dst.p, dst.nb, dst.rows,
-                                                  dst.K, dst.ld);
-  return cudaGetLastError();
+  return launch_behind(split_f64_t_kernel, grid, dim3(32, 8), 0, s, src, sb, kstride, conj, dst.p, dst.nb,
+                       dst.rows, dst.K, dst.ld);
 }
 
 cudaError_t mix_split(const MixTable& T, int Ma, int d, int Mb, const float* X, long long xs,
@@ -786,10 +798,9 @@ cudaError_t mix_split(const MixTable& T, int Ma, int d, int Mb, const float* X, 
 #define TDMRG_MIX_COLS(DD)                                                                    \
   case DD:                                                                                   \
     if (cols >= (1LL << 31) - 256LL * 152 * 32) break;                                       \
-    mix_split_cols_kernel<DD><<<grid_for(cols), 256, 0, s>>>(T.Dout, Ma, Mb, T.start, T.chan, \
-                                                             T.ops32, T.nblk, X, xs, xplane, \
-                                                             dst.p, dst.ld, trans);          \
-    return cudaGetLastError();
+    return launch_behind(mix_split_cols_kernel<DD>, dim3(grid_for(cols)), 256, 0, s, T.Dout, \
+                         Ma, Mb, T.start, T.chan, T.ops32, T.nblk, X, xs, xplane, dst.p,     \
+                         dst.ld, trans);
   switch (d) {
     TDMRG_MIX_COLS(2)
     TDMRG_MIX_COLS(3)
@@ -804,16 +815,15 @@ cudaError_t mix_split(const MixTable& T, int Ma, int d, int Mb, const float* X, 
       break;
   }
 #undef TDMRG_MIX_COLS
-  mix_split_kernel<<<grid_for(total), 256, 0, s>>>(T.Dout, Ma, d, Mb, T.start, T.chan, T.ops32,
-                                                   T.nblk, X, xs, xplane, dst.p, dst.ld, trans);
-  return cudaGetLastError();
+  return launch_behind(mix_split_kernel, dim3(grid_for(total)), 256, 0, s, T.Dout, Ma, d, Mb, T.start,
+                       T.chan, T.ops32, T.nblk, X, xs, xplane, dst.p, dst.ld, trans);
 }
 
 cudaError_t planes_to_f64(const TcOperand& P, cplx* out, cudaStream_t s) {
   const long long total = (long long)P.nb * P.rows * P.K;
   count_launch();
-  planes_to_f64_kernel<<<grid_for(total), 256, 0, s>>>(P.p, P.nb, P.rows, P.K, P.ld, out);
-  return cudaGetLastError();
+  return launch_behind(planes_to_f64_kernel, dim3(grid_for(total)), 256, 0, s, P.p, P.nb, P.rows, P.K,
+                       P.ld, out);
 }
 
 }  // namespace tdmrg

@@ -17,6 +17,34 @@ void set_global_error(const char* msg);
 long long launch_count();
 void count_launch(int n = 1);
 
+// Kernels of a chain split -> product -> reduction: launched with programmatic stream
+// serialisation, so that a kernel's CTAs take their SM and set up (barriers, TMEM) while the one
+// before it still runs.  The kernel calls behind_wait() before it touches memory (which waits until
+// the kernel before it has finished, its writes visible) and behind_next() to let the next one in.
+#ifdef __CUDACC__
+__device__ __forceinline__ void behind_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void behind_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
+
 // Strided view of a matrix operand: element (i, j) = p[i * rs + j * cs] (conjugated if conj),
 // batch b / reduction term r shift the pointer by b * sb + r * sr.
 struct MixTable;

@@ -84,6 +84,8 @@ constexpr int S_LD = KC + 1;
 
 // One block: 16 rows x one chunk of 128 k of one operand.
 __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
+  behind_next();
+  behind_wait();
   if (A.skip && *A.skip) return;
   __shared__ cplx s_v[SR * S_LD];
   __shared__ int s_e[SR];
@@ -187,7 +189,7 @@ struct GemmArgs {
 };
 
 __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __grid_constant__ GemmArgs A) {
-  if (A.skip && *A.skip) return;
+  behind_next();
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
@@ -225,6 +227,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  behind_wait();
+  if (A.skip && *A.skip) {
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(TMEM_COLS));
+    return;
+  }
 
   if (threadIdx.x == 0) {
     // producer: one contiguous block of each operand per k step
@@ -386,6 +395,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
 
 // C = alpha sum_s part_s + beta C, splits in order
 __global__ void __launch_bounds__(256) digit_reduce_kernel(GemmArgs A) {
+  behind_next();
+  behind_wait();
   if (A.skip && *A.skip) return;
   const long long mn = (long long)A.p_rows * A.q_rows, total = mn * A.nbatch;
   for (long long e = blockIdx.x * 256LL + threadIdx.x; e < total; e += (long long)gridDim.x * 256) {
@@ -556,8 +567,7 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
         sa.blocks0 = (int)blk0;
         if (blk0 + blk1 > 0x7fffffffLL) return cudaErrorInvalidValue;
         count_launch();
-        digit_split_kernel<<<(unsigned)(blk0 + blk1), 256, 0, s>>>(sa);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_behind(digit_split_kernel, dim3((unsigned)(blk0 + blk1)), 256, 0, s, sa);
         if (e != cudaSuccess) return e;
         GemmArgs g{};
         g.pd = p.dig;
@@ -595,14 +605,15 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
         g.part = reinterpret_cast<cplx*>(w);
         if ((long long)bb * g.ksplit > 65535 || p.tiles > 65535) return cudaErrorInvalidValue;
         count_launch();
-        digit_gemm_kernel<<<dim3(q.tiles, p.tiles, bb * g.ksplit), GEMM_THREADS, GEMM_SMEM, s>>>(g);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_behind(digit_gemm_kernel, dim3(q.tiles, p.tiles, bb * g.ksplit), GEMM_THREADS,
+                          GEMM_SMEM, s, g);
+        if (e != cudaSuccess) return e;
         if (g.ksplit > 1) {
           long long blocks = ((long long)p.rows * q.rows * bb + 255) / 256;
           if (blocks > 152 * 8) blocks = 152 * 8;
           count_launch();
-          digit_reduce_kernel<<<(int)blocks, 256, 0, s>>>(g);
-          if ((e = cudaGetLastError()) != cudaSuccess) return e;
+          e = launch_behind(digit_reduce_kernel, dim3((unsigned)blocks), 256, 0, s, g);
+          if (e != cudaSuccess) return e;
         }
       }
   *taken = true;
