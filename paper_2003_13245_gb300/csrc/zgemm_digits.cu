@@ -81,6 +81,8 @@ struct SplitArgs {
 
 constexpr int SR = 16;                        // rows of a split block
 constexpr int S_LD = KC + 1;
+constexpr int PER = 4;                        // entries a thread loads at a time
+static_assert(SR * KC % (256 * PER) == 0, "split block");
 
 // One block: 16 rows x one chunk of 128 k of one operand.
 __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
@@ -103,23 +105,61 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
   const int steps = (kn + KS - 1) / KS;
   const cplx* src = o.p + (long long)b * o.sb + (long long)red * o.sr;
   if (threadIdx.x < SR) s_e[threadIdx.x] = 0;
-  // load in the order that is contiguous in memory
+  // load in the order that is contiguous in memory, PER entries of a thread at a time: their loads
+  // (and, mixed on the fly, the chains table row -> term -> X) are in flight together
   const bool kfast = o.ks == 1;
-  for (int e = threadIdx.x; e < SR * KC; e += 256) {
-    const int r = kfast ? e / KC : e % SR, k = kfast ? e % KC : e / SR;
-    cplx v = make_double2(0.0, 0.0);
-    if (r0 + r < o.rows && k < kn) {
-      const long long off = (long long)(r0 + r) * o.rs + (long long)(k0 + k) * o.ks;
-      if (!o.mix_start) {
-        v = src[off];
-      } else {
-        const int idx = (int)(off + o.off0), sig = (idx / o.dmb) % o.d;
-        const int* st = o.mix_start + (o.by_red ? red : b + o.b0) * o.d + sig;
-        v = mix_entries(__ldg(st), __ldg(st + 1), o.mix_cu, o.mix_val, o.p + (idx - sig * o.dmb),
-                        o.xs, o.dmb);
+  const int* rows = o.mix_start ? o.mix_start + (o.by_red ? red : b + o.b0) * o.d : nullptr;
+#pragma unroll 1
+  for (int e0 = threadIdx.x; e0 < SR * KC; e0 += 256 * PER) {
+    cplx v[PER];
+    const cplx* x[PER];
+    int at[PER], end[PER], dst[PER];
+    bool more = false;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = e0 + i * 256;
+      const int r = kfast ? e / KC : e % SR, k = kfast ? e % KC : e / SR;
+      dst[i] = r * S_LD + k;
+      v[i] = make_double2(0.0, 0.0);
+      x[i] = o.p;
+      at[i] = end[i] = 0;
+      if (r0 + r < o.rows && k < kn) {
+        const long long off = (long long)(r0 + r) * o.rs + (long long)(k0 + k) * o.ks;
+        if (!rows) {
+          v[i] = src[off];
+        } else {
+          const int idx = (int)(off + o.off0), sig = (idx / o.dmb) % o.d;
+          x[i] = o.p + (idx - sig * o.dmb);
+          at[i] = __ldg(rows + sig);
+          end[i] = __ldg(rows + sig + 1);
+        }
       }
     }
-    s_v[r * S_LD + k] = v;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) more = more || at[i] < end[i];
+    for (bool first = true; more; first = false) {
+      cplx f[PER], z[PER];
+      int2 c[PER];
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {          // (a term that is not wanted: term 0 and X[0])
+        const int t = at[i] < end[i] ? at[i] : 0;
+        c[i] = __ldg(o.mix_cu + t);
+        f[i] = __ldg(o.mix_val + t);
+      }
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        z[i] = at[i] < end[i] ? x[i][c[i].x * o.xs + (long long)c[i].y * o.dmb] : o.p[0];
+      more = false;
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        if (at[i] < end[i]) {
+          mix_add(v[i], f[i], z[i], first);
+          ++at[i];
+          more = more || at[i] < end[i];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) s_v[dst[i]] = v[i];
   }
   __syncthreads();
   const int r = threadIdx.x & (SR - 1), g = threadIdx.x / SR;      // row, group of 8 k
