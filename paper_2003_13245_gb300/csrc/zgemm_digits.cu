@@ -11,9 +11,9 @@
 // arithmetic.  Re and im parts share E.  The digits are stored as the shared-memory image of the
 // tile they will be staged in (8 x 16 byte core matrices), so a stage is one contiguous block.
 //
-// Product (digit_gemm_kernel): one CTA computes a 128 x 32 tile of C.  For every digit i of the
-// 128-row operand one tcgen05.mma (kind::f16, FP32 accumulation) multiplies it with the digits
-// j = 0 .. min(6, 7 - i) of the 32-column operand at once (N = 32 per digit), because digit pair
+// Product (digit_gemm_kernel): one CTA computes a 128 x 32 (or 128 x 16) tile of C.  For every digit
+// i of the 128-row operand one tcgen05.mma (kind::f16, FP32 accumulation) multiplies it with the
+// digits j = 0 .. min(6, 7 - i) of the 32-column operand at once (N = 32 per digit), because pair
 // (i, j) goes to the accumulator of level i + j and both the digits in shared memory and the
 // levels in TMEM are contiguous: 4 x 7 instructions per 16-deep k step.  A digit product is at
 // most 2^14; over one chunk of 128 k a level of p pairs sums to at most p 2^22, an integer that
@@ -25,11 +25,15 @@
 // one rounding; the FMA kernel rounds every partial sum.
 //
 // Bound: the tensor pipe in the main loop (28 instructions, ~2300 clocks per k step of 128 x 32),
-// plus the integer epilogue, which cannot overlap it (eight re and im levels fill all 512 TMEM
-// columns).  72 KB per stage from L2, three stages, one CTA per SM.  Measured on GB300 against the
-// FMA kernel: 896 x 8192 x 128 0.28 against 6.2 ms (27 TFLOP/s, tensor pipe 39 %); 8192 x 128 x 128
-// summed over seven channels 0.35 against 7.3 ms; 128 x 128 x 8192, seven batches, 0.55 against
-// 34 ms; 64 x 64 x 256, seven batches, 35 against 1048 us; 16 x 16 x 4 21 against 68 us.
+// plus the integer epilogue, which cannot overlap it (eight re and im levels of 32 columns fill all
+// 512 TMEM columns).  72 KB per stage from L2, three stages, one CTA per SM.  A small product is
+// latency: a launch each for split, product and reduction, set up while the one before runs, half
+// the instructions' time with 16-column tiles.
+//
+// Measured on GB300 against the FMA kernel, split and reduction included: 896 x 8192 x 128 0.255
+// against 6.2 ms (29 TFLOP/s, tensor pipe 39 %); 8192 x 128 x 128 summed over seven channels 0.310
+// against 7.3 ms; 128 x 128 x 8192, seven batches, 0.486 against 34 ms; 64 x 64 x 256, seven
+// batches, 27 against 1049 us (32 with tiles of 32); 16 x 16 x 4 11 against 21 us (15).
 #include "mix.cuh"
 #include "umma.cuh"
 
@@ -41,24 +45,25 @@ using namespace dig;
 
 namespace {
 
-constexpr int PT = 128, QT = 32;              // tile rows (operand P) and columns (operand Q)
+constexpr int PT = 128;                       // tile rows (operand P)
+// tile columns (operand Q): 32, or 16 where the tiles of 32 leave SMs idle
 constexpr int KS = 16;                        // k per stage
 constexpr int KC = 128;                       // k per chunk (one scale per row and chunk)
 constexpr int STEPS = KC / KS;
 constexpr int P_BLOCK = 2 * ND * PT * KS * 2; // 57344 bytes per stage
-constexpr int Q_BLOCK = 2 * ND * QT * KS * 2; // 14336
-constexpr int STAGE = P_BLOCK + Q_BLOCK;
+__host__ __device__ constexpr int q_block(int qt) { return 2 * ND * qt * KS * 2; }     // 14336, 7168
 constexpr int NST = 3;
 constexpr int GEMM_THREADS = 320;             // TMA warp, MMA warp, eight epilogue warps
-constexpr size_t GEMM_SMEM = (size_t)NST * STAGE + 256 + 128;
-constexpr int TMEM_COLS = 512;
+constexpr size_t gemm_smem(int qt) {
+  return (size_t)NST * (P_BLOCK + q_block(qt)) + 256 + 128;
+}
 
 struct Operand {
   const cplx* p;
   long long rs, ks, sb, sr;   // strides of row, k, batch, reduction term
   int conj;
   int rows, nb;               // rows; batches stored (1 when the batches share the operand)
-  int tile;                   // PT or QT
+  int tile;                   // PT, or the width of a Q tile
   int tiles;                  // row tiles
   unsigned char* dig;         // [nb][tiles][steps] blocks
   int* ex;                    // [nb][chunks][tiles * tile]
@@ -201,7 +206,7 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
       if (wide)                      // [part][digit][k half][row group][8 rows][16 B]
         off = (((part * ND + l) * 2 + kh) * (PT / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
       else                           // [part][k half][digit][row group][8 rows][16 B]
-        off = (((part * 2 + kh) * ND + l) * (QT / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
+        off = (((part * 2 + kh) * ND + l) * (o.tile / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
       *reinterpret_cast<uint4*>(dst + off) = make_uint4(h[0], h[1], h[2], h[3]);
     }
   }
@@ -228,7 +233,11 @@ struct GemmArgs {
   const int* skip;
 };
 
+template <int QT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __grid_constant__ GemmArgs A) {
+  constexpr int Q_BLOCK = q_block(QT), STAGE = P_BLOCK + Q_BLOCK;
+  constexpr int TMEM_COLS = 2 * NL * QT;
+  constexpr int CW = QT / 2;                   // columns of an epilogue warp
   behind_next();
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
@@ -344,29 +353,29 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
       if (live) mma_commit(acc_full);
     }
   } else if (warp >= 2) {
-    // epilogue: warp w reads TMEM lanes 32 (w mod 4)..; warps 2-5 the first 16 columns of every
-    // level, warps 6-9 the others
+    // epilogue: warp w reads TMEM lanes 32 (w mod 4)..; warps 2-5 the first half of every
+    // level's columns, warps 6-9 the other
     const int quad = warp & 3, half = (warp - 2) >> 2;
     const int prow = pt * PT + quad * 32 + lane;
-    const int qcol0 = qt * QT + half * 16;
+    const int qcol0 = qt * QT + half * CW;
     const long long pext = (long long)A.p_tiles * PT, qext = (long long)A.q_tiles * QT;
     const int* pe = A.pe + bz * A.pe_b + prow;
     const int* qe = A.qe + bz * A.qe_b + qcol0;
-    const uint32_t base = tmem + ((uint32_t)(quad * 32) << 16) + half * 16;
-    double re[16], im[16];
+    const uint32_t base = tmem + ((uint32_t)(quad * 32) << 16) + half * CW;
+    double re[CW], im[CW];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) re[c] = im[c] = 0.0;
+    for (int c = 0; c < CW; ++c) re[c] = im[c] = 0.0;
     bool ok = true;
     for (int ch = cbeg; ch < cend; ++ch) {
       const int local = ch - cbeg;
       const int ep = __ldg(pe + ch * pext);
-      const int eqv = __ldg(qe + ch * qext + (lane & 15));      // column lane & 15
+      const int eqv = __ldg(qe + ch * qext + (lane & (CW - 1)));      // column lane mod CW
       ok = mbar_wait(acc_full, local & 1, fail, A.status, 3);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-      for (int blk = 0; blk < 8; ++blk) {          // four columns of re, then of im
+      for (int blk = 0; blk < CW / 2; ++blk) {     // four columns of re, then of im
         const int c0 = (blk >> 1) * 4;
         const bool imag = blk & 1;
         int eq[4];
@@ -388,12 +397,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
       if (A.ksplit > 1) {
         cplx* D = A.part + (((long long)sp * A.nbatch + bz) * A.q_rows) * A.p_rows + prow;
 #pragma unroll
-        for (int c = 0; c < 16; ++c)
+        for (int c = 0; c < CW; ++c)
           if (qcol0 + c < A.q_rows) D[(long long)(qcol0 + c) * A.p_rows] = make_double2(re[c], im[c]);
       } else {
         cplx* D = A.C + bz * A.sc + prow * A.cp;
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
+        for (int c = 0; c < CW; ++c) {
           if (qcol0 + c < A.q_rows) {
             cplx v = make_double2(re[c], im[c]);
             cplx* d = D + (qcol0 + c) * A.cq;
@@ -466,21 +475,25 @@ size_t up(size_t x) { return (x + ALIGN - 1) & ~(ALIGN - 1); }
 
 struct Plan {
   int ksteps, chunks, tc;
-  size_t row_p, row_q;       // bytes of one 128-row tile of P, one 32-row tile of Q (with scales)
+  size_t row_p, row_q;       // bytes of one 128-row tile of P, one tile of Q (with scales)
 };
-Plan plan_of(int k, int nred) {
+Plan plan_of(int k, int nred, int qt = 32) {
   Plan p;
   p.ksteps = (k + KS - 1) / KS;
   p.chunks = (k + KC - 1) / KC;
   p.tc = p.chunks * nred;
   p.row_p = (size_t)p.ksteps * nred * P_BLOCK + (size_t)p.tc * PT * sizeof(int);
-  p.row_q = (size_t)p.ksteps * nred * Q_BLOCK + (size_t)p.tc * QT * sizeof(int);
+  p.row_q = (size_t)p.ksteps * nred * q_block(qt) + (size_t)p.tc * qt * sizeof(int);
   return p;
 }
 
 }  // namespace
 
 namespace {
+// Most CTAs with 16-column tiles: one per SM.  They read the 128-row operand twice as often, which
+// L2 has room for as long as they run side by side; a second wave would cost more than the shorter
+// main loop gives.  448 x 256 x 64 (64 CTAs) 15.0 against 20.1 us, 128 x 128 x 128 19.5 against 25.2.
+constexpr int NARROW = 152;
 // splits of the chunk loop that fill the GPU when there are few tiles
 int splits_of(long long ntile, int chunks) {
   const long long ks = (148 + ntile - 1) / ntile;
@@ -491,7 +504,7 @@ int splits_of(long long ntile, int chunks) {
 size_t zgemm_digits_bytes(int m, int n, int k, int nbatch, int nred, int nbA, int nbB) {
   const Plan p = plan_of(k, nred);
   auto need = [&](int pr, int qr, int nbp, int nbq) {
-    const size_t tp = (pr + PT - 1) / PT, tq = (qr + QT - 1) / QT;
+    const size_t tp = (pr + PT - 1) / PT, tq = (qr + 31) / 32;      // (tiles of 16 need no more)
     const int ks = splits_of((long long)(tp * tq) * nbatch, p.tc);
     return tp * nbp * p.row_p + tq * nbq * p.row_q +
            (ks > 1 ? sizeof(cplx) * (size_t)pr * qr * nbatch * ks : 0);
@@ -508,17 +521,19 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
   *taken = false;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(digit_gemm_kernel,
+    cudaError_t e = cudaFuncSetAttribute(digit_gemm_kernel<32>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)GEMM_SMEM);
+                                         (int)gemm_smem(32));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(digit_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)gemm_smem(16));
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const Plan pl = plan_of(k, nred);
   // the 128-row operand P is the side that pads least; on a tie the columns of C, whose stores
   // are then contiguous across the lanes
   auto tiles = [](int a, int t) { return (long long)(a + t - 1) / t; };
-  const bool swap = tiles(n, PT) * tiles(m, QT) <= tiles(m, PT) * tiles(n, QT);
+  const bool swap = tiles(n, PT) * tiles(m, 32) <= tiles(m, PT) * tiles(n, 32);
   auto operand = [&](const MatRef& M, int rows, long long rs, long long ks) {
     Operand o{};
     o.p = M.p;
@@ -543,6 +558,10 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
   const Operand a = operand(A, m, A.rs, A.cs), b = operand(B, n, B.cs, B.rs);
   Operand P = swap ? b : a, Q = swap ? a : b;
   const long long cp = swap ? 1 : ldc, cq = swap ? ldc : 1;
+  const int tc = (k + KC - 1) / KC * nred;
+  const long long narrow = tiles(P.rows, PT) * tiles(Q.rows, 16) * nbatch;
+  const int QT = narrow * splits_of(narrow, tc) <= NARROW ? 16 : 32;
+  const Plan pl = plan_of(k, nred, QT);
   P.tile = PT;
   Q.tile = QT;
   const int pt_all = (int)tiles(P.rows, PT), qt_all = (int)tiles(Q.rows, QT);
@@ -585,7 +604,7 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
         unsigned char* end = static_cast<unsigned char*>(ws.p) + ws.bytes;
         const long long tsteps = (long long)nred * pl.ksteps;
         const size_t pbytes = (size_t)p.tiles * tsteps * P_BLOCK;
-        const size_t qbytes = (size_t)q.tiles * tsteps * Q_BLOCK;
+        const size_t qbytes = (size_t)q.tiles * tsteps * q_block(QT);
         p.dig = w;
         w += up(pbytes * p.nb);
         q.dig = w;
@@ -645,8 +664,8 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
         g.part = reinterpret_cast<cplx*>(w);
         if ((long long)bb * g.ksplit > 65535 || p.tiles > 65535) return cudaErrorInvalidValue;
         count_launch();
-        e = launch_behind(digit_gemm_kernel, dim3(q.tiles, p.tiles, bb * g.ksplit), GEMM_THREADS,
-                          GEMM_SMEM, s, g);
+        e = launch_behind(QT == 16 ? digit_gemm_kernel<16> : digit_gemm_kernel<32>,
+                          dim3(q.tiles, p.tiles, bb * g.ksplit), GEMM_THREADS, gemm_smem(QT), s, g);
         if (e != cudaSuccess) return e;
         if (g.ksplit > 1) {
           long long blocks = ((long long)p.rows * q.rows * bb + 255) / 256;

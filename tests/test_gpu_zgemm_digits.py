@@ -56,6 +56,14 @@ def test_integers_are_exact(Ml, Mr, Dl, Dr):
     assert np.array_equal(heff(L, W, R, A), ref)
 
 
+@pytest.mark.parametrize("Ml,Mr,Dl,Dr", [(400, 530, 1, 1), (513, 561, 1, 1), (497, 640, 1, 1),
+                                         (260, 257, 7, 2)])
+def test_tile_widths(Ml, Mr, Dl, Dr):
+    """The 32-column tiles are taken where 16-column ones would be more than the SMs: sizes on both
+    sides of that line, with 1, 2, 17 and 32 columns in the last tile."""
+    test_integers_are_exact(Ml, Mr, Dl, Dr)
+
+
 @pytest.mark.parametrize("Ml,Mr,Dl,Dr", SHAPES)
 def test_matches_numpy(Ml, Mr, Dl, Dr):
     """Rows and columns of very different size.  Both sides round sums of Ml and Dr Mr products:
