@@ -10,7 +10,9 @@
 //
 // Per Krylov vector j (CTA g owns the contiguous slice [g*S, g*S + S) of every vector):
 //  A.  T_w = L_w q_j for every channel w: complex FP32 FMA on 32 x 32 output tiles with the
-//      whole K = M extent staged in shared memory (M <= 256; the contraction is 2 Dw M^3
+//      whole K = M extent staged in shared memory, all operands read as FP32 copies (L, R converted
+//      once, q_j by the CTA that owns the slice, scaled by a power of two and by the rest of 1/beta
+//      in FP64 after the channel sum) (M <= 256; the contraction is 2 Dw M^3
 //      complex MACs, too small to keep a tensor-core pipeline busy);
 //  B.  P_w = T_w R_w^T, one partial per channel (the channel sum is taken in C1, in order);
 //  C1. w = sum_w P_w in FP64 on the own slice; partial dots against q_{j-1}, q_j;
@@ -23,6 +25,10 @@
 // significands: no coarser than the 3xTF32 tensor-core products), every Lanczos quantity,
 // the small exponential and all norms in FP64.  All reductions have a fixed order: the
 // result does not depend on timing.
+//
+// Bound: latency (barriers of ~1.4 us, loads of a tile's operands, serial FP64 of one warp) and,
+// before the FP32 copies, conversions and scalings of 24,000 numbers per tile pair at the FP64 rate.
+// The call at M = 128, seven channels: 353 us with conversions at every load, 309 us now.
 #include "lanczos_coop.cuh"
 
 namespace tdmrg {
@@ -42,7 +48,8 @@ struct BondArgs {
   const cplx* v;       // [M][M]
   cplx* out;           // [M][M]
   cplx* V;             // kcap vectors of n
-  cplx* W;             // n: the projected, unnormalised new vector
+  float2* W;           // n: the projected new vector in FP32, scaled by a power of two
+  float2* LR;          // [2][Dw][n]: L and R in FP32
   float2* T;           // [Dw][n]
   float2* P;           // [Dw][n]
   cplx* part;          // 2 * G * NV
@@ -123,6 +130,10 @@ __device__ __forceinline__ float2 to_f2(cplx z) {
   return make_float2(__double2float_rn(z.x), __double2float_rn(z.y));
 }
 
+// a power of two near the norm (from the norm^2), for a vector's FP32 copy
+__device__ __forceinline__ int scale_of(double nrm2) { return (bexp(nrm2) - 1023) >> 1; }
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
 __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
   extern __shared__ __align__(16) unsigned char dyn[];
   float2* at = reinterpret_cast<float2*>(dyn);        // [KT][TP]
@@ -143,6 +154,13 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
   cplx* part1 = A.part;
   cplx* part2 = A.part + (size_t)A.G * NV;
 
+  // L and R in FP32 once: a conversion runs at the FP64 rate, and each tile of each vector reads
+  // them again
+  for (long long e = (long long)blockIdx.x * BT + threadIdx.x; e < (long long)Dw * n;
+       e += (long long)A.G * BT) {
+    A.LR[e] = to_f2(__ldg(&A.L[e]));
+    A.LR[(long long)Dw * n + e] = to_f2(__ldg(&A.R[e]));
+  }
   // ||v||: q_0 = v / ||v||
   for (int e = threadIdx.x; e < len; e += BT) ws[e] = A.v[e0 + e];
   __syncthreads();
@@ -160,31 +178,31 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
     return;
   }
   double inv = 1.0 / b0;
-  for (int e = threadIdx.x; e < len; e += BT)
+  int kw = scale_of(s_nrm);
+  for (int e = threadIdx.x; e < len; e += BT) {
     A.V[e0 + e] = make_double2(ws[e].x * inv, ws[e].y * inv);
-  const cplx* src = A.v;        // q_j = src * inv (src is read by every CTA)
+    A.W[e0 + e] = to_f2(make_double2(ws[e].x * pow2(-kw), ws[e].y * pow2(-kw)));
+  }
+  if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
+  double fac = inv * pow2(kw);  // q_j = W * fac (W is read by every CTA)
 
   int k = 0;
   for (int j = 0; j < A.kcap; ++j) {
-    // ---- A: T_w = L_w q_j
+    // ---- A: T_w = L_w q_j / fac
     for (int it = blockIdx.x; it < items; it += A.G) {
       const int w = it / (nt * nt), rem = it - w * nt * nt;
       const int ra = (rem / nt) * TL, cb = (rem % nt) * TL;
-      const cplx* Lw = A.L + (size_t)w * M * M;
-      const double sc = inv;
+      const float2* Lw = A.LR + (size_t)w * n;
       float2 acc[2][2] = {};
       tile_cgemm<false>(
           M,
           [&](int r, int kk) {
             const int a = ra + r;
-            return (a < M && kk < M) ? to_f2(__ldg(&Lw[(size_t)a * M + kk]))
-                                     : make_float2(0.f, 0.f);
+            return (a < M && kk < M) ? __ldcg(&Lw[(size_t)a * M + kk]) : make_float2(0.f, 0.f);
           },
           [&](int kk, int c) {
             const int b = cb + c;
-            if (kk >= M || b >= M) return make_float2(0.f, 0.f);
-            const cplx z = __ldcg(&src[(size_t)kk * M + b]);
-            return make_float2(__double2float_rn(z.x * sc), __double2float_rn(z.y * sc));
+            return (kk < M && b < M) ? __ldcg(&A.W[(size_t)kk * M + b]) : make_float2(0.f, 0.f);
           },
           at, bt, acc);
       const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -203,7 +221,7 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
       const int w = it / (nt * nt), rem = it - w * nt * nt;
       const int ra = (rem / nt) * TL, cb = (rem % nt) * TL;
       const float2* Tw = A.T + (size_t)w * n;
-      const cplx* Rw = A.R + (size_t)w * M * M;
+      const float2* Rw = A.LR + (size_t)(Dw + w) * n;
       float2 acc[2][2] = {};
       tile_cgemm<true>(
           M,
@@ -213,8 +231,7 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
           },
           [&](int kk, int c) {
             const int b = cb + c;
-            return (kk < M && b < M) ? to_f2(__ldg(&Rw[(size_t)b * M + kk]))
-                                     : make_float2(0.f, 0.f);
+            return (kk < M && b < M) ? __ldcg(&Rw[(size_t)b * M + kk]) : make_float2(0.f, 0.f);
           },
           at, bt, acc);
       const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -236,7 +253,7 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
         x += (double)p.x;
         y += (double)p.y;
       }
-      ws[e] = make_double2(x, y);
+      ws[e] = make_double2(x * fac, y * fac);
     }
     __syncthreads();
     const int lo = j > 0 ? j - 1 : 0;
@@ -247,6 +264,7 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
     // (the criterion of Daniel, Gragg, Kaufman and Stewart), the second one against q_0 .. q_j
     lzc::reduce_dots(part1, A.G, lo, j + 1, h1);
     lzc::reduce_norm(A.partn + A.G, A.G, &s_nrm);
+    kw = scale_of(s_nrm);         // of w before the projection: known in time for the last barrier
     lzc::slice_project(A.V, n, ws, e0, len, lo, j + 1, h1);
     if (threadIdx.x == 0) {
       double rem = s_nrm;
@@ -265,7 +283,8 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
       __syncthreads();
     }
     // ---- ||w||^2
-    for (int e = threadIdx.x; e < len; e += BT) A.W[e0 + e] = ws[e];
+    for (int e = threadIdx.x; e < len; e += BT)
+      A.W[e0 + e] = to_f2(make_double2(ws[e].x * pow2(-kw), ws[e].y * pow2(-kw)));
     lzc::slice_norm(ws, len, red, A.partn);
     if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
     // ---- C4: tridiagonal bookkeeping and the small exponential (warp 0 of every CTA)
@@ -288,9 +307,9 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
     k = s_k;
     if (s_done) break;
     inv = s_inv;
+    fac = inv * pow2(kw);
     for (int e = threadIdx.x; e < len; e += BT)
       A.V[(size_t)(j + 1) * n + e0 + e] = make_double2(ws[e].x * inv, ws[e].y * inv);
-    src = A.W;
   }
   // out = sum_{i < k} c_i q_i on the own slice
   for (int e = threadIdx.x; e < len; e += BT) {
@@ -348,7 +367,7 @@ cudaError_t bond_exp_fused(int M, int Dw, const cplx* L, const cplx* R, const cp
   a.S = (int)((a.n + G - 1) / G);
   a.kcap = kcap; a.fixed = fixed;
   a.L = L; a.R = R; a.v = C; a.out = out; a.V = V;
-  a.W = W.W; a.T = W.T; a.P = W.P; a.part = W.part; a.partn = W.partn; a.bar = W.bar;
+  a.W = reinterpret_cast<float2*>(W.W); a.LR = W.LR; a.T = W.T; a.P = W.P; a.part = W.part; a.partn = W.partn; a.bar = W.bar;
   a.status = status; a.mv = W.mv;
   a.wait = W.wait > 0 ? W.wait : kBarrierWaitCycles;
   a.tr = tr; a.ti = ti; a.tol = tol;

@@ -1173,6 +1173,7 @@ int tdmrg_kernel_bond_exp(int M, int Dw, const void* L, const void* R, const voi
     W.W = mem.get(n);
     W.T = (float2*)mem.bytes(sizeof(float2) * (size_t)Dw * n);
     W.P = (float2*)mem.bytes(sizeof(float2) * (size_t)Dw * n);
+    W.LR = (float2*)mem.bytes(sizeof(float2) * 2 * (size_t)Dw * n);
     W.part = mem.get(2 * (long long)sms * (tdmrg::KMAX + 1));
     W.partn = (double*)mem.bytes(sizeof(double) * 2 * (size_t)sms);   // 2 * gmax
     W.bar = (unsigned*)mem.bytes(sizeof(unsigned) * 2);

@@ -515,7 +515,7 @@ Engine::~Engine() {
     if (e) cudaEventDestroy(e);
   for (float* p : {tcb_.envA, tcb_.envB, tcb_.siteA, tcb_.siteB, tcb_.x32, tcb_.mix, tcb_.kpart})
     if (p) cudaFree(p);
-  for (void* p : {(void*)bs_.W, (void*)bs_.T, (void*)bs_.P, (void*)bs_.part, (void*)bs_.partn,
+  for (void* p : {(void*)bs_.W, (void*)bs_.T, (void*)bs_.P, (void*)bs_.LR, (void*)bs_.part, (void*)bs_.partn,
                   (void*)bs_.bar, (void*)bs_.mv})
     if (p) cudaFree(p);
   if (h_mv_) cudaFreeHost(h_mv_);
@@ -805,13 +805,14 @@ void Engine::ensure_bond_scratch(int maxbond) {
   const long long maxn = (long long)maxbond * maxbond;
   const int maxDw = std::max(H_.maxD, J_.maxD);
   if (maxn <= bs_.maxn && maxDw <= bs_.maxDw) return;
-  for (void* p : {(void*)bs_.W, (void*)bs_.T, (void*)bs_.P})
+  for (void* p : {(void*)bs_.W, (void*)bs_.T, (void*)bs_.P, (void*)bs_.LR})
     if (p) cudaFree(p);
   bs_.W = nullptr;
-  bs_.T = bs_.P = nullptr;
+  bs_.T = bs_.P = bs_.LR = nullptr;
   CK(cudaMalloc(&bs_.W, sizeof(cplx) * (size_t)maxn));
   CK(cudaMalloc(&bs_.T, sizeof(float2) * (size_t)maxDw * maxn));
   CK(cudaMalloc(&bs_.P, sizeof(float2) * (size_t)maxDw * maxn));
+  CK(cudaMalloc(&bs_.LR, sizeof(float2) * 2 * (size_t)maxDw * maxn));
   if (!bs_.part) {
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));

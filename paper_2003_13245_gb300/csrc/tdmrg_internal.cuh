@@ -158,6 +158,7 @@ struct BondScratch {
   cplx* W = nullptr;                 // maxn
   float2* T = nullptr;               // maxDw * maxn
   float2* P = nullptr;               // maxDw * maxn
+  float2* LR = nullptr;              // 2 * maxDw * maxn
   cplx* part = nullptr;              // 2 * gmax * (KMAX + 1)
   double* partn = nullptr;           // 2 * gmax (lz_step: the norms before and after)
   unsigned* bar = nullptr;           // 2 (barrier counter, generation)
