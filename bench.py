@@ -28,12 +28,12 @@ sys.path.insert(0, ROOT)
 
 WORKLOAD = dict(name="holstein-N16-2mode-M128", N=16, omega=[0.2, 1.0], g=[1.5, 0.8],
                 nmax=[8, 4], V=0.5, kT=2.0, dtau=0.05, M=128, dt=0.05)
-# GB300 dense FP64 from unit counts and clock (152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz;
-# nominal 1.25 TFLOP/s); no FP64 figure is measured on this machine
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+# FP64 contractions (and the projections of the gauge QR) are taken as exact products of 8-bit
+# digits in fp16 on the tensor cores: 34 digit products per real product
+DIGIT_PRODUCTS = 34
 METRIC = "TDVP site-updates/s (real-time, both states, N=16 2-mode Holstein chain, M=128)"
 # DRAM bytes (read + write) of one 8192 x 128 gauge-QR launch, measured by ncu
-QR_BULK_TRAFFIC = 17378560 + 225792
+QR_BULK_TRAFFIC = 19006976 + 29809408
 
 
 def parse():
@@ -341,20 +341,21 @@ def run_ours(args):
 
     value = total_units / (ms_max / 1e3)
     heff_tflops = st["heff_flops"] / (st["heff_ms"] / 1e3) / 1e12 if st["heff_ms"] > 0 else None
+    peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
+    digit_peak = peaks["bf16_tflops_sustained"] / DIGIT_PRODUCTS
     if prec == PREC_C128:
-        roof = {"bound": "alu", "achieved": heff_tflops, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "frac": heff_tflops / FP64_PEAK_TFLOPS if heff_tflops else None,
+        roof = {"bound": "tensor", "achieved": heff_tflops, "peak": digit_peak,
+                "unit": "TFLOP/s", "frac": heff_tflops / digit_peak if heff_tflops else None,
                 "traffic": None,
-                "kernel": "zgemm_kernel (H_eff contractions, FP64 DFMA)",
-                "peak_source": "GB300 FP64 rate from unit counts and clock: 152 SMs x 2 DFMA/clk "
-                               "x 2 flops x 2.07 GHz = 1.26 (nominal 1.25) TFLOP/s; no FP64 "
-                               "figure is measured on this pool",
+                "kernel": "digit_split_kernel + digit_gemm_kernel (H_eff contractions, FP64 operands "
+                          "as seven 8-bit digits on tcgen05 kind::f16)",
+                "peak_source": "MEASURED_PEAKS bf16_tflops_sustained / 34 digit products per real "
+                               "product, of measured",
                 "per_launch": "algorithmic H_eff flops 8*(Dl*Ml^2*d^2*Mr + Dr*Ml*d^2*Mr^2) "
                               "per matvec / event-timed matvec duration"}
     else:
         # the H_eff matvec runs inside a long step: sustained bf16 peak of measured, TF32 at half
         # the bf16 rate (nominal ratio 1.1 : 2.25 PFLOP/s dense)
-        peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
         tf32 = peaks["bf16_tflops_sustained"] / 2.0
         iso = heff_iso["tflops"] if heff_iso else None
         heff_roof = {"bound": "tensor", "achieved": iso, "peak": tf32, "unit": "TFLOP/s",
@@ -377,34 +378,35 @@ def run_ours(args):
         qr_all = st["qr_flops"] / (st["qr_ms"] / 1e3) / 1e12 if st["qr_ms"] > 0 else None
         qr_tflops = (st["qr_bulk_flops"] / (st["qr_bulk_ms"] / 1e3) / 1e12
                      if st["qr_bulk_ms"] > 0 else None)
-        lane_peak = FP64_PEAK_TFLOPS * lane_sms / sms
-        roof = {"bound": "alu", "achieved": qr_tflops, "peak": lane_peak,
+        lane_peak = digit_peak * lane_sms / sms
+        roof = {"bound": "tensor", "achieved": qr_tflops, "peak": lane_peak,
                 "unit": "TFLOP/s", "frac": qr_tflops / lane_peak if qr_tflops else None,
                 "traffic": QR_BULK_TRAFFIC,
                 "launch": "8192 x 128 complex (the bulk sites), %d launches in the timed region"
                           % int(st["qr_bulk_n"]),
                 "all_launches": {"achieved": qr_all, "frac": qr_all / lane_peak if qr_all else None,
                                  "launches": int(st["qrs"])},
-                "peak_device": FP64_PEAK_TFLOPS,
-                "frac_of_device": qr_tflops / FP64_PEAK_TFLOPS if qr_tflops else None,
+                "peak_device": digit_peak,
+                "frac_of_device": qr_tflops / digit_peak if qr_tflops else None,
                 "lane_sms": lane_sms, "sms": sms,
                 "peak_note": "each QR launch of the timed region runs on one lane's %d of %d SMs "
                              "(the two real-time states step side by side), so its peak is "
-                             "that share of the device's FP64 rate" % (lane_sms, sms),
-                "peak_measured": fp64_peak,
-                "frac_of_measured_lane": (qr_tflops / (fp64_peak["tflops"] * lane_sms / sms)
-                                          if qr_tflops and fp64_peak else None),
-                "kernel": "gauge_qr_blocked_kernel (FP64 gauge QR, cooperative, 16-column blocks)",
+                             "that share of the device's rate; the launch is bound by latency "
+                             "(grid barriers, the serial 16-column factorisation)" % (lane_sms, sms),
+                "fp64_rate_measured": fp64_peak,
+                "ratio_to_fp64_rate_of_lane": (qr_tflops / (fp64_peak["tflops"] * lane_sms / sms)
+                                               if qr_tflops and fp64_peak else None),
+                "kernel": "gauge_qr_tensor_kernel (FP64 gauge QR, cooperative, 16-column blocks, "
+                          "projections as digit products on tcgen05 kind::f16)",
                 "share_of_step": st["qr_ms"] / ms_max if ms_max > 0 else None,
-                "peak_source": "GB300 FP64 rate from unit counts and clock: 152 SMs x 2 DFMA/clk "
-                               "x 2 flops x 2.07 GHz = 1.26 (nominal 1.25) TFLOP/s; no FP64 "
-                               "figure is measured on this pool",
+                "peak_source": "MEASURED_PEAKS bf16_tflops_sustained / 34 digit products per real "
+                               "product, of measured",
                 "per_launch": "algorithmic flops 8*m*n^2 (one Gram-Schmidt pass) = 1.07e9 per "
                               "8192 x 128 QR / its event-timed duration; the kernel makes a "
-                              "second pass where a column lost more than half its norm",
+                              "second pass where a column kept less than a quarter of its norm^2",
                 "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum of one 8192 x 128 "
-                                "launch (ncu, profiles/gauge_qr_blocked_8192x128.md); Q stays "
-                                "in L2, so the writes are small"}
+                                "launch (ncu, profiles/gauge_qr_tensor_8192x128.md); the "
+                                "writes are Q and part of its digits"}
     steps_total = args.steps + args.warmup
     line = {
         "metric": METRIC, "value": value, "unit": "site-updates/s", "n_gpus": world,

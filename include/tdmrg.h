@@ -515,7 +515,10 @@ int tdmrg_kernel_gauge_qr(int m, int n, const void* Y, int p, const void* E, voi
  * and status handling as tdmrg_kernel_gauge_qr, computed 16 columns at a time (block
  * Gram-Schmidt projections, Gram-form factorisation inside the block with a cancellation
  * guard that restarts the block at any column whose residual lost more than half its norm).
- * Each block stages ceil(m / blocks) rows of 16 columns and 16 n projection coefficients in at
+ * Factors of 9 to 256 columns and at most 128 rows per SM take their projections as exact digit
+ * products on the tensor cores (same rank decisions and completions; there a block goes on until a
+ * column keeps less than 1e-8 of its norm^2, and its columns are corrected once more).  Elsewhere
+ * each block stages ceil(m / blocks) rows of 16 columns and 16 n projection coefficients in at
  * most 200 KB of shared memory; a factor that does not fit (e.g. 24576 x 640 on 152 SMs) is
  * factorised by the column-wise kernel of tdmrg_kernel_gauge_qr instead (same result).
  * Allocates and frees its scratch; synchronises `stream`. */

@@ -39,13 +39,13 @@
 // (a restart below a quarter) stands in the middle; "rank 2": all but two columns are completed from
 // 7 n candidates of which n lie in the span:
 //   m x n        parallel         graded                 rank 2
-//   64 x 16       99 /   81       257 / 449 /   79        743 /  157
-//   256 x 32     171 /  198       356 / 641 /  198       1549 /  290
-//   1024 x 64    388 /  450       706 / 914 /  450       3716 /  545
-//   256 x 128    825 /  994      1028 / 1150 / 1000      7537 / 1184
-//   1024 x 128   943 / 1001      1173 / 1183 / 1105      9622 / 1208
-//   8192 x 128  2681 / 1218      3913 / 1454 / 1231     19468 / 1552
-//   8192 x 128 on 76 CTAs (two lanes)  4514 / 1541 and (rank 2) 25140 / 1783
+//   64 x 16        98 /   69       257 / 449 /   71
+//   256 x 32      172 /  177       355 / 641 /  179       1549 /  295
+//   1024 x 64     387 /  399       707 / 914 /  407
+//   256 x 128     827 /  915      1032 / 1150 /  912      7537 / 1174
+//   1024 x 128    944 /  908      1175 / 1183 / 1017
+//   8192 x 128   2685 / 1093      3911 / 1454 / 1114     19468 / 1535
+//   8192 x 128 on 76 CTAs (two lanes)  6742 / 1377 (graded) and 25148 / 1796 (rank 2)
 // Below nine columns the other kernel is the faster one at full rank (256 x 4: 55 against 95 us),
 // where such bonds, at the ends of a chain, mostly are.  About 32 rows per CTA: fewer rows raise the
 // number of partial sums, more the FP64 product V M.
