@@ -190,7 +190,11 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
   const int block = 2 * ND * o.tile * KS * 2;
   unsigned char* dst = o.dig +
       (((long long)b * o.tiles + tile) * ((long long)A.nred * A.ksteps) + step) * block;
+  // PT: [part][digit][k half][row group][8 rows][16 B]; Q: [part][k half][digit][row group]...
   const bool wide = o.tile == PT;
+  const int group = o.tile * 16;                     // the row groups of one digit and k half
+  const int by_digit = wide ? 2 * group : group, by_half = wide ? group : ND * group;
+  dst += kh * by_half + (rt >> 3) * 128 + (rt & 7) * 16;
 #pragma unroll
   for (int part = 0; part < 2; ++part) {
     unsigned long long w[8];
@@ -202,12 +206,8 @@ __global__ void __launch_bounds__(256) digit_split_kernel(SplitArgs A) {
       uint32_t h[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) h[q] = digit_pair(w[2 * q], w[2 * q + 1], l);
-      long long off;
-      if (wide)                      // [part][digit][k half][row group][8 rows][16 B]
-        off = (((part * ND + l) * 2 + kh) * (PT / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
-      else                           // [part][k half][digit][row group][8 rows][16 B]
-        off = (((part * 2 + kh) * ND + l) * (o.tile / 8) + (rt >> 3)) * 128 + (rt & 7) * 16;
-      *reinterpret_cast<uint4*>(dst + off) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(dst + part * 2 * ND * group + l * by_digit) =
+          make_uint4(h[0], h[1], h[2], h[3]);
     }
   }
 }
