@@ -11,8 +11,8 @@
 // Per Krylov vector j (CTA g owns the contiguous slice [g*S, g*S + S) of every vector):
 //  A.  T_w = L_w q_j for every channel w: complex FP32 FMA on 32 x 32 output tiles with the
 //      whole K = M extent staged in shared memory, all operands read as FP32 copies (L, R converted
-//      once, q_j by the CTA that owns the slice, scaled by a power of two and by the rest of 1/beta
-//      in FP64 after the channel sum) (M <= 256; the contraction is 2 Dw M^3
+//      once, q_j by the CTA that owns the slice once its norm is known, which costs a barrier)
+//      (M <= 256; the contraction is 2 Dw M^3
 //      complex MACs, too small to keep a tensor-core pipeline busy);
 //  B.  P_w = T_w R_w^T, one partial per channel (the channel sum is taken in C1, in order);
 //  C1. w = sum_w P_w in FP64 on the own slice; partial dots against q_{j-1}, q_j;
@@ -48,7 +48,7 @@ struct BondArgs {
   const cplx* v;       // [M][M]
   cplx* out;           // [M][M]
   cplx* V;             // kcap vectors of n
-  float2* W;           // n: the projected new vector in FP32, scaled by a power of two
+  float2* W;           // n: q_j in FP32
   float2* LR;          // [2][Dw][n]: L and R in FP32
   float2* T;           // [Dw][n]
   float2* P;           // [Dw][n]
@@ -130,10 +130,6 @@ __device__ __forceinline__ float2 to_f2(cplx z) {
   return make_float2(__double2float_rn(z.x), __double2float_rn(z.y));
 }
 
-// a power of two near the norm (from the norm^2), for a vector's FP32 copy
-__device__ __forceinline__ int scale_of(double nrm2) { return (bexp(nrm2) - 1023) >> 1; }
-__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
-
 __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
   extern __shared__ __align__(16) unsigned char dyn[];
   float2* at = reinterpret_cast<float2*>(dyn);        // [KT][TP]
@@ -178,17 +174,16 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
     return;
   }
   double inv = 1.0 / b0;
-  int kw = scale_of(s_nrm);
   for (int e = threadIdx.x; e < len; e += BT) {
-    A.V[e0 + e] = make_double2(ws[e].x * inv, ws[e].y * inv);
-    A.W[e0 + e] = to_f2(make_double2(ws[e].x * pow2(-kw), ws[e].y * pow2(-kw)));
+    const cplx q = make_double2(ws[e].x * inv, ws[e].y * inv);
+    A.V[e0 + e] = q;
+    A.W[e0 + e] = to_f2(q);     // read by every CTA
   }
   if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
-  double fac = inv * pow2(kw);  // q_j = W * fac (W is read by every CTA)
 
   int k = 0;
   for (int j = 0; j < A.kcap; ++j) {
-    // ---- A: T_w = L_w q_j / fac
+    // ---- A: T_w = L_w q_j
     for (int it = blockIdx.x; it < items; it += A.G) {
       const int w = it / (nt * nt), rem = it - w * nt * nt;
       const int ra = (rem / nt) * TL, cb = (rem % nt) * TL;
@@ -253,7 +248,7 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
         x += (double)p.x;
         y += (double)p.y;
       }
-      ws[e] = make_double2(x * fac, y * fac);
+      ws[e] = make_double2(x, y);
     }
     __syncthreads();
     const int lo = j > 0 ? j - 1 : 0;
@@ -264,7 +259,6 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
     // (the criterion of Daniel, Gragg, Kaufman and Stewart), the second one against q_0 .. q_j
     lzc::reduce_dots(part1, A.G, lo, j + 1, h1);
     lzc::reduce_norm(A.partn + A.G, A.G, &s_nrm);
-    kw = scale_of(s_nrm);         // of w before the projection: known in time for the last barrier
     lzc::slice_project(A.V, n, ws, e0, len, lo, j + 1, h1);
     if (threadIdx.x == 0) {
       double rem = s_nrm;
@@ -283,8 +277,6 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
       __syncthreads();
     }
     // ---- ||w||^2
-    for (int e = threadIdx.x; e < len; e += BT)
-      A.W[e0 + e] = to_f2(make_double2(ws[e].x * pow2(-kw), ws[e].y * pow2(-kw)));
     lzc::slice_norm(ws, len, red, A.partn);
     if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
     // ---- C4: tridiagonal bookkeeping and the small exponential (warp 0 of every CTA)
@@ -307,9 +299,12 @@ __global__ void __launch_bounds__(BT, 1) bond_exp_kernel(BondArgs A) {
     k = s_k;
     if (s_done) break;
     inv = s_inv;
-    fac = inv * pow2(kw);
-    for (int e = threadIdx.x; e < len; e += BT)
-      A.V[(size_t)(j + 1) * n + e0 + e] = make_double2(ws[e].x * inv, ws[e].y * inv);
+    for (int e = threadIdx.x; e < len; e += BT) {
+      const cplx q = make_double2(ws[e].x * inv, ws[e].y * inv);
+      A.V[(size_t)(j + 1) * n + e0 + e] = q;
+      A.W[e0 + e] = to_f2(q);
+    }
+    if (!lzc::barrier(A.bar, A.G, epoch, A.status, A.wait)) return;
   }
   // out = sum_{i < k} c_i q_i on the own slice
   for (int e = threadIdx.x; e < len; e += BT) {

@@ -21,6 +21,15 @@ constexpr long long NOSPLIT = 1LL << 60;
 // gauge-QR rank threshold of the mixed path (a larger threshold, at the 3xTF32 noise level,
 // changes neither C(t) nor log Z measurably but sends many columns through completion)
 constexpr double kMixedRankTol = 1e-12;
+// Largest hopping integral times step for which the mixed path takes the tensor-core gauge QR.  With
+// that threshold, columns that hold only contraction noise are kept, and their directions follow the
+// last bits of the QR; strong hopping carries that into C(t).  Measured as the relative change of
+// C(t = 0, dt) between the two QRs over 1500 truncated chains (rounding to complex64 is 1e-7; the FMA
+// QR alone, with eight rows per CTA instead of four, changes C(t) as much): up to 0.1 at most 5e-6, up
+// to 0.16 99 % below 3e-6 and one 1.3e-5, 2.5e-5 at 0.17, 3e-4 at 0.5.  Beyond the line the FMA QR
+// gives the same bits as ever; its price is 1.25 instead of 0.48 s for C(t) of the six-site two-mode
+// chain.
+constexpr double kTensorQrHopping = 0.1;
 const cplx ONE = {1.0, 0.0};
 const cplx ZERO = {0.0, 0.0};
 
@@ -876,9 +885,14 @@ void Engine::check_status() {
 void Engine::gauge_qr_dev(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* R, int* src) {
   const double t0 = tic();
   const bool timed = !capturing_;
-  CK(zg_reserve(qws_, gauge_qr_tensor_bytes(m, n, qr_.gmax), st_));
-  qr_.dig = static_cast<unsigned char*>(qws_.p);
-  qr_.dig_bytes = qws_.bytes;
+  if (fma_qr_) {
+    qr_.dig = nullptr;
+    qr_.dig_bytes = 0;
+  } else {
+    CK(zg_reserve(qws_, gauge_qr_tensor_bytes(m, n, qr_.gmax), st_));
+    qr_.dig = static_cast<unsigned char*>(qws_.p);
+    qr_.dig_bytes = qws_.bytes;
+  }
   if (timed) {
     if (qr_ev_n_ == QR_EV) harvest_qr_events();
     CK(cudaEventRecord(qr_ev_[2 * qr_ev_n_], st_));
@@ -1204,6 +1218,10 @@ void Engine::tdvp_step_body(DevMps& s, double tr, double ti, int half) {
   const double hr = 0.5 * tr, hi = 0.5 * ti;
   const bool imag = (ti == 0.0);
   const int L = s.L();
+  // (a bond mode modulates V by 1 + alpha (b + b^H))
+  const double hop = std::fabs(P.V) *
+                     (1.0 + (P.peierls ? 2.0 * std::fabs(P.alpha) * std::sqrt((double)P.nmax_p) : 0.0));
+  fma_qr_ = mixed() && !(hop * std::hypot(tr, ti) <= kTensorQrHopping);
   Ctx c = ctx();
   double t0;
   for (int k = 0; k < L && half != 2; ++k) {

@@ -357,6 +357,7 @@ class Engine {
   int lz_ev_n_ = 0;
   ZgWork zws_{};                         // FP64 contractions (digit products)
   ZgWork qws_{};                         // digits of the gauge QR
+  bool fma_qr_ = false;                  // this step's gauge QRs are taken in FP64 FMAs
   TcBufs tcb_{};
   BondScratch bs_{};
   unsigned long long* h_mv_ = nullptr;   // pinned copy of the device Krylov-vector counter

@@ -75,16 +75,18 @@ __device__ __forceinline__ void slice_dots(const cplx* V, long long n, const cpl
   }
 }
 
-// The same partial dots with every thread of the CTA on every vector (for large slices), and
-// with `norm` the slice's ||w||^2: the vectors are taken four at a time, each thread sums its
-// elements (stride blockDim), then warp v adds the threads' sums of value v in a fixed order (one
-// warp per value: a tree in every warp would cost each of them five FP64 additions per value).
-// red: 9 * blockDim doubles of shared memory.
+// The same partial dots with every thread of the CTA on every vector (for large slices), and with
+// `norm` the slice's ||w||^2: the vectors are taken four at a time, each thread sums its elements
+// (stride blockDim), the threads of a warp are added by a tree (lane offsets 16 .. 1), the warps in
+// order.  One warp forms the trees of one value for all warps, halving the values it holds at every
+// offset: 16 FP64 additions of a warp where a tree in every warp takes 80, with the same bits (the
+// order is part of the result: C(t) of a truncated chain on the mixed path follows the last bit).
+// red: 9 * blockDim doubles of shared memory; blockDim is 512.
 __device__ __forceinline__ void slice_dots_block(const cplx* V, long long n, const cplx* w,
                                                  long long e0, int len, int i0, int i1,
                                                  cplx* part, double* norm, double* red) {
-  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int T = blockDim.x;
+  constexpr int T = 512, nw = T / 32;
+  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
   for (int c0 = i0; c0 < i1; c0 += 4) {
     const int nv = min(4, i1 - c0);
     const bool nrm = norm && c0 == i0;
@@ -111,16 +113,42 @@ __device__ __forceinline__ void slice_dots_block(const cplx* V, long long n, con
       }
     if (nrm) red[8 * T + threadIdx.x] = sn;
     __syncthreads();
-    const int live = min(T, (len + 31) & ~31);      // threads that summed anything
+    const int live = min(T, len);                   // threads that summed anything (the rest: +0)
     for (int v = wv; v < 9; v += nw) {
       if (v < 8 ? v >= 2 * nv : !nrm) continue;
-      double x = 0.0;
-      for (int u = lane; u < live; u += 32) x += red[v * T + u];
-      x = wsum(x);
-      if (lane == 0) {
-        if (v == 8) norm[blockIdx.x] = x;
-        else reinterpret_cast<double*>(part + (size_t)blockIdx.x * NV + c0 + (v >> 1))[v & 1] = x;
+      double* r = red + v * T;
+      // offset 16: lanes 0-15 take warp 2 i, lanes 16-31 warp 2 i + 1
+      double s[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const double* t = r + i * 64 + (lane & 16) * 2 + (lane & 15);
+        s[i] = i * 64 < live ? t[0] + t[16] : 0.0;
       }
+      // offsets 8, 4, 2: the lanes of either half keep one of two warps each and give the other away
+#pragma unroll
+      for (int h = 4; h > 0; h >>= 1) {
+        const int o = 2 * h;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+          const bool up = lane & o;
+          const double keep = up ? s[2 * i + 1] : s[2 * i], give = up ? s[2 * i] : s[2 * i + 1];
+          s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+      }
+      s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+      __syncwarp();
+      // the warp this lane ended with: bit 0 from lane bit 4, then bits 3, 2, 1
+      if (!(lane & 1))
+        r[((lane >> 4) & 1) + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1) * 4 + ((lane >> 1) & 1) * 8] = s[0];
+    }
+    __syncthreads();
+    if (threadIdx.x < 9 && (threadIdx.x < 8 ? (int)threadIdx.x < 2 * nv : nrm)) {
+      const int v = threadIdx.x;
+      double x = 0.0;
+#pragma unroll
+      for (int u = 0; u < nw; ++u) x += red[v * T + u];
+      if (v == 8) norm[blockIdx.x] = x;
+      else reinterpret_cast<double*>(part + (size_t)blockIdx.x * NV + c0 + (v >> 1))[v & 1] = x;
     }
     __syncthreads();
   }
@@ -201,13 +229,8 @@ __device__ __forceinline__ void tridiag_step(int j, double aj, double nrm2, doub
                                              double& inv) {
   const int lane = threadIdx.x & 31;
   const int kk = j + 1;
-  if (bexp(nrm2) > 0 && bexp(nrm2) < 0x7ff && nrm2 > 0.0) {
-    inv = rsqrt_series(nrm2);
-    nb = nrm2 * inv;
-  } else {
-    nb = sqrt(nrm2);
-    inv = 1.0 / nb;
-  }
+  nb = sqrt(nrm2);
+  inv = 1.0 / nb;
   const double a = lane < j ? alpha[lane] : (lane == j ? aj : 0.0);
   const double bl = (lane >= 1 && lane < kk) ? beta[lane] : 0.0;
   const double br = (lane + 1 < kk) ? beta[lane + 1] : 0.0;
