@@ -368,8 +368,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
     bool ok = true;
     for (int ch = cbeg; ch < cend; ++ch) {
       const int local = ch - cbeg;
-      const int ep = __ldg(pe + ch * pext);
-      const int eqv = __ldg(qe + ch * qext + (lane & (CW - 1)));      // column lane mod CW
+      // (not __ldg: the split that writes the scales ends after this kernel has started)
+      const int ep = __ldcg(pe + ch * pext);
+      const int eqv = __ldcg(qe + ch * qext + (lane & (CW - 1)));      // column lane mod CW
       ok = mbar_wait(acc_full, local & 1, fail, A.status, 3);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
