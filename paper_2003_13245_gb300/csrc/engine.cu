@@ -1214,14 +1214,19 @@ void Engine::renormalize(cplx* A, long long n) {
   CK(znormalize_log(n, A, scal_ + 2, scal_ + 3, st_));
 }
 
+// which gauge QR a step takes (kTensorQrHopping)
+void Engine::choose_qr(double step) {
+  // (a bond mode modulates V by 1 + alpha (b + b^H))
+  const double hop = std::fabs(P.V) *
+                     (1.0 + (P.peierls ? 2.0 * std::fabs(P.alpha) * std::sqrt((double)P.nmax_p) : 0.0));
+  fma_qr_ = mixed() && !(hop * step <= kTensorQrHopping);
+}
+
 void Engine::tdvp_step_body(DevMps& s, double tr, double ti, int half) {
   const double hr = 0.5 * tr, hi = 0.5 * ti;
   const bool imag = (ti == 0.0);
   const int L = s.L();
-  // (a bond mode modulates V by 1 + alpha (b + b^H))
-  const double hop = std::fabs(P.V) *
-                     (1.0 + (P.peierls ? 2.0 * std::fabs(P.alpha) * std::sqrt((double)P.nmax_p) : 0.0));
-  fma_qr_ = mixed() && !(hop * std::hypot(tr, ti) <= kTensorQrHopping);
+  choose_qr(std::hypot(tr, ti));
   Ctx c = ctx();
   double t0;
   for (int k = 0; k < L && half != 2; ++k) {
@@ -1418,6 +1423,7 @@ void Engine::thermal_prepare(double beta, double dtau, int M) {
   }
   cudaFree(d_ent);
   CK(cudaMemsetAsync(scal_ + 3, 0, sizeof(double), st_));
+  choose_qr(dtau);
   right_canonicalize(psi_b_);
   check_status();
   double n2 = norm2_dev(psi_b_.A[0], psi_b_.size(0));

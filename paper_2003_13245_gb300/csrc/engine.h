@@ -357,7 +357,8 @@ class Engine {
   int lz_ev_n_ = 0;
   ZgWork zws_{};                         // FP64 contractions (digit products)
   ZgWork qws_{};                         // digits of the gauge QR
-  bool fma_qr_ = false;                  // this step's gauge QRs are taken in FP64 FMAs
+  bool fma_qr_ = false;                  // the gauge QRs are taken in FP64 FMAs
+  void choose_qr(double step);           // sets it for a step of this length
   TcBufs tcb_{};
   BondScratch bs_{};
   unsigned long long* h_mv_ = nullptr;   // pinned copy of the device Krylov-vector counter
