@@ -65,8 +65,14 @@ constexpr int TILE = 128;                       // accepted vectors of one produ
 constexpr int MINN = 9;                         // fewer: qr_blocked.cu (one block, no projection)
 constexpr int GROUP = 2 * ND * 2 * 128;         // digits of 8 rows x 16 k: 3584 bytes
 constexpr int RING = 16 * GROUP;                // one k step of 128 rows: 57344 bytes
-constexpr int BSTEP = 2 * ND * 2 * 2 * 128;     // 16 columns x 16 k: 7168 bytes
-constexpr int BDIG = 8 * BSTEP;                 // 57344 bytes
+// digits of B (16 columns): four runs (part, k half) per k step, a block of zeros before each and one
+// behind the last.  Four level groups (16 x 4 instructions per k step) because they need no longer
+// lead: one group (7 x 4) would take 41 KB more shared memory than there is
+using Levels = Groups<4, 0x85310>;
+constexpr int RUN = (Levels::lead() + ND) * 256;   // one run: 2048 bytes
+constexpr int BSTEP = 4 * RUN;                  // 16 columns x 16 k: 8192 bytes
+constexpr int LEAD = Levels::lead() * 256;
+constexpr int BDIG = 8 * BSTEP + 256;           // 65792 bytes
 constexpr int PASSES = 4;                       // projections of a block, at most (and a second round)
 // smallest part of a norm^2 that may be left where the rest is taken off in the Gram matrix
 // (rounding of 2^-53 is then up to 1e-8 of what is left; the second round takes that out)
@@ -216,33 +222,12 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
     bulk_load(ring + st * RING + off, src + s * stride, bytes, &P.full[st]);
     ++issued;
   };
-  auto tile = [&](uint32_t a, uint32_t lbo, uint32_t sbo, uint32_t apart, uint32_t adig, uint32_t b,
-                  uint32_t d, bool first, bool cj) {
-    const uint64_t br = sdesc(b, ND * 256), bi = sdesc(b + BSTEP / 2, ND * 256);
-#pragma unroll
-    for (int i = 0; i < ND; ++i) {
-      const uint32_t n = QB * (NL - i < ND ? NL - i : ND);
-      const uint32_t acc = (!first || i > 0) ? 1u : 0u;
-      const bool cut = i == 1 && first;          // level 7 starts with digit pair (1, 6)
-      const uint32_t mm = cut ? n - QB : n;
-      const uint64_t ar = sdesc(a + i * adig, lbo, sbo), ai = sdesc(a + apart + i * adig, lbo, sbo);
-      const uint32_t dr = d + i * QB, di = d + IM + i * QB;
-      mma_f16(dr, ar, br, idesc(0, mm), acc);
-      mma_f16(di, ar, bi, idesc(0, mm), acc);
-      if (cut) {
-        mma_f16(dr + mm, ar, sdesc(b + (ND - 1) * 256, ND * 256), idesc(0, QB), 0u);
-        mma_f16(di + mm, ar, sdesc(b + BSTEP / 2 + (ND - 1) * 256, ND * 256), idesc(0, QB), 0u);
-      }
-      mma_f16(dr, ai, bi, idesc(cj ? 0 : 1, n), 1u);
-      mma_f16(di, ai, br, idesc(cj ? 1 : 0, n), 1u);
-    }
-  };
   for (int s = 0; s < S && s < 2; ++s) load(s);
-  const uint32_t b0 = smem_u32(bdig);
+  const uint32_t b0 = smem_u32(bdig) + LEAD;
   auto gram = [&] {
     for (int s = 0; s < gram_steps; ++s)
-      tile(b0 + s * BSTEP, ND * 256, 128, BSTEP / 2, 256, b0 + s * BSTEP, tmem + 2 * IM, s == 0,
-           true);
+      mma_levels<Levels, QB>(tmem + 2 * IM, IM, b0 + s * BSTEP, RUN, 128, 2 * RUN, 256,
+                             b0 + s * BSTEP, RUN, s == 0, true);
   };
   if (conj) gram();
   for (int s = 0; s < S; ++s) {
@@ -253,8 +238,8 @@ __device__ void qt_gemm(Pipe& P, uint32_t tmem, unsigned char* ring, int off,
       break;
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tile(smem_u32(ring + st * RING), 128, GROUP, GROUP / 2, 256, b0 + s * BSTEP, tmem, s == 0,
-         conj);
+    mma_levels<Levels, QB>(tmem, IM, smem_u32(ring + st * RING), 128, GROUP, GROUP / 2, 256,
+                           b0 + s * BSTEP, RUN, s == 0, conj);
     mma_commit(&P.empty[st]);
     if (s + 2 < S) {
       if (!mbar_wait(&P.empty[st], par, P.fail, P.status, 1)) {
@@ -316,7 +301,6 @@ struct Shared {
   int em[QB];                // largest biased exponent of a column (digit scale)
   int ev[QB];                // its digit scale E
   short idx[MAXN];           // column of Q of every accepted vector, in order of acceptance
-  cplx own[OWN];             // sums of a small reduction
   int ec[MAXN];              // form 1: scale of every accepted vector (this CTA's rows)
   int er[MAXR];              // form 2: scale of every row (E_EMPTY: nothing but zeros so far)
   int rnew[MAXR];            // largest biased exponent of a row's new entries
@@ -340,7 +324,10 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
   unsigned char* bdig = base + 2 * RING;                        // BDIG
   cplx* V = reinterpret_cast<cplx*>(bdig + BDIG);               // [QB][MAXR + 1]
   constexpr int LDV = MAXR + 1;
-  cplx* H = reinterpret_cast<cplx*>(ring + RING);               // [MAXN][QB], in stage 1
+  cplx* H = reinterpret_cast<cplx*>(ring + RING);               // [TILE][QB], in stage 1
+  // sums of a small reduction, behind it: read before the next product's copies are issued
+  cplx* own = H + TILE * QB;                                    // [OWN]
+  static_assert(sizeof(cplx) * (TILE * QB + OWN) <= RING, "stage 1");
   __shared__ Shared S;
 
   const int m = A.m, n = A.n;
@@ -374,6 +361,9 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
     for (int e = tid; e < n * n; e += QT_THREADS) A.R[e] = make_double2(0.0, 0.0);
   for (int i = tid; i < n; i += QT_THREADS) S.acc[i] = 0;
   for (int i = tid; i < MAXR; i += QT_THREADS) S.er[i] = E_EMPTY;
+  // the zeros around the runs of bdig (the digits are written over the rest)
+  for (int e = tid; e < BDIG / 16; e += QT_THREADS)
+    reinterpret_cast<uint4*>(bdig)[e] = make_uint4(0u, 0u, 0u, 0u);
   // ||Y||_F (summed over the CTAs with the first block's Gram matrix)
   {
     double s = 0.0;
@@ -459,8 +449,8 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
             const int u = k & 1, part = (k >> 1) & 1, q = k >> 2;
             const int t = 2 * warp + u, em = u ? e2[1] : e2[0];
             qt_store(V + t * LDV + q * 4, 1, min(4, nr - q * 4), part, max(em, 1), em == 0x7ff,
-                     bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
-                         t * 16 + (q & 1) * 8);
+                     bdig + LEAD + (q >> 2) * BSTEP + (2 * part + ((q >> 1) & 1)) * RUN + t * 16 +
+                         (q & 1) * 8);
           }
         }
         asm volatile("fence.proxy.async;" ::: "memory");
@@ -505,16 +495,16 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         if (!alive) break;
         cplx* fin = A.fin + (long long)pass * A.PS;
         const int cnt = na * QB + QB * QB + (started ? 0 : 1);
-        const cplx* sum = qt_reduce(A, cnt, part, fin, S.own, ep, &S.ok);
+        const cplx* sum = qt_reduce(A, cnt, part, fin, own, ep, &S.ok);
         if (!sum) {
           alive = false;
           break;
         }
         mypart += part == A.part ? pset : -pset;
         part = part == A.part ? A.part + pset : A.part;
-        if (sum == S.own) private_r = true;
+        if (sum == own) private_r = true;
         if (!refine) npass = pass + 1;
-        auto take_sum = [&](int e) { return sum == S.own ? S.own[e] : __ldcg(sum + e); };
+        auto take_sum = [&](int e) { return sum == own ? own[e] : __ldcg(sum + e); };
         if (!started) {
           started = true;
           const double y2 = take_sum(QB * QB).x;
@@ -620,8 +610,8 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
             for (int k = tid >> 4; k < 8 * isteps; k += 16) {     // part, group of 4 columns of Q
               const int part = k & 1, q = k >> 1;
               qt_store(H + q * 4 * QB + t, QB, min(4, ni - q * 4), part, em, bad,
-                       bdig + (q >> 2) * BSTEP + part * (BSTEP / 2) + ((q >> 1) & 1) * (ND * 256) +
-                           t * 16 + (q & 1) * 8);
+                       bdig + LEAD + (q >> 2) * BSTEP + (2 * part + ((q >> 1) & 1)) * RUN + t * 16 +
+                           (q & 1) * 8);
             }
           }
           asm volatile("fence.proxy.async;" ::: "memory");
@@ -694,14 +684,14 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
             q = wsum(q);
             if (lane == 0) mypart[t] = make_double2(q, 0.0);
           }
-          if (!qt_reduce(A, QB, part, nullptr, S.own, ep, &S.ok)) {
+          if (!qt_reduce(A, QB, part, nullptr, own, ep, &S.ok)) {
             alive = false;
             break;
           }
           mypart += part == A.part ? pset : -pset;
           part = part == A.part ? A.part + pset : A.part;
           if (tid < QB) {
-            const int drop = S.drop[tid] || !(S.own[tid].x > thr2);
+            const int drop = S.drop[tid] || !(own[tid].x > thr2);
             S.drop[tid] = drop;
             const unsigned dd = __ballot_sync(0xffffu, !drop);
             if (tid == 0) S.any = dd != 0;
@@ -802,7 +792,7 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
         // below 1e-12, in FP32)
         const int a = tid >> 4, b = tid & 15;
         const bool on = a <= b && b < S.done && S.take[a] > 0 && S.take[b] > 0;
-        float2* F = reinterpret_cast<float2*>(S.own);      // U to first order, U, then W
+        float2* F = reinterpret_cast<float2*>(own);      // U to first order, U, then W
         cplx g = make_double2(0.0, 0.0);
         if (on) {
           g = S.G[a][b];
@@ -842,7 +832,7 @@ __global__ void __launch_bounds__(QT_THREADS, 1) gauge_qr_tensor_kernel(QtArgs A
       // lanes the rows (MAXR / 32 rows each).  A second round that changes little: v_t - sum v_s W_st,
       // the sum in FP32
       if (small) {
-        const float2* W = reinterpret_cast<const float2*>(S.own) + 512;
+        const float2* W = reinterpret_cast<const float2*>(own) + 512;
         float2* F = reinterpret_cast<float2*>(ring);       // V, [QB][MAXR + 1]
         for (int e = tid; e < QB * nr; e += QT_THREADS) {
           const int t = e / nr, r = e - t * nr;

@@ -84,6 +84,51 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b,
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
       "l"(a), "l"(b), "r"(id), "r"(acc));
 }
+// Groups of levels: group g holds the levels lo(g) .. lo(g + 1) - 1 (PACK: four bits each).  The
+// order of tcgen05.mma instructions into TMEM columns they share is defined only where accumulator
+// and shape are the same, so every instruction of a group writes all of its columns: digit i of A
+// meets the digits lo(g) - i .. lo(g + 1) - 1 - i of B, and those outside 0 .. ND - 1 are blocks of
+// zeros in shared memory, LEAD of them before each run of ND digits (the one behind a run is the
+// next run's first).  Fewer, wider groups need fewer instructions (each reads the 4 KB of A again)
+// and a longer lead.
+template <int N, unsigned PACK>
+struct Groups {
+  static constexpr int n = N;
+  __host__ __device__ static constexpr int lo(int g) { return (int)(PACK >> (4 * g)) & 15; }
+  __host__ __device__ static constexpr int lead() {
+    int l = 1;
+    for (int g = 0; g < N; ++g) {
+      const int i = lo(g + 1) - 1 < ND - 1 ? lo(g + 1) - 1 : ND - 1;     // the last digit of A
+      if (i - lo(g) > l) l = i - lo(g);
+    }
+    return l;
+  }
+};
+// One 16-deep k step: d (re levels; im levels `im` columns further) += A B, QT columns per level.
+// A: digit 0 of re at `a` (im `apart`, the next digit `adig` bytes further).  B: digit 0 of re at
+// `b`, its runs of ND digits `pitch` bytes apart: re k half 0, re k half 1, im, im.
+// conj: conj(A) B (re = ArBr + AiBi, im = ArBi - AiBr).  first: the levels start from zero.
+template <class G, int QT>
+__device__ __forceinline__ void mma_levels(uint32_t d, uint32_t im, uint32_t a, uint32_t lbo,
+                                           uint32_t sbo, uint32_t apart, uint32_t adig, uint32_t b,
+                                           uint32_t pitch, bool first, bool conj) {
+#pragma unroll
+  for (int i = 0; i < ND; ++i) {
+    const uint64_t ar = sdesc(a + i * adig, lbo, sbo), ai = sdesc(a + apart + i * adig, lbo, sbo);
+    const uint32_t acc = (!first || i > 0) ? 1u : 0u;
+#pragma unroll
+    for (int g = 0; g < G::n; ++g) {
+      if (i >= G::lo(g + 1)) continue;
+      const int n = QT * (G::lo(g + 1) - G::lo(g));
+      const uint32_t w = b + (G::lo(g) - i) * (QT * 16), dr = d + G::lo(g) * QT, di = dr + im;
+      const uint64_t br = sdesc(w, pitch), bi = sdesc(w + 2 * pitch, pitch);
+      mma_f16(dr, ar, br, idesc(0, n), acc);
+      mma_f16(di, ar, bi, idesc(0, n), acc);
+      mma_f16(dr, ai, bi, idesc(conj ? 0 : 1, n), 1u);
+      mma_f16(di, ai, br, idesc(conj ? 1 : 0, n), 1u);
+    }
+  }
+}
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(

@@ -11,11 +11,12 @@
 // arithmetic.  Re and im parts share E.  The digits are stored as the shared-memory image of the
 // tile they will be staged in (8 x 16 byte core matrices), so a stage is one contiguous block.
 //
-// Product (digit_gemm_kernel): one CTA computes a 128 x 32 (or 128 x 16) tile of C.  For every digit
-// i of the 128-row operand one tcgen05.mma (kind::f16, FP32 accumulation) multiplies it with the
-// digits j = 0 .. min(6, 7 - i) of the 32-column operand at once (N = 32 per digit), because pair
-// (i, j) goes to the accumulator of level i + j and both the digits in shared memory and the
-// levels in TMEM are contiguous: 4 x 7 instructions per 16-deep k step.  A digit product is at
+// Product (digit_gemm_kernel): one CTA computes a 128 x 32 (or 128 x 16) tile of C.  Digit i of the
+// 128-row operand times digit j of the 32-column operand goes to the accumulator of level i + j <= 7.
+// Both the digits in shared memory and the levels in TMEM are contiguous, so one tcgen05.mma
+// (kind::f16, FP32 accumulation) takes a digit i with several j at once: a group of levels per
+// instruction (Groups in umma.cuh), 4 x 12 instructions per 16-deep k step with 32-column tiles,
+// 4 x 7 with 16-column ones, zeros in the place of digits a group does not have.  A digit product is at
 // most 2^14; over one chunk of 128 k a level of p pairs sums to at most p 2^22, an integer that
 // FP32 holds exactly.  After each chunk eight warps read the levels back and combine them in
 // 64-bit integers; the chunk's result is rounded once to FP64 and the chunks are added in FP64.
@@ -38,6 +39,7 @@
 #include "umma.cuh"
 
 #include <mutex>
+#include <type_traits>
 
 namespace tdmrg {
 
@@ -52,11 +54,20 @@ constexpr int KC = 128;                       // k per chunk (one scale per row 
 constexpr int STEPS = KC / KS;
 constexpr int P_BLOCK = 2 * ND * PT * KS * 2; // 57344 bytes per stage
 __host__ __device__ constexpr int q_block(int qt) { return 2 * ND * qt * KS * 2; }     // 14336, 7168
+// level groups (lead 2 and 6): 16-column tiles have all levels in one, the wider ones as many as
+// leave room for three stages
+template <int QT>
+using LevelsOf = std::conditional_t<QT == 16, Groups<1, 0x80>, Groups<3, 0x8410>>;
+template <int QT>
+__host__ __device__ constexpr int q_pitch() { return (LevelsOf<QT>::lead() + ND) * QT * 16; }    // between the runs of digits
+template <int QT>
+__host__ __device__ constexpr int q_stage() { return 4 * q_pitch<QT>() + QT * 16; }              // 18944, 13568
 constexpr int NST = 3;
 constexpr int GEMM_THREADS = 320;             // TMA warp, MMA warp, eight epilogue warps
 constexpr size_t gemm_smem(int qt) {
-  return (size_t)NST * (P_BLOCK + q_block(qt)) + 256 + 128;
+  return (size_t)NST * (P_BLOCK + (qt == 16 ? q_stage<16>() : q_stage<32>())) + 256 + 128;
 }
+static_assert(gemm_smem(16) <= 227 * 1024 && gemm_smem(32) <= 227 * 1024, "shared memory");
 
 struct Operand {
   const cplx* p;
@@ -235,7 +246,8 @@ struct GemmArgs {
 
 template <int QT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __grid_constant__ GemmArgs A) {
-  constexpr int Q_BLOCK = q_block(QT), STAGE = P_BLOCK + Q_BLOCK;
+  constexpr int PITCH = q_pitch<QT>(), LEAD = LevelsOf<QT>::lead() * QT * 16;
+  constexpr int Q_BLOCK = q_block(QT), STAGE = P_BLOCK + q_stage<QT>();
   constexpr int TMEM_COLS = 2 * NL * QT;
   constexpr int CW = QT / 2;                   // columns of an epilogue warp
   behind_next();
@@ -272,6 +284,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
                  "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  // the zeros around the runs of Q's digits (the copies write only the runs)
+  for (int e = threadIdx.x; e < NST * (q_stage<QT>() / 16); e += GEMM_THREADS)
+    *reinterpret_cast<uint4*>(smem + e / (q_stage<QT>() / 16) * STAGE + P_BLOCK +
+                              e % (q_stage<QT>() / 16) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  asm volatile("fence.proxy.async;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -302,9 +319,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
         }
         const long long step = (long long)red * A.ksteps + c * STEPS + k;
         unsigned char* st = smem + s * STAGE;
-        mbar_expect_tx(&full[s], STAGE);
+        mbar_expect_tx(&full[s], P_BLOCK + Q_BLOCK);
         bulk_load(st, P + step * P_BLOCK, P_BLOCK, &full[s]);
-        bulk_load(st + P_BLOCK, Q + step * Q_BLOCK, Q_BLOCK, &full[s]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          bulk_load(st + P_BLOCK + LEAD + u * PITCH, Q + step * Q_BLOCK + u * (Q_BLOCK / 4),
+                    Q_BLOCK / 4, &full[s]);
       }
     }
     *issued = t;
@@ -324,30 +344,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t p0 = smem_u32(smem + s * STAGE), q0 = p0 + P_BLOCK;
-        const uint64_t qr = sdesc(q0, ND * QT * 16), qi = sdesc(q0 + Q_BLOCK / 2, ND * QT * 16);
-#pragma unroll
-        for (int i = 0; i < ND; ++i) {
-          // digits j = 0 .. min(6, 7 - i) of Q: levels i .. i + j
-          const uint32_t n = QT * (NL - i < ND ? NL - i : ND);
-          // a chunk's first write of a level does not accumulate: digit 0 starts levels 0-6;
-          // level 7 starts with digit pair (1, 6), which is cut off the others of digit 1
-          const uint32_t acc = (k > 0 || i > 0) ? 1u : 0u;
-          const bool cut = i == 1 && k == 0;
-          const uint32_t m = cut ? n - QT : n;
-          const uint64_t pr = sdesc(p0 + i * (PT * KS * 2), PT * 16);
-          const uint64_t pi = sdesc(p0 + (ND + i) * (PT * KS * 2), PT * 16);
-          const uint32_t d_re = tmem + i * QT, d_im = tmem + NL * QT + i * QT;
-          mma_f16(d_re, pr, qr, idesc(0, m), acc);
-          mma_f16(d_im, pr, qi, idesc(0, m), acc);
-          if (cut) {
-            constexpr uint32_t last = (ND - 1) * QT * 16;       // digit 6 of Q
-            mma_f16(d_re + m, pr, sdesc(q0 + last, ND * QT * 16), idesc(0, QT), 0u);
-            mma_f16(d_im + m, pr, sdesc(q0 + Q_BLOCK / 2 + last, ND * QT * 16), idesc(0, QT), 0u);
-          }
-          mma_f16(d_re, pi, qi, idesc(1, n), 1u);
-          mma_f16(d_im, pi, qr, idesc(0, n), 1u);
-        }
+        const uint32_t p0 = smem_u32(smem + s * STAGE);
+        mma_levels<LevelsOf<QT>, QT>(tmem, NL * QT, p0, PT * 16, 128, ND * (PT * KS * 2),
+                                     PT * KS * 2, p0 + P_BLOCK + LEAD, PITCH, k == 0, false);
         mma_commit(&empty[s]);
       }
       if (live) mma_commit(acc_full);
