@@ -1369,9 +1369,11 @@ int tdmrg_kernel_qr_vjp(int m, int n, const void* Q, const void* R, const void* 
     // entries of Rbar below the diagonal are structural zeros of R
     CK(cudaMemcpyAsync(Ru, Rbar, sizeof(cplx) * (size_t)n * n, cudaMemcpyDeviceToDevice, s));
     CK(tdmrg::triu_inplace(n, Ru, s));
-    // M = R Rbar^H - Qbar^H Q
+    // M = R Rbar^H - Qbar^H Q.  The first product takes FP64 FMAs: a cotangent is large where R is
+    // small, and each term counts in the solve that follows, however small beside the largest
+    // entries of its row and column (digit products are accurate beside those)
     CK(tdmrg::zgemm(n, n, n, 1, 1, one, MatRef{(const cplx*)R, n, 1, 0, 0, 0},
-                    MatRef{Ru, 1, n, 0, 0, 1}, zero, M, n, 0, nullptr, s, &zg.w));
+                    MatRef{Ru, 1, n, 0, 0, 1}, zero, M, n, 0, nullptr, s));
     CK(tdmrg::zgemm(n, n, m, 1, 1, mone, MatRef{(const cplx*)Qbar, 1, n, 0, 0, 1},
                     MatRef{(const cplx*)Q, n, 1, 0, 0, 0}, one, M, n, 0, nullptr, s, &zg.w));
     CK(tdmrg::herm_lower(n, M, S, s));
@@ -1584,10 +1586,10 @@ int tdmrg_kernel_qr_vjp_completed(int m, int n, const int* accepted, const void*
     CK(tdmrg::triu_inplace(n, Rp, s));
     for (int j = 0; j < ns; ++j)
       CK(cudaMemcpy2DAsync(Rp + j, cb * n, RS + S[j], cb * n, cb, (size_t)ns, dd, s));
-    // Qbar_S += Y Rbar_S^H  (the R_S = Q_S^H Y term)
+    // Qbar_S += Y Rbar_S^H  (the R_S = Q_S^H Y term), in FP64 FMAs like M of tdmrg_kernel_qr_vjp
     if (ns > 0)
       CK(tdmrg::zgemm(m, ns, n, 1, 1, one, mat(Yr, n, 1), mat(RbS, 1, n, 0, 0, 1), one, Qbp, n, 0,
-                      nullptr, s, &zg.w));
+                      nullptr, s));
     // Zbar = full-rank QR VJP of Z = Qp R_Z with Rbar_Z = 0:
     //   M = -Qbp^H Qp, S = Hermitian fold of M, Zbar R_Z^H = Qbp + Qp S
     CK(tdmrg::zgemm(n, n, m, 1, 1, mone, mat(Qbp, 1, n, 0, 0, 1), mat(Qp, n, 1), zero, Mt, n, 0,
