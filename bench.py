@@ -28,7 +28,7 @@ sys.path.insert(0, ROOT)
 
 WORKLOAD = dict(name="holstein-N16-2mode-M128", N=16, omega=[0.2, 1.0], g=[1.5, 0.8],
                 nmax=[8, 4], V=0.5, kT=2.0, dtau=0.05, M=128, dt=0.05)
-# FP64 contractions (and the projections of the gauge QR) are taken as exact products of 8-bit
+# FP64 contractions (and the projections of the gauge QR) are taken as products of 8-bit
 # digits in fp16 on the tensor cores: 34 digit products per real product
 DIGIT_PRODUCTS = 34
 METRIC = "TDVP site-updates/s (real-time, both states, N=16 2-mode Holstein chain, M=128)"

@@ -333,6 +333,14 @@ const char* tdmrg_last_global_error(void);
  * the library for the length of the call; the pool keeps at most 512 MB between calls and gives
  * it back when the last model is destroyed.  TDMRG_ERR_TIMEOUT if a bounded pipeline wait of a
  * contraction gave up.
+ *
+ * Accuracy of a complex FP64 contraction C = A B: each operand is rounded to 56 bits below the
+ * largest component of its row of A (column of B) among 128 consecutive k, and the products are
+ * summed in integers, rounded once per 128 k.  The error of an entry is thus about
+ * 2^-56 (max|a| sum|b| + max|b| sum|a|) and one rounding: FP64 accuracy relative to the largest
+ * entries of the row and the column.  It is not relative to sum |a||b|: where a row of A falls along
+ * k while the column of B rises, the small terms lose digits.  Single-term contractions, and in the
+ * QR reverse passes the products of R (or Y) with the cotangent of R, use FP64 FMAs.
  * ---------------------------------------------------------------------------------- */
 
 /* Effective Hamiltonian of one site (the site step of Eq. S1):
@@ -515,7 +523,7 @@ int tdmrg_kernel_gauge_qr(int m, int n, const void* Y, int p, const void* E, voi
  * and status handling as tdmrg_kernel_gauge_qr, computed 16 columns at a time (block
  * Gram-Schmidt projections, Gram-form factorisation inside the block with a cancellation
  * guard that restarts the block at any column whose residual lost more than half its norm).
- * Factors of 9 to 256 columns and at most 128 rows per SM take their projections as exact digit
+ * Factors of 9 to 256 columns and at most 128 rows per SM take their projections as digit
  * products on the tensor cores (same rank decisions and completions; there a block goes on until a
  * column keeps less than 1e-8 of its norm^2, and its columns are corrected once more).  Elsewhere
  * each block stages ceil(m / blocks) rows of 16 columns and 16 n projection coefficients in at

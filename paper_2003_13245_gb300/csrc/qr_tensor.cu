@@ -1,6 +1,6 @@
 // Gauge QR with its projections on the tensor cores: the factorisation, skipping and completion of
 // qr_blocked.cu (blocked Gram-Schmidt of 16 columns at a time, deterministic completion) in one
-// cooperative launch, with Q^H V, V^H V and Q P taken as exact digit products (the scheme of
+// cooperative launch, with Q^H V, V^H V and Q P taken as digit products (the scheme of
 // zgemm_digits.cu) instead of FP64 FMAs.
 //
 // CTA g owns a slice of at most 128 rows of Y, Q and the working block V (shared memory, FP64).

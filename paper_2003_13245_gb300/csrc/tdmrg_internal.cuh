@@ -81,7 +81,8 @@ void zg_pool_trim();
 
 // C_b = alpha * sum_{r < nred} op(A_{b,r}) op(B_{b,r}) + beta * C_b, b < nbatch.
 // C row-major with leading dimension ldc and batch stride sc.  With a workspace the product is
-// taken on the tensor cores in exact digit products (zgemm_digits.cu), otherwise (and for the
+// taken on the tensor cores in digit products (zgemm_digits.cu, which states the error: relative to
+// the largest entries of a row and a column, not to the sum of |a||b|), otherwise (and for the
 // shapes where that is not faster) by FP64 FMAs.
 cudaError_t zgemm(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef A, MatRef B,
                   cplx beta, cplx* C, long long ldc, long long sc, const int* skip,

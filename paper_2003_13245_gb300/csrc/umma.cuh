@@ -168,8 +168,8 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned lo
   return d;
 }
 
-// One accumulated product sum from its eight level sums (FP32 bits holding integers below 2^24;
-// level l counts units of 2^(E_A + E_B - 14 - 8 l)), rounded to nearest.  General form, with the
+// One accumulated product sum from its eight level sums (FP32 bits holding integers below 2^25, even
+// above 2^24; level l counts units of 2^(E_A + E_B - 14 - 8 l)), rounded to nearest.  General form, with the
 // library's scaling where the result leaves the normal range.
 static __device__ __noinline__ double from_levels_any(const uint32_t* v, int eA, int eB) {
   if (eA == E_NONFINITE || eB == E_NONFINITE) return __longlong_as_double(0x7ff8000000000000LL);

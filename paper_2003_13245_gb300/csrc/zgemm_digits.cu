@@ -1,6 +1,6 @@
-// Complex FP64 GEMM on the tensor cores: both operands are written as sums of 8-bit digits and
-// the digit products are summed exactly (the splitting of Ozaki, Ogita, Oishi and Rump,
-// "Error-free transformations of matrix multiplication", with a truncated product sum).
+// Complex FP64 GEMM on the tensor cores: both operands are rounded to sums of 8-bit digits, whose
+// products are summed in integers (the splitting of Ozaki, Ogita, Oishi and Rump, "Error-free
+// transformations of matrix multiplication", with a truncated product sum).
 //
 // Why: GB300 issues about 2 FP64 FMAs per clock per SM, so a 64 x 64 x 64 complex tile of
 // zgemm_kernel holds an SM for ~0.27 ms; its tensor cores take 4096 fp16 multiply-adds per clock.
@@ -17,13 +17,24 @@
 // (kind::f16, FP32 accumulation) takes a digit i with several j at once: a group of levels per
 // instruction (Groups in umma.cuh), 4 x 12 instructions per 16-deep k step with 32-column tiles,
 // 4 x 7 with 16-column ones, zeros in the place of digits a group does not have.  A digit product is at
-// most 2^14; over one chunk of 128 k a level of p pairs sums to at most p 2^22, an integer that
-// FP32 holds exactly.  After each chunk eight warps read the levels back and combine them in
+// most 2^14; over one chunk of 128 k a level of p pairs sums to an integer of at most p 2^22, exact
+// in FP32 up to 2^24.  After each chunk eight warps read the levels back and combine them in
 // 64-bit integers; the chunk's result is rounded once to FP64 and the chunks are added in FP64.
 //
-// Error: the operands carry 56 bits below the chunk's largest entry and the dropped pairs
-// (i + j > 7) are below 2^-62 of it, so an entry is off by about 2^-56 sqrt(K) max|a| max|b| and
-// one rounding; the FMA kernel rounds every partial sum.
+// Error of a component, per chunk with 2^EA and 2^EB the powers of two above the largest components
+// of the row of A and the column of B (|a|_1 = |re| + |im|):
+//   operands   sum_k 2^(EA-56) |b|_1 + 2^(EB-56) |a|_1    (entries above 1/8 of 2^E are exact)
+//   pairs i + j > 7    2^-60 2^(EA+EB) per k
+//   rounding   2^-53 of the chunk's sum, and of the partial sums over the chunks.
+// Levels 4 to 7 (five to seven pairs) pass 2^24 only where nearly all digits are near 127 and the
+// products of one sign; a chunk can then lose 2^-39 2^(EA+EB), which for such entries is 2^-45 of the
+// sum of |a||b| (operands built for it: 2^-55, the rounding of the result).
+// So the error is relative to the largest entries of a row and a column, that of FMAs to the sum of
+// |a||b|.  The same or less where rows of A and columns of B are even or fall together along k, as in
+// a sweep; where one rises as the other falls, by e^s in all, digits lose up to e^s: relative to the
+// sum of |a||b|, K = 128, 2e-14 at e^9, 1e-10 at e^18, 2e-6 at e^28 against 2e-16 (falling together
+// by e^28: 7e-17 against 1e-15).  Products whose operands are so by their nature, as R and its
+// cotangent, take the FMA kernel (capi.cu, QR reverse passes).
 //
 // Bound: the tensor pipe in the main loop (28 instructions, ~2300 clocks per k step of 128 x 32),
 // plus the integer epilogue, which cannot overlap it (eight re and im levels of 32 columns fill all
