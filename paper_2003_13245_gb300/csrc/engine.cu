@@ -574,9 +574,9 @@ void Engine::ensure_workspace(long long maxsite, long long maxxy, int maxbond, i
       if (*b) cudaFree(*b);
       *b = nullptr;
     }
-    CK(cudaMalloc(&V_, sizeof(cplx) * (size_t)(KMAX + 1) * maxsite));
-    CK(cudaMalloc(&Kout_, sizeof(cplx) * (size_t)maxsite));
-    CK(cudaMalloc(&T1_, sizeof(cplx) * (size_t)maxsite));
+    dev_alloc(&V_, sizeof(cplx) * (size_t)(KMAX + 1) * maxsite);
+    dev_alloc(&Kout_, sizeof(cplx) * (size_t)maxsite);
+    dev_alloc(&T1_, sizeof(cplx) * (size_t)maxsite);
     ws_site_ = maxsite;
   }
   if (maxxy > ws_xy_) {
@@ -584,8 +584,8 @@ void Engine::ensure_workspace(long long maxsite, long long maxxy, int maxbond, i
       if (*b) cudaFree(*b);
       *b = nullptr;
     }
-    CK(cudaMalloc(&X_, sizeof(cplx) * (size_t)maxxy));
-    CK(cudaMalloc(&Y_, sizeof(cplx) * (size_t)maxxy));
+    dev_alloc(&X_, sizeof(cplx) * (size_t)maxxy);
+    dev_alloc(&Y_, sizeof(cplx) * (size_t)maxxy);
     ws_xy_ = maxxy;
   }
   if (maxbond > ws_bond_) {
@@ -593,8 +593,8 @@ void Engine::ensure_workspace(long long maxsite, long long maxxy, int maxbond, i
       if (*b) cudaFree(*b);
       *b = nullptr;
     }
-    CK(cudaMalloc(&Cb_, sizeof(cplx) * (size_t)maxbond * maxbond));
-    CK(cudaMalloc(&Rb_, sizeof(cplx) * (size_t)maxbond * maxbond));
+    dev_alloc(&Cb_, sizeof(cplx) * (size_t)maxbond * maxbond);
+    dev_alloc(&Rb_, sizeof(cplx) * (size_t)maxbond * maxbond);
     ws_bond_ = maxbond;
   }
   ensure_bond_scratch(maxbond);
@@ -607,14 +607,14 @@ void Engine::ensure_workspace(long long maxsite, long long maxxy, int maxbond, i
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     qr_.gmax = sms;
     qr_.nmax = maxm;
-    CK(cudaMalloc(&qr_.part, sizeof(cplx) * 2 * (size_t)sms * (maxm + 1)));
-    CK(cudaMalloc(&qr_.partn, sizeof(double) * 2 * (size_t)sms));
-    CK(cudaMalloc(&qr_.bar, sizeof(unsigned) * 2));
+    dev_alloc(&qr_.part, sizeof(cplx) * 2 * (size_t)sms * (maxm + 1));
+    dev_alloc(&qr_.partn, sizeof(double) * 2 * (size_t)sms);
+    dev_alloc(&qr_.bar, sizeof(unsigned) * 2);
     if (qb_scratch_) cudaFree(qb_scratch_);
     if (qb_acc_) cudaFree(qb_acc_);
     qb_len_ = gauge_qr_blocked_scratch(maxm, sms);
-    CK(cudaMalloc(&qb_scratch_, sizeof(cplx) * (size_t)qb_len_));
-    CK(cudaMalloc(&qb_acc_, (size_t)maxm + 16));
+    dev_alloc(&qb_scratch_, sizeof(cplx) * (size_t)qb_len_);
+    dev_alloc(&qb_acc_, (size_t)maxm + 16);
     ws_m_ = maxm;
   }
 }
@@ -637,9 +637,9 @@ void Engine::alloc_mps(DevMps& s, int M) {
   for (int k = 0; k < L; ++k) {
     s.d[k] = sites_[k].d;
     s.D[k] = sites_[k].d * sites_[k].d;
-    CK(cudaMalloc(&s.A[k], sizeof(cplx) * (size_t)s.size(k)));
-    CK(cudaMalloc(&s.Lenv[k], sizeof(cplx) * (size_t)env_size(s, k, H_.s[k].Dl, true)));
-    CK(cudaMalloc(&s.Renv[k], sizeof(cplx) * (size_t)env_size(s, k, H_.s[k].Dr, false)));
+    dev_alloc(&s.A[k], sizeof(cplx) * (size_t)s.size(k));
+    dev_alloc(&s.Lenv[k], sizeof(cplx) * (size_t)env_size(s, k, H_.s[k].Dl, true));
+    dev_alloc(&s.Renv[k], sizeof(cplx) * (size_t)env_size(s, k, H_.s[k].Dr, false));
   }
   long long maxsite = 1, maxxy = 1, maxenv = 1;
   int maxbond = 1;
@@ -658,14 +658,36 @@ void Engine::alloc_mps(DevMps& s, int M) {
   if (maxenv > env_tmp_size_) {
     for (int i = 0; i < 2; ++i) {
       if (env_tmp_[i]) cudaFree(env_tmp_[i]);
-      CK(cudaMalloc(&env_tmp_[i], sizeof(cplx) * (size_t)maxenv));
+      dev_alloc(&env_tmp_[i], sizeof(cplx) * (size_t)maxenv);
     }
     env_tmp_size_ = maxenv;
   }
 }
 
+// The digit workspaces, and what the library's pool holds for later calls, are the only memory that an
+// engine can do without: they make room for everything else.
+void Engine::dev_alloc_bytes(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    zg_pool_trim();
+    if (!zws_.fixed) {
+      zg_free(zws_, st_);
+      zg_free(qws_, st_);
+    }
+    e = cudaMalloc(p, bytes);
+  }
+  CK(e);
+}
+
+void Engine::reserve(ZgWork& w, size_t bytes) {
+  const cudaError_t e = zg_reserve(w, bytes, st_);
+  if (e != cudaErrorMemoryAllocation) CK(e);
+}
+
 // The digit workspaces of the largest contraction and gauge QR of a sweep, so that they do not
-// grow between captured steps (graph mode holds their addresses).
+// grow between captured steps (graph mode holds their addresses).  Where there is no memory for them,
+// the contractions run in slabs or in FP64 FMAs and the gauge QR in FMAs.
 void Engine::alloc_zg(const DevMps& s) {
   size_t need = 0;
   const int Dm = std::max(H_.maxD, J_.maxD);
@@ -684,8 +706,8 @@ void Engine::alloc_zg(const DevMps& s) {
     qneed = std::max(qneed, gauge_qr_tensor_bytes(D * Mr, Ml, qr_.gmax));
   }
   zws_.fixed = qws_.fixed = false;
-  if (!mixed()) CK(zg_reserve(zws_, need, st_));
-  CK(zg_reserve(qws_, qneed, st_));
+  if (!mixed()) reserve(zws_, need);
+  reserve(qws_, qneed);
   zws_.fixed = qws_.fixed = graphs_;
 }
 
@@ -706,15 +728,15 @@ void Engine::alloc_tc(const DevMps& s) {
       if (*p) cudaFree(*p);
       *p = nullptr;
     }
-    CK(cudaMalloc(&tcb_.envA, sizeof(float) * 4 * env));
-    CK(cudaMalloc(&tcb_.envB, sizeof(float) * 4 * env));
-    CK(cudaMalloc(&tcb_.siteA, sizeof(float) * 4 * site));
-    CK(cudaMalloc(&tcb_.siteB, sizeof(float) * 4 * site));
-    CK(cudaMalloc(&tcb_.x32, sizeof(float) * 2 * x));
-    CK(cudaMalloc(&tcb_.mix, sizeof(float) * 4 * (long long)Dmax * site));
+    dev_alloc(&tcb_.envA, sizeof(float) * 4 * env);
+    dev_alloc(&tcb_.envB, sizeof(float) * 4 * env);
+    dev_alloc(&tcb_.siteA, sizeof(float) * 4 * site);
+    dev_alloc(&tcb_.siteB, sizeof(float) * 4 * site);
+    dev_alloc(&tcb_.x32, sizeof(float) * 2 * x);
+    dev_alloc(&tcb_.mix, sizeof(float) * 4 * (long long)Dmax * site);
     if (!tcb_.kpart) {
       tcb_.kpart_len = 4LL << 20;
-      CK(cudaMalloc(&tcb_.kpart, sizeof(float) * tcb_.kpart_len));
+      dev_alloc(&tcb_.kpart, sizeof(float) * tcb_.kpart_len);
     }
     tc_site_ = site;
     tc_env_ = env;
@@ -763,9 +785,9 @@ void Engine::copy_mps(const DevMps& src, DevMps& dst) {
     dst.Lenv.assign(L, nullptr);
     dst.Renv.assign(L, nullptr);
     for (int k = 0; k < L; ++k) {
-      CK(cudaMalloc(&dst.A[k], sizeof(cplx) * (size_t)src.size(k)));
-      CK(cudaMalloc(&dst.Lenv[k], sizeof(cplx) * (size_t)env_size(src, k, H_.s[k].Dl, true)));
-      CK(cudaMalloc(&dst.Renv[k], sizeof(cplx) * (size_t)env_size(src, k, H_.s[k].Dr, false)));
+      dev_alloc(&dst.A[k], sizeof(cplx) * (size_t)src.size(k));
+      dev_alloc(&dst.Lenv[k], sizeof(cplx) * (size_t)env_size(src, k, H_.s[k].Dl, true));
+      dev_alloc(&dst.Renv[k], sizeof(cplx) * (size_t)env_size(src, k, H_.s[k].Dr, false));
     }
   }
   for (int k = 0; k < src.L(); ++k)
@@ -818,19 +840,19 @@ void Engine::ensure_bond_scratch(int maxbond) {
     if (p) cudaFree(p);
   bs_.W = nullptr;
   bs_.T = bs_.P = bs_.LR = nullptr;
-  CK(cudaMalloc(&bs_.W, sizeof(cplx) * (size_t)maxn));
-  CK(cudaMalloc(&bs_.T, sizeof(float2) * (size_t)maxDw * maxn));
-  CK(cudaMalloc(&bs_.P, sizeof(float2) * (size_t)maxDw * maxn));
-  CK(cudaMalloc(&bs_.LR, sizeof(float2) * 2 * (size_t)maxDw * maxn));
+  dev_alloc(&bs_.W, sizeof(cplx) * (size_t)maxn);
+  dev_alloc(&bs_.T, sizeof(float2) * (size_t)maxDw * maxn);
+  dev_alloc(&bs_.P, sizeof(float2) * (size_t)maxDw * maxn);
+  dev_alloc(&bs_.LR, sizeof(float2) * 2 * (size_t)maxDw * maxn);
   if (!bs_.part) {
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     bs_.gmax = sms;
-    CK(cudaMalloc(&bs_.part, sizeof(cplx) * 2 * (size_t)sms * (KMAX + 1)));
-    CK(cudaMalloc(&bs_.partn, sizeof(double) * 2 * (size_t)sms));   // 2 * gmax: lz_step
-    CK(cudaMalloc(&bs_.bar, sizeof(unsigned) * 2));
-    CK(cudaMalloc(&bs_.mv, sizeof(unsigned long long)));
+    dev_alloc(&bs_.part, sizeof(cplx) * 2 * (size_t)sms * (KMAX + 1));
+    dev_alloc(&bs_.partn, sizeof(double) * 2 * (size_t)sms);   // 2 * gmax: lz_step
+    dev_alloc(&bs_.bar, sizeof(unsigned) * 2);
+    dev_alloc(&bs_.mv, sizeof(unsigned long long));
     CK(cudaMemset(bs_.mv, 0, sizeof(unsigned long long)));
     CK(cudaMallocHost(&h_mv_, sizeof(unsigned long long)));
     mv_seen_ = 0;
@@ -889,7 +911,7 @@ void Engine::gauge_qr_dev(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx* 
     qr_.dig = nullptr;
     qr_.dig_bytes = 0;
   } else {
-    CK(zg_reserve(qws_, gauge_qr_tensor_bytes(m, n, qr_.gmax), st_));
+    reserve(qws_, gauge_qr_tensor_bytes(m, n, qr_.gmax));
     qr_.dig = static_cast<unsigned char*>(qws_.p);
     qr_.dig_bytes = qws_.bytes;
   }
@@ -1335,8 +1357,8 @@ void Engine::fit_apply(const DevMpo& W, const DevMps& psi, DevMps& phi, int swee
     }
   } guard{Lf, Rf};
   for (int k = 0; k < L; ++k) {
-    CK(cudaMalloc(&Lf[k], sizeof(cplx) * (size_t)env_size(psi, k, W.s[k].Dl, true)));
-    CK(cudaMalloc(&Rf[k], sizeof(cplx) * (size_t)env_size(psi, k, W.s[k].Dr, false)));
+    dev_alloc(&Lf[k], sizeof(cplx) * (size_t)env_size(psi, k, W.s[k].Dl, true));
+    dev_alloc(&Rf[k], sizeof(cplx) * (size_t)env_size(psi, k, W.s[k].Dr, false));
   }
   set_ones(Lf[0]);
   set_ones(Rf[L - 1]);
@@ -1413,7 +1435,7 @@ void Engine::thermal_prepare(double beta, double dtau, int M) {
   int* d_ent = nullptr;
   size_t maxe = 0;
   for (auto& e : ent) maxe = std::max(maxe, e.size());
-  CK(cudaMalloc(&d_ent, sizeof(int) * std::max<size_t>(maxe, 1)));
+  dev_alloc(&d_ent, sizeof(int) * std::max<size_t>(maxe, 1));
   for (int k = 0; k < psi_b_.L(); ++k) {
     CK(cudaMemcpy(d_ent, ent[k].data(), sizeof(int) * ent[k].size(), cudaMemcpyHostToDevice));
     stats.h2d_bytes += sizeof(int) * ent[k].size();
@@ -1641,8 +1663,8 @@ void Engine::reduced_density(double* sigma) {
       if (t) cudaFree(t);
     }
   } guard{ops, buf, tr};
-  for (auto& p : buf) CK(cudaMalloc(&p, sizeof(cplx) * (size_t)maxe));
-  CK(cudaMalloc(&tr, sizeof(cplx) * (size_t)N * N));
+  for (auto& p : buf) dev_alloc(&p, sizeof(cplx) * (size_t)maxe);
+  dev_alloc(&tr, sizeof(cplx) * (size_t)N * N);
   CK(cudaMemsetAsync(tr, 0, sizeof(cplx) * (size_t)N * N, st_));
   // slot 0: E; slots 1 + 2p, 2 + 2p: c_p and c+_p inserted; two banks (current, next)
   int bank = 0;

@@ -202,6 +202,12 @@ class Engine {
   cudaStream_t stream() const { return st_; }
   cplx* X() { return X_; }
   ZgWork* zg() { return &zws_; }
+  // device memory; takes back the digit workspaces where there is no other
+  template <class T>
+  void dev_alloc(T** p, size_t bytes) {
+    dev_alloc_bytes(reinterpret_cast<void**>(p), bytes);
+  }
+  void dev_alloc_bytes(void** p, size_t bytes);
   cplx* Y() { return Y_; }
 
   // Lanczos exponential exp(tau M) v for a matvec callback (device pointers); returns the
@@ -278,6 +284,7 @@ class Engine {
                      const cplx* Renv, const cplx* bra, const cplx* ket, cplx* Rout);
   void alloc_tc(const DevMps& s);
   void alloc_zg(const DevMps& s);
+  void reserve(ZgWork& w, size_t bytes);   // what memory allows of it
   void absorb_left(const cplx* C, int M, cplx* A, long long ncols);
   void absorb_right(cplx* A, long long nrows, const cplx* C, int M);
   void set_ones(cplx* p);

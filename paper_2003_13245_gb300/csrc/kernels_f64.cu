@@ -140,8 +140,7 @@ cudaError_t zgemm_mixed(int m, int n, int k, int nbatch, int nred, MatRef A, Mat
     x.dmb = T.d * Mb;
     cudaError_t e = zg_reserve(*ws, zgemm_digits_bytes(m, n, k, nbatch, nred, A.sb == 0 ? 1 : nbatch,
                                                        B.sb == 0 ? 1 : nbatch), s);
-    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
-    else if (e != cudaSuccess) return e;
+    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return e;
     bool taken = false;
     if (ws->p) e = zgemm_digits(m, n, k, nbatch, nred, one, a, b, zero, C, ldc, sc, skip, *ws, s,
                                 &taken);
@@ -172,8 +171,8 @@ cudaError_t zgemm(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef 
     const size_t need = zgemm_digits_bytes(m, n, k, nbatch, nred, A.sb == 0 ? 1 : nbatch,
                                            B.sb == 0 ? 1 : nbatch);
     cudaError_t e = zg_reserve(*ws, need, s);
-    if (e == cudaErrorMemoryAllocation) cudaGetLastError();   // what there is may do in slabs
-    else if (e != cudaSuccess) return e;
+    // (out of memory: what there is may do in slabs)
+    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return e;
     bool taken = false;
     if (ws->p) e = zgemm_digits(m, n, k, nbatch, nred, alpha, A, B, beta, C, ldc, sc, skip, *ws,
                                 s, &taken);

@@ -54,16 +54,19 @@ QrRef qr(const cplx* p, long long rs, long long cs, long long cb, long long cbs,
 
 // device allocations of one call, freed on return
 struct Tape {
+  Engine& eng;
   std::vector<void*> p;
+  explicit Tape(Engine& e) : eng(e) {}
+  Tape(const Tape&) = delete;
   cplx* get(long long n) {
     void* q = nullptr;
-    CK(cudaMalloc(&q, sizeof(cplx) * (size_t)(n > 0 ? n : 1)));
+    eng.dev_alloc(&q, sizeof(cplx) * (size_t)(n > 0 ? n : 1));
     p.push_back(q);
     return (cplx*)q;
   }
   int* geti(long long n) {
     void* q = nullptr;
-    CK(cudaMalloc(&q, sizeof(int) * (size_t)(n > 0 ? n : 1)));
+    eng.dev_alloc(&q, sizeof(int) * (size_t)(n > 0 ? n : 1));
     p.push_back(q);
     return (int*)q;
   }
@@ -294,7 +297,7 @@ void Engine::exp_vjp_nodes(long long n, const cplx* v, const cplx* ybar, double 
     zb[q] = sq[q] * Cx(tr, ti);
     za[q] = (1.0 - sq[q]) * Cx(tr, -ti);
   }
-  Tape tp;
+  Tape tp(*this);
   if (k1 > 0 && b1 > 0.0) {
     tridiag_exp_e1(k1, a1.data(), e1.data(), nodes, zb.data(), cb.data());
     std::vector<cplx> h((size_t)nodes * k1);
@@ -364,7 +367,7 @@ void Engine::step_vjp(int M, const cplx* const* A_in, double tr, double ti,
     CK(cudaMemcpyAsync(dst, src, sizeof(cplx) * (size_t)cnt, d2d, st_));
   };
   Ctx c = ctx();
-  Tape tp;
+  Tape tp(*this);
 
   // ---- forward with the tape ----
   std::vector<cplx*> A(L), Lenv(L), Rin(L), Rnew(L);
@@ -859,7 +862,7 @@ void Engine::overlap_vjp(const std::vector<cplx*>& bra, const std::vector<cplx*>
     maxsite = std::max(maxsite, n[k]);
   }
   ne[L] = 1;
-  Tape tp;
+  Tape tp(*this);
   std::vector<cplx*> e(L + 1);
   for (int k = 0; k <= L; ++k) e[k] = tp.get(ne[k]);
   Ctx c = ctx();
@@ -921,7 +924,7 @@ void Engine::correlation_states_vjp(int M, const cplx* const* psi1, const cplx* 
   const std::vector<int>& Mb = s1.Mb;
   std::vector<long long> n(L);
   for (int k = 0; k < L; ++k) n[k] = s1.size(k);
-  Tape tp;
+  Tape tp(*this);
   auto snapshot = [&](const DevMps& s) {
     std::vector<cplx*> out(L);
     for (int k = 0; k < L; ++k) {
@@ -982,7 +985,7 @@ void Engine::correlation_states_vjp(int M, const cplx* const* psi1, const cplx* 
     const int e0 = (i + 1 < (int)ck.size()) ? ck[i + 1].n : nsteps;
     if (e0 <= s0) continue;
     std::vector<std::vector<cplx*>> st1{ck[i].a}, st2{ck[i].b};
-    Tape seg;
+    Tape seg(*this);
     load(s1, ck[i].a);
     load(s2, ck[i].b);
     for (int t = s0 + 1; t <= e0; ++t) {
@@ -1073,7 +1076,7 @@ void Engine::canonicalize_vjp(int M, cplx* const* psi0, const cplx* const* gbar,
     CK(cudaMemcpyAsync(dst, src, sizeof(cplx) * (size_t)cnt, cudaMemcpyDeviceToDevice, st_));
   };
   Ctx c = ctx();
-  Tape tp;
+  Tape tp(*this);
   std::vector<cplx*> A(L), Renv(L), ain(L), Q2(L), R2(L), Qs(L), Cm(L), nxt(L);
   std::vector<std::vector<unsigned char>> acc(L);
   std::vector<std::vector<int>> src(L);
@@ -1221,7 +1224,7 @@ void Engine::fit_vjp(int M, const cplx* const* psi, cplx* const* phi, const cplx
     nRj[k] = (long long)J_.s[k].Dr * z.Mb[k + 1] * z.Mb[k + 1];
   }
   Ctx c = ctx();
-  Tape tp;
+  Tape tp(*this);
   int* src_dev = tp.geti(z.maxbond);
   auto flags = [&](int cols, std::vector<unsigned char>& acc, std::vector<int>& src) {
     acc.resize(cols);
@@ -1429,7 +1432,7 @@ void Engine::correlation_vjp(double beta, double dtau, int M, double dt, int nst
   const int L = (int)sites_.size();
   const int np = parameter_count(P);
   const Dims z = make_dims(sites_, M, std::max(H_.maxD, J_.maxD));
-  Tape tp;
+  Tape tp(*this);
   auto state = [&]() {
     std::vector<cplx*> a(L);
     for (int k = 0; k < L; ++k) a[k] = tp.get(z.n[k]);

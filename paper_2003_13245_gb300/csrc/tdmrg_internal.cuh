@@ -71,7 +71,8 @@ struct ZgWork {
   bool fixed = false, pooled = false;
 };
 constexpr size_t kZgMaxBytes = (size_t)2 << 30;
-// grows w to at least min(bytes, kZgMaxBytes) (contents lost); leaves it as it is when fixed
+// grows w to at least min(bytes, kZgMaxBytes) (contents lost); leaves it as it is when fixed.  Where
+// memory runs out it keeps what it had, and the error is cudaErrorMemoryAllocation (cleared)
 cudaError_t zg_reserve(ZgWork& w, size_t bytes, cudaStream_t s);
 void zg_free(ZgWork& w, cudaStream_t s);
 // a block of the library's stream-ordered pool (cudaFreeAsync gives it back)

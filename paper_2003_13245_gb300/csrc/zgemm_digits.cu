@@ -48,6 +48,7 @@
 // batches, 27 against 1049 us (32 with tiles of 32); 16 x 16 x 4 11 against 21 us (15).
 #include "mix.cuh"
 #include "umma.cuh"
+#include "workspace.h"
 
 #include <mutex>
 #include <type_traits>
@@ -737,14 +738,14 @@ cudaError_t zg_reserve(ZgWork& w, size_t bytes, cudaStream_t s) {
   if (bytes > kZgMaxBytes) bytes = kZgMaxBytes;
   if (w.fixed || bytes <= w.bytes) return cudaSuccess;
   bytes = up(bytes + bytes / 8);      // room to grow without a new allocation
-  zg_free(w, s);
-  const cudaError_t e = w.pooled ? zg_pool_alloc(&w.p, bytes, s) : cudaMalloc(&w.p, bytes);
-  if (e != cudaSuccess) {
-    w.p = nullptr;
-    return e;
-  }
-  w.bytes = bytes;
-  return cudaSuccess;
+  const bool pooled = w.pooled;
+  const cudaError_t e = grow_block<cudaError_t>(
+      w.p, w.bytes, bytes,
+      [&](void** q, size_t n) { return pooled ? zg_pool_alloc(q, n, s) : cudaMalloc(q, n); },
+      [&](void* q) { pooled ? cudaFreeAsync(q, s) : cudaFree(q); },
+      [](cudaError_t r) { return r == cudaErrorMemoryAllocation; });
+  if (e == cudaErrorMemoryAllocation) cudaGetLastError();      // the caller goes on with what there is
+  return e;
 }
 
 void zg_free(ZgWork& w, cudaStream_t s) {
