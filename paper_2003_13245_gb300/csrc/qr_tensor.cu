@@ -50,6 +50,7 @@
 // where such bonds, at the ends of a chain, mostly are.  About 32 rows per CTA: fewer rows raise the
 // number of partial sums, more the FP64 product V M.
 #include "umma.cuh"
+#include "workspace.h"
 
 namespace tdmrg {
 
@@ -1098,14 +1099,15 @@ cudaError_t gauge_qr_tensor(int m, int n, QrRef Y, int p, QrRef E, cplx* Q, cplx
   if (!W.dig || !qt_plan(m, n, cap, pl)) return cudaSuccess;
   const long long PS = (long long)n * QB + QB + QB * QB;
   if ((size_t)pl.G * pl.dig_cta > W.dig_bytes || (2 * (long long)pl.G + PASSES + 1) * PS > scratch_len) return cudaSuccess;
-  static bool attr = false;
-  cudaError_t e;
-  if (!attr) {
-    e = cudaFuncSetAttribute(gauge_qr_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)QT_SMEM);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice smem;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = smem.run(dev, cudaErrorInvalidDevice, [] {
+      return cudaFuncSetAttribute(gauge_qr_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)QT_SMEM);
+    });
+  if (e != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(W.bar, 0, 2 * sizeof(unsigned), s)) != cudaSuccess) return e;
   QtArgs a{};
   a.m = m; a.n = n; a.p = p;

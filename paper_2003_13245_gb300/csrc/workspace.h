@@ -1,7 +1,8 @@
 // Host bookkeeping without CUDA calls of its own (it compiles and is tested with a plain C++
-// compiler): the growth of a workspace where memory may run out.
+// compiler): the growth of a workspace where memory may run out, and work done once per device.
 #pragma once
 #include <cstddef>
+#include <mutex>
 
 namespace tdmrg {
 
@@ -39,5 +40,25 @@ Err grow_block(void*& p, std::size_t& bytes, std::size_t want, Get get, Put put,
   }
   return e;
 }
+
+// f() once for every device (its error is returned and tried again by the next call); safe with
+// several threads
+class OncePerDevice {
+ public:
+  template <class Err, class F>
+  Err run(int dev, Err bad_device, F f) {
+    if (dev < 0 || dev >= kDevices) return bad_device;
+    std::lock_guard<std::mutex> lock(mu_);
+    if (done_[dev]) return Err(0);
+    const Err e = f();
+    done_[dev] = e == Err(0);
+    return e;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::mutex mu_;
+  bool done_[kDevices] = {};
+};
 
 }  // namespace tdmrg

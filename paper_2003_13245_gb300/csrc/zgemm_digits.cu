@@ -531,17 +531,19 @@ cudaError_t zgemm_digits(int m, int n, int k, int nbatch, int nred, cplx alpha, 
                          cplx beta, cplx* C, long long ldc, long long sc, const int* skip,
                          const ZgWork& ws, cudaStream_t s, bool* taken) {
   *taken = false;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(digit_gemm_kernel<32>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)gemm_smem(32));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(digit_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)gemm_smem(16));
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice smem;
+  int dev = 0;
+  cudaError_t ea = cudaGetDevice(&dev);
+  if (ea == cudaSuccess)
+    ea = smem.run(dev, cudaErrorInvalidDevice, [] {
+      const cudaError_t e = cudaFuncSetAttribute(
+          digit_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(32));
+      return e != cudaSuccess ? e
+                              : cudaFuncSetAttribute(digit_gemm_kernel<16>,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     (int)gemm_smem(16));
+    });
+  if (ea != cudaSuccess) return ea;
   // the 128-row operand P is the side that pads least; on a tie the columns of C, whose stores
   // are then contiguous across the lanes
   auto tiles = [](int a, int t) { return (long long)(a + t - 1) / t; };

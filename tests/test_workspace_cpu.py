@@ -1,5 +1,5 @@
-"""The library's host bookkeeping (csrc/workspace.h) on a device that is a counter: a workspace that
-cannot grow keeps what it had."""
+"""The library's host bookkeeping (csrc/workspace.h) on devices that are counters: a workspace that
+cannot grow keeps what it had; a kernel's shared-memory limit is raised once on every device."""
 import os
 import shutil
 import subprocess
@@ -78,6 +78,49 @@ int main() {
 '''
 
 
+ONCE = r'''
+#include "workspace.h"
+#include <atomic>
+#include <chrono>
+#include <cassert>
+#include <cstdio>
+#include <thread>
+#include <vector>
+enum Err { OK = 0, BROKEN = 9, BAD = 7 };
+int main() {
+  tdmrg::OncePerDevice once;
+  std::atomic<int> calls[3] = {{0}, {0}, {0}};
+  assert(once.run(0, BAD, [&] { ++calls[0]; return OK; }) == OK);
+  assert(once.run(0, BAD, [&] { ++calls[0]; return OK; }) == OK);
+  assert(calls[0] == 1);
+  // another device has its own, a failed one is tried again
+  assert(once.run(1, BAD, [&] { ++calls[1]; return BROKEN; }) == BROKEN);
+  assert(once.run(1, BAD, [&] { ++calls[1]; return OK; }) == OK);
+  assert(once.run(1, BAD, [&] { ++calls[1]; return BROKEN; }) == OK);
+  assert(calls[1] == 2);
+  assert(once.run(-1, BAD, [] { return OK; }) == BAD && once.run(64, BAD, [] { return OK; }) == BAD);
+  // several threads: nobody goes on before the one call is through
+  std::vector<std::thread> t;
+  std::atomic<bool> through{false};
+  std::atomic<int> early{0};
+  for (int i = 0; i < 8; ++i)
+    t.emplace_back([&] {
+      once.run(2, BAD, [&] {
+        ++calls[2];
+        std::this_thread::sleep_for(std::chrono::milliseconds(20));
+        through = true;
+        return OK;
+      });
+      if (!through) ++early;
+    });
+  for (auto& x : t) x.join();
+  assert(calls[2] == 1 && early == 0);
+  std::puts("ok");
+  return 0;
+}
+'''
+
+
 def compile_and_run(tmp_path, text, extra=()):
     cxx = shutil.which("g++") or shutil.which("c++")
     if not cxx:
@@ -92,6 +135,19 @@ def compile_and_run(tmp_path, text, extra=()):
 
 def test_a_workspace_that_cannot_grow_keeps_what_it_had(tmp_path):
     compile_and_run(tmp_path, GROW)
+
+
+def test_once_per_device(tmp_path):
+    compile_and_run(tmp_path, ONCE, ["-pthread"])
+
+
+def test_shared_memory_limits_are_raised_per_device():
+    """A limit raised with one flag for the process leaves the other devices without it."""
+    for f in ("zgemm_digits.cu", "qr_tensor.cu"):
+        with open(os.path.join(CSRC, f)) as fh:
+            text = fh.read()
+        assert "static bool attr" not in text, f
+        assert "static OncePerDevice" in text, f
 
 
 def test_the_engine_goes_on_without_the_workspace():
