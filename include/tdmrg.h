@@ -149,6 +149,11 @@ int tdmrg_model_set_profiling(tdmrg_model* h, int on);
 
 int tdmrg_model_destroy(tdmrg_model* h);
 
+/* Gives the memory that the library's pool keeps for later kernel-level calls (at most 512 MB a
+ * device) back to the device; for callers that hold no model, whose last one would do it.
+ * Synchronises the device. */
+int tdmrg_release_memory(void);
+
 /* Imaginary-time preparation of Psi_beta (Eq. 5): |I> restricted to the one-carrier sector,
  * bond dimensions M_k = min(M, prod of local dims on either side), right-canonicalised, then
  * round(beta / (2 dtau)) symmetric projector-splitting steps of exp(-dtau H), normalised
@@ -331,7 +336,7 @@ const char* tdmrg_last_global_error(void);
  * except where noted; each entry states whether it synchronises `stream`.  Complex FP64
  * contractions take a workspace (the digits of their operands) from a stream-ordered pool of
  * the library for the length of the call; the pool keeps at most 512 MB between calls and gives
- * it back when the last model is destroyed.  TDMRG_ERR_TIMEOUT if a bounded pipeline wait of a
+ * it back when the last model is destroyed or tdmrg_release_memory is called.  TDMRG_ERR_TIMEOUT if a bounded pipeline wait of a
  * contraction gave up.
  *
  * Accuracy of a complex FP64 contraction C = A B: each operand is rounded to 56 bits below the

@@ -41,6 +41,7 @@ _SIGS = {
     "tdmrg_model_set_krylov": [_p, _d, _i, _i],
     "tdmrg_model_set_stream": [_p, _p],
     "tdmrg_model_destroy": [_p],
+    "tdmrg_release_memory": [],
     "tdmrg_model_set_profiling": [_p, _i],
     "tdmrg_model_set_wait_cycles": [_p, ctypes.c_longlong],
     "tdmrg_model_set_concurrent": [_p, _i],
@@ -358,6 +359,11 @@ class Batch:
             self.close()
         except Exception:
             pass
+
+
+def release_memory():
+    """Give the memory that the kernel-level calls keep between them back to the device."""
+    _check(load().tdmrg_release_memory())
 
 
 def mobility(t_grid, C, kT):

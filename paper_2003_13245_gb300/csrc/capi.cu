@@ -490,6 +490,13 @@ int tdmrg_model_destroy(tdmrg_model* h) {
   return TDMRG_OK;
 }
 
+int tdmrg_release_memory(void) {
+  return guarded(nullptr, [] {
+    CK(cudaDeviceSynchronize());      // blocks given back on a stream are the pool's when it gets there
+    tdmrg::zg_pool_trim();
+  });
+}
+
 int tdmrg_thermal_prepare(tdmrg_model* h, double beta, double dtau, int M) {
   if (!h) return fail(nullptr, TDMRG_ERR_ARG, "NULL handle");
   return guarded(h, [&] { h->eng->thermal_prepare(beta, dtau, M); });
