@@ -510,6 +510,18 @@ int tdmrg_kernel_env_left(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int
                           const double* W_host, const void* L, const void* bra,
                           const void* ket, void* Lout, void* X, void* Y, void* stream);
 
+/* tdmrg_kernel_heff (TDMRG_PREC_C128) and tdmrg_kernel_env_left with at most work_bytes of workspace
+ * for the digits of the operands.  A product that needs more runs in slabs of its batches and
+ * rows; where one tile of each operand does not fit (0: always) it takes FP64 FMAs, whose error is
+ * relative to sum |a||b|. */
+int tdmrg_kernel_heff_work(int Ml, int Mr, int d, int Dl, int Dr, const double* W_host,
+                           const void* L, const void* R, const void* A, void* out, void* X, void* Y,
+                           long long work_bytes, void* stream);
+int tdmrg_kernel_env_left_work(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int Dr,
+                               const double* W_host, const void* L, const void* bra,
+                               const void* ket, void* Lout, void* X, void* Y, long long work_bytes,
+                               void* stream);
+
 /* Gauge QR of the shifts of Eq. S1: Y (m x n row-major, m >= n) = Q R with a deterministic
  * completion: accepted columns are Gram-Schmidt residuals (twice) above
  * 1e-12 ||Y||_F; skipped positions are filled from the columns of E (m x p row-major, may

@@ -74,6 +74,10 @@ _SIGS = {
     "tdmrg_reset_stats": [_p],
     "tdmrg_kernel_heff": [_i, _i, _i, _i, _i, _dp, _p, _p, _p, _p, _p, _p, _p, _i, _p],
     "tdmrg_kernel_env_left": [_i, _i, _i, _i, _i, _i, _i, _dp, _p, _p, _p, _p, _p, _p, _p],
+    "tdmrg_kernel_heff_work": [_i, _i, _i, _i, _i, _dp, _p, _p, _p, _p, _p, _p,
+                               ctypes.c_longlong, _p],
+    "tdmrg_kernel_env_left_work": [_i, _i, _i, _i, _i, _i, _i, _dp, _p, _p, _p, _p, _p, _p,
+                                   ctypes.c_longlong, _p],
     "tdmrg_kernel_gauge_qr": [_i, _i, _p, _i, _p, _p, _p, _p, _p],
     "tdmrg_kernel_krylov_dense": [_i, _p, _p, _p, _d, _d, _d, _i, _ip, _p],
     "tdmrg_kernel_bond_exp": [_i, _i, _p, _p, _p, _p, _d, _d, _d, _i, _ip, _p],
@@ -537,6 +541,17 @@ def kernel_heff(L, W, R, A, out, X, Y, d, precision=PREC_C128, ws32=None, stream
                                  _stream_ptr(stream)))
 
 
+def kernel_heff_work(L, W, R, A, out, X, Y, d, work_bytes, stream=None):
+    """kernel_heff in complex128 with at most work_bytes of digit workspace (0: FP64 FMAs)."""
+    lib = load()
+    Dl, Ml, _ = L.shape
+    Dr, Mr, _ = R.shape
+    Wc = np.ascontiguousarray(W, dtype=np.complex128).view(np.float64)
+    _check(lib.tdmrg_kernel_heff_work(Ml, Mr, d, Dl, Dr, _dptr(Wc), _ptr(L), _ptr(R), _ptr(A),
+                                      _ptr(out), _ptr(X), _ptr(Y), int(work_bytes),
+                                      _stream_ptr(stream)))
+
+
 def kernel_heff_timed(L, W, R, A, out, d, precision=PREC_C64_3XTF32, reps=20, stream=None):
     """Average milliseconds of the sweep's H_eff product (tdmrg_kernel_heff_timed)."""
     lib = load()
@@ -667,6 +682,19 @@ def kernel_env_left(L, W, bra, ket, Lout, X, Y, d, stream=None):
     _check(lib.tdmrg_kernel_env_left(Ml1, Mr1, Ml2, Mr2, d, Dl, Dr, _dptr(Wc), _ptr(L),
                                      _ptr(bra), _ptr(ket), _ptr(Lout), _ptr(X), _ptr(Y),
                                      _stream_ptr(stream)))
+
+
+def kernel_env_left_work(L, W, bra, ket, Lout, X, Y, d, work_bytes, stream=None):
+    """kernel_env_left with at most work_bytes of digit workspace (0: FP64 FMAs)."""
+    lib = load()
+    Dl = L.shape[0]
+    Dr = Lout.shape[0]
+    Ml1, _, Mr1 = bra.shape
+    Ml2, _, Mr2 = ket.shape
+    Wc = np.ascontiguousarray(W, dtype=np.complex128).view(np.float64)
+    _check(lib.tdmrg_kernel_env_left_work(Ml1, Mr1, Ml2, Mr2, d, Dl, Dr, _dptr(Wc), _ptr(L),
+                                          _ptr(bra), _ptr(ket), _ptr(Lout), _ptr(X), _ptr(Y),
+                                          int(work_bytes), _stream_ptr(stream)))
 
 
 def kernel_gauge_qr(Y, Q, R, E=None, status=None, stream=None):

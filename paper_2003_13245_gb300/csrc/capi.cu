@@ -115,8 +115,9 @@ tdmrg::MatRef mat(const void* p, long long rs, long long cs, long long sb = 0, l
 struct ZgHold {
   tdmrg::ZgWork w;
   cudaStream_t s;
-  explicit ZgHold(cudaStream_t st) : s(st) {
+  explicit ZgHold(cudaStream_t st, size_t limit = tdmrg::kZgMaxBytes) : s(st) {
     w.pooled = true;
+    w.limit = limit;
     CK(tdmrg::zg_pool_alloc(reinterpret_cast<void**>(&w.status), sizeof(int), s));
     CK(cudaMemsetAsync(w.status, 0, sizeof(int), s));
   }
@@ -781,6 +782,57 @@ long long tdmrg_heff_workspace_floats(int Ml, int Mr, int d, int Dl, int Dr) {
   return tdmrg::heff_tc_floats(Ml, Mr, d * d, Dl, Dr);
 }
 
+}  // extern "C"
+
+namespace {
+// most bytes of digits of an entry point's workspace, from a caller's limit (checked to be >= 0)
+size_t work_limit(long long work_bytes) {
+  return std::min((size_t)work_bytes, tdmrg::kZgMaxBytes);
+}
+
+void heff_c128(int Ml, int Mr, int d, int Dl, int Dr, const double* W_host, const void* L,
+               const void* R, const void* A, void* out, void* X, void* Y, size_t limit,
+               cudaStream_t s) {
+  TempMpo W(Dl, Dr, d, W_host, s);
+  ZgHold zg(s, limit);
+  tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y, &zg.w};
+  tdmrg::heff_f64(c, W.m.s[0], Ml, Mr, d * d, d, (const cplx*)L, (const cplx*)R, (const cplx*)A,
+                  (cplx*)out, nullptr);
+  zg.finish();
+}
+
+int env_left_c128(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int Dr, const double* W_host,
+                  const void* L, const void* bra, const void* ket, void* Lout, void* X, void* Y,
+                  long long work_bytes, void* stream) {
+  if (Ml1 < 1 || Mr1 < 1 || Ml2 < 1 || Mr2 < 1 || d < 1 || Dl < 1 || Dr < 1 || !W_host || !L ||
+      !bra || !ket || !Lout || !X || !Y || work_bytes < 0)
+    return fail(nullptr, TDMRG_ERR_ARG, "env_left: bad arguments");
+  return guarded(nullptr, [&] {
+    cudaStream_t s = (cudaStream_t)stream;
+    TempMpo W(Dl, Dr, d, W_host, s);
+    ZgHold zg(s, work_limit(work_bytes));
+    tdmrg::Ctx c{s, (cplx*)X, (cplx*)Y, &zg.w};
+    tdmrg::env_left_f64(c, W.m.s[0], Ml1, Mr1, Ml2, Mr2, d * d, d, (const cplx*)L,
+                        (const cplx*)bra, (const cplx*)ket, (cplx*)Lout);
+    zg.finish();
+  });
+}
+}  // namespace
+
+extern "C" {
+
+int tdmrg_kernel_heff_work(int Ml, int Mr, int d, int Dl, int Dr, const double* W_host,
+                           const void* L, const void* R, const void* A, void* out, void* X, void* Y,
+                           long long work_bytes, void* stream) {
+  if (Ml < 1 || Mr < 1 || d < 1 || Dl < 1 || Dr < 1 || !W_host || !L || !R || !A || !out || !X ||
+      !Y || work_bytes < 0)
+    return fail(nullptr, TDMRG_ERR_ARG, "heff: bad arguments");
+  return guarded(nullptr, [&] {
+    heff_c128(Ml, Mr, d, Dl, Dr, W_host, L, R, A, out, X, Y, work_limit(work_bytes),
+              (cudaStream_t)stream);
+  });
+}
+
 int tdmrg_kernel_heff(int Ml, int Mr, int d, int Dl, int Dr, const double* W_host, const void* L,
                       const void* R, const void* A, void* out, void* X, void* Y, void* ws32,
                       int precision, void* stream) {
@@ -793,15 +845,11 @@ int tdmrg_kernel_heff(int Ml, int Mr, int d, int Dl, int Dr, const double* W_hos
   if (precision != TDMRG_PREC_C128 && precision != TDMRG_PREC_C64_3XTF32)
     return fail(nullptr, TDMRG_ERR_ARG, "heff: unknown precision");
   return guarded(nullptr, [&] {
-    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
     cudaStream_t s = (cudaStream_t)stream;
     if (precision == TDMRG_PREC_C128) {
-      ZgHold zg(s);
-      tdmrg::Ctx c{s, (tdmrg::cplx*)X, (tdmrg::cplx*)Y, &zg.w};
-      tdmrg::heff_f64(c, W.m.s[0], Ml, Mr, d * d, d, (const tdmrg::cplx*)L,
-                      (const tdmrg::cplx*)R, (const tdmrg::cplx*)A, (tdmrg::cplx*)out, nullptr);
-      zg.finish();
+      heff_c128(Ml, Mr, d, Dl, Dr, W_host, L, R, A, out, X, Y, tdmrg::kZgMaxBytes, s);
     } else {
+      TempMpo W(Dl, Dr, d, W_host, s);
       DevBufs mem(s);
       int* st = (int*)mem.bytes(sizeof(int));
       CK(cudaMemsetAsync(st, 0, sizeof(int), s));
@@ -1063,17 +1111,16 @@ int tdmrg_kernel_zgemm_tc(int M, int N, int K, const void* A, const void* B, int
 int tdmrg_kernel_env_left(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int Dr,
                           const double* W_host, const void* L, const void* bra, const void* ket,
                           void* Lout, void* X, void* Y, void* stream) {
-  if (Ml1 < 1 || Mr1 < 1 || Ml2 < 1 || Mr2 < 1 || d < 1 || Dl < 1 || Dr < 1 || !W_host || !L ||
-      !bra || !ket || !Lout || !X || !Y)
-    return fail(nullptr, TDMRG_ERR_ARG, "env_left: bad arguments");
-  return guarded(nullptr, [&] {
-    TempMpo W(Dl, Dr, d, W_host, (cudaStream_t)stream);
-    ZgHold zg((cudaStream_t)stream);
-    tdmrg::Ctx c{(cudaStream_t)stream, (tdmrg::cplx*)X, (tdmrg::cplx*)Y, &zg.w};
-    tdmrg::env_left_f64(c, W.m.s[0], Ml1, Mr1, Ml2, Mr2, d * d, d, (const tdmrg::cplx*)L,
-                        (const tdmrg::cplx*)bra, (const tdmrg::cplx*)ket, (tdmrg::cplx*)Lout);
-    zg.finish();
-  });
+  return env_left_c128(Ml1, Mr1, Ml2, Mr2, d, Dl, Dr, W_host, L, bra, ket, Lout, X, Y,
+                       (long long)tdmrg::kZgMaxBytes, stream);
+}
+
+int tdmrg_kernel_env_left_work(int Ml1, int Mr1, int Ml2, int Mr2, int d, int Dl, int Dr,
+                               const double* W_host, const void* L, const void* bra,
+                               const void* ket, void* Lout, void* X, void* Y, long long work_bytes,
+                               void* stream) {
+  return env_left_c128(Ml1, Mr1, Ml2, Mr2, d, Dl, Dr, W_host, L, bra, ket, Lout, X, Y, work_bytes,
+                       stream);
 }
 
 int tdmrg_kernel_gauge_qr(int m, int n, const void* Y, int p, const void* E, void* Q, void* R,

@@ -60,18 +60,18 @@ struct MatRef {
 };
 
 // Workspace of the digit products of zgemm (zgemm_digits.cu) for calls on one stream at a time:
-// the digits of both operands and split-K partials.  It grows on demand up to kZgMaxBytes unless
-// `fixed` (captured graphs hold its address).  `pooled` workspaces live for one call of a
+// the digits of both operands and split-K partials.  It grows on demand up to `limit` unless
+// `fixed` (captured graphs hold its address); what does not fit runs in slabs.  `pooled` workspaces live for one call of a
 // kernel-level entry point and come from the library's stream-ordered pool; the others belong to
 // an engine.  *status (device) is set to 3 when a bounded pipeline wait gives up.
+constexpr size_t kZgMaxBytes = (size_t)2 << 30;
 struct ZgWork {
   void* p = nullptr;
-  size_t bytes = 0;
+  size_t bytes = 0, limit = kZgMaxBytes;
   int* status = nullptr;
   bool fixed = false, pooled = false;
 };
-constexpr size_t kZgMaxBytes = (size_t)2 << 30;
-// grows w to at least min(bytes, kZgMaxBytes) (contents lost); leaves it as it is when fixed.  Where
+// grows w to at least min(bytes, w.limit) (contents lost); leaves it as it is when fixed.  Where
 // memory runs out it keeps what it had, and the error is cudaErrorMemoryAllocation (cleared)
 cudaError_t zg_reserve(ZgWork& w, size_t bytes, cudaStream_t s);
 void zg_free(ZgWork& w, cudaStream_t s);

@@ -737,9 +737,10 @@ cudaError_t zg_pool_alloc(void** p, size_t bytes, cudaStream_t s) {
 }
 
 cudaError_t zg_reserve(ZgWork& w, size_t bytes, cudaStream_t s) {
-  if (bytes > kZgMaxBytes) bytes = kZgMaxBytes;
+  if (bytes > w.limit) bytes = w.limit;
   if (w.fixed || bytes <= w.bytes) return cudaSuccess;
   bytes = up(bytes + bytes / 8);      // room to grow without a new allocation
+  if (bytes > w.limit) bytes = w.limit;
   const bool pooled = w.pooled;
   const cudaError_t e = grow_block<cudaError_t>(
       w.p, w.bytes, bytes,
