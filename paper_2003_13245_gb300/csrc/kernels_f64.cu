@@ -190,14 +190,15 @@ cudaError_t zgemm(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef 
 // blockIdx.y is one output channel and level (wo, s), whose few nonzero entries are the same for
 // the whole block; the threads run over (a, t, b), contiguous in t and b.  Bound by the reads of X
 // (mostly from L2) and the write of Y; entries of 1 cost no FP64 instruction, real ones two.
-__global__ void __launch_bounds__(256) mpo_mix_kernel(int Ma, int d, int Mb, const int* start,
+// (wos0: the first (wo, s) of a launch)
+__global__ void __launch_bounds__(256) mpo_mix_kernel(int wos0, int Ma, int d, int Mb, const int* start,
                                                       const int2* cu, const cplx* val,
                                                       const cplx* X, long long xs, cplx* Y,
                                                       long long ys, const int* skip) {
   if (skip && *skip) return;
   const int dmb = d * Mb, ddmb = d * dmb;
-  const int wo = blockIdx.y / d, sig = blockIdx.y % d;
-  const int lo = start[blockIdx.y], hi = start[blockIdx.y + 1];
+  const int wos = wos0 + blockIdx.y, wo = wos / d, sig = wos % d;
+  const int lo = start[wos], hi = start[wos + 1];
   const int total = Ma * dmb;
   cplx* y = Y + wo * ys + (long long)sig * dmb;
   for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
@@ -209,16 +210,28 @@ __global__ void __launch_bounds__(256) mpo_mix_kernel(int Ma, int d, int Mb, con
 
 cudaError_t mpo_mix(const MixTable& T, int Ma, int d, int Mb, const cplx* X, long long xs,
                     cplx* Y, long long ys, const int* skip, cudaStream_t s) {
-  const long long total = (long long)Ma * d * Mb;
-  if (total <= 0 || T.Dout <= 0) return cudaSuccess;
-  if (total > 0x7fffffffLL - 256 * 152 * 32 || (long long)T.Dout * d > 65535)
-    return cudaErrorInvalidValue;
-  long long blocks = (total + 255) / 256;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  count_launch();
-  mpo_mix_kernel<<<dim3((unsigned)blocks, T.Dout * d), 256, 0, s>>>(Ma, d, Mb, T.sp_start, T.sp_cu,
-                                                                    T.sp_val, X, xs, Y, ys, skip);
-  return cudaGetLastError();
+  const long long row = (long long)d * Mb, wos = (long long)T.Dout * d;
+  if (Ma <= 0 || row <= 0 || wos <= 0) return cudaSuccess;
+  // the kernel counts (a, t, b) in 32 bits and (wo, s) along the grid's y: rows a and pairs (wo, s) in
+  // as many launches as that takes (one for anything but tensors of 2^31 entries a level)
+  constexpr long long most = 0x7fffffffLL - 256 * 152 * 32;
+  const long long rows = most / row;
+  if (rows < 1 || row * d > 0x7fffffffLL || wos > 0x7fffffffLL) return cudaErrorInvalidValue;
+  for (long long a0 = 0; a0 < Ma; a0 += rows) {
+    const int na = (int)(Ma - a0 < rows ? Ma - a0 : rows);
+    long long blocks = (na * row + 255) / 256;
+    if (blocks > 152 * 16) blocks = 152 * 16;
+    for (long long w0 = 0; w0 < wos; w0 += 65535) {
+      const unsigned nw = (unsigned)(wos - w0 < 65535 ? wos - w0 : 65535);
+      count_launch();
+      mpo_mix_kernel<<<dim3((unsigned)blocks, nw), 256, 0, s>>>(
+          (int)w0, na, d, Mb, T.sp_start, T.sp_cu, T.sp_val, X + a0 * row * d, xs, Y + a0 * row * d,
+          ys, skip);
+      const cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
 }
 
 // ------------------------------------------------------------------------------------

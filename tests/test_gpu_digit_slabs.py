@@ -93,3 +93,18 @@ def test_no_workspace_means_fmas():
     scale = np.abs(L[0]) @ np.abs(A[:, :, 0])
     err = np.abs(out.cpu().numpy()[:, :, 0] - L[0] @ A[:, :, 0])
     assert np.all(err <= 4 * m * 2.0 ** -53 * scale)     # two sums of 2 m rounded products
+
+
+def test_many_channels():
+    """More pairs of output channel and level than a grid has rows (65535)."""
+    from paper_2003_13245_gb300 import binding
+    rng = np.random.default_rng(4)
+    d, Dr = 2, 33000
+    L, R, A = ints(rng, (1, 1, 1)), ints(rng, (Dr, 1, 1)), ints(rng, (1, d, d, 1))
+    W = rng.integers(-2, 3, (1, Dr, d, d)) + 0j
+    ref = np.einsum("w,wvsu,ut,v->st", L[:, 0, 0], W, A[0, :, :, 0], R[:, 0, 0], optimize=True)
+    out = torch.zeros((1, d * d, 1), dtype=torch.complex128, device="cuda")
+    x = torch.zeros(Dr * d * d, dtype=torch.complex128, device="cuda")
+    binding.kernel_heff_work(dev(L), W, dev(R), dev(A.reshape(1, d * d, 1)), out, x,
+                             torch.zeros_like(x), d, 0)
+    assert np.array_equal(out.cpu().numpy()[0, :, 0], ref.reshape(-1))
