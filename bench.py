@@ -33,7 +33,7 @@ WORKLOAD = dict(name="holstein-N16-2mode-M128", N=16, omega=[0.2, 1.0], g=[1.5, 
 DIGIT_PRODUCTS = 34
 METRIC = "TDVP site-updates/s (real-time, both states, N=16 2-mode Holstein chain, M=128)"
 # DRAM bytes (read + write) of one 8192 x 128 gauge-QR launch, measured by ncu
-QR_BULK_TRAFFIC = 19006976 + 29809408
+QR_BULK_TRAFFIC = 19095296 + 29693696
 
 
 def parse():

@@ -152,16 +152,16 @@ cudaError_t zgemm_mixed(int m, int n, int k, int nbatch, int nred, MatRef A, Mat
 }
 
 // With a workspace every product of two or more terms goes to the digit products: measured on
-// GB300 they are faster from the smallest shapes (4 x 4 x 4: 10.4 against 20.6 us;
-// 64 x 64 x 256, 7 batches: 27 against 1049 us) to the largest (896 x 8192 x 128: 0.255 against
+// GB300 they are faster from the smallest shapes (4 x 4 x 4: 10.4 against 20.7 us;
+// 64 x 64 x 256, 7 batches: 26 against 1048 us) to the largest (896 x 8192 x 128: 0.290 against
 // 6.2 ms), and their error against 113-bit sums
 // is no larger where rows of A and columns of B are even or graded together along k, as in a sweep
 // (normal entries, K = 16: 6.1e-17 against 1.9e-16 relative, K = 128: 6.1e-17 against
 // 5.4e-16; entries graded over e^-28: 1.2e-16 against 2.2e-16 and 1.3e-16 against 8.0e-16).  Where one
 // rises as the other falls it is larger (zgemm_digits.cu has the bound and figures): such products
 // are called without a workspace.  A
-// single term (K = 1) is one rounding here and keeps the FMA kernel (16 x 16 8.9 against 10.8 us,
-// 1024 x 1024 22.7 against 27.0), as do callers without a
+// single term (K = 1) is one rounding here and keeps the FMA kernel (16 x 16 8.9 against 10.7 us,
+// 1024 x 1024 22.9 against 28.3), as do callers without a
 // workspace (dot products of the reverse pass).
 cudaError_t zgemm(int m, int n, int k, int nbatch, int nred, cplx alpha, MatRef A, MatRef B,
                   cplx beta, cplx* C, long long ldc, long long sc, const int* skip,

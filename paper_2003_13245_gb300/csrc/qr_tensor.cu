@@ -29,26 +29,31 @@
 // unit vectors); the first pass rejects every candidate in the span of the accepted columns at
 // once (residual^2 = ||e||^2 - |P|^2 <= 1e-4 ||e||^2), so 16 rejections cost one pass.
 //
-// Bound: latency.  A pass of a block takes ~25 us (two to four grid barriers of ~1.3 us, two
-// tensor-core products of 4-10 us, reading their levels back, the digits), the serial 16-column
-// factorisation ~16 us and the FP64 product V M 3-10 us; the FP64 work per column does not grow
-// with the number of accepted columns.
+// Bound: latency.  A block of 8192 x 128 takes ~165 us: two to four grid barriers of ~1.3 us a pass,
+// two tensor-core products a pass (64 instructions a k step, the ring's copies from L2), reading their
+// levels back, the digits, the serial 16-column factorisation (~16 us) and the FP64 product V M
+// (3-10 us); the FP64 work per column does not grow with the number of accepted columns.
 //
 // Measured on GB300 against qr_blocked.cu (FP64 FMAs), us.  "parallel": random columns, nearly
-// parallel; "graded": singular values from 1 to e^-9, mixed, for which the same kernel with one round
-// (a restart below a quarter) stands in the middle; "rank 2": all but two columns are completed from
-// 7 n candidates of which n lie in the span:
-//   m x n        parallel         graded                 rank 2
-//   64 x 16        98 /   69       257 / 449 /   71
-//   256 x 32      172 /  177       355 / 641 /  179       1549 /  295
-//   1024 x 64     387 /  399       707 / 914 /  407
-//   256 x 128     827 /  915      1032 / 1150 /  912      7537 / 1174
-//   1024 x 128    944 /  908      1175 / 1183 / 1017
-//   8192 x 128   2685 / 1093      3911 / 1454 / 1114     19468 / 1535
-//   8192 x 128 on 76 CTAs (two lanes)  6742 / 1377 (graded) and 25148 / 1796 (rank 2)
-// Below nine columns the other kernel is the faster one at full rank (256 x 4: 55 against 95 us),
-// where such bonds, at the ends of a chain, mostly are.  About 32 rows per CTA: fewer rows raise the
-// number of partial sums, more the FP64 product V M.
+// parallel; "graded": singular values from 1 to e^-9, mixed; "rank 2": all but two columns are
+// completed from 7 n candidates of which n lie in the span:
+//   m x n        parallel       graded         rank 2
+//   64 x 16        87 /   74     257 /   77     676 /  177
+//   256 x 32      161 /  194     358 /  198    1546 /  326
+//   1024 x 64     336 /  429     706 /  460    3702 /  615
+//   256 x 128     803 / 1056    1028 / 1064    7546 / 1362
+//   1024 x 128    871 / 1032    1174 / 1193    9628 / 1392
+//   2048 x 128   1062 / 1002    1523 / 1057   12481 / 1392
+//   8192 x 128   2360 / 1164    3912 / 1330   19450 / 1706
+//   8192 x 128 on 76 CTAs (two lanes)  3949 / 1442 (parallel), 6746 / 1644, 25157 / 2204
+// The rule goes by size alone, since neither the grading nor the rank is known before the call.  What a
+// sweep brings is graded or rank deficient (center matrices of truncated chains): there this kernel is
+// at par for 128 columns of few rows and faster elsewhere; columns that are nearly parallel and few
+// rows (0.76-0.84 of the FMA kernel's speed) are the price.  Below nine columns the other kernel is the
+// faster one at full rank (256 x 4: 55 against 95 us), where such bonds, at the ends of a chain,
+// mostly are.  About 32 rows per CTA: fewer rows raise the number of partial sums, more the FP64
+// product V M.  With the digit pairs of all levels in 28 instructions of different width on shared
+// columns (an order that is not promised) 8192 x 128 took 1114 (graded).
 #include "umma.cuh"
 #include "workspace.h"
 

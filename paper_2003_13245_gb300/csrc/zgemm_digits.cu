@@ -36,16 +36,18 @@
 // by e^28: 7e-17 against 1e-15).  Products whose operands are so by their nature, as R and its
 // cotangent, take the FMA kernel (capi.cu, QR reverse passes).
 //
-// Bound: the tensor pipe in the main loop (28 instructions, ~2300 clocks per k step of 128 x 32),
-// plus the integer epilogue, which cannot overlap it (eight re and im levels of 32 columns fill all
-// 512 TMEM columns).  72 KB per stage from L2, three stages, one CTA per SM.  A small product is
-// latency: a launch each for split, product and reduction, set up while the one before runs, half
-// the instructions' time with 16-column tiles.
+// Bound: the tensor pipe in the main loop (48 instructions per k step of 128 x 32; narrow ones wait for
+// the 4 KB of A that each reads), plus the integer epilogue, which cannot overlap it (eight re and im
+// levels of 32 columns fill all 512 TMEM columns).  70 KB per stage from L2, three stages, one CTA per
+// SM.  A small product is latency: a launch each for split, product and reduction, set up while the one
+// before runs.
 //
-// Measured on GB300 against the FMA kernel, split and reduction included: 896 x 8192 x 128 0.255
-// against 6.2 ms (29 TFLOP/s, tensor pipe 39 %); 8192 x 128 x 128 summed over seven channels 0.310
-// against 7.3 ms; 128 x 128 x 8192, seven batches, 0.486 against 34 ms; 64 x 64 x 256, seven
-// batches, 27 against 1049 us (32 with tiles of 32); 16 x 16 x 4 11 against 21 us (15).
+// Measured on GB300 against the FMA kernel, split and reduction included: 896 x 8192 x 128 0.290
+// against 6.2 ms (26 TFLOP/s, tensor pipe 46 %); 8192 x 128 x 128 summed over seven channels 0.342
+// against 7.3 ms; 128 x 128 x 8192, seven batches, 0.531 against 34 ms; 64 x 64 x 256, seven
+// batches, 26 against 1049 us; 16 x 16 x 4 11 against 21 us.  With the digit pairs of all levels in
+// instructions of different width on shared columns (28 a k step, an order that is not promised) the
+// first three took 0.255, 0.310 and 0.486 ms.
 #include "mix.cuh"
 #include "umma.cuh"
 #include "workspace.h"
@@ -502,13 +504,15 @@ Plan plan_of(int k, int nred, int qt = 32) {
 }  // namespace
 
 namespace {
+constexpr int SMS = 152;                      // of this chip
 // Most CTAs with 16-column tiles: one per SM.  They read the 128-row operand twice as often, which
 // L2 has room for as long as they run side by side; a second wave would cost more than the shorter
-// main loop gives.  448 x 256 x 64 (64 CTAs) 15.0 against 20.1 us, 128 x 128 x 128 19.5 against 25.2.
-constexpr int NARROW = 152;
-// splits of the chunk loop that fill the GPU when there are few tiles
+// main loop gives.  448 x 256 x 64 (64 CTAs) 15 against 21 us, 128 x 128 x 128 19 against 27.
+constexpr int NARROW = SMS;
+// Splits of the chunk loop that fill the GPU when there are few tiles: as many CTAs as leave at most
+// four SMs idle where a whole number of splits does (50 tiles take three, 150 CTAs, and not four)
 int splits_of(long long ntile, int chunks) {
-  const long long ks = (148 + ntile - 1) / ntile;
+  const long long ks = (SMS - 4 + ntile - 1) / ntile;
   return (int)(ks < chunks ? ks : chunks);
 }
 }  // namespace
