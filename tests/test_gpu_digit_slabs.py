@@ -108,3 +108,26 @@ def test_many_channels():
     binding.kernel_heff_work(dev(L), W, dev(R), dev(A.reshape(1, d * d, 1)), out, x,
                              torch.zeros_like(x), d, 0)
     assert np.array_equal(out.cpu().numpy()[0, :, 0], ref.reshape(-1))
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, complex(0.0, np.inf)])
+@pytest.mark.parametrize("where", ["L", "A", "R"])
+def test_nonfinite_entries_as_with_fmas(where, bad):
+    """An Inf or NaN of an operand reaches the same entries on both routes, and as NaN on both: the FMA
+    sums of a complex product mix re and im, and alpha = 1 + 0 i multiplies both parts."""
+    from paper_2003_13245_gb300 import binding
+    rng = np.random.default_rng(5)
+    m, n, d = 140, 30, 2
+    ops = {"L": ints(rng, (1, m, m)), "R": ints(rng, (1, n, n)), "A": ints(rng, (m, d * d, n))}
+    ops[where][(0, 7, 3) if where != "A" else (131, 2, 7)] = bad
+    W = np.eye(d).reshape(1, 1, d, d) + 0j
+    got = []
+    for work in (0, 1 << 30):
+        out = torch.zeros((m, d * d, n), dtype=torch.complex128, device="cuda")
+        x = torch.zeros(ops["A"].size, dtype=torch.complex128, device="cuda")
+        binding.kernel_heff_work(dev(ops["L"]), W, dev(ops["R"]), dev(ops["A"]), out, x,
+                                 torch.zeros_like(x), d, work)
+        got.append(out.cpu().numpy())
+    assert not np.isfinite(got[0]).all()
+    for part in (np.real, np.imag):
+        assert np.array_equal(part(got[0]), part(got[1]), equal_nan=True)
